@@ -1,11 +1,10 @@
 // Similarity-based merging (Sec. 3.2.2; Algorithm 1, the loop over V_merge and
-// the removal of the merged positions), everything except the tensor-core
-// similarity kernel:
+// the removal of the merged positions), everything except the similarity itself
+// (gemm_tc.cu; proj_simt.cu for fp32 storage):
 //
 //   prepare   slot of every visual token in the kept list (-1 = pruned), 1/|h| of
 //             every visual row, and a packed copy of the kept rows (the second
 //             operand of the similarity)
-//   sim_simt  cosine + arg-max on CUDA cores (fp32 storage, debugging aid)
 //   finish    destination slots, per-slot member lists, aggregation in a fixed
 //             order and compaction into the shortened sequence
 //
@@ -107,56 +106,6 @@ prepare_rows_kernel(const T* __restrict__ hidden, const int32_t* __restrict__ cu
     assign[g] = slot;
     best[g] = 0ull;
     if (slot >= 0) inv_norm_kept[k0 + slot] = inv;
-  }
-}
-
-// ---------------------------------------------------------------- similarity on CUDA cores
-// one block per pruned row; warp w scores slots w, w+8, ...
-template <typename T>
-__global__ void __launch_bounds__(256)
-sim_simt_kernel(const T* __restrict__ hidden, const T* __restrict__ kept_rows,
-                const int32_t* __restrict__ cu_seqlens, const int32_t* __restrict__ cu_vis,
-                const int32_t* __restrict__ cu_kept, const int32_t* __restrict__ assign,
-                const float* __restrict__ inv_norm, const float* __restrict__ inv_norm_kept,
-                int D, int max_kept, unsigned long long* __restrict__ best, float* __restrict__ sim_debug) {
-  constexpr int kVec = Storage<T>::kVec;
-  grid_dependency_enter();
-  const int b = blockIdx.y, m = blockIdx.x;
-  const int v0 = cu_vis[b];
-  if (m >= cu_vis[b + 1] - v0) return;
-  const int g = v0 + m;
-  if (assign[g] >= 0) return;                      // kept token
-  const int k0 = cu_kept[b], kb = cu_kept[b + 1] - k0;
-  const T* hm = hidden + (size_t)(cu_seqlens[b] + m) * D;
-  const float inm = inv_norm[g];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  unsigned long long mine = 0ull;
-  for (int s = warp; s < kb; s += 8) {
-    const T* hk = kept_rows + (size_t)(k0 + s) * D;
-    float acc = 0.f;
-    for (int c = lane * kVec; c < D; c += 32 * kVec) {
-      float x[kVec], y[kVec];
-      Storage<T>::load(hm + c, x);
-      Storage<T>::load(hk + c, y);
-#pragma unroll
-      for (int i = 0; i < kVec; ++i) acc = fmaf(x[i], y[i], acc);
-    }
-    acc = warp_sum(acc);
-    const float sim = (acc * inm) * inv_norm_kept[k0 + s] + 0.0f;   // the value the arg-max compares (never -0)
-    if (lane == 0) {
-      const unsigned long long packed = ((unsigned long long)ordered_key(sim) << 32) | (0xffffffffu - (unsigned)s);
-      mine = packed > mine ? packed : mine;
-      if (sim_debug != nullptr) sim_debug[(size_t)g * max_kept + s] = sim;
-    }
-  }
-  __shared__ unsigned long long red[8];
-  if (lane == 0) red[warp] = mine;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned long long r = red[0];
-#pragma unroll
-    for (int w = 1; w < 8; ++w) r = red[w] > r ? red[w] : r;
-    best[g] = r;
   }
 }
 
@@ -512,22 +461,6 @@ int launch_merge_prepare(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
                                           static_cast<const __nv_bfloat16*>(a.hidden), a.cu_seqlens, a.cu_vis,
                                           a.kept_idx, a.cu_kept, a.D, a.assign, ctx->best, ctx->inv_norm,
                                           ctx->inv_norm_kept, static_cast<__nv_bfloat16*>(ctx->kept_rows), ctx->n_heavy));
-  return D3TOM_OK;
-}
-
-int launch_sim_simt(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
-  dim3 grid(a.max_visual, a.B);
-  if (a.dt == D3TOM_FP32)
-    D3TOM_CUDA_TRY(ctx, launch_serialized(sim_simt_kernel<float>, grid, 256, 0, s, static_cast<const float*>(a.hidden),
-                                          static_cast<const float*>(ctx->kept_rows), a.cu_seqlens, a.cu_vis, a.cu_kept,
-                                          a.assign, ctx->inv_norm, ctx->inv_norm_kept, a.D, a.max_kept, ctx->best,
-                                          a.sim_debug));
-  else
-    D3TOM_CUDA_TRY(ctx, launch_serialized(sim_simt_kernel<__nv_bfloat16>, grid, 256, 0, s,
-                                          static_cast<const __nv_bfloat16*>(a.hidden),
-                                          static_cast<const __nv_bfloat16*>(ctx->kept_rows), a.cu_seqlens, a.cu_vis,
-                                          a.cu_kept, a.assign, ctx->inv_norm, ctx->inv_norm_kept, a.D, a.max_kept,
-                                          ctx->best, a.sim_debug));
   return D3TOM_OK;
 }
 

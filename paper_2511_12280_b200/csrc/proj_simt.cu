@@ -1,105 +1,269 @@
-// Q,K,V projection and the other dense layers of a block on CUDA cores (Sec. 3.2.1,
-// Q = H W_Q, K = H W_K; Algorithm 1, FFN_l): the fp32 storage path and a debugging aid for bf16.  C[n, 3D] = X[n, D] * W[3D, D]^T,
-// fp32 accumulation, 32x32 output tile per block staged through shared memory.
+// "NT" matrix products on CUDA cores, C[m, n] = sum_k A[m, k] B[n, k] with fp32 arithmetic: the fp32 storage path (and,
+// for bf16, a debugging aid) of the dense layers (Sec. 3.2.1, Q = H W_Q, K = H W_K; Algorithm 1, FFN_l) and of the
+// similarity with its arg-max (Sec. 3.2.2).
+//
+// A CTA of 8 warps computes a (16 WM) x (32 WN) tile; WK warps share a 16 x 32 register tile (f32_tile.cuh) and cut
+// every k-block of 32 WK between them, so that small products, which have few tiles, keep short chains.  k-blocks come
+// through a ring of kStages buffers by 16-byte asynchronous copies.  Bound: the fp32 pipe and shared memory (a lane reads
+// 8 vectors per 64 multiply-adds): 42 TFLOP/s at 1152 x 12288 x 4096, 30 at 384 x 1536 x 512 (20 us; one output per
+// thread and two shared-memory reads per multiply-add took 83).
 #include "common.cuh"
+#include "f32_tile.cuh"
 
 namespace {
 
-template <typename T>
-__global__ void __launch_bounds__(1024)
-proj_simt_kernel(const T* __restrict__ x, const T* __restrict__ w, int n, int D,
-                 T* __restrict__ q, T* __restrict__ k, T* __restrict__ v) {
-  __shared__ float xs[32][33];
-  __shared__ float ws[32][33];
-  grid_dependency_enter();
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int row = blockIdx.y * 32 + ty;       // token
-  const int col = blockIdx.x * 32 + tx;       // output feature in [0, 3D)
-  float acc = 0.f;
-  for (int c0 = 0; c0 < D; c0 += 32) {
-    const int xr = blockIdx.y * 32 + ty, wr = blockIdx.x * 32 + ty;
-    xs[ty][tx] = (xr < n && c0 + tx < D) ? Storage<T>::to_float(x[(size_t)xr * D + c0 + tx]) : 0.f;
-    ws[ty][tx] = (wr < 3 * D && c0 + tx < D) ? Storage<T>::to_float(w[(size_t)wr * D + c0 + tx]) : 0.f;
-    __syncthreads();
-#pragma unroll
-    for (int c = 0; c < 32; ++c) acc = fmaf(xs[ty][c], ws[tx][c], acc);
-    __syncthreads();
-  }
-  if (row < n && col < 3 * D) {
-    T* dst = col < D ? q : (col < 2 * D ? k : v);
-    dst[(size_t)row * D + (col % D)] = Storage<T>::from_float(acc);
-  }
-}
+constexpr int kStages = 3;
+enum { kSimtProj = 0, kSimtLinear = 1, kSimtGateUp = 2, kSimtSim = 3 };
 
-// y[n, N] = residual + x[n, K] w[N, K]^T (kGateUp == false), or the first half of the gated feed-forward network,
-// act[n, m] = silu(x Wg^T) * (x Wu^T) with w = [Wg; Wu] of 2m rows (kGateUp == true, N = m): Algorithm 1, FFN_l.
-template <typename T, bool kGateUp>
-__global__ void __launch_bounds__(1024)
-linear_simt_kernel(const T* __restrict__ x, const T* __restrict__ w, const T* residual, int n, int K, int N, T* out) {
-  __shared__ float xs[32][33];
-  __shared__ float ws[32][33];
-  __shared__ float us[kGateUp ? 32 : 1][33];
+template <typename T> struct SimtGemm {
+  const T* a; const T* b;          // A rows of the products, B rows (for the gate-up pass: gate rows, then the up rows from row n_cols on)
+  int rows, n_cols, K;             // (similarity: the bounds over all requests)
+  bool vec;                        // 16-byte copies are possible
+  T* out[3];                       // projection: q, k, v; otherwise out[0]
+  const T* residual;
+  int D;                           // projection: columns of one output
+  // similarity
+  const int32_t* cu_seqlens; const int32_t* cu_vis; const int32_t* cu_kept; const int32_t* assign;
+  const float* inv_norm; const float* inv_norm_kept; int max_kept;
+  unsigned long long* best; float* sim_debug;
+};
+
+template <int EPI, int WM, int WN, int WK> struct SimtGemmSmem {
+  static constexpr int kBM = 16 * WM, kBN = 32 * WN, kBK = 32 * WK, kLd = kBK + 4;
+  static constexpr int kB = kBN * (EPI == kSimtGateUp ? 2 : 1);
+  static constexpr int kStage = (kBM + kB) * kLd;        // floats
+  static constexpr int kBytes = kStages * kStage * 4;
+  static_assert(WM * WN * WK == 8, "eight warps");
+  static_assert(kStages * kStage >= (WK - 1) * kBM * kB, "the slices' sums are exchanged in the ring");
+};
+
+template <typename T, int EPI, int WM, int WN, int WK>
+__global__ void __launch_bounds__(256, 1)
+gemm_simt_kernel(SimtGemm<T> p) {
+  using S = SimtGemmSmem<EPI, WM, WN, WK>;
+  constexpr int kLd = S::kLd, kMats = EPI == kSimtGateUp ? 2 : 1;
+  extern __shared__ float4 smem_f4[];
+  float* ring = reinterpret_cast<float*>(smem_f4);
   grid_dependency_enter();
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int row = blockIdx.y * 32 + ty;
-  const int col = blockIdx.x * 32 + tx;
-  float acc = 0.f, acc_u = 0.f;
-  for (int c0 = 0; c0 < K; c0 += 32) {
-    const int wr = blockIdx.x * 32 + ty;
-    const bool in_k = c0 + tx < K;
-    xs[ty][tx] = (row < n && in_k) ? Storage<T>::to_float(x[(size_t)row * K + c0 + tx]) : 0.f;
-    ws[ty][tx] = (wr < N && in_k) ? Storage<T>::to_float(w[(size_t)wr * K + c0 + tx]) : 0.f;
-    if (kGateUp) us[ty][tx] = (wr < N && in_k) ? Storage<T>::to_float(w[(size_t)(N + wr) * K + c0 + tx]) : 0.f;
-    __syncthreads();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = f32::lane_ty(lane), tx = f32::lane_tx(lane);
+  const int wk = warp % WK, wn = (warp / WK) % WN, wm = warp / (WK * WN);
+  const int m0 = blockIdx.y * S::kBM, n0 = blockIdx.x * S::kBN;
+  int rows = p.rows, cols = p.n_cols, v0 = 0, k0 = 0;
+  const T* a = p.a;
+  const T* b = p.b;
+  if (EPI == kSimtSim) {
+    const int rq = blockIdx.z;
+    v0 = p.cu_vis[rq]; rows = p.cu_vis[rq + 1] - v0;
+    k0 = p.cu_kept[rq]; cols = p.cu_kept[rq + 1] - k0;
+    if (cols >= rows || m0 >= rows || n0 >= cols) return;      // nothing pruned in this request, or outside it
+    a += (size_t)p.cu_seqlens[rq] * p.K;
+    b += (size_t)k0 * p.K;
+  }
+  const int nkb = (p.K + S::kBK - 1) / S::kBK;
+  // this thread's vectors of every k-block: the same column of rows lrow, lrow + kStep, ... of the A and B tiles
+  constexpr int kV = S::kBK / 4, kStep = 256 / kV, kLoads = (S::kBM + S::kB) / kStep;
+  static_assert((S::kBM + S::kB) % kStep == 0, "every thread loads the same number of vectors");
+  const int lrow = tid / kV, lcol = (tid % kV) * 4;
+  const T* src[kLoads];
+  unsigned src_ok = 0u;
 #pragma unroll
-    for (int c = 0; c < 32; ++c) {
-      acc = fmaf(xs[ty][c], ws[tx][c], acc);
-      if (kGateUp) acc_u = fmaf(xs[ty][c], us[tx][c], acc_u);
+  for (int u = 0; u < kLoads; ++u) {
+    const int r = lrow + u * kStep;
+    bool ok;
+    if (r < S::kBM) {
+      ok = m0 + r < rows;
+      src[u] = a + (size_t)(ok ? m0 + r : 0) * p.K;
+    } else {
+      const int rb = r - S::kBM, mat = rb / S::kBN, col = n0 + rb - mat * S::kBN;
+      ok = col < cols;
+      src[u] = b + (size_t)(ok ? mat * cols + col : 0) * p.K;
+    }
+    src_ok |= (ok ? 1u : 0u) << u;
+  }
+  auto load_block = [&](int kb) {
+    if (kb < nkb) {
+      float* dst = ring + (kb % kStages) * S::kStage + lrow * kLd + lcol;
+      const int c = kb * S::kBK + lcol;
+#pragma unroll
+      for (int u = 0; u < kLoads; ++u) f32::load4<T>(dst + u * kStep * kLd, src[u], c, p.K, (src_ok >> u) & 1u, p.vec);
+    }
+    f32::cp_async_commit();
+  };
+  float2 acc[kMats][4][4];
+#pragma unroll
+  for (int t = 0; t < kMats; ++t)
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[t][r][j] = make_float2(0.f, 0.f);
+  for (int kb = 0; kb < kStages - 1; ++kb) load_block(kb);
+  for (int kb = 0; kb < nkb; ++kb) {
+    f32::cp_async_wait<kStages - 2>();
+    __syncthreads();                       // block kb is there for everyone, and everyone is done with block kb - 1
+    load_block(kb + kStages - 1);
+    const float* st = ring + (kb % kStages) * S::kStage;
+    const float* aw = st + wm * 16 * kLd + wk * 32;
+    const float* bw = st + (S::kBM + wn * 32) * kLd + wk * 32;
+#pragma unroll
+    for (int t = 0; t < kMats; ++t) f32::dot_16x32<kLd, kLd, 8>(acc[t], aw, bw + t * S::kBN * kLd, ty, tx);
+  }
+  float c[kMats][4][4];
+#pragma unroll
+  for (int t = 0; t < kMats; ++t)
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) c[t][r][j] = acc[t][r][j].x + acc[t][r][j].y;
+  if (WK > 1) {
+    // the WK slices of a register tile meet in shared memory and are added in slice order by the first
+    f32::cp_async_wait<0>();
+    __syncthreads();
+    constexpr int kTile = kMats * 16 * 32;
+    float* mine = ring + ((wm * WN + wn) * (WK - 1) + (wk - 1)) * kTile;
+    if (wk > 0) {
+#pragma unroll
+      for (int t = 0; t < kMats; ++t)
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) mine[((t * 4 + r) * 4 + j) * 32 + lane] = c[t][r][j];
     }
     __syncthreads();
+    if (wk > 0) return;
+    for (int q = 0; q < WK - 1; ++q) {
+      const float* other = ring + ((wm * WN + wn) * (WK - 1) + q) * kTile;
+#pragma unroll
+      for (int t = 0; t < kMats; ++t)
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) c[t][r][j] += other[((t * 4 + r) * 4 + j) * 32 + lane];
+    }
   }
-  if (row < n && col < N) {
-    const size_t o = (size_t)row * N + col;
-    if (kGateUp) out[o] = Storage<T>::from_float(acc / (1.f + expf(-acc)) * acc_u);
-    else out[o] = Storage<T>::from_float(residual != nullptr ? acc + Storage<T>::to_float(residual[o]) : acc);
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int row = m0 + wm * 16 + ty + 4 * r;
+    if (EPI == kSimtSim) {
+      const int g = v0 + row;
+      const bool active = row < rows && p.assign[g] < 0;       // a pruned token
+      const float inm = active ? p.inv_norm[g] : 0.f;
+      unsigned long long mine = 0ull;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int s = n0 + wn * 32 + tx + 8 * j;
+        if (active && s < cols) {
+          const float sim = (c[0][r][j] * inm) * p.inv_norm_kept[k0 + s] + 0.0f;   // the value the arg-max compares (never -0)
+          const unsigned long long packed = ((unsigned long long)ordered_key(sim) << 32) | (0xffffffffu - (unsigned)s);
+          mine = packed > mine ? packed : mine;
+          if (p.sim_debug != nullptr) p.sim_debug[(size_t)g * p.max_kept + s] = sim;
+        }
+      }
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 2) {
+        const unsigned long long o = __shfl_xor_sync(0xffffffffu, mine, d);
+        mine = o > mine ? o : mine;
+      }
+      if (tx == 0 && mine != 0ull) atomicMax(p.best + g, mine);
+    } else if (row < rows) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int col = n0 + wn * 32 + tx + 8 * j;
+        if (col >= cols) continue;
+        if (EPI == kSimtProj) {
+          const int which = col / p.D;
+          p.out[which][(size_t)row * p.D + (col - which * p.D)] = Storage<T>::from_float(c[0][r][j]);
+        } else {
+          const size_t o = (size_t)row * cols + col;
+          float y = c[0][r][j];
+          if (EPI == kSimtGateUp) y = y / (1.f + expf(-y)) * c[kMats - 1][r][j];
+          else if (p.residual != nullptr) y += Storage<T>::to_float(p.residual[o]);
+          p.out[0][o] = Storage<T>::from_float(y);
+        }
+      }
+    }
   }
 }
 
-template <typename T, bool kGateUp>
-int launch_linear_simt_t(d3tom_ctx* ctx, const void* x, const void* w, const void* residual, int rows, int K, int N,
-                         void* out, cudaStream_t s) {
-  dim3 grid(ceil_div(N, 32), ceil_div(rows, 32));
-  D3TOM_CUDA_TRY(ctx, launch_serialized(linear_simt_kernel<T, kGateUp>, grid, 1024, 0, s, static_cast<const T*>(x),
-                                        static_cast<const T*>(w), static_cast<const T*>(residual), rows, K, N,
-                                        static_cast<T*>(out)));
+template <typename T, int EPI, int WM, int WN, int WK>
+int launch_shape(d3tom_ctx* ctx, const SimtGemm<T>& p, int batch, cudaStream_t s) {
+  using S = SimtGemmSmem<EPI, WM, WN, WK>;
+  dim3 grid(ceil_div(p.n_cols, S::kBN), ceil_div(p.rows, S::kBM), batch);
+  // (the attribute belongs to the current device: set on every call, a process may drive several GPUs)
+  D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(gemm_simt_kernel<T, EPI, WM, WN, WK>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kBytes));
+  D3TOM_CUDA_TRY(ctx, launch_serialized(gemm_simt_kernel<T, EPI, WM, WN, WK>, grid, 256, S::kBytes, s, p));
   return D3TOM_OK;
+}
+
+// Tile shape: the fewest rounds over the SMs weighted by the tile's area and by what a finer tile costs per element (its
+// operands are read more often: measured 1.5 for 32 x 32 at 640 x 1536 x 512), so that only a product with few 64 x 64
+// tiles is cut finer, its k-blocks shared by two or four warps.
+template <typename T, int EPI>
+int launch_simt_gemm(d3tom_ctx* ctx, SimtGemm<T> p, int batch, cudaStream_t s) {
+  if (p.rows <= 0 || p.n_cols <= 0) return D3TOM_OK;
+  const uintptr_t bits = (uintptr_t)p.a | (uintptr_t)p.b;
+  p.vec = sizeof(T) == 4 && p.K % 4 == 0 && bits % 16 == 0;
+  const long long sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
+  auto cost = [&](int bm, int bn, double scale) {
+    const long long tiles = (long long)ceil_div(p.rows, bm) * ceil_div(p.n_cols, bn) * batch;
+    return scale * (double)((tiles + sms - 1) / sms) * bm * bn;
+  };
+  const double large = cost(64, 64, 1.0), middle = cost(32, 64, 1.2), small = cost(32, 32, 1.5);
+  if (large <= middle && large <= small) return launch_shape<T, EPI, 4, 2, 1>(ctx, p, batch, s);
+  if (middle <= small) return launch_shape<T, EPI, 2, 2, 2>(ctx, p, batch, s);
+  return launch_shape<T, EPI, 2, 1, 4>(ctx, p, batch, s);
+}
+
+template <typename T>
+int proj_t(d3tom_ctx* ctx, const void* x, const void* w, int total, int D, void* q, void* k, void* v, cudaStream_t s) {
+  SimtGemm<T> p = {};
+  p.a = static_cast<const T*>(x); p.b = static_cast<const T*>(w);
+  p.rows = total; p.n_cols = 3 * D; p.K = D; p.D = D;
+  p.out[0] = static_cast<T*>(q); p.out[1] = static_cast<T*>(k); p.out[2] = static_cast<T*>(v);
+  return launch_simt_gemm<T, kSimtProj>(ctx, p, 1, s);
+}
+
+template <typename T, int EPI>
+int linear_t(d3tom_ctx* ctx, const void* x, const void* w, const void* residual, int rows, int K, int N, void* out,
+             cudaStream_t s) {
+  SimtGemm<T> p = {};
+  p.a = static_cast<const T*>(x); p.b = static_cast<const T*>(w);
+  p.rows = rows; p.n_cols = N; p.K = K;
+  p.residual = static_cast<const T*>(residual); p.out[0] = static_cast<T*>(out);
+  return launch_simt_gemm<T, EPI>(ctx, p, 1, s);
+}
+
+template <typename T>
+int sim_t(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
+  SimtGemm<T> p = {};
+  p.a = static_cast<const T*>(a.hidden); p.b = static_cast<const T*>(ctx->kept_rows);
+  p.rows = a.max_visual; p.n_cols = a.max_kept; p.K = a.D;
+  p.cu_seqlens = a.cu_seqlens; p.cu_vis = a.cu_vis; p.cu_kept = a.cu_kept; p.assign = a.assign;
+  p.inv_norm = ctx->inv_norm; p.inv_norm_kept = ctx->inv_norm_kept; p.max_kept = a.max_kept;
+  p.best = ctx->best; p.sim_debug = a.sim_debug;
+  return launch_simt_gemm<T, kSimtSim>(ctx, p, a.B, s);
 }
 
 }  // namespace
 
 int launch_linear_simt(d3tom_ctx* ctx, d3tom_dtype dt, const void* x, const void* w, const void* residual, int rows,
                        int K, int N, void* out, cudaStream_t s) {
-  if (dt == D3TOM_FP32) return launch_linear_simt_t<float, false>(ctx, x, w, residual, rows, K, N, out, s);
-  return launch_linear_simt_t<__nv_bfloat16, false>(ctx, x, w, residual, rows, K, N, out, s);
+  if (dt == D3TOM_FP32) return linear_t<float, kSimtLinear>(ctx, x, w, residual, rows, K, N, out, s);
+  return linear_t<__nv_bfloat16, kSimtLinear>(ctx, x, w, residual, rows, K, N, out, s);
 }
 
 int launch_gate_up_simt(d3tom_ctx* ctx, d3tom_dtype dt, const void* x, const void* w_gate_up, int rows, int D, int m,
                         void* act, cudaStream_t s) {
-  if (dt == D3TOM_FP32) return launch_linear_simt_t<float, true>(ctx, x, w_gate_up, nullptr, rows, D, m, act, s);
-  return launch_linear_simt_t<__nv_bfloat16, true>(ctx, x, w_gate_up, nullptr, rows, D, m, act, s);
+  if (dt == D3TOM_FP32) return linear_t<float, kSimtGateUp>(ctx, x, w_gate_up, nullptr, rows, D, m, act, s);
+  return linear_t<__nv_bfloat16, kSimtGateUp>(ctx, x, w_gate_up, nullptr, rows, D, m, act, s);
 }
 
-int launch_proj_simt(d3tom_ctx* ctx, d3tom_dtype dt, const void* x, const void* w, int total, int D,
-                     void* q, void* k, void* v, cudaStream_t s) {
-  dim3 grid(ceil_div(3 * D, 32), ceil_div(total, 32));
-  if (dt == D3TOM_FP32)
-    D3TOM_CUDA_TRY(ctx, launch_serialized(proj_simt_kernel<float>, grid, 1024, 0, s, static_cast<const float*>(x),
-                                          static_cast<const float*>(w), total, D, static_cast<float*>(q),
-                                          static_cast<float*>(k), static_cast<float*>(v)));
-  else
-    D3TOM_CUDA_TRY(ctx, launch_serialized(proj_simt_kernel<__nv_bfloat16>, grid, 1024, 0, s,
-                                          static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(w),
-                                          total, D, static_cast<__nv_bfloat16*>(q), static_cast<__nv_bfloat16*>(k),
-                                          static_cast<__nv_bfloat16*>(v)));
-  return D3TOM_OK;
+int launch_proj_simt(d3tom_ctx* ctx, d3tom_dtype dt, const void* x, const void* w, int total, int D, void* q, void* k,
+                     void* v, cudaStream_t s) {
+  if (dt == D3TOM_FP32) return proj_t<float>(ctx, x, w, total, D, q, k, v, s);
+  return proj_t<__nv_bfloat16>(ctx, x, w, total, D, q, k, v, s);
+}
+
+int launch_sim_simt(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
+  if (a.dt == D3TOM_FP32) return sim_t<float>(ctx, a, s);
+  return sim_t<__nv_bfloat16>(ctx, a, s);
 }
