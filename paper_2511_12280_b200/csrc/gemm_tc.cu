@@ -20,6 +20,8 @@
 // stages and keep streaming across tile boundaries; one thread of warp 1 issues tcgen05.mma
 // (M = 128, N = BN, K = 16) into one of TWO TMEM accumulators; warps 2..5 read the other
 // accumulator back with tcgen05.ld (one row per thread) and run the epilogue meanwhile.
+#include <math.h>
+
 #include "common.cuh"
 #include "ptx.cuh"
 
@@ -53,6 +55,7 @@ struct GemmParams {
   const int32_t* cu_seqlens; const int32_t* cu_vis; const int32_t* cu_kept; const int32_t* assign;
   const float* inv_norm; const float* inv_norm_kept;
   unsigned long long* best; float* sim_debug; int max_kept;
+  int bn, stages;             // CTA pairs: columns of a tile (a multiple of 32, at most 256) and ring stages
   int* dev_status;
 };
 
@@ -529,11 +532,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 }
 
 // ---------------------------------------------------------------- CTA pairs
-// Two CTAs of a cluster (ranks 0 and 1, neighbouring SMs) compute one 256 x BN tile with `cta_group::2` MMAs: each CTA
-// holds its own 128 rows of A and HALF of the B tile (BN / 2 rows) in shared memory, the tensor cores of both read both
-// halves, and each CTA's 128 x BN accumulator lands in its own tensor memory.  Per k-block a CTA pulls 16 + BN / 4 KB out
-// of L2 instead of 16 + BN / 2 KB: 32 KB for 512 tensor cycles at BN = 256, where the single-CTA 128 x 256 tile needs 48 KB
+// Two CTAs of a cluster (ranks 0 and 1, neighbouring SMs) compute one 256 x bn tile with `cta_group::2` MMAs: each CTA
+// holds its own 128 rows of A and HALF of the B tile (bn / 2 rows) in shared memory, the tensor cores of both read both
+// halves, and each CTA's 128 x bn accumulator lands in its own tensor memory.  Per k-block a CTA pulls 16 + bn / 16 KB out
+// of L2: 32 KB for 512 tensor cycles at bn = 256, where the single-CTA 128 x 256 tile needs 48 KB
 // and is bound by what an SM can pull out of L2 (about 56 B per cycle).
+// The width is chosen at run time (any multiple of 32 up to 256: the instruction descriptor, the tensor map's box and the
+// ring's strides are data), because what separates the widths is how the tiles fill the rounds over the pairs.
 //   * both CTAs run the same warp roles; each loader thread waits on its OWN `empty` barrier and loads its own boxes, whose
 //     bytes are counted on rank 0's `full` barrier (rank 0's loader threads expect the bytes of both CTAs);
 //   * one thread of rank 0 issues every MMA and commits to the `empty` / `acc_full` barriers of BOTH CTAs;
@@ -541,27 +546,40 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 //   * before a CTA leaves, its loaders have seen every commit aimed at it, rank 0 has seen every epilogue arrival, and
 //     the two CTAs meet in a cluster barrier; tensor memory is allocated and freed by warp 2 of both CTAs together.
 // Whole tiles only (no K split); every mbarrier wait is bounded as elsewhere.
-template <int BN> struct PairSmem {
-  static constexpr int kABytes = kBM * kBK * 2, kBBytes = (BN / 2) * kBK * 2;
-  static constexpr int kStages = 6;
-  static constexpr int kBytes = kStages * (kABytes + kBBytes) + 1024 /*alignment slack*/ + 256 /*barriers*/;
+// 64-deep boxes of each operand per stage.  Two for the narrower tiles: a barrier check and a commit then serve eight MMAs
+// instead of four, whose overhead shows where an MMA is short (128 columns: 0.33 -> 0.29 us per 64 of K, 192: 0.35 -> 0.31);
+// one for the wider ones, whose ring would be left with three stages (256 columns: 0.32 against 0.33 us).
+__host__ __device__ constexpr int pair_sub(int bn) { return bn <= 192 ? 2 : 1; }
+constexpr int kPairMaxStages = 8;
+constexpr int kPairSmemLimit = 227 * 1024;
+__host__ __device__ constexpr int pair_stage_bytes(int bn) { return pair_sub(bn) * (kBM * kBK * 2 + (bn / 2) * kBK * 2); }
+constexpr int pair_stages(int bn) {
+  const int fit = (kPairSmemLimit - 1024 - 256) / pair_stage_bytes(bn);
+  return fit < kPairMaxStages ? fit : kPairMaxStages;
+}
+constexpr int pair_smem_bytes(int bn) { return pair_stages(bn) * pair_stage_bytes(bn) + 1024 /*alignment slack*/ + 256 /*barriers*/; }
+
+// stage index and phase of a ring of p.stages buffers
+struct RingPos {
+  int s = 0;
+  uint32_t phase = 0;
+  __device__ __forceinline__ void next(int stages) { if (++s == stages) { s = 0; phase ^= 1u; } }
 };
 
-template <int BN, int EPI>
+template <int EPI, int kSub>           // kSub == pair_sub(p.bn)
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b, GemmParams p) {
-  static_assert(BN % 32 == 0 && BN <= 256 && (BN / 2) % 8 == 0, "half of the B tile is a whole number of 8-row swizzle groups");
   static_assert(EPI != kEpiSim, "the dense layers only");
-  using S = PairSmem<BN>;
-  constexpr int kStages = S::kStages;
+  constexpr int kABytes = kBM * kBK * 2;                   // one box of A; of B: bn / 2 rows of 128 bytes (whole 8-row swizzle groups)
+  const int bn = p.bn, stages = p.stages, b_bytes = (bn / 2) * kBK * 2;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* a_s = smem;
-  uint8_t* b_s = smem + kStages * S::kABytes;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * (S::kABytes + S::kBBytes));
-  uint64_t* empty = full + kStages;
-  uint64_t* acc_full = empty + kStages;       // [2]
-  uint64_t* acc_empty = acc_full + 2;         // [2] (rank 0's are the ones in use)
+  uint8_t* b_s = smem + stages * kSub * kABytes;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + stages * kSub * (kABytes + b_bytes));
+  uint64_t* empty = full + kPairMaxStages;
+  uint64_t* acc_full = empty + kPairMaxStages;   // [2]
+  uint64_t* acc_empty = acc_full + 2;            // [2] (rank 0's are the ones in use)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -569,7 +587,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
   const uint32_t rank = ptx::cluster_ctarank();
   const bool leader = rank == 0;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) { ptx::mbar_init(&full[s], 2); ptx::mbar_init(&empty[s], 1); }   // A and B loaders of rank 0; one commit
+    for (int s = 0; s < stages; ++s) { ptx::mbar_init(&full[s], 2); ptx::mbar_init(&empty[s], 1); }   // A and B loaders of rank 0; one commit
     for (int i = 0; i < 2; ++i) { ptx::mbar_init(&acc_full[i], 1); ptx::mbar_init(&acc_empty[i], 8); }   // four epilogue warps in each CTA
     *abort_flag = 0;
     ptx::fence_mbar_init();
@@ -585,7 +603,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
   const int n_pairs = gridDim.x >> 1, pair = blockIdx.x >> 1;
   // tile t: M fastest, so that the pairs of a round share their B tiles in L2
   auto tile_m0 = [&](int t) { return (t % p.m_tiles) * (2 * kBM); };
-  auto tile_n0 = [&](int t) { return (t / p.m_tiles) * (EPI == kEpiGateUp ? BN / 2 : BN); };
+  auto tile_n0 = [&](int t) { return (t / p.m_tiles) * (EPI == kEpiGateUp ? bn / 2 : bn); };
 
   if (warp == 0 || warp == 6) {
     // ------------------------------------------------------------ TMA producers: warp 0 streams A, warp 6 streams B
@@ -593,34 +611,38 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
       const bool is_a = warp == 0;
       const CUtensorMap* tm = is_a ? &tmap_a : &tmap_b;
       uint8_t* ring = is_a ? a_s : b_s;
-      const int stage_bytes = is_a ? S::kABytes : S::kBBytes;
+      const int box_bytes = is_a ? kABytes : b_bytes;
       ptx::prefetch_tensormap(tm);
       int it = 0;
+      RingPos r;
       bool ok = true;
       for (int t = pair; t < tiles && ok; t += n_pairs) {
         const int n0 = tile_n0(t);
         // this CTA's rows: its half of the 256 rows of A; its half of the B tile (gate rows for rank 0, up rows for rank 1)
         const int row0 = is_a ? tile_m0(t) + (int)rank * kBM
-                              : (EPI == kEpiGateUp ? (leader ? n0 : p.up_row_offset + n0) : n0 + (int)rank * (BN / 2));
-        for (int kbk = 0; kbk < p.num_k_blocks; ++kbk, ++it) {
-          const int s = it % kStages;
-          ok = ptx::mbar_wait(&empty[s], ((it / kStages) & 1) ^ 1, abort_flag, p.dev_status);
+                              : (EPI == kEpiGateUp ? (leader ? n0 : p.up_row_offset + n0) : n0 + (int)rank * (bn / 2));
+        for (int kbk = 0; kbk < p.num_k_blocks; kbk += kSub, ++it, r.next(stages)) {
+          const int sub = min(kSub, p.num_k_blocks - kbk);
+          ok = ptx::mbar_wait(&empty[r.s], r.phase ^ 1u, abort_flag, p.dev_status);
           if (!ok) break;
-          if (leader) ptx::mbar_arrive_expect_tx(&full[s], 2 * stage_bytes);     // this operand's boxes of both CTAs
-          ptx::tma_load_2d_pair(ring + s * stage_bytes, tm, &full[s], kbk * kBK, row0);
+          if (leader) ptx::mbar_arrive_expect_tx(&full[r.s], 2 * sub * box_bytes);     // this operand's boxes of both CTAs
+#pragma unroll
+          for (int b = 0; b < kSub; ++b)
+            if (b < sub) ptx::tma_load_2d_pair(ring + (r.s * kSub + b) * box_bytes, tm, &full[r.s], (kbk + b) * kBK, row0);
         }
       }
       // every commit aimed at this CTA's `empty` barriers has landed before the CTA may leave
-      for (int j = it > kStages ? it - kStages : 0; j < it && ok; ++j)
-        ok = ptx::mbar_wait(&empty[j % kStages], (j / kStages) & 1, abort_flag, p.dev_status);
+      for (int j = it > stages ? it - stages : 0; j < it && ok; ++j)
+        ok = ptx::mbar_wait(&empty[j % stages], (j / stages) & 1, abort_flag, p.dev_status);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (rank 0 only)
     if (lane == 0 && leader) {
-      constexpr uint32_t idesc = ptx::idesc_bf16_f32(2 * kBM, BN, 0, 0);
+      const uint32_t idesc = ptx::idesc_bf16_f32(2 * kBM, bn, 0, 0);
       const ptx::SmemDesc a_desc0 = ptx::smem_desc_kmajor_sw128(ptx::smem_u32(a_s));
       const ptx::SmemDesc b_desc0 = ptx::smem_desc_kmajor_sw128(ptx::smem_u32(b_s));
-      int it = 0, lt = 0;
+      int lt = 0;
+      RingPos r;
       bool ok = true;
       for (int t = pair; t < tiles && ok; t += n_pairs, ++lt) {
         const int buf = lt & 1;
@@ -628,17 +650,23 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
         if (!ok) break;
         ptx::tc_fence_after_sync();
         const uint32_t tmem_acc = tmem_base + (uint32_t)buf * 256u;
-        for (int kbk = 0; kbk < p.num_k_blocks; ++kbk, ++it) {
-          const int s = it % kStages;
-          ok = ptx::mbar_wait(&full[s], (it / kStages) & 1, abort_flag, p.dev_status);
+        for (int kbk = 0; kbk < p.num_k_blocks; kbk += kSub, r.next(stages)) {
+          ok = ptx::mbar_wait(&full[r.s], r.phase, abort_flag, p.dev_status);
           if (!ok) break;
           ptx::tc_fence_after_sync();
-          const ptx::SmemDesc ad = ptx::smem_desc_advance(a_desc0, s * S::kABytes), bd = ptx::smem_desc_advance(b_desc0, s * S::kBBytes);
+          const ptx::SmemDesc ad = ptx::smem_desc_advance(a_desc0, r.s * kSub * kABytes);
+          const ptx::SmemDesc bd = ptx::smem_desc_advance(b_desc0, r.s * kSub * b_bytes);
 #pragma unroll
           for (int kk = 0; kk < kBK / 16; ++kk)
             ptx::mma_ss_pair(tmem_acc, ptx::smem_desc_advance(ad, kk * 32), ptx::smem_desc_advance(bd, kk * 32), idesc,
                              (kbk > 0 || kk > 0) ? 1u : 0u);
-          ptx::mma_commit_pair(&empty[s], 3);      // frees the stage in both CTAs once these MMAs have read it
+          if (kSub > 1 && kbk + 1 < p.num_k_blocks) {
+            const ptx::SmemDesc ad1 = ptx::smem_desc_advance(ad, kABytes), bd1 = ptx::smem_desc_advance(bd, b_bytes);
+#pragma unroll
+            for (int kk = 0; kk < kBK / 16; ++kk)
+              ptx::mma_ss_pair(tmem_acc, ptx::smem_desc_advance(ad1, kk * 32), ptx::smem_desc_advance(bd1, kk * 32), idesc, 1u);
+          }
+          ptx::mma_commit_pair(&empty[r.s], 3);      // frees the stage in both CTAs once these MMAs have read it
         }
         if (ok) ptx::mma_commit_pair(&acc_full[buf], 3);
       }
@@ -648,6 +676,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
     }
   } else {
     // ------------------------------------------------------------ epilogue: warp w may touch TMEM lanes 32*(w%4) .. +31
+    // 32 columns at a time, stored as two pieces of 16 (half of a gate-up tile may end in half a piece of 32)
     const int quarter = warp & 3;
     const int row = quarter * 32 + lane;
     int lt = 0;
@@ -659,75 +688,55 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
       const uint32_t t_row = tmem_base + (uint32_t)buf * 256u + ((uint32_t)(quarter * 32) << 16);
       const int grow = tile_m0(t) + (int)rank * kBM + row;
       const int n0 = tile_n0(t);
-      if (EPI == kEpiProj) {
+      // columns of the tile that exist
+      const int width = EPI == kEpiGateUp ? min(bn / 2, p.ld_out - n0) : min(bn, (EPI == kEpiProj ? 3 * p.out_cols : p.ld_out) - n0);
+      const bool live = grow < p.out_rows;
 #pragma unroll 1
-        for (int c = 0; c < BN; c += 32) {
-          uint32_t r[32];
-          ptx::tmem_ld32(t_row + c, r);
+      for (int c = 0; c < width; c += 32) {
+        uint32_t r[32];
+        ptx::tmem_ld32(t_row + c, r);
+        if (EPI == kEpiGateUp) {
+          uint32_t up[32];
+          ptx::tmem_ld32(t_row + bn / 2 + c, up);
           ptx::tmem_wait_ld();
-          const int gcol = n0 + c, which = gcol / p.out_cols;
-          if (grow < p.out_rows && which < 3) {
-            __nv_bfloat16* dst = p.out[which] + (size_t)grow * p.out_cols + (gcol - which * p.out_cols);
 #pragma unroll
-            for (int i = 0; i < 32; i += 8) {
-              uint32_t w[4];
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(r[i + 2 * j]), __uint_as_float(r[i + 2 * j + 1]));
-                w[j] = *reinterpret_cast<uint32_t*>(&h2);
-              }
-              *reinterpret_cast<uint4*>(dst + i) = make_uint4(w[0], w[1], w[2], w[3]);
-            }
+          for (int i = 0; i < 32; ++i) {
+            const float g = __uint_as_float(r[i]);
+            // silu(g) = g / (1 + exp(-g)); for very negative g the divisor is inf and the quotient 0
+            r[i] = __float_as_uint(__fdividef(g, 1.f + __expf(-g)) * __uint_as_float(up[i]));
           }
-        }
-      } else if (EPI == kEpiLinear) {
-#pragma unroll 1
-        for (int c = 0; c < BN; c += 32) {
-          uint32_t r[32];
-          ptx::tmem_ld32(t_row + c, r);
+        } else {
           ptx::tmem_wait_ld();
-          if (grow < p.out_rows && n0 + c < p.ld_out) {
-            const size_t off = (size_t)grow * p.ld_out + n0 + c;
+        }
 #pragma unroll
-            for (int i = 0; i < 32; i += 8) {
-              uint32_t w[4] = {0u, 0u, 0u, 0u};
-              if (p.residual != nullptr) {
-                const uint4 rr = *reinterpret_cast<const uint4*>(p.residual + off + i);
-                w[0] = rr.x; w[1] = rr.y; w[2] = rr.z; w[3] = rr.w;
-              }
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const float lo = __uint_as_float(r[i + 2 * j]) + __uint_as_float(w[j] << 16);
-                const float hi = __uint_as_float(r[i + 2 * j + 1]) + __uint_as_float(w[j] & 0xffff0000u);
-                __nv_bfloat162 h2 = __floats2bfloat162_rn(lo, hi);
-                w[j] = *reinterpret_cast<uint32_t*>(&h2);
-              }
-              *reinterpret_cast<uint4*>(p.lin_out + off + i) = make_uint4(w[0], w[1], w[2], w[3]);
-            }
+        for (int hf = 0; hf < 2; ++hf) {
+          const int col = c + hf * 16;
+          if (!live || col >= width) continue;
+          __nv_bfloat16* dst;
+          const __nv_bfloat16* res = nullptr;
+          if (EPI == kEpiProj) {
+            const int gcol = n0 + col, which = gcol / p.out_cols;
+            dst = p.out[which] + (size_t)grow * p.out_cols + (gcol - which * p.out_cols);
+          } else {
+            const size_t off = (size_t)grow * p.ld_out + n0 + col;
+            dst = p.lin_out + off;
+            if (EPI == kEpiLinear && p.residual != nullptr) res = p.residual + off;
           }
-        }
-      } else {
-#pragma unroll 1
-        for (int c = 0; c < BN / 2; c += 32) {
-          uint32_t g[32], up[32];
-          ptx::tmem_ld32(t_row + c, g);
-          ptx::tmem_ld32(t_row + BN / 2 + c, up);
-          ptx::tmem_wait_ld();
-          if (grow < p.out_rows) {
-            __nv_bfloat16* dst = p.lin_out + (size_t)grow * p.ld_out + n0 + c;
 #pragma unroll
-            for (int i = 0; i < 32; i += 8) {
-              uint32_t w[4];
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const float g0 = __uint_as_float(g[i + 2 * j]), g1 = __uint_as_float(g[i + 2 * j + 1]);
-                const float a0 = __fdividef(g0, 1.f + __expf(-g0)) * __uint_as_float(up[i + 2 * j]);
-                const float a1 = __fdividef(g1, 1.f + __expf(-g1)) * __uint_as_float(up[i + 2 * j + 1]);
-                __nv_bfloat162 h2 = __floats2bfloat162_rn(a0, a1);
-                w[j] = *reinterpret_cast<uint32_t*>(&h2);
-              }
-              *reinterpret_cast<uint4*>(dst + i) = make_uint4(w[0], w[1], w[2], w[3]);
+          for (int i = 0; i < 16; i += 8) {
+            uint32_t w[4] = {0u, 0u, 0u, 0u};
+            if (EPI == kEpiLinear && res != nullptr) {
+              const uint4 rr = *reinterpret_cast<const uint4*>(res + i);
+              w[0] = rr.x; w[1] = rr.y; w[2] = rr.z; w[3] = rr.w;
             }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              float lo = __uint_as_float(r[hf * 16 + i + 2 * j]), hi = __uint_as_float(r[hf * 16 + i + 2 * j + 1]);
+              if (EPI == kEpiLinear) { lo += __uint_as_float(w[j] << 16); hi += __uint_as_float(w[j] & 0xffff0000u); }
+              __nv_bfloat162 h2 = __floats2bfloat162_rn(lo, hi);
+              w[j] = *reinterpret_cast<uint32_t*>(&h2);
+            }
+            *reinterpret_cast<uint4*>(dst + i) = make_uint4(w[0], w[1], w[2], w[3]);
           }
         }
       }
@@ -825,21 +834,21 @@ int launch_gemm(d3tom_ctx* ctx, const CUtensorMap& ta, const CUtensorMap& tb, Ge
 
 // How many CTA pairs of this kernel the device holds at once (asked once per device; 0 = clusters of two cannot be
 // launched here, and the caller keeps single-CTA tiles).
-template <int BN, int EPI>
+template <int EPI>
 int resident_pairs(d3tom_ctx* ctx) {
   static int cached[64] = {};
   int& pairs = cached[ctx->device & 63];
   if (pairs == 0) {
-    auto kernel = gemm_pair_kernel<BN, EPI>;
+    auto kernel = gemm_pair_kernel<EPI, 1>;      // (both forms: one CTA per SM, the same shared memory)
     pairs = -1;
     if (ctx->sm_count >= 2 &&
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PairSmem<BN>::kBytes) == cudaSuccess) {
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemLimit) == cudaSuccess) {
       cudaLaunchAttribute attr[1];
       attr[0].id = cudaLaunchAttributeClusterDimension;
       attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3((unsigned)(ctx->sm_count & ~1)); cfg.blockDim = dim3(kGemmThreads);
-      cfg.dynamicSmemBytes = PairSmem<BN>::kBytes; cfg.attrs = attr; cfg.numAttrs = 1;
+      cfg.dynamicSmemBytes = kPairSmemLimit; cfg.attrs = attr; cfg.numAttrs = 1;
       int n = 0;
       if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0)
         pairs = n < ctx->sm_count / 2 ? n : ctx->sm_count / 2;
@@ -849,15 +858,17 @@ int resident_pairs(d3tom_ctx* ctx) {
   return pairs > 0 ? pairs : 0;
 }
 
-template <int BN, int EPI>
+template <int EPI>
 int launch_gemm_pair(d3tom_ctx* ctx, const CUtensorMap& ta, const CUtensorMap& tb, GemmParams p, cudaStream_t s) {
   const long long tiles = (long long)p.m_tiles * p.n_tiles;
   if (tiles <= 0) return D3TOM_OK;
-  const int pairs = resident_pairs<BN, EPI>(ctx);
+  const int pairs = resident_pairs<EPI>(ctx);
   if (pairs <= 0) return D3TOM_ERR_UNSUPPORTED;
-  auto kernel = gemm_pair_kernel<BN, EPI>;
+  p.stages = pair_stages(p.bn);
+  const int smem = pair_smem_bytes(p.bn);
+  auto kernel = pair_sub(p.bn) == 2 ? gemm_pair_kernel<EPI, 2> : gemm_pair_kernel<EPI, 1>;
   // (the attribute belongs to the current device: set on every call, a process may drive several GPUs)
-  D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PairSmem<BN>::kBytes));
+  D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemLimit));
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
@@ -865,24 +876,53 @@ int launch_gemm_pair(d3tom_ctx* ctx, const CUtensorMap& ta, const CUtensorMap& t
   attr[1].val.programmaticStreamSerializationAllowed = g_d3tom_launch_overlap ? 1 : 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(2 * (tiles < pairs ? tiles : pairs))); cfg.blockDim = dim3(kGemmThreads);
-  cfg.dynamicSmemBytes = PairSmem<BN>::kBytes; cfg.stream = s; cfg.attrs = attr; cfg.numAttrs = 2;
+  cfg.dynamicSmemBytes = smem; cfg.stream = s; cfg.attrs = attr; cfg.numAttrs = 2;
   D3TOM_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, kernel, ta, tb, p));
   return D3TOM_OK;
 }
 
-// Whether a dense layer of `rows` x `ncols` outputs runs as 256 x 256 tiles on CTA pairs.  Measured against the
-// single-CTA shapes, alternating the two in one process (projection / output projection / feed-forward network at
-// D = 4096, m = 12288, us): 1216 rows 94 / 51 / 294 against 92 / 56 / 303, 1152 rows 98 / 59 / 297 against
-// 87 / 39 / 257, 2176 rows 147 / 56 / 453 against 156 / 62 / 480, 4288 rows 281 / 105 / 914 against 303 / 132 / 1076,
-// 7800 rows 543 / 212 / 1715 against 583 / 290 / 1988.  A round of 74 pair tiles costs what a round of 148 tiles of
-// 256 x 256 costs per flop (both run at the tensor rate the board's power limit allows), so short layers, which are
-// decided by how the tiles fill the last round, keep their shapes; from about two thousand rows on the pairs win on
-// every layer: half the operand traffic per SM leaves more of the power budget to the tensor cores.
-bool use_pair_tiles(const d3tom_ctx* ctx, int rows, int ncols) {
-  if (ncols % 256 != 0 || ctx->sm_count < 2) return false;
-  if (g_d3tom_pair_tiles == 0) return false;
-  if (g_d3tom_pair_tiles == 256) return true;
-  return rows >= 2048;
+// Width of the CTA-pair tiles for a dense layer of `rows` x `ncols` outputs (for the gate-up pass the columns of both
+// matrices), or 0 for single-CTA tiles.  A round of pair tiles costs the times below per 64 of K whatever it computes, so
+// the width that fills the rounds best wins; against it stand rounds of single-CTA tiles, whose last, partial round is
+// cheaper, and K slices for a long K (plan_tail_split).  All figures in us per 64 of K, fitted to the four layers of a
+// block (D = 4096, m = 12288) at 128 .. 4288 rows.  What it changes, old shapes / pairs (us): projection 640 rows
+// 56 / 51; output projection 1216 rows 69 / 55, 1536 rows 57 / 49, 2600 rows 81 / 75 (224 columns; 83 with 256); down
+// projection 640 rows 82 / 62, 1800 rows 171 / 155; feed-forward network 1216 rows 308 / 282.  The factor
+// 1.08 is for power: the pairs move half the operand bytes, and the board's limit sets the clock under these layers.
+// From 2048 rows on the pairs are always taken.
+int pair_tile_width(const d3tom_ctx* ctx, int rows, int ncols, int num_k_blocks, int pairs, bool gate_up) {
+  if (pairs <= 0 || g_d3tom_pair_tiles == 0) return 0;
+  if (g_d3tom_pair_tiles == 256) return ncols % 256 == 0 ? 256 : 0;
+  const int sms = ctx->sm_count;
+  constexpr int kWidths[] = {256, 224, 192, 160, 128};
+  constexpr double kPerBlock[] = {0.36, 0.345, 0.31, 0.30, 0.29};
+  double best = 1e30;
+  int width = 0;
+  for (int i = 0; i < 5; ++i) {
+    const long long tiles = (long long)ceil_div(rows, 2 * kBM) * ceil_div(ncols, kWidths[i]);
+    const double cost = kPerBlock[i] * (double)((tiles + pairs - 1) / pairs);
+    if (cost < best) { best = cost; width = kWidths[i]; }
+  }
+  if (rows >= 2048) return width;
+  auto rounds = [&](int bm, int bn, double full, double last0, double last_r) {
+    const long long tiles = (long long)ceil_div(rows, bm) * ceil_div(ncols, bn);
+    const long long r = tiles % sms;
+    return full * (double)(tiles / sms) + (r > 0 ? last0 + last_r * (double)r : 0.0);
+  };
+  double single = rounds(kBM, 256, 0.40, 0.26, 0.0009);
+  if (!gate_up) {      // (the pass of two matrices walks whole tiles)
+    const long long tiles = (long long)ceil_div(rows, kBM) * ceil_div(ncols, 256);
+    const int rem = (int)(tiles % sms);
+    for (int sp = 2; sp <= kMaxKSplits && rem > 0; ++sp) {
+      if (num_k_blocks / sp < 8 || rem * sp > 2 * sms) break;
+      const double cut = (double)(ceil_div(rem * sp, sms) * ceil_div(num_k_blocks, sp) + 30 + 5 * sp) / num_k_blocks;
+      if (cut < 1.0) single = fmin(single, 0.40 * (double)(tiles / sms) + 0.42 * cut);
+    }
+    single = fmin(single, rounds(2 * kBM, 224, 0.65, 0.41, 0.0016));
+  }
+  single = fmin(single, rounds(2 * kBM, 256, 0.73, 0.46, 0.0018));
+  // (a pair launch costs about 1.5 us more: with a short K the single-CTA tiles keep small layers, 319 x 3072 x 1024: 9.0 / 9.9)
+  return best * num_k_blocks + 1.5 < 1.08 * single * num_k_blocks ? width : 0;
 }
 
 }  // namespace
@@ -924,11 +964,11 @@ int launch_proj_tc(d3tom_ctx* ctx, const void* x, const void* w, int total, int 
     const double cost = rounds * (cand == 256 ? 667.0 : cand == 192 ? 633.0 : 600.0);
     if (cost < best_cost) { best_cost = cost; bn = cand; }
   }
-  if (use_pair_tiles(ctx, total, 3 * D) && resident_pairs<256, kEpiProj>(ctx) > 0) {
-    r = make_tmap_bf16_2d(&tb, w, (uint64_t)3 * D, (uint64_t)D, (uint64_t)D, 128);       // a CTA's half of the weight tile
+  if (const int bn2 = pair_tile_width(ctx, total, 3 * D, p.num_k_blocks, resident_pairs<kEpiProj>(ctx), false)) {
+    r = make_tmap_bf16_2d(&tb, w, (uint64_t)3 * D, (uint64_t)D, (uint64_t)D, (uint32_t)bn2 / 2);   // a CTA's half of the weight tile
     if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
-    p.m_tiles = ceil_div(total, 2 * kBM); p.n_tiles = 3 * D / 256;
-    return launch_gemm_pair<256, kEpiProj>(ctx, ta, tb, p, s);
+    p.bn = bn2; p.m_tiles = ceil_div(total, 2 * kBM); p.n_tiles = ceil_div(3 * D, bn2);
+    return launch_gemm_pair<kEpiProj>(ctx, ta, tb, p, s);
   }
   if (const int w2 = two_m_tile_width(ctx, total, 3 * D, D % 32 == 0)) {
     r = make_tmap_bf16_2d(&ta, x, (uint64_t)total, (uint64_t)D, (uint64_t)D, 2 * kBM);
@@ -967,11 +1007,11 @@ int launch_linear_tc(d3tom_ctx* ctx, const void* x, const void* w, const void* r
     const double cost = rounds * (cand == 256 ? 667.0 : cand == 192 ? 633.0 : 600.0);
     if (cost < best_cost) { best_cost = cost; bn = cand; }
   }
-  if (use_pair_tiles(ctx, rows, N) && resident_pairs<256, kEpiLinear>(ctx) > 0) {
-    r = make_tmap_bf16_2d(&tb, w, (uint64_t)N, (uint64_t)K, (uint64_t)K, 128);
+  if (const int bn2 = pair_tile_width(ctx, rows, N, p.num_k_blocks, resident_pairs<kEpiLinear>(ctx), false)) {
+    r = make_tmap_bf16_2d(&tb, w, (uint64_t)N, (uint64_t)K, (uint64_t)K, (uint32_t)bn2 / 2);
     if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
-    p.m_tiles = ceil_div(rows, 2 * kBM); p.n_tiles = N / 256;
-    return launch_gemm_pair<256, kEpiLinear>(ctx, ta, tb, p, s);
+    p.bn = bn2; p.m_tiles = ceil_div(rows, 2 * kBM); p.n_tiles = ceil_div(N, bn2);
+    return launch_gemm_pair<kEpiLinear>(ctx, ta, tb, p, s);
   }
   if (const int w2 = two_m_tile_width(ctx, rows, N, true)) {
     r = make_tmap_bf16_2d(&ta, x, (uint64_t)rows, (uint64_t)K, (uint64_t)K, 2 * kBM);
@@ -1001,9 +1041,11 @@ int launch_gate_up_tc(d3tom_ctx* ctx, const void* x, const void* w_gate_up, int 
   p.lin_out = static_cast<__nv_bfloat16*>(act); p.ld_out = m; p.up_row_offset = m; p.out_rows = rows;
   p.dev_status = ctx->dev_status;
   p.m_tiles = ceil_div(rows, kBM); p.n_tiles = m / 128; p.batch = 1; p.k_splits = 1;
-  if (use_pair_tiles(ctx, rows, 2 * m) && resident_pairs<256, kEpiGateUp>(ctx) > 0) {       // (the B map's box is already 128 rows: one CTA's half)
-    p.m_tiles = ceil_div(rows, 2 * kBM);
-    return launch_gemm_pair<256, kEpiGateUp>(ctx, ta, tb, p, s);
+  if (const int bn2 = pair_tile_width(ctx, rows, 2 * m, p.num_k_blocks, resident_pairs<kEpiGateUp>(ctx), true)) {
+    r = make_tmap_bf16_2d(&tb, w_gate_up, (uint64_t)2 * m, (uint64_t)D, (uint64_t)D, (uint32_t)bn2 / 2);   // gate rows or up rows
+    if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
+    p.bn = bn2; p.m_tiles = ceil_div(rows, 2 * kBM); p.n_tiles = ceil_div(m, bn2 / 2);
+    return launch_gemm_pair<kEpiGateUp>(ctx, ta, tb, p, s);
   }
   {
     if (two_m_tile_width(ctx, rows, 2 * m, false) == 256) {

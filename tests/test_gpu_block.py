@@ -112,6 +112,23 @@ def test_long_dense_layers_take_cta_pairs_by_default():
     run_ffn(2100, 256, 256, "bf16", seed=9)
 
 
+# nine 256-row tiles on 74 pairs: eight column tiles fill one round, so the width follows the number of columns: 128, 160,
+# 160 with an overhang, 192, 192 with an overhang, 224, 224 with an overhang, 256; K of one, three and four 64-deep blocks
+# (the narrower tiles take two blocks per ring stage)
+@pytest.mark.parametrize("N,K", [(1024, 192), (1280, 64), (1152, 192), (1536, 256), (1408, 192), (1792, 192), (1664, 256), (2048, 192)])
+def test_pair_tiles_of_every_width(N, K):
+    run_linear(2100, K, N, "bf16", residual=True, seed=N)
+
+
+def test_pair_tiles_of_every_width_projection_and_gate_up():
+    run_proj(2100, 4, 128, seed=21)          # 3 D = 1536: width 192 straddles q | k and k | v
+    run_proj(2100, 3, 128, seed=22)          # 3 D = 1152: width 160, overhang
+    run_ffn(2100, 128, 640, "bf16", seed=23)        # 160: halves of 80 gate and 80 up rows
+    run_ffn(2100, 256, 896, "bf16", seed=24)        # 224: halves of 112
+    run_ffn(2100, 128, 1152, "bf16", seed=25)       # 160 in two rounds, the last tile hangs over the edge of both matrices
+    run_linear(600, 320, 5120, "bf16", residual=True, seed=26)      # below 2048 rows: pairs where their rounds are cheaper
+
+
 def test_linear_fp32_odd_sizes():
     run_linear(70, 50, 45, "fp32", residual=True)
     run_linear(33, 7, 3, "fp32", residual=False)
