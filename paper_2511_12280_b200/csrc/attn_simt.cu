@@ -1,59 +1,57 @@
 // Bidirectional attention on CUDA cores (fp32 arithmetic) and the importance
 // finishing kernel shared with the tensor-core attention.
 //
-// One CTA owns BM = 128 / KG query rows of one (request, head) and visits the keys 32 KG at a time.  Its 8 warps are
-// 8 / KG row groups of 16 rows times KG key groups of 32 keys: a warp runs the online softmax (log2 domain) of its
-// own 16 rows over its own keys, and the KG partial results (m, l, O) of a row are combined once at the end, in key
-// group order.  Scores and P V both run as 16 x 32 register tiles out of shared memory (f32_tile.cuh); P passes from
-// lane to lane through 2 KB of shared memory per warp.  K and V have one buffer each: the next K tile is copied while
-// the softmax and P V of this one run, the next V tile under the next scores.
-//
-// Bound: the fp32 pipe and the latency of one or two warps per scheduler (FMA pipe about half busy).  One warp per
-// query row, every lane walking a key of its own through global memory, took 1139 us at 1152 rows x 8 heads x 64 where
-// this takes 82, and 111 us at 288 x 4 x 64 where this takes 14.
-//
+// A warp owns RW (16 or 8) query rows of one (request, head) and visits the keys 32 at a time with an online softmax
+// (log2 domain); the NW warps of a CTA share the K and V tiles, which come by asynchronous copies into two stages.  Scores
+// and P V run as register tiles out of shared memory (lane layout of f32_tile.cuh); P passes from lane to lane through
+// shared memory of the warp.  Every score is one chain of multiply-adds over head_dim, every output one chain over the
+// keys, and the row sums are added in the order of a butterfly over 32 keys: the arithmetic does not depend on how rows
+// are spread over warps.
 // Decider rows additionally write their raw q.k scores over the visual keys to
 // the score scratch and their final (M, l) pair to the lse scratch; the
 // finishing kernel turns those into S_j = sum_h sum_{i in D} A_ij.
+//
+// Bound: the fp32 pipe and the latency of one to three warps per scheduler.  One warp per query row, every lane walking a
+// key of its own through global memory, took 1139 us at 1152 rows x 8 heads x 64 where this takes 98, and 111 us at
+// 288 x 4 x 64 where this takes 20.
 #include "common.cuh"
 #include "f32_tile.cuh"
 
 namespace {
 
-constexpr int kSimtWarps = 8;
-constexpr int kPStride = 36;         // floats per row of a warp's P tile (32 + 4: see f32_tile.cuh)
+constexpr int kKeyTile = 32;
+constexpr int kPStride = kKeyTile + 4;         // floats per row of a warp's P tile (see f32_tile.cuh)
 
-// DHP: head_dim rounded up to 32, 64 or 128 (padding columns are zero); KG: key groups
-template <int DHP, int KG> struct SimtSmem {
-  static constexpr int kBM = 128 / KG, kKeys = 32 * KG, kLd = DHP + 4;
-  static constexpr int kQ = kBM * kLd, kK = kKeys * kLd, kP = kSimtWarps * 16 * kPStride;
-  static constexpr int kBytes = (kQ + 2 * kK + kP) * 4 + kBM * 4;
-  static_assert(2 * kK >= 128 * DHP, "the partial outputs of all key groups are combined in the K and V buffers");
+// DHP: head_dim rounded up to 32, 64 or 128 (padding columns are zero)
+template <int DHP, int RW, int NW> struct SimtSmem {
+  static constexpr int kBM = RW * NW, kLd = DHP + 4;
+  static constexpr int kQ = kBM * kLd, kKv = kKeyTile * kLd, kP = NW * RW * kPStride;
+  static constexpr int kBytes = (kQ + 4 * kKv + kP) * 4 + kBM * 4;
 };
 
-template <typename T, int DHP, int KG>
-__global__ void __launch_bounds__(kSimtWarps * 32, 1)
+template <typename T, int DHP, int RW, int NW>
+__global__ void __launch_bounds__(NW * 32)
 attn_simt_kernel(AttnArgs a, bool vec) {
-  using S = SimtSmem<DHP, KG>;
-  constexpr int kLd = S::kLd, kCols = DHP / 32;         // 4-column groups of the output per lane
+  using S = SimtSmem<DHP, RW, NW>;
+  constexpr int kLd = S::kLd, kCols = DHP / 32, kR = RW / 4;      // 4-column groups of the output and rows per lane
   extern __shared__ float4 smem_f4[];
   float* q_s = reinterpret_cast<float*>(smem_f4);
-  float* k_s = q_s + S::kQ;
-  float* v_s = k_s + S::kK;
-  float* p_all = v_s + S::kK;
+  float* kv_s = q_s + S::kQ;                              // stage st: K tile, V tile
+  float* p_all = kv_s + 4 * S::kKv;
   int* dec_s = reinterpret_cast<int*>(p_all + S::kP);
   grid_dependency_enter();
   const int b = blockIdx.z, h = blockIdx.y, tid = threadIdx.x;
   const int lo = a.cu_seqlens[b], n = a.cu_seqlens[b + 1] - lo;
   const int q0 = blockIdx.x * S::kBM;
   if (q0 >= n) return;
-  const int H = a.H, dh = a.dh;
-  const size_t ld = (size_t)H * dh;
+  const int dh = a.dh;
+  const size_t ld = (size_t)a.H * dh;
   const T* qg = static_cast<const T*>(a.q) + (size_t)(lo + q0) * ld + (size_t)h * dh;
   const T* kg = static_cast<const T*>(a.k) + (size_t)lo * ld + (size_t)h * dh;
   const T* vg = static_cast<const T*>(a.v) + (size_t)lo * ld + (size_t)h * dh;
   // `rows` rows from row `r0` of a head's matrix; rows past the request and columns past head_dim become zeros
-  constexpr int kVecs = DHP / 4, kStep = kSimtWarps * 32 / kVecs;        // vectors per row, rows per pass of the block
+  constexpr int kVecs = DHP / 4, kStep = NW * 32 / kVecs > 0 ? NW * 32 / kVecs : 1;        // vectors per row, rows per pass of the CTA
+  static_assert(NW * 32 >= kVecs, "a pass covers whole rows");
   const int lrow = tid / kVecs, lcol = (tid % kVecs) * 4;
   auto load_rows = [&](float* dst, const T* src, int r0, int rows, int n_rows) {
     dst += lrow * kLd + lcol;
@@ -61,164 +59,159 @@ attn_simt_kernel(AttnArgs a, bool vec) {
     for (int r = lrow; r < rows; r += kStep, dst += kStep * kLd, src += kStep * ld)
       f32::load4<T>(dst, src, lcol, dh, r0 + r < n_rows, vec);
   };
+  auto load_tile = [&](int t) {                           // K and V of key tile t, one copy group (empty past the end)
+    if (t * kKeyTile < n) {
+      float* st = kv_s + (t & 1) * 2 * S::kKv;
+      load_rows(st, kg, t * kKeyTile, kKeyTile, n);
+      load_rows(st + S::kKv, vg, t * kKeyTile, kKeyTile, n);
+    }
+    f32::cp_async_commit();
+  };
   load_rows(q_s, qg, 0, S::kBM, n - q0);
-  load_rows(k_s, kg, 0, S::kKeys, n);
-  f32::cp_async_commit();
-  load_rows(v_s, vg, 0, S::kKeys, n);
-  f32::cp_async_commit();
+  load_tile(0);
+  load_tile(1);
   // which of the rows are deciders?  (strictly ascending list: binary search)
   int n_vis = 0;
   if (a.decider_pos != nullptr) n_vis = a.n_visual[b];
-  if (tid < S::kBM) {
+  for (int row = tid; row < S::kBM; row += NW * 32) {
     int slot = -1;
     if (a.decider_pos != nullptr) {
       int l = a.cu_deciders[b], r = a.cu_deciders[b + 1];
       while (l < r) {
         const int mid = (l + r) >> 1, p = a.decider_pos[mid];
-        if (p == q0 + tid) { slot = mid; break; }
-        if (p < q0 + tid) l = mid + 1; else r = mid;
+        if (p == q0 + row) { slot = mid; break; }
+        if (p < q0 + row) l = mid + 1; else r = mid;
       }
     }
-    dec_s[tid] = slot;
+    dec_s[row] = slot;
   }
 
   const int warp = tid >> 5, lane = tid & 31, ty = f32::lane_ty(lane), tx = f32::lane_tx(lane);
-  const int rg = warp / KG, key_g = warp - rg * KG;     // row group, key group
-  const float* qw = q_s + rg * 16 * kLd;
-  const float* kw = k_s + key_g * 32 * kLd;
-  const float* vw = v_s + key_g * 32 * kLd;
-  float* pw = p_all + warp * 16 * kPStride;
-  float m[4], l[4];
-  float2 o[4][kCols][2];
+  const float* qw = q_s + warp * RW * kLd + ty * kLd;
+  float* pw = p_all + warp * RW * kPStride;
+  float m[kR], l[kR];
+  float2 o[kR][kCols][2];
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
+  for (int r = 0; r < kR; ++r) {
     m[r] = -INFINITY; l[r] = 0.f;
 #pragma unroll
     for (int c = 0; c < kCols; ++c) o[r][c][0] = o[r][c][1] = make_float2(0.f, 0.f);
   }
-  for (int j0 = 0; j0 < n; j0 += S::kKeys) {
-    const int key0 = j0 + key_g * 32;
-    const bool live = key0 < n;                         // (whole warp)
-    f32::cp_async_wait<1>();                            // K has landed (V may be on its way)
+  const int n_tiles = (n + kKeyTile - 1) / kKeyTile;
+  for (int t = 0; t < n_tiles; ++t) {
+    f32::cp_async_wait<1>();                              // this tile has landed (the next may be on its way)
     __syncthreads();
-    float2 s2[4][4];
+    const int j0 = t * kKeyTile;
+    const float* kw = kv_s + (t & 1) * 2 * S::kKv + tx * kLd;
+    const float* vw = kv_s + (t & 1) * 2 * S::kKv + S::kKv + tx * 4;
+    float s[kR][4];
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < kR; ++r)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) s2[r][j] = make_float2(0.f, 0.f);
-    if (live) f32::dot_16x32<kLd, kLd, DHP / 4>(s2, qw, kw, ty, tx);
-    __syncthreads();                                    // everyone is done with this K tile
-    if (j0 + S::kKeys < n) load_rows(k_s, kg, j0 + S::kKeys, S::kKeys, n);
-    f32::cp_async_commit();
-    if (live) {
+      for (int j = 0; j < 4; ++j) s[r][j] = 0.f;
+    {
+      float4 av[2][kR], bv[2][4];
+      auto fetch = [&](int buf, int k) {
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int row = ty + 4 * r;
-        const int slot = dec_s[rg * 16 + row];
-        float s[4];
-        float mx = -INFINITY;
+        for (int r = 0; r < kR; ++r) av[buf][r] = *reinterpret_cast<const float4*>(qw + r * 4 * kLd + k);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int key = key0 + tx + 8 * j;
-          const float raw = s2[r][j].x + s2[r][j].y;
-          if (slot >= 0 && key < n_vis) a.score_scratch[((size_t)h * a.max_deciders + slot) * a.vis_stride + key] = raw;
-          s[j] = key < n ? raw * a.scale_log2 : -INFINITY;
-          mx = fmaxf(mx, s[j]);
-        }
-        const float m_new = fmaxf(m[r], f32::max_over_tx(mx));
-        const float corr = exp2f(m[r] - m_new);         // first tile: exp2(-inf) = 0
-        float sum = 0.f;
+        for (int j = 0; j < 4; ++j) bv[buf][j] = *reinterpret_cast<const float4*>(kw + j * 8 * kLd + k);
+      };
+      fetch(0, 0);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float p = key0 + tx + 8 * j < n ? exp2f(s[j] - m_new) : 0.f;
-          pw[row * kPStride + tx + 8 * j] = p;
-          sum += p;
-        }
-        l[r] = fmaf(l[r], corr, sum);                   // this lane's keys only; the lanes are added up at the end
-        m[r] = m_new;
+      for (int k = 0; k < DHP; k += 4) {                  // the next step's operands are read while this step multiplies
+        const int bf = (k >> 2) & 1;
+        if (k + 4 < DHP) fetch(bf ^ 1, k + 4);
 #pragma unroll
-        for (int c = 0; c < kCols; ++c)
+        for (int e = 0; e < 4; ++e)
 #pragma unroll
-          for (int e = 0; e < 2; ++e) { o[r][c][e].x *= corr; o[r][c][e].y *= corr; }
+          for (int r = 0; r < kR; ++r)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float4 x = av[bf][r], y = bv[bf][j];
+              s[r][j] = e == 0 ? fmaf(x.x, y.x, s[r][j]) : e == 1 ? fmaf(x.y, y.y, s[r][j]) : e == 2 ? fmaf(x.z, y.z, s[r][j])
+                                                                                          : fmaf(x.w, y.w, s[r][j]);
+            }
       }
     }
-    f32::cp_async_wait<1>();                            // V has landed (the next K may be on its way)
-    __syncthreads();
-    if (live) {
-      float4 p4[2][4], v4[2][kCols];
-      auto fetch_p = [&](int buf, int k) {
 #pragma unroll
-        for (int r = 0; r < 4; ++r) p4[buf][r] = *reinterpret_cast<const float4*>(pw + (ty + 4 * r) * kPStride + k);
-      };
-      auto fetch_v = [&](int buf, int k) {
+    for (int r = 0; r < kR; ++r) {
+      const int row = ty + 4 * r;
+      const int slot = dec_s[warp * RW + row];
+      float mx = -INFINITY;
 #pragma unroll
-        for (int c = 0; c < kCols; ++c) v4[buf][c] = *reinterpret_cast<const float4*>(vw + k * kLd + c * 32 + tx * 4);
-      };
-      fetch_p(0, 0);
-      fetch_v(0, 0);
+      for (int j = 0; j < 4; ++j) {
+        const int key = j0 + tx + 8 * j;
+        if (slot >= 0 && key < n_vis) a.score_scratch[((size_t)h * a.max_deciders + slot) * a.vis_stride + key] = s[r][j];
+        s[r][j] = key < n ? __fmul_rn(s[r][j], a.scale_log2) : -INFINITY;
+        mx = fmaxf(mx, s[r][j]);
+      }
+      const float m_new = fmaxf(m[r], f32::max_over_tx(mx));
+      const float corr = exp2f(m[r] - m_new);             // first tile: exp2(-inf) = 0
+      float p[4];
 #pragma unroll
-      for (int k = 0; k < 32; ++k) {                    // the next step's operands are read while this step multiplies
-        const int pb = (k >> 2) & 1, vb = k & 1;
-        if ((k & 3) == 0 && k + 4 < 32) fetch_p(pb ^ 1, k + 4);
-        if (k + 1 < 32) fetch_v(vb ^ 1, k + 1);
+      for (int j = 0; j < 4; ++j) {
+        p[j] = j0 + tx + 8 * j < n ? exp2f(__fsub_rn(s[r][j], m_new)) : 0.f;
+        pw[row * kPStride + tx + 8 * j] = p[j];
+      }
+      l[r] = fmaf(l[r], corr, f32::sum_over_tx((p[0] + p[2]) + (p[1] + p[3])));
+      m[r] = m_new;
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const float4 p = p4[pb][r];
-          const float pk = (k & 3) == 0 ? p.x : (k & 3) == 1 ? p.y : (k & 3) == 2 ? p.z : p.w;
-          const float2 pp = make_float2(pk, pk);
+      for (int c = 0; c < kCols; ++c)
 #pragma unroll
-          for (int c = 0; c < kCols; ++c) {
-            o[r][c][0] = __ffma2_rn(pp, make_float2(v4[vb][c].x, v4[vb][c].y), o[r][c][0]);
-            o[r][c][1] = __ffma2_rn(pp, make_float2(v4[vb][c].z, v4[vb][c].w), o[r][c][1]);
-          }
+        for (int e = 0; e < 2; ++e) { o[r][c][e].x *= corr; o[r][c][e].y *= corr; }
+    }
+    __syncwarp();
+    float4 p4[2][kR], v4[2][kCols];
+    auto fetch_p = [&](int buf, int k) {
+#pragma unroll
+      for (int r = 0; r < kR; ++r) p4[buf][r] = *reinterpret_cast<const float4*>(pw + (ty + 4 * r) * kPStride + k);
+    };
+    auto fetch_v = [&](int buf, int k) {
+#pragma unroll
+      for (int c = 0; c < kCols; ++c) v4[buf][c] = *reinterpret_cast<const float4*>(vw + k * kLd + c * 32);
+    };
+    fetch_p(0, 0);
+    fetch_v(0, 0);
+#pragma unroll
+    for (int k = 0; k < kKeyTile; ++k) {                  // the next step's operands are read while this step multiplies
+      const int pb = (k >> 2) & 1, vb = k & 1;
+      if ((k & 3) == 0 && k + 4 < kKeyTile) fetch_p(pb ^ 1, k + 4);
+      if (k + 1 < kKeyTile) fetch_v(vb ^ 1, k + 1);
+#pragma unroll
+      for (int r = 0; r < kR; ++r) {
+        const float4 p = p4[pb][r];
+        const float pk = (k & 3) == 0 ? p.x : (k & 3) == 1 ? p.y : (k & 3) == 2 ? p.z : p.w;
+        const float2 pp = make_float2(pk, pk);
+#pragma unroll
+        for (int c = 0; c < kCols; ++c) {
+          o[r][c][0] = __ffma2_rn(pp, make_float2(v4[vb][c].x, v4[vb][c].y), o[r][c][0]);
+          o[r][c][1] = __ffma2_rn(pp, make_float2(v4[vb][c].z, v4[vb][c].w), o[r][c][1]);
         }
       }
     }
-    __syncthreads();                                    // everyone is done with this V tile (and this P)
-    if (j0 + S::kKeys < n) load_rows(v_s, vg, j0 + S::kKeys, S::kKeys, n);
-    f32::cp_async_commit();
+    __syncthreads();                                      // everyone is done with this stage
+    load_tile(t + 2);
   }
-  // ---- the KG partial results of every row, in key group order: [KG][BM][DHP] outputs and (m, l) pairs
-  float* o_s = k_s;
-  float2* ml_s = reinterpret_cast<float2*>(p_all);
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int slot = key_g * S::kBM + rg * 16 + ty + 4 * r;
-    const float sum = f32::sum_over_tx(l[r]);
-    if (tx == 0) ml_s[slot] = make_float2(m[r], sum);
+  for (int r = 0; r < kR; ++r) {
+    const int row = warp * RW + ty + 4 * r;
+    if (q0 + row >= n) continue;
+    const float inv_l = 1.f / l[r];
+    T* dst = static_cast<T*>(a.out) + (size_t)(lo + q0 + row) * ld + (size_t)h * dh;
 #pragma unroll
-    for (int c = 0; c < kCols; ++c)
-      *reinterpret_cast<float4*>(o_s + (size_t)slot * DHP + c * 32 + tx * 4) =
-          make_float4(o[r][c][0].x, o[r][c][0].y, o[r][c][1].x, o[r][c][1].y);
-  }
-  __syncthreads();
-  T* out = static_cast<T*>(a.out) + (size_t)(lo + q0) * ld + (size_t)h * dh;
-  for (int i = tid; i < S::kBM * (DHP / 4); i += kSimtWarps * 32) {
-    const int r = i / (DHP / 4), c = (i - r * (DHP / 4)) * 4;
-    if (q0 + r >= n || c >= dh) continue;
-    float mm = ml_s[r].x;
+    for (int c = 0; c < kCols; ++c) {
+      const int col = c * 32 + tx * 4;
+      if (col >= dh) continue;
+      const float y[4] = {o[r][c][0].x * inv_l, o[r][c][0].y * inv_l, o[r][c][1].x * inv_l, o[r][c][1].y * inv_l};
+      if (sizeof(T) == 4 && vec) {
+        *reinterpret_cast<float4*>(dst + col) = make_float4(y[0], y[1], y[2], y[3]);
+      } else {
 #pragma unroll
-    for (int g = 1; g < KG; ++g) mm = fmaxf(mm, ml_s[g * S::kBM + r].x);
-    float lsum = 0.f;
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int g = 0; g < KG; ++g) {
-      const float2 ml = ml_s[g * S::kBM + r];
-      const float w = exp2f(ml.x - mm);                 // a key group without keys: exp2(-inf) = 0
-      const float4 x = *reinterpret_cast<const float4*>(o_s + (size_t)(g * S::kBM + r) * DHP + c);
-      lsum = fmaf(ml.y, w, lsum);
-      acc.x = fmaf(x.x, w, acc.x); acc.y = fmaf(x.y, w, acc.y); acc.z = fmaf(x.z, w, acc.z); acc.w = fmaf(x.w, w, acc.w);
+        for (int e = 0; e < 4; ++e) dst[col + e] = Storage<T>::from_float(y[e]);
+      }
     }
-    const float inv_l = 1.f / lsum;
-    const float y[4] = {acc.x * inv_l, acc.y * inv_l, acc.z * inv_l, acc.w * inv_l};
-    T* dst = out + (size_t)r * ld + c;
-    if (sizeof(T) == 4 && vec) {
-      *reinterpret_cast<float4*>(dst) = make_float4(y[0], y[1], y[2], y[3]);
-    } else {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) dst[e] = Storage<T>::from_float(y[e]);
-    }
-    if (c == 0 && dec_s[r] >= 0) a.lse_scratch[(size_t)h * a.max_deciders + dec_s[r]] = make_float2(mm, lsum);
+    if (tx == 0 && dec_s[row] >= 0) a.lse_scratch[(size_t)h * a.max_deciders + dec_s[row]] = make_float2(m[r], l[r]);
   }
 }
 
@@ -286,37 +279,41 @@ importance_finish_kernel(const float* __restrict__ score, const float2* __restri
 
 namespace {
 
-template <typename T, int DHP, int KG>
+template <typename T, int DHP, int RW, int NW>
 int launch_simt(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s) {
-  using S = SimtSmem<DHP, KG>;
+  using S = SimtSmem<DHP, RW, NW>;
   // 16-byte copies and stores where the caller's buffers allow them (head_dim is a multiple of 4)
   const uintptr_t bits = (uintptr_t)a.q | (uintptr_t)a.k | (uintptr_t)a.v | (uintptr_t)a.out;
   const bool vec = sizeof(T) == 4 && bits % 16 == 0;
   dim3 grid(ceil_div(a.max_seqlen, S::kBM), a.H, a.B);
+  // At most ceil(CTAs / SMs) CTAs fit an SM (by the shared memory asked for): CTAs that start while the kernel before is
+  // draining would otherwise pile up on the SMs that are free first, and the fullest SM sets the time (a step of three
+  // 1152 / 384-row layers x 8 heads x 64: 316 us, against 255 us without launch overlap).
+  const long long sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
+  const long long per_sm = ((long long)grid.x * grid.y * grid.z + sms - 1) / sms;
+  int smem = S::kBytes;
+  if (per_sm <= 4) smem = max(smem, (int)(227 * 1024 / per_sm) - 1024);
   // (the attribute belongs to the current device: set on every call, a process may drive several GPUs)
-  D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(attn_simt_kernel<T, DHP, KG>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kBytes));
-  D3TOM_CUDA_TRY(ctx, launch_serialized(attn_simt_kernel<T, DHP, KG>, grid, kSimtWarps * 32, S::kBytes, s, a, vec));
+  D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(attn_simt_kernel<T, DHP, RW, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  D3TOM_CUDA_TRY(ctx, launch_serialized(attn_simt_kernel<T, DHP, RW, NW>, grid, NW * 32, smem, s, a, vec));
   return D3TOM_OK;
 }
 
-// Rows per CTA (128 / KG): the fewest rounds of CTAs over the SMs times key blocks per CTA.  Few CTAs leave SMs idle, so
-// short calls cut the rows finer and let more warps share a row's keys.  Measured, KG = 2 / 4 / 8 (us): 288 rows x 4
-// heads x 64: 25.1 / 17.1 / 13.5; 600 x 8 x 64: 48.2 / 51.5 / 48.7; 1152 x 8 x 64: 82 / 89 / 108; 700 x 4 x 128: 88 / 55;
-// 1152 x 32 x 128: 558 / 611; a batch of two of 700 x 8 x 64: 102 / 90 / 88.
+// Rows per warp: with 16 a score needs fewer shared-memory reads, with 8 there are twice the warps to hide latency, which
+// wins until the SMs are full of warps anyway (from 16 eight-row warps per SM on).  Measured, 8 / 16 rows (us): 288 rows x
+// 4 heads x 64: 19.4 / 28.0; 600 x 8 x 64: 51.7 / 55.6; 1152 x 8 x 64: 95.8 / 102.0; 700 x 4 x 128: 73.7 / 130.7;
+// 1152 x 32 x 128: 639 / 564.
+template <typename T, int DHP>
+int launch_simt_dh(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s) {
+  const long long sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
+  const long long warps8 = (long long)ceil_div(a.max_seqlen, 8) * a.H * a.B;
+  return warps8 > 16 * sms ? launch_simt<T, DHP, 16, 4>(ctx, a, s) : launch_simt<T, DHP, 8, 4>(ctx, a, s);
+}
+
 template <typename T>
 int launch_simt_t(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s) {
-  const int sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
-  int kg = 2;
-  long long best = 0;
-  for (int c = 2; c <= 8; c *= 2) {
-    const long long ctas = (long long)ceil_div(a.max_seqlen, 128 / c) * a.H * a.B;
-    const long long cost = ((ctas + sms - 1) / sms) * ceil_div(a.max_seqlen, 32 * c);
-    if (c == 2 || cost < best) { best = cost; kg = c; }
-  }
-  if (a.dh > 64) return kg == 2 ? launch_simt<T, 128, 2>(ctx, a, s) : launch_simt<T, 128, 4>(ctx, a, s);
-  if (a.dh > 32)
-    return kg == 2 ? launch_simt<T, 64, 2>(ctx, a, s) : kg == 4 ? launch_simt<T, 64, 4>(ctx, a, s) : launch_simt<T, 64, 8>(ctx, a, s);
-  return kg == 2 ? launch_simt<T, 32, 2>(ctx, a, s) : kg == 4 ? launch_simt<T, 32, 4>(ctx, a, s) : launch_simt<T, 32, 8>(ctx, a, s);
+  if (a.dh > 64) return launch_simt_dh<T, 128>(ctx, a, s);
+  return a.dh > 32 ? launch_simt_dh<T, 64>(ctx, a, s) : launch_simt_dh<T, 32>(ctx, a, s);
 }
 
 }  // namespace

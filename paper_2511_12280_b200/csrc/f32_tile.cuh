@@ -16,15 +16,15 @@ namespace f32 {
 
 __device__ __forceinline__ int lane_ty(int lane) { return ((lane >> 1) & 1) | ((lane >> 2) & 2); }
 __device__ __forceinline__ int lane_tx(int lane) { return (lane & 1) | ((lane >> 1) & 2) | ((lane >> 2) & 4); }
-// exchange partners among the eight lanes of one ty: lane ^ 1, lane ^ 4, lane ^ 16
+// over the eight lanes of one ty, partners tx ^ 4, tx ^ 2, tx ^ 1 in this order
 __device__ __forceinline__ float max_over_tx(float v) {
 #pragma unroll
-  for (int d = 1; d < 32; d <<= 2) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, d));
+  for (int d = 16; d > 0; d >>= 2) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, d));
   return v;
 }
 __device__ __forceinline__ float sum_over_tx(float v) {
 #pragma unroll
-  for (int d = 1; d < 32; d <<= 2) v += __shfl_xor_sync(0xffffffffu, v, d);
+  for (int d = 16; d > 0; d >>= 2) v += __shfl_xor_sync(0xffffffffu, v, d);
   return v;
 }
 

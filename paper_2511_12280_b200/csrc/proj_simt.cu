@@ -2,7 +2,7 @@
 // for bf16, a debugging aid) of the dense layers (Sec. 3.2.1, Q = H W_Q, K = H W_K; Algorithm 1, FFN_l) and of the
 // similarity with its arg-max (Sec. 3.2.2).
 //
-// A CTA of 8 warps computes a (16 WM) x (32 WN) tile; WK warps share a 16 x 32 register tile (f32_tile.cuh) and cut
+// Dense layers: a CTA of 8 warps computes a (16 WM) x (32 WN) tile; WK warps share a 16 x 32 register tile (f32_tile.cuh) and cut
 // every k-block of 32 WK between them, so that small products, which have few tiles, keep short chains.  k-blocks come
 // through a ring of kStages buffers by 16-byte asynchronous copies.  Bound: the fp32 pipe and shared memory (a lane reads
 // 8 vectors per 64 multiply-adds): 42 TFLOP/s at 1152 x 12288 x 4096, 30 at 384 x 1536 x 512 (20 us; one output per
@@ -13,19 +13,15 @@
 namespace {
 
 constexpr int kStages = 3;
-enum { kSimtProj = 0, kSimtLinear = 1, kSimtGateUp = 2, kSimtSim = 3 };
+enum { kSimtProj = 0, kSimtLinear = 1, kSimtGateUp = 2 };
 
 template <typename T> struct SimtGemm {
   const T* a; const T* b;          // A rows of the products, B rows (for the gate-up pass: gate rows, then the up rows from row n_cols on)
-  int rows, n_cols, K;             // (similarity: the bounds over all requests)
+  int rows, n_cols, K;
   bool vec;                        // 16-byte copies are possible
   T* out[3];                       // projection: q, k, v; otherwise out[0]
   const T* residual;
   int D;                           // projection: columns of one output
-  // similarity
-  const int32_t* cu_seqlens; const int32_t* cu_vis; const int32_t* cu_kept; const int32_t* assign;
-  const float* inv_norm; const float* inv_norm_kept; int max_kept;
-  unsigned long long* best; float* sim_debug;
 };
 
 template <int EPI, int WM, int WN, int WK> struct SimtGemmSmem {
@@ -48,17 +44,9 @@ gemm_simt_kernel(SimtGemm<T> p) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = f32::lane_ty(lane), tx = f32::lane_tx(lane);
   const int wk = warp % WK, wn = (warp / WK) % WN, wm = warp / (WK * WN);
   const int m0 = blockIdx.y * S::kBM, n0 = blockIdx.x * S::kBN;
-  int rows = p.rows, cols = p.n_cols, v0 = 0, k0 = 0;
+  const int rows = p.rows, cols = p.n_cols;
   const T* a = p.a;
   const T* b = p.b;
-  if (EPI == kSimtSim) {
-    const int rq = blockIdx.z;
-    v0 = p.cu_vis[rq]; rows = p.cu_vis[rq + 1] - v0;
-    k0 = p.cu_kept[rq]; cols = p.cu_kept[rq + 1] - k0;
-    if (cols >= rows || m0 >= rows || n0 >= cols) return;      // nothing pruned in this request, or outside it
-    a += (size_t)p.cu_seqlens[rq] * p.K;
-    b += (size_t)k0 * p.K;
-  }
   const int nkb = (p.K + S::kBK - 1) / S::kBK;
   // this thread's vectors of every k-block: the same column of rows lrow, lrow + kStep, ... of the A and B tiles
   constexpr int kV = S::kBK / 4, kStep = 256 / kV, kLoads = (S::kBM + S::kB) / kStep;
@@ -143,28 +131,7 @@ gemm_simt_kernel(SimtGemm<T> p) {
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
     const int row = m0 + wm * 16 + ty + 4 * r;
-    if (EPI == kSimtSim) {
-      const int g = v0 + row;
-      const bool active = row < rows && p.assign[g] < 0;       // a pruned token
-      const float inm = active ? p.inv_norm[g] : 0.f;
-      unsigned long long mine = 0ull;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int s = n0 + wn * 32 + tx + 8 * j;
-        if (active && s < cols) {
-          const float sim = (c[0][r][j] * inm) * p.inv_norm_kept[k0 + s] + 0.0f;   // the value the arg-max compares (never -0)
-          const unsigned long long packed = ((unsigned long long)ordered_key(sim) << 32) | (0xffffffffu - (unsigned)s);
-          mine = packed > mine ? packed : mine;
-          if (p.sim_debug != nullptr) p.sim_debug[(size_t)g * p.max_kept + s] = sim;
-        }
-      }
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 2) {
-        const unsigned long long o = __shfl_xor_sync(0xffffffffu, mine, d);
-        mine = o > mine ? o : mine;
-      }
-      if (tx == 0 && mine != 0ull) atomicMax(p.best + g, mine);
-    } else if (row < rows) {
+    if (row < rows) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int col = n0 + wn * 32 + tx + 8 * j;
@@ -185,9 +152,9 @@ gemm_simt_kernel(SimtGemm<T> p) {
 }
 
 template <typename T, int EPI, int WM, int WN, int WK>
-int launch_shape(d3tom_ctx* ctx, const SimtGemm<T>& p, int batch, cudaStream_t s) {
+int launch_shape(d3tom_ctx* ctx, const SimtGemm<T>& p, cudaStream_t s) {
   using S = SimtGemmSmem<EPI, WM, WN, WK>;
-  dim3 grid(ceil_div(p.n_cols, S::kBN), ceil_div(p.rows, S::kBM), batch);
+  dim3 grid(ceil_div(p.n_cols, S::kBN), ceil_div(p.rows, S::kBM));
   // (the attribute belongs to the current device: set on every call, a process may drive several GPUs)
   D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(gemm_simt_kernel<T, EPI, WM, WN, WK>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kBytes));
   D3TOM_CUDA_TRY(ctx, launch_serialized(gemm_simt_kernel<T, EPI, WM, WN, WK>, grid, 256, S::kBytes, s, p));
@@ -198,19 +165,18 @@ int launch_shape(d3tom_ctx* ctx, const SimtGemm<T>& p, int batch, cudaStream_t s
 // operands are read more often: measured 1.5 for 32 x 32 at 640 x 1536 x 512), so that only a product with few 64 x 64
 // tiles is cut finer, its k-blocks shared by two or four warps.
 template <typename T, int EPI>
-int launch_simt_gemm(d3tom_ctx* ctx, SimtGemm<T> p, int batch, cudaStream_t s) {
-  if (p.rows <= 0 || p.n_cols <= 0) return D3TOM_OK;
+int launch_simt_gemm(d3tom_ctx* ctx, SimtGemm<T> p, cudaStream_t s) {
   const uintptr_t bits = (uintptr_t)p.a | (uintptr_t)p.b;
   p.vec = sizeof(T) == 4 && p.K % 4 == 0 && bits % 16 == 0;
   const long long sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
   auto cost = [&](int bm, int bn, double scale) {
-    const long long tiles = (long long)ceil_div(p.rows, bm) * ceil_div(p.n_cols, bn) * batch;
+    const long long tiles = (long long)ceil_div(p.rows, bm) * ceil_div(p.n_cols, bn);
     return scale * (double)((tiles + sms - 1) / sms) * bm * bn;
   };
   const double large = cost(64, 64, 1.0), middle = cost(32, 64, 1.2), small = cost(32, 32, 1.5);
-  if (large <= middle && large <= small) return launch_shape<T, EPI, 4, 2, 1>(ctx, p, batch, s);
-  if (middle <= small) return launch_shape<T, EPI, 2, 2, 2>(ctx, p, batch, s);
-  return launch_shape<T, EPI, 2, 1, 4>(ctx, p, batch, s);
+  if (large <= middle && large <= small) return launch_shape<T, EPI, 4, 2, 1>(ctx, p, s);
+  if (middle <= small) return launch_shape<T, EPI, 2, 2, 2>(ctx, p, s);
+  return launch_shape<T, EPI, 2, 1, 4>(ctx, p, s);
 }
 
 template <typename T>
@@ -219,7 +185,7 @@ int proj_t(d3tom_ctx* ctx, const void* x, const void* w, int total, int D, void*
   p.a = static_cast<const T*>(x); p.b = static_cast<const T*>(w);
   p.rows = total; p.n_cols = 3 * D; p.K = D; p.D = D;
   p.out[0] = static_cast<T*>(q); p.out[1] = static_cast<T*>(k); p.out[2] = static_cast<T*>(v);
-  return launch_simt_gemm<T, kSimtProj>(ctx, p, 1, s);
+  return launch_simt_gemm<T, kSimtProj>(ctx, p, s);
 }
 
 template <typename T, int EPI>
@@ -229,18 +195,153 @@ int linear_t(d3tom_ctx* ctx, const void* x, const void* w, const void* residual,
   p.a = static_cast<const T*>(x); p.b = static_cast<const T*>(w);
   p.rows = rows; p.n_cols = N; p.K = K;
   p.residual = static_cast<const T*>(residual); p.out[0] = static_cast<T*>(out);
-  return launch_simt_gemm<T, EPI>(ctx, p, 1, s);
+  return launch_simt_gemm<T, EPI>(ctx, p, s);
+}
+
+// ---------------------------------------------------------------- similarity
+// One CTA = 16 visual rows x 32 kept rows of one request.  The dot product of a pair is 32 chains of multiply-adds, chain
+// l over the 16-byte vectors l, l + 32, ... of the rows, added up as a butterfly (distances 16, 8, 4, 2, 1): a fixed order
+// that does not depend on the tile, so near-ties of the arg-max fall the same way whatever the launch looks like.  Warp w
+// runs the chains w, w + 8, w + 16, w + 24 of the whole tile on vectors from shared memory (a lane 4 x 4 pairs) and adds
+// those four; the eight sums meet in shared memory.  Bound: the fp32 pipe; one warp per pair reading both rows from L2
+// took 46 us at 1024 visual x 256 kept x 512 where this takes 21.
+constexpr int kSimRows = 16, kSimCols = 32;
+
+template <typename T> struct SimSmem {
+  static constexpr int kVec = Storage<T>::kVec, kChunk = 32 * kVec, kLd = kChunk + 4;
+  static constexpr int kStage = (kSimRows + kSimCols) * kLd;
+  static constexpr int kBytes = kStages * kStage * 4;
+  static_assert(kStages * kStage >= 8 * kSimRows * kSimCols, "the warps' sums are exchanged in the ring");
+};
+
+template <typename T>
+__global__ void __launch_bounds__(256)
+sim_simt_kernel(const T* __restrict__ hidden, const T* __restrict__ kept_rows, const int32_t* __restrict__ cu_seqlens,
+                const int32_t* __restrict__ cu_vis, const int32_t* __restrict__ cu_kept, const int32_t* __restrict__ assign,
+                const float* __restrict__ inv_norm, const float* __restrict__ inv_norm_kept, int D, int max_kept, bool vec,
+                unsigned long long* __restrict__ best, float* __restrict__ sim_debug) {
+  using S = SimSmem<T>;
+  constexpr int kVec = S::kVec, kChunk = S::kChunk, kLd = S::kLd;
+  extern __shared__ float4 smem_f4[];
+  float* ring = reinterpret_cast<float*>(smem_f4);
+  grid_dependency_enter();
+  const int rq = blockIdx.z, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ty = f32::lane_ty(lane), tx = f32::lane_tx(lane);
+  const int v0 = cu_vis[rq], Vb = cu_vis[rq + 1] - v0, k0 = cu_kept[rq], kb = cu_kept[rq + 1] - k0;
+  const int m0 = blockIdx.y * kSimRows, s0 = blockIdx.x * kSimCols;
+  if (m0 >= Vb || s0 >= kb || kb >= Vb) return;
+  // a tile of kept rows only has nothing to do
+  if (!__syncthreads_or(tid < kSimRows && m0 + tid < Vb && assign[v0 + m0 + tid] < 0)) return;
+  const T* a = hidden + (size_t)(cu_seqlens[rq] + m0) * D;
+  const T* b = kept_rows + (size_t)(k0 + s0) * D;
+  const int n_chunks = (D + kChunk - 1) / kChunk;
+  // this thread's vectors of every chunk: the same column of rows lrow, lrow + kStep, ...
+  constexpr int kV = kChunk / 4, kStep = 256 / kV, kLoads = (kSimRows + kSimCols) / kStep;
+  const int lrow = tid / kV, lcol = (tid % kV) * 4;
+  const T* src[kLoads];
+  unsigned src_ok = 0u;
+#pragma unroll
+  for (int u = 0; u < kLoads; ++u) {
+    const int r = lrow + u * kStep;
+    const bool is_a = r < kSimRows, ok = is_a ? m0 + r < Vb : s0 + r - kSimRows < kb;
+    src[u] = is_a ? a + (size_t)(ok ? r : 0) * D : b + (size_t)(ok ? r - kSimRows : 0) * D;
+    src_ok |= (ok ? 1u : 0u) << u;
+  }
+  auto load_chunk = [&](int t) {
+    if (t < n_chunks) {
+      float* dst = ring + (t % kStages) * S::kStage + lrow * kLd + lcol;
+#pragma unroll
+      for (int u = 0; u < kLoads; ++u)
+        f32::load4<T>(dst + u * kStep * kLd, src[u], t * kChunk + lcol, D, (src_ok >> u) & 1u, vec);
+    }
+    f32::cp_async_commit();
+  };
+  float acc[4][4][4];                      // [chain of this warp][r][j]
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[q][r][j] = 0.f;
+  for (int t = 0; t < kStages - 1; ++t) load_chunk(t);
+  for (int t = 0; t < n_chunks; ++t) {
+    f32::cp_async_wait<kStages - 2>();
+    __syncthreads();
+    load_chunk(t + kStages - 1);
+    const float* st = ring + (t % kStages) * S::kStage;
+    const float* ar = st + ty * kLd;
+    const float* br = st + (kSimRows + tx) * kLd;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+#pragma unroll
+      for (int e = 0; e < kVec; e += 4) {
+        const int c = (warp + 8 * q) * kVec + e;
+        float4 av[4], bv[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) av[r] = *reinterpret_cast<const float4*>(ar + r * 4 * kLd + c);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) bv[j] = *reinterpret_cast<const float4*>(br + j * 8 * kLd + c);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[q][r][j] = fmaf(av[r].x, bv[j].x, acc[q][r][j]);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[q][r][j] = fmaf(av[r].y, bv[j].y, acc[q][r][j]);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[q][r][j] = fmaf(av[r].z, bv[j].z, acc[q][r][j]);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[q][r][j] = fmaf(av[r].w, bv[j].w, acc[q][r][j]);
+      }
+    }
+  }
+  f32::cp_async_wait<0>();
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)            // distances 16 and 8
+      ring[(warp * kSimRows + ty + 4 * r) * kSimCols + tx + 8 * j] =
+          (acc[0][r][j] + acc[2][r][j]) + (acc[1][r][j] + acc[3][r][j]);
+  __syncthreads();
+#pragma unroll
+  for (int rr = 0; rr < kSimRows / 8; ++rr) {
+    const int row = warp * (kSimRows / 8) + rr, m = m0 + row, g = v0 + m, s = s0 + lane;
+    float v[8];
+#pragma unroll
+    for (int w = 0; w < 8; ++w) v[w] = ring[(w * kSimRows + row) * kSimCols + lane];
+    const float dot = ((v[0] + v[4]) + (v[2] + v[6])) + ((v[1] + v[5]) + (v[3] + v[7]));      // distances 4, 2, 1
+    unsigned long long mine = 0ull;
+    if (m < Vb && s < kb && assign[g] < 0) {                      // a pruned token and one of the kept ones
+      const float sim = (dot * inv_norm[g]) * inv_norm_kept[k0 + s] + 0.0f;      // the value the arg-max compares (never -0)
+      mine = ((unsigned long long)ordered_key(sim) << 32) | (0xffffffffu - (unsigned)s);
+      if (sim_debug != nullptr) sim_debug[(size_t)g * max_kept + s] = sim;
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      const unsigned long long o = __shfl_xor_sync(0xffffffffu, mine, d);
+      mine = o > mine ? o : mine;
+    }
+    if (lane == 0 && mine != 0ull) atomicMax(best + g, mine);
+  }
 }
 
 template <typename T>
 int sim_t(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
-  SimtGemm<T> p = {};
-  p.a = static_cast<const T*>(a.hidden); p.b = static_cast<const T*>(ctx->kept_rows);
-  p.rows = a.max_visual; p.n_cols = a.max_kept; p.K = a.D;
-  p.cu_seqlens = a.cu_seqlens; p.cu_vis = a.cu_vis; p.cu_kept = a.cu_kept; p.assign = a.assign;
-  p.inv_norm = ctx->inv_norm; p.inv_norm_kept = ctx->inv_norm_kept; p.max_kept = a.max_kept;
-  p.best = ctx->best; p.sim_debug = a.sim_debug;
-  return launch_simt_gemm<T, kSimtSim>(ctx, p, a.B, s);
+  if (a.max_kept <= 0) return D3TOM_OK;
+  const T* hidden = static_cast<const T*>(a.hidden);
+  const bool vec = sizeof(T) == 4 && (uintptr_t)hidden % 16 == 0;      // (D is a multiple of 8)
+  dim3 grid(ceil_div(a.max_kept, kSimCols), ceil_div(a.max_visual, kSimRows), a.B);
+  D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(sim_simt_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, SimSmem<T>::kBytes));
+  D3TOM_CUDA_TRY(ctx, launch_serialized(sim_simt_kernel<T>, grid, 256, SimSmem<T>::kBytes, s, hidden,
+                                        static_cast<const T*>(ctx->kept_rows), a.cu_seqlens, a.cu_vis, a.cu_kept, a.assign,
+                                        ctx->inv_norm, ctx->inv_norm_kept, a.D, a.max_kept, vec, ctx->best, a.sim_debug));
+  return D3TOM_OK;
 }
 
 }  // namespace
