@@ -32,7 +32,7 @@ constexpr int kGemmThreads = 224;      // warps: 0 A loads, 1 MMA, 2..5 epilogue
 
 enum { kEpiProj = 0, kEpiSim = 1, kEpiLinear = 2, kEpiGateUp = 3 };
 constexpr int kMaxKSplits = 4;        // K slices per tile at most when the last slice to arrive adds them all
-constexpr int kCoopSlices = 16;       // K slices per similarity tile at most when every slice adds its own share of the columns (8 or 16)
+constexpr int kCoopSlices = 16;       // K slices per similarity tile at most when every slice adds its own share of the columns
 
 struct GemmParams {
   int num_k_blocks;           // K / 64
@@ -41,7 +41,6 @@ struct GemmParams {
   int full_tiles;             // the first tiles of the walk are whole work units (0: every tile is cut)
   float* split_ws;            // [(tiles - full_tiles) * k_splits][BN][128] fp32 partial tiles (column-major: coalesced per warp)
   int* split_counters;        // [tiles] parts done; zero between launches
-  int coop;                   // similarity, few tiles: 8 or 16 slices per tile, all resident; each reduces BN / k_splits columns
   // projection
   __nv_bfloat16* out[3];      // q, k, v
   int out_rows;               // total tokens
@@ -81,6 +80,8 @@ template <int BN, int MT = 1> struct GemmSmem {
   static constexpr int kAccStride = BN <= 128 ? 128 : 256;              // TMEM columns between the two accumulators
   static constexpr int kBytes = kStages * (kABytes + kBBytes) + 1024 /*alignment slack*/ + 256 /*barriers*/ + BN * 4;
 };
+
+template <int N> struct Const { static constexpr int value = N; };
 
 // Where tile `t` of the walk lies: rows of A, rows of B, and for the similarity the request
 // it belongs to.  Returns false for a tile of the bounding grid that a request does not reach.
@@ -278,13 +279,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       // counter, left at zero again) adds the parts in the order of the K slices and runs the epilogue on
       // the sums: same values whichever unit comes last.
       const bool split = un.nsp > 1;
-      const bool coop = EPI == kEpiSim && p.coop != 0;
+      constexpr bool coop = EPI == kEpiSim;                     // every slice adds up a share of the columns, or the last one adds all
       const int ws_tile = t - p.full_tiles;                     // cut tiles are numbered from zero in the workspace
       bool last = true;
       if (split) {
         float* part = p.split_ws + (size_t)(ws_tile * un.nsp + sp) * BN * kBM;
+        const int live_cols = EPI == kEpiSim ? min(BN, tc.kb - tc.n0) : BN;      // (columns past the kept set are never read)
 #pragma unroll 1
-        for (int c = 0; c < BN; c += 32) {
+        for (int c = 0; c < live_cols; c += 32) {
           uint32_t r[32];
           ptx::tmem_ld32(t_row + c, r);
           ptx::tmem_wait_ld();
@@ -328,7 +330,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       }
       // 32 accumulator columns of this thread's row: from tensor memory, or the sum of the slices
       auto load32 = [&](int c, float (&acc)[32]) {
-        if (!split) {
+        if (EPI == kEpiSim || !split) {          // (the similarity's slices never come here: they add up their columns above)
           uint32_t r[32];
           ptx::tmem_ld32(t_row + c, r);
           ptx::tmem_wait_ld();
@@ -356,12 +358,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         }
       };
       if (!last) { ++lt; continue; }
-      if (EPI == kEpiSim && coop) {
-        // this slice's share of the tile's columns, eight at a time: the sums over all slices (ascending slice
+      if (coop && split) {
+        // this slice's share of the tile's live columns in groups of eight: the sums over all slices (ascending slice
         // order), then the arg-max over those columns; the 64-bit maximum over slices and tiles is order-independent
-        const int nsp = un.nsp;                                  // 8 or 16
-        const int cw = BN / nsp;
-        const int cb = sp * cw;
+        const int nsp = un.nsp;                                  // 2 .. 16
+        const int groups = (min(BN, tc.kb - tc.n0) + 7) >> 3;
+        const int cb = sp * groups / nsp * 8, ce = (sp + 1) * groups / nsp * 8;
         const int m = m_base + row;
         const int g = tc.v0 + m;
         const bool active = m < tc.Vb && p.assign[g] < 0;
@@ -369,37 +371,48 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         float best_sim = -INFINITY;
         int best_slot = 0;
         float* dbg = (p.sim_debug != nullptr && active) ? p.sim_debug + (size_t)g * p.max_kept + tc.n0 : nullptr;
+        const float* tile_ws = p.split_ws + (size_t)ws_tile * nsp * BN * kBM + row;
+        // kQ slices x kC columns of loads in flight (64 words a thread)
+        auto add_up = [&](auto q_tag, auto c_tag) {
+          constexpr int kQ = decltype(q_tag)::value, kC = decltype(c_tag)::value;
 #pragma unroll 1
-        for (int c8 = cb; c8 < cb + cw; c8 += 8) {
-          float dot[8];
+          for (int c = cb; c < ce; c += kC) {
+            float dot[kC];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) dot[i] = 0.f;
+            for (int i = 0; i < kC; ++i) dot[i] = 0.f;
 #pragma unroll 1
-          for (int q0 = 0; q0 < nsp; q0 += 8) {                  // eight slices' loads in flight at a time
-            float part[8][8];
+            for (int q0 = 0; q0 < nsp; q0 += kQ) {
+              float part[kQ][kC];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-              const float* src = p.split_ws + ((size_t)(ws_tile * nsp + q0 + q) * BN + c8) * kBM + row;
+              for (int q = 0; q < kQ; ++q)
+                if (q0 + q < nsp) {
+                  const float* src = tile_ws + ((size_t)(q0 + q) * BN + c) * kBM;
 #pragma unroll
-              for (int i = 0; i < 8; ++i) part[q][i] = __ldcg(src + (size_t)i * kBM);
+                  for (int i = 0; i < kC; ++i)
+                    if (c + (i & ~7) < ce) part[q][i] = __ldcg(src + (size_t)i * kBM);
+                }
+#pragma unroll
+              for (int q = 0; q < kQ; ++q)
+                if (q0 + q < nsp) {
+#pragma unroll
+                  for (int i = 0; i < kC; ++i)
+                    if (c + (i & ~7) < ce) dot[i] += part[q][i];
+                }
             }
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-#pragma unroll
-              for (int q = 0; q < 8; ++q) dot[i] += part[q][i];
+            for (int i = 0; i < kC; ++i) {
+              const int sidx = tc.n0 + c + i;
+              if (active && c + i < ce && sidx < tc.kb) {
+                const float sim = (dot[i] * inm) * ink_s[c + i] + 0.0f;
+                if (sim > best_sim) { best_sim = sim; best_slot = sidx; }
+                if (dbg != nullptr) dbg[c + i] = sim;
+              }
             }
           }
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int sidx = tc.n0 + c8 + i;
-            if (active && sidx < tc.kb) {
-              const float sim = (dot[i] * inm) * ink_s[c8 + i] + 0.0f;
-              if (sim > best_sim) { best_sim = sim; best_slot = sidx; }
-              if (dbg != nullptr) dbg[c8 + i] = sim;
-            }
-          }
-        }
-        if (active && tc.n0 + cb < tc.kb) {
+        };
+        if (nsp > 4) add_up(Const<8>{}, Const<8>{});
+        else add_up(Const<4>{}, Const<16>{});
+        if (active && cb < ce) {
           const unsigned long long mine =
               ((unsigned long long)ordered_key(best_sim) << 32) | (0xffffffffu - (unsigned)best_slot);
           atomicMax(p.best + g, mine);
@@ -1072,29 +1085,22 @@ int launch_sim_tc(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
   p.inv_norm = ctx->inv_norm; p.inv_norm_kept = ctx->inv_norm_kept; p.best = ctx->best; p.sim_debug = a.sim_debug;
   p.max_kept = a.max_kept; p.dev_status = ctx->dev_status;
   p.m_tiles = ceil_div(a.max_visual, kBM); p.batch = a.B;
-  // Few tiles (short requests, small kept sets): a tile is 64 k-blocks of serial work on one SM while
-  // most SMs idle, so each tile's K range is cut into slices for different SMs (see the epilogue).
-  {
-    const int bn = a.max_kept > 128 ? 256 : 128;
-    const long long tiles = (long long)p.m_tiles * ceil_div(a.max_kept, bn) * p.batch;
-    int splits = (int)(ctx->sm_count / (tiles > 0 ? tiles : 1));
-    if (splits > kMaxKSplits) splits = kMaxKSplits;
-    if (splits > p.num_k_blocks) splits = p.num_k_blocks;
-    if (splits < 2 || tiles * splits > 2LL * ctx->sm_count) splits = 1;
-    // very few tiles (a small kept set, one short request): eight or sixteen slices per tile, each a CTA of its
-    // own, and every slice adds up its share of the tile's columns itself instead of the last one adding all
-    for (int c = kCoopSlices; c >= 8; c /= 2) {
-      if (tiles * c <= ctx->sm_count && p.num_k_blocks >= 2 * c) {
-        splits = c;
-        p.coop = 1;
-        break;
-      }
-    }
-    p.k_splits = splits;
-    p.full_tiles = 0;                                   // every tile is cut (or none: one slice)
-    p.split_ws = ctx->gemm_split_ws; p.split_counters = ctx->gemm_split_counters;
-  }
-  if (a.max_kept > 128) {      // 256-wide tiles: the A tile is streamed once per 256 kept rows and each MMA covers twice the work
+  // Few tiles (short requests, small kept sets): a tile is 64 k-blocks of serial work on one SM while most SMs idle, so
+  // each tile's K range is cut into slices, each a CTA of its own, all resident at once (units <= SMs), and every slice
+  // adds up its share of the tile's columns over all slices.  The last arriver adding all columns alone cost more than the
+  // main loop: 2048 visual x 512 kept x 4096 (32 tiles, 4 slices) 28.6 us,
+  // shared 20.1.
+  // 128-wide tiles also serve larger kept sets while eight slices of each still fit: half the exchange per slice
+  // (577 x 173 x 1024: 13.6 -> 10.3 us).
+  const long long narrow_tiles = (long long)p.m_tiles * ceil_div(a.max_kept, 128) * p.batch;
+  const int bn = a.max_kept <= 128 || narrow_tiles * 8 <= ctx->sm_count ? 128 : 256;
+  const long long tiles = (long long)p.m_tiles * ceil_div(a.max_kept, bn) * p.batch;
+  p.k_splits = 1;
+  for (int c : {kCoopSlices, 8, 4, 3, 2})
+    if (tiles * c <= ctx->sm_count && p.num_k_blocks >= 2 * c) { p.k_splits = c; break; }
+  p.full_tiles = 0;                                     // every tile is cut (or none: one slice)
+  p.split_ws = ctx->gemm_split_ws; p.split_counters = ctx->gemm_split_counters;
+  if (bn == 256) {             // 256-wide tiles: the A tile is streamed once per 256 kept rows and each MMA covers twice the work
     r = make_tmap_bf16_2d(&tb, ctx->kept_rows, (uint64_t)kept_rows_bound, (uint64_t)a.D, (uint64_t)a.D, 256);
     if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
     p.n_tiles = ceil_div(a.max_kept, 256);

@@ -119,6 +119,18 @@ def test_few_similarity_tiles_are_cut_along_k_and_every_slice_reduces_its_column
     pu.check_step(w, mode=B_.AGG_SUM, full_attention=False, n_sample_rows=24)
 
 
+@pytest.mark.parametrize("H,reqs", [
+    (16, [dict(V=1500, P=5, O=8, n_dec=3, r=0.3)]),       # 12 x 2 tiles of 256: four slices each
+    (16, [dict(V=2500, P=5, O=8, n_dec=3, r=0.2)]),       # 20 x 2 tiles: three slices
+    (16, [dict(V=3000, P=5, O=8, n_dec=3, r=0.25)]),      # 24 x 3 tiles: two slices
+    (8, [dict(V=577, P=5, O=8, n_dec=3, r=0.3)]),         # 173 kept in 5 x 2 tiles of 128: eight slices of two k-blocks
+    (8, [dict(V=700, P=5, O=8, n_dec=3, r=0.4), dict(V=200, P=3, O=8, n_dec=3, r=0.9), dict(V=300, P=3, O=8, n_dec=0, r=1.0)]),
+], ids=["256x4", "256x3", "256x2", "128x8", "batch"])
+def test_similarity_tiles_cut_into_two_to_four_slices(H, reqs):
+    w = small(H=H, dh=128, reqs=reqs, post=0)
+    pu.check_step(w, full_attention=False, n_sample_rows=8)
+
+
 def run_attention_only(lens, H, seed=0):
     """d3tom_attn_varlen on random Q, K, V of a ragged batch against the oracle, every row."""
     dev = torch.device("cuda", 0)
