@@ -352,6 +352,7 @@ static int merge_common(d3tom_ctx* ctx, d3tom_dtype dt, d3tom_agg mode, const vo
   a.kept_idx = kept_idx; a.cu_kept = cu_kept; a.B = B; a.D = D; a.total_tokens = total_tokens; a.total_out = total_out;
   a.max_visual = max_visual; a.max_kept = max_kept; a.hidden_out = hidden_out; a.cu_seqlens_out = cu_seqlens_out;
   a.assign = assign; a.member_count = member_count; a.src_of_dst = src_of_dst; a.sim_debug = sim_debug;
+  a.second = second; a.second_out = second_out;
   int st = D3TOM_OK;
   if (max_visual > 0) {
     st = launch_merge_prepare(ctx, a, s);
@@ -362,10 +363,7 @@ static int merge_common(d3tom_ctx* ctx, d3tom_dtype dt, d3tom_agg mode, const vo
       if (st != D3TOM_OK) return st;
     }
   }
-  st = launch_merge_finish(ctx, a, s);
-  if (st != D3TOM_OK || second == nullptr) return st;
-  a.hidden = second; a.hidden_out = second_out;       // same routing, second payload
-  return launch_merge_aggregate(ctx, a, s);
+  return launch_merge_finish(ctx, a, s);
 }
 
 int d3tom_merge(d3tom_ctx* ctx, d3tom_dtype dt, d3tom_agg mode, const void* hidden, const int32_t* cu_seqlens,

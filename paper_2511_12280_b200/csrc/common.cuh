@@ -177,13 +177,14 @@ struct MergeArgs {
   const int32_t* kept_idx; const int32_t* cu_kept;
   int B, D, total_tokens, total_out, max_visual, max_kept;
   void* hidden_out; const int32_t* cu_seqlens_out;
+  const void* second; void* second_out;      // a second payload of the same rows (the V cache), or null
   int32_t* assign; int32_t* member_count; int32_t* src_of_dst; float* sim_debug;
 };
 int launch_merge_prepare(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s);     // slots, norms, kept-row gather
 int launch_sim_simt(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s);          // similarity + argmax, CUDA cores
 int launch_sim_tc(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s);            // similarity + argmax, tcgen05
 int launch_merge_finish(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s);      // members, aggregate, compact
-int launch_merge_aggregate(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s);   // aggregate, compact (lists already built)
+int launch_merge_aggregate(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s);   // aggregate, compact (lists already built), both payloads
 int launch_merge_aggregate_stream(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s);   // the same as a bulk-copy pipeline
 
 int launch_wait_timeout_selftest(d3tom_ctx* ctx, long long limit_ns, cudaStream_t s);   // a wait that cannot end

@@ -316,18 +316,23 @@ __device__ __forceinline__ void add_rows(float (&acc)[Storage<T>::kVec], const T
 // ascending; warp w adds the kept row (w = 0) and the 32-member segments w, w + 8, ...,
 // and the eight partial sums are added in warp order.  Every order is a fixed function of
 // the sorted list, so results do not depend on scheduling.
+// blockIdx.y = 1: the same for a second payload (the V cache beside the K cache), in the same launch: the two share
+// nothing but the lists, and either alone leaves the SMs waiting on latency (4096 + 128 rows of 8 KB: 2 x 12.1 us one
+// after the other).
 template <typename T>
 __global__ void __launch_bounds__(kAggWarps * 32)
-aggregate_compact_kernel(const T* __restrict__ hidden, const int32_t* __restrict__ cu_seqlens,
+aggregate_compact_kernel(const T* __restrict__ hidden_1, const T* __restrict__ hidden_2, const int32_t* __restrict__ cu_seqlens,
                          const int32_t* __restrict__ n_visual, const int32_t* __restrict__ kept_idx,
                          const int32_t* __restrict__ cu_kept, const int32_t* __restrict__ cu_seqlens_out, int B, int D,
                          int chunks, int total_out, int heavy_blocks, int mean,
                          const int32_t* __restrict__ member_count, const int32_t* __restrict__ member_off,
                          const int32_t* __restrict__ member_list, const int32_t* __restrict__ heavy_slots,
-                         const int* __restrict__ n_heavy, const int4* __restrict__ row_desc, T* __restrict__ hidden_out,
-                         int32_t* __restrict__ src_of_dst) {
+                         const int* __restrict__ n_heavy, const int4* __restrict__ row_desc, T* __restrict__ out_1,
+                         T* __restrict__ out_2, int32_t* __restrict__ src_of_dst) {
   constexpr int kVec = Storage<T>::kVec;
   grid_dependency_enter();
+  const T* __restrict__ hidden = blockIdx.y == 0 ? hidden_1 : hidden_2;      // (the second payload: same lists, same rows)
+  T* __restrict__ hidden_out = blockIdx.y == 0 ? out_1 : out_2;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float acc[kVec];
 #pragma unroll
@@ -369,7 +374,7 @@ aggregate_compact_kernel(const T* __restrict__ hidden, const int32_t* __restrict
       for (int e = 0; e < kVec; ++e) acc[e] *= inv_denom;
       Storage<T>::store(hidden_out + (size_t)row * D + c, acc);
     }
-    if (ch == 0 && threadIdx.x == 0) src_of_dst[row] = lo + pos;
+    if (ch == 0 && blockIdx.y == 0 && threadIdx.x == 0) src_of_dst[row] = lo + pos;
     __syncthreads();                                            // `part` is reused by the next item
     }
     return;
@@ -393,7 +398,7 @@ aggregate_compact_kernel(const T* __restrict__ hidden, const int32_t* __restrict
   }
   const T* req = hidden + (size_t)lo * D;
   T* dst = hidden_out + (size_t)row * D;
-  if (cg == 0 && lane == 0) src_of_dst[row] = desc.x;
+  if (cg == 0 && blockIdx.y == 0 && lane == 0) src_of_dst[row] = desc.x;
 
   if (cnt < 0) {                                                // prompt / response row: copy
     uint4 raw[kAggCpw];
@@ -484,11 +489,26 @@ int launch_merge_finish(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
   return launch_merge_aggregate(ctx, a, s);
 }
 
-// aggregation + compaction of a.hidden into a.hidden_out with the member lists the context holds
-// (may run again on another tensor of the same rows: the V cache after the K cache)
+// aggregation + compaction of a.hidden into a.hidden_out (and of a.second into a.second_out) with the member lists the
+// context holds
 int launch_merge_aggregate(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
   const int mean = a.mode == D3TOM_AGG_MEAN ? 1 : 0;
   if (a.total_out <= 0) return D3TOM_OK;
+  if (a.second != nullptr) {
+    // one payload's output may lie where the other's input was (the V cache written over the K cache): then one after the other
+    const size_t esize = a.dt == D3TOM_FP32 ? 4 : 2, in = (size_t)a.total_tokens * a.D * esize, out = (size_t)a.total_out * a.D * esize;
+    auto overlap = [&](const void* x, const void* y) {
+      return (uintptr_t)x < (uintptr_t)y + in && (uintptr_t)y < (uintptr_t)x + out;
+    };
+    if (overlap(a.second_out, a.hidden) || overlap(a.hidden_out, a.second)) {
+      MergeArgs one = a;
+      one.second = nullptr; one.second_out = nullptr;
+      const int st = launch_merge_aggregate(ctx, one, s);
+      if (st != D3TOM_OK) return st;
+      one.hidden = a.second; one.hidden_out = a.second_out;
+      return launch_merge_aggregate(ctx, one, s);
+    }
+  }
   {   // the streaming pipeline takes every row size it supports; the kernel below is the general one
     const int st = launch_merge_aggregate_stream(ctx, a, s);
     if (st != D3TOM_ERR_UNSUPPORTED) return st;
@@ -499,18 +519,21 @@ int launch_merge_aggregate(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
   const int light_blocks = (int)((warps + kAggWarps - 1) / kAggWarps);
   // at most (pruned tokens) / kHeavy kept tokens can be heavy; the blocks beyond the actual number leave at once
   const int max_heavy = (a.total_tokens - a.total_out) / kHeavy;
-  int heavy_blocks = max_heavy * chunks;
-  if (heavy_blocks > ctx->sm_count) heavy_blocks = ctx->sm_count;
-  const int blocks = light_blocks + heavy_blocks;
+  // (one block per SM, and more once so many are possible that one per SM would walk over dozens of (row, chunk) items:
+  // 12287 visual tokens, 10 % kept, 55 -> 42 us; four per SM for everyone delays the light rows of short requests, 9.4 -> 10.8)
+  const int heavy_items = max_heavy * chunks, sms = ctx->sm_count;
+  const int heavy_blocks = min(heavy_items, max(sms, min(4 * sms, heavy_items / 8)));
+  const dim3 blocks(light_blocks + heavy_blocks, a.second != nullptr ? 2 : 1);
   if (a.dt == D3TOM_FP32)
     D3TOM_CUDA_TRY(ctx, launch_serialized(aggregate_compact_kernel<float>, blocks, kAggWarps * 32, 0, s,
-        static_cast<const float*>(a.hidden), a.cu_seqlens, a.n_visual, a.kept_idx, a.cu_kept, a.cu_seqlens_out, a.B, a.D,
+        static_cast<const float*>(a.hidden), static_cast<const float*>(a.second), a.cu_seqlens, a.n_visual, a.kept_idx, a.cu_kept, a.cu_seqlens_out, a.B, a.D,
         chunks, a.total_out, heavy_blocks, mean, a.member_count, ctx->member_off, ctx->member_list, ctx->heavy_slots,
-        ctx->n_heavy, ctx->row_desc, static_cast<float*>(a.hidden_out), a.src_of_dst));
+        ctx->n_heavy, ctx->row_desc, static_cast<float*>(a.hidden_out), static_cast<float*>(a.second_out), a.src_of_dst));
   else
     D3TOM_CUDA_TRY(ctx, launch_serialized(aggregate_compact_kernel<__nv_bfloat16>, blocks, kAggWarps * 32, 0, s,
-        static_cast<const __nv_bfloat16*>(a.hidden), a.cu_seqlens, a.n_visual, a.kept_idx, a.cu_kept, a.cu_seqlens_out,
+        static_cast<const __nv_bfloat16*>(a.hidden), static_cast<const __nv_bfloat16*>(a.second), a.cu_seqlens, a.n_visual, a.kept_idx, a.cu_kept, a.cu_seqlens_out,
         a.B, a.D, chunks, a.total_out, heavy_blocks, mean, a.member_count, ctx->member_off, ctx->member_list,
-        ctx->heavy_slots, ctx->n_heavy, ctx->row_desc, static_cast<__nv_bfloat16*>(a.hidden_out), a.src_of_dst));
+        ctx->heavy_slots, ctx->n_heavy, ctx->row_desc, static_cast<__nv_bfloat16*>(a.hidden_out),
+        static_cast<__nv_bfloat16*>(a.second_out), a.src_of_dst));
   return D3TOM_OK;
 }

@@ -46,6 +46,7 @@ template <> __device__ __forceinline__ void add_vec<__nv_bfloat16>(float (&acc)[
 
 struct StreamParams {
   const void* hidden; void* hidden_out;
+  const void* second; void* second_out;      // a second payload of the same rows, or null: its work items follow the first's
   const int4* row_desc;            // per output row: {source row, members or -1 (copy), list offset, request's first row}
   const int32_t* member_list;
   int32_t* src_of_dst;
@@ -54,7 +55,7 @@ struct StreamParams {
   int total_out, D, col_splits, seg_bytes, slots, mean;
 };
 
-// slot header: x = output row (-1: no more work), y = bit 0 first source, bit 1 last source, bits 8.. column segment,
+// slot header: x = output row (-1: no more work), y = bit 0 first source, bit 1 last source, bit 2 second payload, bits 8.. column segment,
 //              z = member count of the row, w = source row of the output row (for src_of_dst)
 template <typename T>
 __global__ void __launch_bounds__(kStreamThreads)
@@ -77,11 +78,12 @@ aggregate_stream_kernel(StreamParams p) {
   grid_dependency_release();
   __syncthreads();
   const int seg_elems = p.seg_bytes / (int)sizeof(T);
-  const long long n_items = (long long)p.total_out * p.col_splits;
+  const long long n_first = (long long)p.total_out * p.col_splits, n_items = p.second != nullptr ? 2 * n_first : n_first;
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer warp
-    const T* hidden = static_cast<const T*>(p.hidden);
+    const T* hidden = nullptr;                        // payload of the item in hand
+    int payload_bit = 0;
     int it = 0;                                       // slots filled so far
     bool ok = true;
     // pushes one source segment; lane 0 does the waiting and the copy
@@ -90,7 +92,7 @@ aggregate_stream_kernel(StreamParams p) {
         const int s = it % R;
         ok = ptx::mbar_wait(&empty[s], ((it / R) & 1) ^ 1, abort_flag, p.dev_status);
         if (ok) {
-          header[s] = make_int4(out_row, flags | (cq << 8), cnt, src_of_row);
+          header[s] = make_int4(out_row, flags | payload_bit | (cq << 8), cnt, src_of_row);
           ptx::mbar_arrive_expect_tx(&full[s], (uint32_t)p.seg_bytes);
           bulk_load(ring + (size_t)s * p.seg_bytes, hidden + (size_t)src_row * p.D + (size_t)cq * seg_elems,
                     (uint32_t)p.seg_bytes, &full[s]);
@@ -104,6 +106,9 @@ aggregate_stream_kernel(StreamParams p) {
       item = __shfl_sync(0xffffffffu, item, 0);
       ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
       if (item >= n_items || !ok) break;
+      hidden = static_cast<const T*>(item < n_first ? p.hidden : p.second);
+      payload_bit = item < n_first ? 0 : 4;
+      if (item >= n_first) item -= n_first;
       const int row = (int)(item / p.col_splits), cq = (int)(item - (long long)row * p.col_splits);
       const int4 d = p.row_desc[row];
       const int cnt = d.y < 0 ? 0 : d.y, lo = d.w;
@@ -147,7 +152,6 @@ aggregate_stream_kernel(StreamParams p) {
   } else {
     // ------------------------------------------------------------ consumer warps: 128 threads, 16 bytes per thread and pass
     const int ct = threadIdx.x - 32;
-    T* out = static_cast<T*>(p.hidden_out);
     float acc[kMaxVecPerThread][kVec];
     for (int it = 0;; ++it) {
       const int s = it % R;
@@ -170,7 +174,7 @@ aggregate_stream_kernel(StreamParams p) {
       if (last) {
         const int cq = h.y >> 8;
         const float inv = (p.mean && h.z > 0) ? 1.0f / (float)(1 + h.z) : 1.f;
-        T* dst = out + (size_t)h.x * p.D + (size_t)cq * seg_elems;
+        T* dst = static_cast<T*>((h.y & 4) ? p.second_out : p.hidden_out) + (size_t)h.x * p.D + (size_t)cq * seg_elems;
 #pragma unroll
         for (int v = 0; v < kMaxVecPerThread; ++v) {
           const int byte = (ct + v * 32 * kConsumerWarps) * 16;
@@ -205,12 +209,12 @@ int launch_merge_aggregate_stream(d3tom_ctx* ctx, const MergeArgs& a, cudaStream
   if (slots > kMaxSlots) slots = kMaxSlots;
   if (slots < 4) return D3TOM_ERR_UNSUPPORTED;
   StreamParams p;
-  p.hidden = a.hidden; p.hidden_out = a.hidden_out; p.row_desc = ctx->row_desc; p.member_list = ctx->member_list;
+  p.hidden = a.hidden; p.hidden_out = a.hidden_out; p.second = a.second; p.second_out = a.second_out; p.row_desc = ctx->row_desc; p.member_list = ctx->member_list;
   p.src_of_dst = a.src_of_dst; p.work_counter = ctx->agg_counter; p.dev_status = ctx->dev_status;
   p.total_out = a.total_out; p.D = a.D; p.col_splits = splits; p.seg_bytes = (int)seg; p.slots = slots;
   p.mean = a.mode == D3TOM_AGG_MEAN ? 1 : 0;
   const size_t smem = (size_t)slots * seg + 128;
-  const long long items = (long long)a.total_out * splits;
+  const long long items = (long long)a.total_out * splits * (a.second != nullptr ? 2 : 1);
   long long grid = 6LL * ctx->sm_count;                 // six CTAs fit one SM (32 KB of ring each): what limits the
                                                         // pipeline is the rate at which one producer lane issues copies
   if (grid > items) grid = items;

@@ -265,6 +265,13 @@ def test_select_adversarial_inputs():
     run_select([rng.random(3000), rng.random(100)], [0, 7])                 # keys in registers, keep count 0
 
 
+@pytest.mark.parametrize("V", [8192, 8193, 12287, 16383, 16384, 16385])
+def test_select_at_the_ends_of_the_key_in_registers_range(V):
+    rng = np.random.default_rng(V)
+    run_select([rng.random(V)], [V // 10])
+    run_select([rng.integers(0, 5, V) / 8.0, rng.random(9)], [V - 3, 2])        # long runs of ties
+
+
 def test_host_made_failures_return_status_codes():
     w = small(post=0)
     step = pu.make_step(w, sim_debug=False)

@@ -82,3 +82,31 @@ def test_merge_kv_fp32_path():
 def test_merge_kv_llada_shape():
     # the prefix cache of the LLaDA-8B-shaped config: 1024 visual + 64 prompt rows of width 4096, keep 10 %
     run_case(wl.config("C1"), B_.AGG_MEAN, keep_ratio=0.10)
+
+
+@pytest.mark.parametrize("V,r", [(4700, 0.92), (9000, 0.2), (17000, 0.02)])
+def test_merge_kv_both_caches_in_one_launch_of_either_aggregation(V, r):
+    # 4.3 K output rows take the streaming pipeline; 9 K and 17 K visual tokens with few kept ones have long member lists
+    # (more heavy kept tokens x chunks than blocks) and lie on either side of what the list kernel keeps in registers
+    run_case(wl.make_workload("kvl", "bf16", 2, 64, 43, 64, [dict(V=V, P=9, O=4, n_dec=1, r=r)]), B_.AGG_MEAN)
+
+
+def test_merge_kv_value_cache_written_over_the_key_cache():
+    dev, D, V, P, k = torch.device("cuda", 0), 256, 300, 5, 40
+    g = torch.Generator().manual_seed(3)
+    kc, vc = (torch.randn(V + P, D, generator=g).to(torch.bfloat16).to(dev) for _ in range(2))
+    i32 = lambda *a: torch.tensor(a, dtype=torch.int32, device=dev)
+    kept = torch.arange(0, V, V // k, dtype=torch.int32, device=dev)[:k].contiguous()
+    ctx = B_.Context(V + P, 1, 2, 128, 1, V)
+    idx = [torch.empty(V + P, dtype=torch.int32, device=dev) for _ in range(3)]
+    n = k + P
+    outs = []
+    for over in (False, True):
+        a, b = kc.clone(), vc.clone()
+        k_out, v_out = torch.empty(n, D, dtype=torch.bfloat16, device=dev), a[:n] if over else torch.empty(n, D, dtype=torch.bfloat16, device=dev)
+        ctx.d3tom_merge_kv(B_.AGG_SUM, a, b, i32(0, V + P), i32(V), i32(0, V), kept, i32(0, k), 1, D, V + P, n, V, k, k_out, v_out,
+                           i32(0, n), *idx)
+        torch.cuda.synchronize()
+        outs.append((k_out.clone(), v_out.clone()))
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+    ctx.close()
