@@ -440,10 +440,12 @@ attn_sk_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
           m_used = m;
         }
         const float inv_l = 1.f / l_sum;
-        __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(a.out) + ((size_t)(lo + q_row) * a.H + w.h) * DH;
+        // this warp's 32 rows
+        const int warp_row = q_row - lane;
+        __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(a.out) + ((size_t)(lo + warp_row) * a.H + w.h) * DH;
 #pragma unroll 1
         for (int c0 = 0; c0 < DH; c0 += 32) {
-          uint32_t r[32];
+          uint32_t r[32], wv[16];
           ptx::tmem_ld32(t_o + c0, r);
           ptx::tmem_wait_ld();
           if (is_head) {
@@ -451,16 +453,10 @@ attn_sk_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
             for (int e = 0; e < 32; ++e)
               r[e] = __float_as_uint(__uint_as_float(r[e]) * a1 + __ldcg(other + (size_t)(c0 + e) * kTile + row) * a2);
           }
-          if (valid_row) {
 #pragma unroll
-            for (int e = 0; e < 32; e += 8) {
-              uint32_t wv[4];
-#pragma unroll
-              for (int t = 0; t < 4; ++t)
-                wv[t] = pack_bf16x2(__uint_as_float(r[e + 2 * t]) * inv_l, __uint_as_float(r[e + 2 * t + 1]) * inv_l);
-              *reinterpret_cast<uint4*>(dst + c0 + e) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-            }
-          }
+          for (int t = 0; t < 16; ++t)
+            wv[t] = pack_bf16x2(__uint_as_float(r[2 * t]) * inv_l, __uint_as_float(r[2 * t + 1]) * inv_l);
+          ptx::store_rows_64b(dst + c0, (size_t)a.H * DH * 2, n - warp_row, wv);
         }
         if (dec_slot >= 0) a.lse_scratch[(size_t)w.h * a.max_deciders + dec_slot] = make_float2(m_used, l_sum);
         if (is_head) {                                         // the slot's flag goes back to zero for the next launch

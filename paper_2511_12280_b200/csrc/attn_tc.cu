@@ -375,22 +375,18 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
       if (ok) {
         const float l_sum = l2.x + l2.y;
         const float inv_l = 1.f / l_sum;
-        __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(a.out) + ((size_t)(lo + q_row) * a.H + h) * DH;
+        // this warp's 32 rows
+        const int warp_row = q_row - lane;
+        __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(a.out) + ((size_t)(lo + warp_row) * a.H + h) * DH;
 #pragma unroll 1
         for (int c0 = 0; c0 < DH; c0 += 32) {
-          uint32_t r[32];
+          uint32_t r[32], w[16];
           ptx::tmem_ld32(t_o + c0, r);
           ptx::tmem_wait_ld();
-          if (valid_row) {
 #pragma unroll
-            for (int e = 0; e < 32; e += 8) {
-              uint32_t w[4];
-#pragma unroll
-              for (int t = 0; t < 4; ++t)
-                w[t] = pack_bf16x2(__uint_as_float(r[e + 2 * t]) * inv_l, __uint_as_float(r[e + 2 * t + 1]) * inv_l);
-              *reinterpret_cast<uint4*>(dst + c0 + e) = make_uint4(w[0], w[1], w[2], w[3]);
-            }
-          }
+          for (int t = 0; t < 16; ++t)
+            w[t] = pack_bf16x2(__uint_as_float(r[2 * t]) * inv_l, __uint_as_float(r[2 * t + 1]) * inv_l);
+          ptx::store_rows_64b(dst + c0, (size_t)a.H * DH * 2, n - warp_row, w);
         }
         if (dec_slot >= 0) a.lse_scratch[(size_t)h * a.max_deciders + dec_slot] = make_float2(m_used, l_sum);
       }

@@ -426,78 +426,64 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       // (a 256-row tile: the same epilogue once per 128-row half, each half in its own accumulator)
 #pragma unroll 1
       for (int mh = 0; mh < MT; ++mh, t_row += S::kAccStride, m_base += kBM) {
+      const int warp_row = m_base + quarter * 32, n_valid = p.out_rows - warp_row;      // dense layers: this warp's 32 rows
       if (EPI == kEpiProj) {
-        const int grow = m_base + row;
 #pragma unroll 1
         for (int c = 0; c < BN; c += 32) {
           float r[32];
           load32(c, r);
           // 32 divides D, so a 32-column piece lies in one of q, k, v even when the tile straddles two of them
           const int gcol = tc.n0 + c, which = gcol / p.out_cols;
-          __nv_bfloat16* dst = p.out[which] + (size_t)grow * p.out_cols + (gcol - which * p.out_cols) - c;
-          if (grow < p.out_rows && which < 3) {      // (a tile width that does not divide 3 D: the last tile hangs over)
+          if (which < 3) {                           // (a tile width that does not divide 3 D: the last tile hangs over)
+            uint32_t w[16];
 #pragma unroll
-            for (int i = 0; i < 32; i += 8) {
-              uint32_t w[4];
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                __nv_bfloat162 h2 = __floats2bfloat162_rn(r[i + 2 * j], r[i + 2 * j + 1]);
-                w[j] = *reinterpret_cast<uint32_t*>(&h2);
-              }
-              *reinterpret_cast<uint4*>(dst + c + i) = make_uint4(w[0], w[1], w[2], w[3]);
+            for (int j = 0; j < 16; ++j) {
+              __nv_bfloat162 h2 = __floats2bfloat162_rn(r[2 * j], r[2 * j + 1]);
+              w[j] = *reinterpret_cast<uint32_t*>(&h2);
             }
+            ptx::store_rows_64b(p.out[which] + (size_t)warp_row * p.out_cols + (gcol - which * p.out_cols),
+                                (size_t)p.out_cols * 2, n_valid, w);
           }
         }
       } else if (EPI == kEpiLinear) {
-        const int grow = m_base + row;
 #pragma unroll 1
         for (int c = 0; c < BN; c += 32) {
           float r[32];
           load32(c, r);
-          if (grow < p.out_rows && tc.n0 + c < p.ld_out) {
-            const size_t off = (size_t)grow * p.ld_out + tc.n0 + c;
+          if (tc.n0 + c < p.ld_out) {
+            uint32_t w[16];
+            if (p.residual != nullptr) {
+              ptx::load_rows_64b(p.residual + (size_t)warp_row * p.ld_out + tc.n0 + c, (size_t)p.ld_out * 2, n_valid, w);
+            } else {
 #pragma unroll
-            for (int i = 0; i < 32; i += 8) {
-              uint32_t w[4] = {0u, 0u, 0u, 0u};
-              if (p.residual != nullptr) {
-                const uint4 rr = *reinterpret_cast<const uint4*>(p.residual + off + i);
-                w[0] = rr.x; w[1] = rr.y; w[2] = rr.z; w[3] = rr.w;
-              }
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const float lo = r[i + 2 * j] + __uint_as_float(w[j] << 16);
-                const float hi = r[i + 2 * j + 1] + __uint_as_float(w[j] & 0xffff0000u);
-                __nv_bfloat162 h2 = __floats2bfloat162_rn(lo, hi);
-                w[j] = *reinterpret_cast<uint32_t*>(&h2);
-              }
-              *reinterpret_cast<uint4*>(p.lin_out + off + i) = make_uint4(w[0], w[1], w[2], w[3]);
+              for (int i = 0; i < 16; ++i) w[i] = 0u;
             }
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              __nv_bfloat162 h2 = __floats2bfloat162_rn(r[2 * j] + __uint_as_float(w[j] << 16),
+                                                        r[2 * j + 1] + __uint_as_float(w[j] & 0xffff0000u));
+              w[j] = *reinterpret_cast<uint32_t*>(&h2);
+            }
+            // (out may be the residual buffer: the piece of a row is read and written by the same lane)
+            ptx::store_rows_64b(p.lin_out + (size_t)warp_row * p.ld_out + tc.n0 + c, (size_t)p.ld_out * 2, n_valid, w);
           }
         }
       } else if (EPI == kEpiGateUp) {
-        const int grow = m_base + row;
 #pragma unroll 1
         for (int c = 0; c < BN / 2; c += 32) {
           float g[32], up[32];
           load32(c, g);
           load32(BN / 2 + c, up);
-          if (grow < p.out_rows) {
-            __nv_bfloat16* dst = p.lin_out + (size_t)grow * p.ld_out + tc.n0 + c;
+          uint32_t w[16];
 #pragma unroll
-            for (int i = 0; i < 32; i += 8) {
-              uint32_t w[4];
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const float g0 = g[i + 2 * j], g1 = g[i + 2 * j + 1];
-                // silu(g) = g / (1 + exp(-g)); for very negative g the divisor is inf and the quotient 0
-                const float a0 = __fdividef(g0, 1.f + __expf(-g0)) * up[i + 2 * j];
-                const float a1 = __fdividef(g1, 1.f + __expf(-g1)) * up[i + 2 * j + 1];
-                __nv_bfloat162 h2 = __floats2bfloat162_rn(a0, a1);
-                w[j] = *reinterpret_cast<uint32_t*>(&h2);
-              }
-              *reinterpret_cast<uint4*>(dst + i) = make_uint4(w[0], w[1], w[2], w[3]);
-            }
+          for (int j = 0; j < 16; ++j) {
+            const float g0 = g[2 * j], g1 = g[2 * j + 1];
+            // silu(g) = g / (1 + exp(-g)); for very negative g the divisor is inf and the quotient 0
+            __nv_bfloat162 h2 = __floats2bfloat162_rn(__fdividef(g0, 1.f + __expf(-g0)) * up[2 * j],
+                                                      __fdividef(g1, 1.f + __expf(-g1)) * up[2 * j + 1]);
+            w[j] = *reinterpret_cast<uint32_t*>(&h2);
           }
+          ptx::store_rows_64b(p.lin_out + (size_t)warp_row * p.ld_out + tc.n0 + c, (size_t)p.ld_out * 2, n_valid, w);
         }
       } else {
         const int m = m_base + row;
@@ -689,7 +675,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
     }
   } else {
     // ------------------------------------------------------------ epilogue: warp w may touch TMEM lanes 32*(w%4) .. +31
-    // 32 columns at a time, stored as two pieces of 16 (half of a gate-up tile may end in half a piece of 32)
+    // 32 columns at a time
     const int quarter = warp & 3;
     const int row = quarter * 32 + lane;
     int lt = 0;
@@ -721,36 +707,37 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
         } else {
           ptx::tmem_wait_ld();
         }
+        // the piece's destination: one row of one output; only a gate-up half of 80 or 112 columns ends in half a piece
+        __nv_bfloat16* base;
+        size_t ld;
+        if (EPI == kEpiProj) {
+          const int gcol = n0 + c, which = gcol / p.out_cols;      // (32 divides D: a piece lies in one of q, k, v)
+          base = p.out[which] + (gcol - which * p.out_cols);
+          ld = (size_t)p.out_cols;
+        } else {
+          base = p.lin_out + n0 + c;
+          ld = (size_t)p.ld_out;
+        }
+        uint32_t w[16];
+        if (EPI == kEpiLinear && p.residual != nullptr) {
+          ptx::load_rows_64b(p.residual + (size_t)(grow - lane) * ld + n0 + c, ld * 2, p.out_rows - (grow - lane), w);
+        } else {
 #pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-          const int col = c + hf * 16;
-          if (!live || col >= width) continue;
-          __nv_bfloat16* dst;
-          const __nv_bfloat16* res = nullptr;
-          if (EPI == kEpiProj) {
-            const int gcol = n0 + col, which = gcol / p.out_cols;
-            dst = p.out[which] + (size_t)grow * p.out_cols + (gcol - which * p.out_cols);
-          } else {
-            const size_t off = (size_t)grow * p.ld_out + n0 + col;
-            dst = p.lin_out + off;
-            if (EPI == kEpiLinear && p.residual != nullptr) res = p.residual + off;
-          }
+          for (int i = 0; i < 16; ++i) w[i] = 0u;
+        }
 #pragma unroll
-          for (int i = 0; i < 16; i += 8) {
-            uint32_t w[4] = {0u, 0u, 0u, 0u};
-            if (EPI == kEpiLinear && res != nullptr) {
-              const uint4 rr = *reinterpret_cast<const uint4*>(res + i);
-              w[0] = rr.x; w[1] = rr.y; w[2] = rr.z; w[3] = rr.w;
-            }
+        for (int j = 0; j < 16; ++j) {
+          float lo = __uint_as_float(r[2 * j]), hi = __uint_as_float(r[2 * j + 1]);
+          if (EPI == kEpiLinear) { lo += __uint_as_float(w[j] << 16); hi += __uint_as_float(w[j] & 0xffff0000u); }
+          __nv_bfloat162 h2 = __floats2bfloat162_rn(lo, hi);
+          w[j] = *reinterpret_cast<uint32_t*>(&h2);
+        }
+        if (EPI != kEpiGateUp || c + 32 <= width) {
+          ptx::store_rows_64b(base + (size_t)(grow - lane) * ld, ld * 2, p.out_rows - (grow - lane), w);
+        } else if (live) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              float lo = __uint_as_float(r[hf * 16 + i + 2 * j]), hi = __uint_as_float(r[hf * 16 + i + 2 * j + 1]);
-              if (EPI == kEpiLinear) { lo += __uint_as_float(w[j] << 16); hi += __uint_as_float(w[j] & 0xffff0000u); }
-              __nv_bfloat162 h2 = __floats2bfloat162_rn(lo, hi);
-              w[j] = *reinterpret_cast<uint32_t*>(&h2);
-            }
-            *reinterpret_cast<uint4*>(dst + i) = make_uint4(w[0], w[1], w[2], w[3]);
-          }
+          for (int i = 0; i < 2; ++i)
+            *reinterpret_cast<uint4*>(base + (size_t)grow * ld + i * 8) = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
         }
       }
       // the accumulator may be overwritten once the four warps of both CTAs have read it: tell rank 0
