@@ -117,7 +117,8 @@ int d3tom_set_reference_kernels(d3tom_ctx* ctx, int on);
 int d3tom_set_launch_overlap(int on);
 
 /* Tile shape of the dense layers (d3tom_proj_qkv, d3tom_linear, d3tom_ffn; Sec. 3.2.1 "Q = H W_Q", Algorithm 1
- * FFN_l): -1 (default) lets the library choose per shape (pairs from about two thousand rows on), 0 keeps single-CTA
+ * FFN_l): -1 (default) lets the library choose shape and width per call (pairs from 2048 rows on, and below where
+ * they take less time), 0 keeps single-CTA
  * tiles, 256 forces tiles of 256 x 256 computed by a pair of CTAs (cta_group::2) wherever the number of output columns
  * is a multiple of 256.  Results do not depend on the choice: every output is one fp32 accumulator over K in
  * ascending order, rounded once.  Process-wide; not thread-safe against concurrent launches.

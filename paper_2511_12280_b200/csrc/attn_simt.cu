@@ -293,8 +293,9 @@ int launch_simt(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s) {
   const long long per_sm = ((long long)grid.x * grid.y * grid.z + sms - 1) / sms;
   int smem = S::kBytes;
   if (per_sm <= 4) smem = max(smem, (int)(227 * 1024 / per_sm) - 1024);
-  // (the attribute belongs to the current device: set on every call, a process may drive several GPUs)
-  D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(attn_simt_kernel<T, DHP, RW, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  // (the attribute belongs to the current device: set on every call, a process may drive several GPUs; always to the same
+  // value, since another thread may be launching with another size)
+  D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(attn_simt_kernel<T, DHP, RW, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   D3TOM_CUDA_TRY(ctx, launch_serialized(attn_simt_kernel<T, DHP, RW, NW>, grid, NW * 32, smem, s, a, vec));
   return D3TOM_OK;
 }
