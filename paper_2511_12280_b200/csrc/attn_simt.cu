@@ -1,7 +1,7 @@
 // Bidirectional attention on CUDA cores (fp32 arithmetic) and the importance
 // finishing kernel shared with the tensor-core attention.
 //
-// A warp owns RW (16 or 8) query rows of one (request, head) and visits the keys 32 at a time with an online softmax
+// A warp owns RW (16, 8 or 4) query rows of one (request, head) and visits the keys 32 at a time with an online softmax
 // (log2 domain); the NW warps of a CTA share the K and V tiles, which come by asynchronous copies into two stages.  Scores
 // and P V run as register tiles out of shared memory (lane layout of f32_tile.cuh); P passes from lane to lane through
 // shared memory of the warp.  Every score is one chain of multiply-adds over head_dim, every output one chain over the
@@ -13,7 +13,7 @@
 //
 // Bound: the fp32 pipe and the latency of one to three warps per scheduler.  One warp per query row, every lane walking a
 // key of its own through global memory, took 1139 us at 1152 rows x 8 heads x 64 where this takes 98, and 111 us at
-// 288 x 4 x 64 where this takes 20.
+// 288 x 4 x 64 where this takes 17.
 #include "common.cuh"
 #include "f32_tile.cuh"
 
@@ -303,11 +303,13 @@ int launch_simt(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s) {
 // Rows per warp: with 16 a score needs fewer shared-memory reads, with 8 there are twice the warps to hide latency, which
 // wins until the SMs are full of warps anyway (from 16 eight-row warps per SM on).  Measured, 8 / 16 rows (us): 288 rows x
 // 4 heads x 64: 19.4 / 28.0; 600 x 8 x 64: 51.7 / 55.6; 1152 x 8 x 64: 95.8 / 102.0; 700 x 4 x 128: 73.7 / 130.7;
-// 1152 x 32 x 128: 639 / 564.
+// 1152 x 32 x 128: 639 / 564.  With 4 rows (so few warps that most schedulers would idle): 288 x 4 x 64 17.1, 300 x 4 x 128
+// 25.9 against 40.2, but 384 x 8 x 64 29.0 against 25.9.
 template <typename T, int DHP>
 int launch_simt_dh(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s) {
   const long long sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
   const long long warps8 = (long long)ceil_div(a.max_seqlen, 8) * a.H * a.B;
+  if (warps8 <= 2 * sms) return launch_simt<T, DHP, 4, 4>(ctx, a, s);
   return warps8 > 16 * sms ? launch_simt<T, DHP, 16, 4>(ctx, a, s) : launch_simt<T, DHP, 8, 4>(ctx, a, s);
 }
 

@@ -23,9 +23,10 @@ def _close(got, want):
     assert np.isfinite(err).all() and (err <= 1e-5 + 1e-4 * np.abs(want)).all(), err.max()
 
 
-# rows and heads that take 64-, 32- and 16-row CTAs; head sizes below, at and above the padded widths 32 / 64 / 128
+# rows and heads that take 16, 8 and 4 rows per warp; head sizes below, at and above the padded widths 32 / 64 / 128
 @pytest.mark.parametrize("lens,H,dh", [([1], 2, 64), ([15, 16, 17], 4, 64), ([31, 33], 2, 32), ([255, 257], 1, 36),
-                                       ([130], 3, 128), ([65, 1, 200], 2, 100), ([1152], 8, 64), ([700], 32, 4)])
+                                       ([130], 3, 128), ([65, 1, 200], 2, 100), ([1152], 8, 64), ([700], 32, 4), ([288], 4, 64),
+                                       ([600], 4, 128), ([2400], 8, 32)])
 @pytest.mark.parametrize("aligned", [True, False])
 def test_attention_and_importance_fp32(lens, H, dh, aligned):
     g = torch.Generator().manual_seed(sum(lens) + dh)
