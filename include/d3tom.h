@@ -270,7 +270,9 @@ int d3tom_merge(d3tom_ctx* ctx, d3tom_dtype dt, d3tom_agg mode,
  * equations; MEAN divides both by 1 + members, one reading of "renormalise"), and the
  * positions in M are dropped: k_out, v_out [total_out, D] are the shorter caches, rows
  * ordered as in d3tom_merge.  Every other argument is as in d3tom_merge; assign,
- * member_count and src_of_dst describe the routing shared by both tensors. */
+ * member_count and src_of_dst describe the routing shared by both tensors.
+ * k_out may lie over v_cache and v_out over k_cache (either or both; the two payloads
+ * then run one after the other); k_out must not lie over k_cache, nor v_out over v_cache. */
 int d3tom_merge_kv(d3tom_ctx* ctx, d3tom_dtype dt, d3tom_agg mode,
                    const void* k_cache, const void* v_cache,
                    const int32_t* cu_seqlens, const int32_t* n_visual, const int32_t* cu_vis,

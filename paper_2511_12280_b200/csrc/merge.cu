@@ -495,18 +495,25 @@ int launch_merge_aggregate(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
   const int mean = a.mode == D3TOM_AGG_MEAN ? 1 : 0;
   if (a.total_out <= 0) return D3TOM_OK;
   if (a.second != nullptr) {
-    // one payload's output may lie where the other's input was (the V cache written over the K cache): then one after the other
+    // One payload's output may lie where the other's input is: then they run one after the other, the payload whose input
+    // is about to be overwritten first.  Where each output lies over the other's input no order works, and the second
+    // payload's rows wait in the scratch of the gathered kept rows (free once the similarity has run).
     const size_t esize = a.dt == D3TOM_FP32 ? 4 : 2, in = (size_t)a.total_tokens * a.D * esize, out = (size_t)a.total_out * a.D * esize;
     auto overlap = [&](const void* x, const void* y) {
       return (uintptr_t)x < (uintptr_t)y + in && (uintptr_t)y < (uintptr_t)x + out;
     };
-    if (overlap(a.second_out, a.hidden) || overlap(a.hidden_out, a.second)) {
-      MergeArgs one = a;
-      one.second = nullptr; one.second_out = nullptr;
-      const int st = launch_merge_aggregate(ctx, one, s);
-      if (st != D3TOM_OK) return st;
-      one.hidden = a.second; one.hidden_out = a.second_out;
-      return launch_merge_aggregate(ctx, one, s);
+    const bool over_first = overlap(a.second_out, a.hidden), over_second = overlap(a.hidden_out, a.second);
+    if (over_first || over_second) {
+      MergeArgs first = a, second = a;
+      first.second = second.second = nullptr;
+      first.second_out = second.second_out = nullptr;
+      second.hidden = a.second;
+      second.hidden_out = over_first && over_second ? ctx->kept_rows : a.second_out;
+      int st = launch_merge_aggregate(ctx, over_second ? second : first, s);
+      if (st == D3TOM_OK) st = launch_merge_aggregate(ctx, over_second ? first : second, s);
+      if (st == D3TOM_OK && over_first && over_second)
+        D3TOM_CUDA_TRY(ctx, cudaMemcpyAsync(a.second_out, ctx->kept_rows, out, cudaMemcpyDeviceToDevice, s));
+      return st;
     }
   }
   {   // the streaming pipeline takes every row size it supports; the kernel below is the general one

@@ -110,3 +110,28 @@ def test_merge_kv_value_cache_written_over_the_key_cache():
         outs.append((k_out.clone(), v_out.clone()))
     assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
     ctx.close()
+
+
+@pytest.mark.parametrize("v_over_k", [False, True])
+@pytest.mark.parametrize("V,k", [(300, 40), (5000, 4200)])          # the plain aggregation and the streaming one
+def test_merge_kv_key_cache_written_over_the_value_cache(V, k, v_over_k):
+    dev, D, P = torch.device("cuda", 0), 256, 5
+    g = torch.Generator().manual_seed(V)
+    kc, vc = (torch.randn(V + P, D, generator=g).to(torch.bfloat16).to(dev) for _ in range(2))
+    i32 = lambda *a: torch.tensor(a, dtype=torch.int32, device=dev)
+    kept = torch.randperm(V, generator=g)[:k].sort().values.to(torch.int32).to(dev)
+    ctx = B_.Context(V + P, 1, 2, 128, 1, V)
+    idx = [torch.empty(V + P, dtype=torch.int32, device=dev) for _ in range(3)]
+    n = k + P
+    outs = []
+    for over in (False, True):
+        a, b = kc.clone(), vc.clone()
+        # (five rows into the other cache: the overlap need not start where the cache does)
+        k_out = b[5:5 + n] if over else torch.empty(n, D, dtype=torch.bfloat16, device=dev)
+        v_out = a[:n] if over and v_over_k else torch.empty(n, D, dtype=torch.bfloat16, device=dev)
+        ctx.d3tom_merge_kv(B_.AGG_MEAN, a, b, i32(0, V + P), i32(V), i32(0, V), kept, i32(0, k), 1, D, V + P, n, V, k, k_out, v_out,
+                           i32(0, n), *idx)
+        torch.cuda.synchronize()
+        outs.append((k_out.clone(), v_out.clone()))
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+    ctx.close()
