@@ -31,7 +31,7 @@ struct d3tom_ctx {
   int* agg_counter;             // [2] work and exit counters of the streaming aggregation; the kernel leaves them at zero
   int4* row_desc;               // [max_total_tokens] per output row: {source row, members or -1, list offset, request start}
   float* gemm_split_ws;         // [2 * sm_count][256][128] fp32 partial similarity tiles (K slices of a tile)
-  int* gemm_split_counters;     // [2 * sm_count] slices done per tile; zero between launches
+  int* gemm_split_counters;     // [2 * sm_count] slices arrived per tile (similarity: and shares done / left behind); zero between launches
   float* attn_part_ws;          // [sm_count][2][128 + 2][128] fp32: O tile and (m, l) of an attention item's later key tiles
   int* attn_part_flags;         // [sm_count][2][4] one word per (CTA, query tile, warp); zero between launches
   int* dev_status;              // device status word

@@ -32,7 +32,8 @@ constexpr int kGemmThreads = 224;      // warps: 0 A loads, 1 MMA, 2..5 epilogue
 
 enum { kEpiProj = 0, kEpiSim = 1, kEpiLinear = 2, kEpiGateUp = 3 };
 constexpr int kMaxKSplits = 4;        // K slices per tile at most when the last slice to arrive adds them all
-constexpr int kCoopSlices = 16;       // K slices per similarity tile at most when every slice adds its own share of the columns
+constexpr int kCoopSlices = 16;       // K slices per similarity tile at most (every slice adds its own share of the columns)
+constexpr uint64_t kSliceWaitNs = 200000ull;   // after this long a slice leaves its share of a tile to the last one
 
 struct GemmParams {
   int num_k_blocks;           // K / 64
@@ -274,10 +275,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       ptx::tc_fence_after_sync();
       uint32_t t_row = tmem_base + (uint32_t)buf * S::kAccStride + ((uint32_t)(quarter * 32) << 16);
       int m_base = tc.m0;                                       // first row of the 128-row half in hand
-      // A tile whose K range is cut into slices on different SMs: every unit writes its partial sums out
-      // (column-major, so a warp's 32 rows are one 128-byte line); the unit that completes the tile (a
-      // counter, left at zero again) adds the parts in the order of the K slices and runs the epilogue on
-      // the sums: same values whichever unit comes last.
+      // A tile whose K range is cut into slices on different SMs: every unit writes its partial sums out (column-major, so
+      // a warp's 32 rows are one 128-byte line) and counts itself in.  Dense layers: the unit that completes the tile
+      // adds the parts in the order of the K slices and runs the epilogue on the sums (the counter is left at zero
+      // again).  Similarity: every slice adds up its share of the columns (below).  Same values whichever unit comes last.
       const bool split = un.nsp > 1;
       constexpr bool coop = EPI == kEpiSim;                     // every slice adds up a share of the columns, or the last one adds all
       const int ws_tile = t - p.full_tiles;                     // cut tiles are numbered from zero in the workspace
@@ -298,33 +299,38 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         if (lane == 0) ptx::mbar_arrive(&acc_empty[buf]);          // the accumulator is free again
         __threadfence();
         asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (et == 0) s_prev = atomicAdd(p.split_counters + ws_tile, 1);
-        asm volatile("bar.sync 1, 128;" ::: "memory");
         if (!coop) {
+          if (et == 0) s_prev = atomicAdd(p.split_counters + ws_tile, 1);
+          asm volatile("bar.sync 1, 128;" ::: "memory");
           last = s_prev == un.nsp - 1;
           if (last) {
             if (et == 0) p.split_counters[ws_tile] = 0;
             __threadfence();
           }
         } else {
-          // every slice of the tile is a CTA of its own and all of them are resident: wait (bounded) until all have
-          // written, then each adds up its own share of the columns
+          // The slices of a tile are neighbouring CTAs and normally all resident: wait until all have written, then each
+          // adds up its own share of the columns.  Nothing depends on that, though: a slice that has waited kSliceWaitNs
+          // (the SMs may be held by another stream) leaves its share to the slice that arrives last.
+          // Counter word: bits 0..7 slices arrived, 8..15 shares done, 16..31 shares left behind.
           if (et == 0) {
-            const volatile int* ctr = p.split_counters + ws_tile;
-            const uint64_t t0 = ptx::globaltimer_ns();
-            uint32_t polls = 0;
-            s_prev = 1;
-            while (*ctr < un.nsp) {
-              if ((++polls & 0xffu) == 0u && (*abort_flag || ptx::globaltimer_ns() - t0 > ptx::kWaitLimitNs)) {
-                *abort_flag = 1;
-                atomicExch(p.dev_status, -5);
-                s_prev = 0;
-                break;
+            int* ctr = p.split_counters + ws_tile;
+            const int before = atomicAdd(ctr, 1);
+            s_prev = 1 << sp;                                                    // shares this CTA adds up
+            if ((before & 0xff) == un.nsp - 1) {
+              s_prev |= (int)((uint32_t)before >> 16);
+            } else {
+              const uint64_t t0 = ptx::globaltimer_ns();
+              uint32_t polls = 0;
+              while ((*static_cast<const volatile int*>(ctr) & 0xff) < un.nsp) {
+                if ((++polls & 0x3fu) == 0u && ptx::globaltimer_ns() - t0 > kSliceWaitNs) {
+                  // (had the last slice arrived before this word was set, it did not see it: the share is still ours)
+                  if ((atomicOr(ctr, (int)(1u << (16 + sp))) & 0xff) < un.nsp) s_prev = 0;
+                  break;
+                }
               }
             }
           }
           asm volatile("bar.sync 1, 128;" ::: "memory");
-          if (s_prev == 0) break;
           __threadfence();
         }
       }
@@ -359,17 +365,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       };
       if (!last) { ++lt; continue; }
       if (coop && split) {
-        // this slice's share of the tile's live columns in groups of eight: the sums over all slices (ascending slice
-        // order), then the arg-max over those columns; the 64-bit maximum over slices and tiles is order-independent
+        // shares of the tile's live columns in groups of eight, this slice's own and any left behind: the sums over all
+        // slices (ascending slice order), then the arg-max over those columns; the 64-bit maximum over slices and tiles
+        // is order-independent
         const int nsp = un.nsp;                                  // 2 .. 16
         const int groups = (min(BN, tc.kb - tc.n0) + 7) >> 3;
-        const int cb = sp * groups / nsp * 8, ce = (sp + 1) * groups / nsp * 8;
+        const int shares = s_prev;
         const int m = m_base + row;
         const int g = tc.v0 + m;
         const bool active = m < tc.Vb && p.assign[g] < 0;
         const float inm = active ? p.inv_norm[g] : 0.f;
         float best_sim = -INFINITY;
         int best_slot = 0;
+        int cb, ce;                                              // columns of the share in hand
         float* dbg = (p.sim_debug != nullptr && active) ? p.sim_debug + (size_t)g * p.max_kept + tc.n0 : nullptr;
         const float* tile_ws = p.split_ws + (size_t)ws_tile * nsp * BN * kBM + row;
         // kQ slices x kC columns of loads in flight (64 words a thread)
@@ -410,16 +418,26 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
             }
           }
         };
-        if (nsp > 4) add_up(Const<8>{}, Const<8>{});
-        else add_up(Const<4>{}, Const<16>{});
-        if (active && cb < ce) {
+        bool any = false;
+#pragma unroll 1
+        for (int left = shares; left != 0; left &= left - 1) {   // (ascending columns: the lowest slot wins a tie)
+          const int share = __ffs(left) - 1;
+          cb = share * groups / nsp * 8; ce = (share + 1) * groups / nsp * 8;
+          any |= cb < ce;
+          if (nsp > 4) add_up(Const<8>{}, Const<8>{});
+          else add_up(Const<4>{}, Const<16>{});
+        }
+        if (active && any) {
           const unsigned long long mine =
               ((unsigned long long)ordered_key(best_sim) << 32) | (0xffffffffu - (unsigned)best_slot);
           atomicMax(p.best + g, mine);
         }
-        // the counter goes on to twice the slices as they finish reading; the last one leaves it at zero
+        // whoever finishes the last share leaves the counter at zero (a slice that left its share behind is not coming back)
         asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (et == 0 && atomicAdd(p.split_counters + ws_tile, 1) == 2 * nsp - 1) p.split_counters[ws_tile] = 0;
+        if (et == 0 && shares != 0) {
+          const int n = __popc(shares), before = atomicAdd(p.split_counters + ws_tile, n << 8);
+          if (((before >> 8) & 0xff) + n == nsp) p.split_counters[ws_tile] = 0;
+        }
         ++lt;
         continue;
       }
@@ -1073,10 +1091,9 @@ int launch_sim_tc(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
   p.max_kept = a.max_kept; p.dev_status = ctx->dev_status;
   p.m_tiles = ceil_div(a.max_visual, kBM); p.batch = a.B;
   // Few tiles (short requests, small kept sets): a tile is 64 k-blocks of serial work on one SM while most SMs idle, so
-  // each tile's K range is cut into slices, each a CTA of its own, all resident at once (units <= SMs), and every slice
-  // adds up its share of the tile's columns over all slices.  The last arriver adding all columns alone cost more than the
-  // main loop: 2048 visual x 512 kept x 4096 (32 tiles, 4 slices) 28.6 us,
-  // shared 20.1.
+  // each tile's K range is cut into slices, each a CTA of its own (units <= SMs), and every slice adds up its share of
+  // the tile's columns over all slices.  The last arriver adding all columns alone cost more than the main loop:
+  // 2048 visual x 512 kept x 4096 (32 tiles, 4 slices) 28.6 us, shared 20.1.
   // 128-wide tiles also serve larger kept sets while eight slices of each still fit: half the exchange per slice
   // (577 x 173 x 1024: 13.6 -> 10.3 us).
   const long long narrow_tiles = (long long)p.m_tiles * ceil_div(a.max_kept, 128) * p.batch;

@@ -358,3 +358,44 @@ def test_a_wait_that_cannot_end_reports_timeout_and_leaves_the_context_usable():
     pu.assert_close(pu.f64(step.attn_out[:step.total]), want, w.dtype, "attention output after a timed-out wait")
     pu.assert_guard_rows_untouched(step)
     step.ctx.close()
+
+
+def test_similarity_slices_beside_another_stream_that_holds_the_sms():
+    # the K slices of a similarity tile wait for one another; they may not depend on being resident together.  A long fp32
+    # attention leaves two SMs free (one CTA of 32 rows per SM), and a second stream of higher priority runs merges of its
+    # own; every merge must end with the result it has alone
+    dev = torch.device("cuda", 0)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    i32 = lambda *a: torch.tensor(a, dtype=torch.int32, device=dev)
+    n = 32 * (sms - 2)
+    q, o_att = torch.randn(n, 128, device=dev), torch.empty(n, 128, device=dev)
+    cu, att = i32(0, n), B_.Context(n, 1, 1, 128, 1, n)
+    busy, low, high = torch.cuda.Stream(), torch.cuda.Stream(priority=0), torch.cuda.Stream(priority=-1)
+    for V, k, D, H in ((2048, 512, 4096, 32), (577, 173, 1024, 8), (256, 64, 4096, 32)):       # 4, 8 and 16 slices
+        g = torch.Generator().manual_seed(V)
+        x = torch.randn(V, D, generator=g).to(torch.bfloat16).to(dev)
+        kept = torch.randperm(V, generator=g)[:k].sort().values.to(torch.int32).to(dev)
+        ends, n_vis, cu_kept = i32(0, V), i32(V), i32(0, k)
+        ctxs = [B_.Context(V, 1, H, D // H, 1, V) for _ in range(2)]
+
+        def merge(ctx, stream):
+            o = [torch.empty(k, D, dtype=torch.bfloat16, device=dev), torch.empty(V, dtype=torch.int32, device=dev),
+                 torch.empty(k, dtype=torch.int32, device=dev), torch.empty(k, dtype=torch.int32, device=dev)]
+            assert x.shape == (V, D) and kept.shape == (k,) and o[0].shape == (k, D) and o[1].shape == (V,)
+            torch.cuda.synchronize() if stream is None else stream.wait_stream(torch.cuda.current_stream())
+            ctx.d3tom_merge(B_.AGG_SUM, x, ends, n_vis, ends, kept, cu_kept, 1, D, V, k, V, k, o[0], cu_kept, o[1], o[2], o[3],
+                            stream=stream)
+            return o
+
+        want = merge(ctxs[0], None)
+        torch.cuda.synchronize()
+        for _ in range(4):
+            att.d3tom_attn_varlen(q, q, q, cu, 1, n, n, 0.1, o_att, stream=busy)
+            got = [merge(ctxs[i & 1], (low, high)[i & 1]) for i in range(12)]
+            torch.cuda.synchronize()
+            for o in got:
+                assert all(torch.equal(t, w) for t, w in zip(o, want))
+        for c in ctxs:
+            assert c.device_status() == 0
+            c.close()
+    att.close()
