@@ -286,13 +286,7 @@ int launch_simt(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s) {
   const uintptr_t bits = (uintptr_t)a.q | (uintptr_t)a.k | (uintptr_t)a.v | (uintptr_t)a.out;
   const bool vec = sizeof(T) == 4 && bits % 16 == 0;
   dim3 grid(ceil_div(a.max_seqlen, S::kBM), a.H, a.B);
-  // At most ceil(CTAs / SMs) CTAs fit an SM (by the shared memory asked for): CTAs that start while the kernel before is
-  // draining would otherwise pile up on the SMs that are free first, and the fullest SM sets the time (a step of three
-  // 1152 / 384-row layers x 8 heads x 64: 316 us, against 255 us without launch overlap).
-  const long long sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
-  const long long per_sm = ((long long)grid.x * grid.y * grid.z + sms - 1) / sms;
-  int smem = S::kBytes;
-  if (per_sm <= 4) smem = max(smem, (int)(227 * 1024 / per_sm) - 1024);
+  const int smem = spread_smem(ctx, grid, S::kBytes, 4);
   // (the attribute belongs to the current device: set on every call, a process may drive several GPUs; always to the same
   // value, since another thread may be launching with another size)
   D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(attn_simt_kernel<T, DHP, RW, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));

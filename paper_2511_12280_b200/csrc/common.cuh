@@ -84,6 +84,19 @@ inline cudaError_t launch_serialized(void (*kernel)(Params...), dim3 grid, dim3 
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
 }
 
+// Dynamic shared memory to ask for so that at most ceil(CTAs / SMs) CTAs of a small grid fit an SM (`fit`: CTAs that fit
+// with `bytes` alone).  Under launch overlap, CTAs that start while the kernel before is draining would otherwise pile up
+// on the SMs that are free first, and the fullest SM sets the time (a step of three fp32 1152 / 384-row layers x 8 heads x
+// 64: 316 us, against 255 without launch overlap).  Without overlap nothing piles up, and the shared memory stays free
+// for kernels of other streams.
+inline int spread_smem(const d3tom_ctx* ctx, dim3 grid, int bytes, int fit) {
+  const long long sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
+  const long long per_sm = ((long long)grid.x * grid.y * grid.z + sms - 1) / sms;
+  if (!g_d3tom_launch_overlap || per_sm > fit) return bytes;
+  const int share = (int)(227 * 1024 / per_sm) - 1024;
+  return share > bytes ? share : bytes;
+}
+
 // largest b in [0, B) with cu[b] <= idx  (cu ascending, cu[0] = 0)
 __device__ __forceinline__ int find_segment(const int32_t* __restrict__ cu, int B, int idx) {
   int lo = 0, hi = B;   // invariant: cu[lo] <= idx < cu[hi]

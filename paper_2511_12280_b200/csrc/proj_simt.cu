@@ -155,11 +155,7 @@ template <typename T, int EPI, int WM, int WN, int WK>
 int launch_shape(d3tom_ctx* ctx, const SimtGemm<T>& p, cudaStream_t s) {
   using S = SimtGemmSmem<EPI, WM, WN, WK>;
   dim3 grid(ceil_div(p.n_cols, S::kBN), ceil_div(p.rows, S::kBM));
-  // at most ceil(CTAs / SMs) CTAs fit an SM, so that launch overlap does not pile them up on the SMs that drain first
-  // (a step with two layers of 384 rows x 512: 264 -> 238 us)
-  const long long sms = ctx->sm_count > 0 ? ctx->sm_count : 148, per_sm = ((long long)grid.x * grid.y + sms - 1) / sms;
-  int smem = S::kBytes;
-  if (per_sm <= 3) smem = max(smem, (int)(227 * 1024 / per_sm) - 1024);
+  const int smem = spread_smem(ctx, grid, S::kBytes, 3);      // (a step with two layers of 384 rows x 512: 264 -> 238 us)
   // (the attribute belongs to the current device: set on every call, a process may drive several GPUs; always to the same
   // value, since another thread may be launching with another size)
   D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(gemm_simt_kernel<T, EPI, WM, WN, WK>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));

@@ -74,3 +74,46 @@ def test_linear_and_gate_up_fp32(rows, K, N, aligned):
     h = torch.nn.functional.silu(x.double() @ w[:N].double().T) * (x.double() @ w[N:].double().T)
     _close(act, h)
     _close(out, act.double() @ wd.double().T)
+
+
+def _shared_memory_of_kernels(call):
+    """Dynamic shared memory that each kernel of `call` asks for, read from a recorded graph."""
+    from cuda.bindings import driver
+    call()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    raw = driver.CUgraph(graph.raw_cuda_graph())
+    _, _, n = driver.cuGraphGetNodes(raw)
+    err, nodes, n = driver.cuGraphGetNodes(raw, n)
+    assert err == driver.CUresult.CUDA_SUCCESS
+    out = []
+    for node in nodes[:n]:
+        if driver.cuGraphNodeGetType(node)[1] == driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            out.append(driver.cuGraphKernelNodeGetParams(node)[1].sharedMemBytes)
+    return out
+
+
+def test_small_calls_fill_an_sm_with_shared_memory_only_under_launch_overlap():
+    n, H, dh = 64, 2, 64
+    q, k, v = (torch.randn(n, H * dh, device="cuda") for _ in range(3))
+    out, y, w = torch.empty_like(q), torch.empty_like(q), torch.randn(H * dh, H * dh, device="cuda")
+    cu = torch.tensor([0, n], dtype=torch.int32, device="cuda")
+    ctx = B_.Context(n, 1, H, dh, 1, n)
+
+    def call():
+        ctx.d3tom_attn_varlen(q, k, v, cu, 1, n, n, 0.125, out)
+        ctx.d3tom_linear(q, w, None, n, H * dh, H * dh, y)
+
+    with_overlap = _shared_memory_of_kernels(call)
+    got = out.clone(), y.clone()
+    B_.d3tom_set_launch_overlap(False)
+    try:
+        without = _shared_memory_of_kernels(call)
+        assert torch.equal(got[0], out) and torch.equal(got[1], y)
+    finally:
+        B_.d3tom_set_launch_overlap(True)
+    assert len(with_overlap) == len(without) == 2
+    # one CTA per SM of 227 KB while kernels overlap; otherwise what the kernels use: at most 150 KB
+    assert all(b > 220 * 1024 for b in with_overlap) and all(b < 150 * 1024 for b in without), (with_overlap, without)
