@@ -309,7 +309,11 @@ int d3tom_proj_qkv(d3tom_ctx* ctx, d3tom_dtype dt, const void* x, const void* w_
  * this is the attention output projection.  out may be the residual buffer itself
  * (in-place add) but not x.  All pointers are device memory, caller-owned.
  * bf16 on the tensor-core path needs K % 64 == 0 and N % 128 == 0
- * (D3TOM_ERR_UNSUPPORTED otherwise); fp32 has no such limit. */
+ * (D3TOM_ERR_UNSUPPORTED otherwise); fp32 has no such limit.
+ * With fp32 storage every output is summed over K in one fixed order, here, in d3tom_ffn
+ * and in d3tom_proj_qkv: a row's results do not depend on the other rows of the call.
+ * With bf16 storage they agree to rounding (the fp32 sum over K may be cut into up to
+ * four slices, added in order, depending on the number of rows). */
 int d3tom_linear(d3tom_ctx* ctx, d3tom_dtype dt, const void* x, const void* w, const void* residual,
                  int rows, int K, int N, void* out, d3tom_stream stream);
 

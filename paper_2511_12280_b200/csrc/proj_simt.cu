@@ -4,9 +4,13 @@
 //
 // Dense layers: a CTA of 8 warps computes a (16 WM) x (32 WN) tile; WK warps share a 16 x 32 register tile (f32_tile.cuh) and cut
 // every k-block of 32 WK between them, so that small products, which have few tiles, keep short chains.  k-blocks come
-// through a ring of kStages buffers by 16-byte asynchronous copies.  Bound: the fp32 pipe and shared memory (a lane reads
-// 8 vectors per 64 multiply-adds): 42 TFLOP/s at 1152 x 12288 x 4096, 30 at 384 x 1536 x 512 (20 us; one output per
-// thread and two shared-memory reads per multiply-add took 83).
+// through a ring of kStages buffers by 16-byte asynchronous copies.
+// One order of sums for every tile shape: an output is four chains of multiply-adds (even and odd k apart), chain c over
+// the 32-deep pieces c, c + 4, c + 8, ... of K, and the four are added in this order.  A warp that owns more than one
+// chain walks its k-blocks chain by chain (the sums so far wait in shared memory: in registers they would cost the second
+// CTA per SM).  So a row has the same bits alone and in any batch, whichever tile serves it.
+// Bound: the fp32 pipe and shared memory (a lane reads 8 vectors per 64 multiply-adds): 42 TFLOP/s at 1152 x 12288 x 4096,
+// 30 at 384 x 1536 x 512 (20 us; one output per thread and two shared-memory reads per multiply-add took 83).
 #include "common.cuh"
 #include "f32_tile.cuh"
 
@@ -28,13 +32,15 @@ template <int EPI, int WM, int WN, int WK> struct SimtGemmSmem {
   static constexpr int kBM = 16 * WM, kBN = 32 * WN, kBK = 32 * WK, kLd = kBK + 4;
   static constexpr int kB = kBN * (EPI == kSimtGateUp ? 2 : 1);
   static constexpr int kStage = (kBM + kB) * kLd;        // floats
-  static constexpr int kBytes = kStages * kStage * 4;
+  static constexpr int kMats = EPI == kSimtGateUp ? 2 : 1;
+  static constexpr int kSums = WK == 4 ? 0 : 8 * kMats * 16 * 32;       // floats: sums of each warp's finished chains
+  static constexpr int kBytes = (kStages * kStage + kSums) * 4;
   static_assert(WM * WN * WK == 8, "eight warps");
   static_assert(kStages * kStage >= (WK - 1) * kBM * kB, "the slices' sums are exchanged in the ring");
 };
 
 template <typename T, int EPI, int WM, int WN, int WK>
-__global__ void __launch_bounds__(256, 1)
+__global__ void __launch_bounds__(256, EPI != kSimtGateUp && WK < 4 ? 2 : 1)
 gemm_simt_kernel(SimtGemm<T> p) {
   using S = SimtGemmSmem<EPI, WM, WN, WK>;
   constexpr int kLd = S::kLd, kMats = EPI == kSimtGateUp ? 2 : 1;
@@ -68,45 +74,80 @@ gemm_simt_kernel(SimtGemm<T> p) {
     }
     src_ok |= (ok ? 1u : 0u) << u;
   }
-  auto load_block = [&](int kb) {
-    if (kb < nkb) {
-      float* dst = ring + (kb % kStages) * S::kStage + lrow * kLd + lcol;
-      const int c = kb * S::kBK + lcol;
+  // The walk over the k-blocks: those of residue 0 of the block number modulo kTurns, then residue 1, ... (one chain per
+  // warp each); kb_load is the next one to load, nkb when there is none.
+  constexpr int kTurns = 4 / WK;
+  int kb_load = 0, turn_load = 0;
+  auto load_next = [&](float* stage) {
+    if (kb_load < nkb) {
+      float* dst = stage + lrow * kLd + lcol;
+      const int c = kb_load * S::kBK + lcol;
 #pragma unroll
       for (int u = 0; u < kLoads; ++u) f32::load4<T>(dst + u * kStep * kLd, src[u], c, p.K, (src_ok >> u) & 1u, p.vec);
+      kb_load += kTurns;
+      if (kTurns > 1 && kb_load >= nkb) kb_load = ++turn_load < kTurns ? turn_load : nkb;
     }
     f32::cp_async_commit();
   };
   float2 acc[kMats][4][4];
+  auto clear_acc = [&] {
 #pragma unroll
-  for (int t = 0; t < kMats; ++t)
+    for (int t = 0; t < kMats; ++t)
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+      for (int r = 0; r < 4; ++r)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[t][r][j] = make_float2(0.f, 0.f);
-  for (int kb = 0; kb < kStages - 1; ++kb) load_block(kb);
-  for (int kb = 0; kb < nkb; ++kb) {
-    f32::cp_async_wait<kStages - 2>();
-    __syncthreads();                       // block kb is there for everyone, and everyone is done with block kb - 1
-    load_block(kb + kStages - 1);
-    const float* st = ring + (kb % kStages) * S::kStage;
-    const float* aw = st + wm * 16 * kLd + wk * 32;
-    const float* bw = st + (S::kBM + wn * 32) * kLd + wk * 32;
+        for (int j = 0; j < 4; ++j) acc[t][r][j] = make_float2(0.f, 0.f);
+  };
+  constexpr int kTile = kMats * 16 * 32;
+  float4* sums = reinterpret_cast<float4*>(ring + kStages * S::kStage + warp * kTile) + lane;      // of this lane's outputs
+  auto end_chain = [&](bool first) {
 #pragma unroll
-    for (int t = 0; t < kMats; ++t) f32::dot_16x32<kLd, kLd, 8>(acc[t], aw, bw + t * S::kBN * kLd, ty, tx);
+    for (int t = 0; t < kMats; ++t)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        float4* sum = sums + (t * 4 + r) * 32;
+        float4 v = make_float4(acc[t][r][0].x + acc[t][r][0].y, acc[t][r][1].x + acc[t][r][1].y,
+                               acc[t][r][2].x + acc[t][r][2].y, acc[t][r][3].x + acc[t][r][3].y);
+        if (!first) { const float4 o = *sum; v = make_float4(o.x + v.x, o.y + v.y, o.z + v.z, o.w + v.w); }
+        *sum = v;
+      }
+    clear_acc();
+  };
+  clear_acc();
+#pragma unroll
+  for (int i = 0; i < kStages - 1; ++i) load_next(ring + i * S::kStage);
+  float* st = ring;                                       // this k-block's stage, and the one read before it
+  float* st_before = ring + (kStages - 1) * S::kStage;
+  for (int turn = 0; turn < kTurns && turn < nkb; ++turn) {
+    for (int kb = turn; kb < nkb; kb += kTurns) {
+      f32::cp_async_wait<kStages - 2>();
+      __syncthreads();                     // this block is there for everyone, and everyone is done with the one before
+      load_next(st_before);
+      const float* aw = st + wm * 16 * kLd + wk * 32;
+      const float* bw = st + (S::kBM + wn * 32) * kLd + wk * 32;
+#pragma unroll
+      for (int t = 0; t < kMats; ++t) f32::dot_16x32<kLd, kLd, 8>(acc[t], aw, bw + t * S::kBN * kLd, ty, tx);
+      st_before = st;
+      st = st == ring + (kStages - 1) * S::kStage ? ring : st + S::kStage;
+    }
+    if (turn < kTurns - 1) end_chain(turn == 0);          // (the last chain stays in the accumulators; zeros where K has no piece for it)
   }
   float c[kMats][4][4];
 #pragma unroll
   for (int t = 0; t < kMats; ++t)
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < 4; ++r) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) c[t][r][j] = acc[t][r][j].x + acc[t][r][j].y;
+      if (WK == 1) {
+        const float4 o = sums[(t * 4 + r) * 32];
+        c[t][r][0] = o.x + c[t][r][0]; c[t][r][1] = o.y + c[t][r][1]; c[t][r][2] = o.z + c[t][r][2]; c[t][r][3] = o.w + c[t][r][3];
+      }
+    }
   if (WK > 1) {
-    // the WK slices of a register tile meet in shared memory and are added in slice order by the first
+    // the chains of a register tile meet in shared memory and are added by the first warp
     f32::cp_async_wait<0>();
     __syncthreads();
-    constexpr int kTile = kMats * 16 * 32;
     float* mine = ring + ((wm * WN + wn) * (WK - 1) + (wk - 1)) * kTile;
     if (wk > 0) {
 #pragma unroll
@@ -118,15 +159,22 @@ gemm_simt_kernel(SimtGemm<T> p) {
     }
     __syncthreads();
     if (wk > 0) return;
-    for (int q = 0; q < WK - 1; ++q) {
-      const float* other = ring + ((wm * WN + wn) * (WK - 1) + q) * kTile;
+    const float* others = ring + (wm * WN + wn) * (WK - 1) * kTile + lane;
 #pragma unroll
-      for (int t = 0; t < kMats; ++t)
+    for (int t = 0; t < kMats; ++t)
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+      for (int r = 0; r < 4; ++r) {
+        const float* o = others + (t * 4 + r) * 4 * 32;
+        if (WK == 2) {                     // chain 0 waits here, chain 1 with the other warp
+          const float4 s0 = sums[(t * 4 + r) * 32], s1 = sums[(t * 4 + r) * 32 + kTile / 4];
+          const float s01[4] = {s0.x + s1.x, s0.y + s1.y, s0.z + s1.z, s0.w + s1.w};
 #pragma unroll
-          for (int j = 0; j < 4; ++j) c[t][r][j] += other[((t * 4 + r) * 4 + j) * 32 + lane];
-    }
+          for (int j = 0; j < 4; ++j) c[t][r][j] = (s01[j] + c[t][r][j]) + o[j * 32];
+        } else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) c[t][r][j] = ((c[t][r][j] + o[j * 32]) + o[j * 32 + kTile]) + o[j * 32 + 2 * kTile];
+        }
+      }
   }
 #pragma unroll
   for (int r = 0; r < 4; ++r) {

@@ -117,3 +117,70 @@ def test_small_calls_fill_an_sm_with_shared_memory_only_under_launch_overlap():
     assert len(with_overlap) == len(without) == 2
     # one CTA per SM of 227 KB while kernels overlap; otherwise what the kernels use: at most 150 KB
     assert all(b > 220 * 1024 for b in with_overlap) and all(b < 150 * 1024 for b in without), (with_overlap, without)
+
+
+def _heads_tails(n):
+    """Row ranges to run by themselves: short, middle and long, so that other tiles serve them than the whole batch."""
+    return [(0, 1), (n // 3, n // 3 + 33), (0, n // 2), (n - 200, n)]
+
+
+@pytest.mark.parametrize("n,K,N", [(1500, 512, 768), (640, 130, 200), (2000, 96, 512), (700, 1000, 96), (3000, 33, 64)])
+def test_dense_layers_give_a_row_the_same_bits_alone_and_in_a_batch(n, K, N):
+    g = torch.Generator().manual_seed(n + K)
+    x, w, wd = (torch.randn(*s, generator=g).cuda() * c for s, c in (((n, K), 1.0), ((2 * N, K), 0.05), ((K, N), 0.05)))
+    wq = torch.randn(3 * K, K, generator=g).cuda() * 0.05
+    ctx = B_.Context(n, 1, 1, 4, 1, 1)
+
+    def run(a, b):
+        m = b - a
+        xs = x[a:b].contiguous()
+        y, act, out = torch.empty(m, N, device="cuda"), torch.empty(m, N, device="cuda"), torch.empty(m, K, device="cuda")
+        q, k, v = (torch.empty(m, K, device="cuda") for _ in range(3))
+        ctx.d3tom_linear(xs, w[:N], None, m, K, N, y)
+        ctx.d3tom_ffn(xs, w, wd, xs, m, K, N, act, out)
+        ctx.d3tom_proj_qkv(xs, wq, m, K, q, k, v)
+        return y, act, out, q, k, v
+
+    whole = run(0, n)
+    for a, b in _heads_tails(n):
+        for got, want in zip(run(a, b), whole):
+            assert torch.equal(got, want[a:b]), (a, b)
+
+
+# one request among others, with lengths at which 4, 8 and 16 rows per warp serve the launch
+@pytest.mark.parametrize("lens,H,dh", [([288, 40], 4, 64), ([288, 900, 100], 4, 64), ([288, 1400, 1400], 8, 64), ([150, 700], 32, 128),
+                                       ([75, 31], 2, 36)])
+def test_attention_importance_and_merge_give_a_request_the_same_bits_alone_and_in_a_batch(lens, H, dh):
+    g = torch.Generator().manual_seed(sum(lens))
+    D = H * dh
+    q, k, v = (torch.randn(sum(lens), D, generator=g).cuda() for _ in range(3))
+    vis, keep = [m // 2 for m in lens], [m // 5 for m in lens]
+    cs = lambda a: torch.tensor(np.concatenate([[0], np.cumsum(a)]), dtype=torch.int32, device="cuda")
+    i32 = lambda a: torch.tensor(a, dtype=torch.int32, device="cuda")
+    kept = [torch.randperm(nv, generator=g)[:kc].sort().values.to(torch.int32).cuda() for nv, kc in zip(vis, keep)]
+
+    def run(which):
+        m, B, lo = [lens[i] for i in which], len(which), [sum(lens[:i]) for i in which]
+        n, nv, kc = sum(m), [vis[i] for i in which], [keep[i] for i in which]
+        rows = torch.cat([torch.arange(a, a + b) for a, b in zip(lo, m)]).cuda()
+        qq, kk, vv = (t[rows].contiguous() for t in (q, k, v))
+        dec = i32(np.concatenate([np.arange(b - b // 8, b) for b in m]))
+        cu_dec = [b // 8 for b in m]
+        ctx = B_.Context(n, B, H, dh, int(sum(cu_dec)), max(nv))
+        out, imp = torch.empty(n, D, device="cuda"), torch.empty(sum(nv), device="cuda")
+        ctx.d3tom_attn_importance(qq, kk, vv, cs(m), i32(nv), dec, cs(cu_dec), B, n, max(m), max(nv), int(sum(cu_dec)), dh ** -0.5,
+                                  out, imp, cs(nv))
+        lo_out = [b - c + e for b, c, e in zip(m, nv, kc)]
+        total_out = sum(lo_out)
+        h_out, assign = torch.empty(total_out, D, device="cuda"), torch.empty(sum(nv), dtype=torch.int32, device="cuda")
+        count, src = torch.empty(sum(kc), dtype=torch.int32, device="cuda"), torch.empty(total_out, dtype=torch.int32, device="cuda")
+        ctx.d3tom_merge(B_.AGG_SUM, out, cs(m), i32(nv), cs(nv), torch.cat([kept[i] for i in which]), cs(kc), B, D, n, total_out,
+                        max(nv), max(kc), h_out, cs(lo_out), assign, count, src)
+        torch.cuda.synchronize()
+        assert ctx.device_status() == 0
+        ctx.close()
+        return out[:m[0]], imp[:nv[0]], assign[:nv[0]], count[:kc[0]], h_out[:lo_out[0]]
+
+    alone, together = run([0]), run(list(range(len(lens))))
+    for a, b in zip(alone, together):
+        assert torch.equal(a, b)
