@@ -29,6 +29,8 @@ template <int DHP, int RW, int NW> struct SimtSmem {
   static constexpr int kBytes = (kQ + 4 * kKv + kP) * 4 + kBM * 4;
 };
 
+template <int N> struct Rows { static constexpr int value = N; };
+
 template <typename T, int DHP, int RW, int NW>
 __global__ void __launch_bounds__(NW * 32)
 attn_simt_kernel(AttnArgs a, bool vec) {
@@ -53,21 +55,22 @@ attn_simt_kernel(AttnArgs a, bool vec) {
   constexpr int kVecs = DHP / 4, kStep = NW * 32 / kVecs > 0 ? NW * 32 / kVecs : 1;        // vectors per row, rows per pass of the CTA
   static_assert(NW * 32 >= kVecs, "a pass covers whole rows");
   const int lrow = tid / kVecs, lcol = (tid % kVecs) * 4;
-  auto load_rows = [&](float* dst, const T* src, int r0, int rows, int n_rows) {
-    dst += lrow * kLd + lcol;
+  auto load_rows = [&](auto rows, float* dst, const T* src, int r0, int n_rows) {
+    static_assert(decltype(rows)::value % kStep == 0, "every thread loads the same number of vectors");
     src += (size_t)(r0 + lrow) * ld;
-    for (int r = lrow; r < rows; r += kStep, dst += kStep * kLd, src += kStep * ld)
-      f32::load4<T>(dst, src, lcol, dh, r0 + r < n_rows, vec);
+    f32::load_vecs<T, decltype(rows)::value / kStep>(dst + lrow * kLd + lcol, kStep * kLd, [&](int u) {
+      return f32::RowRef<T>{src + (size_t)u * kStep * ld, r0 + lrow + u * kStep < n_rows};
+    }, lcol, dh, vec);
   };
   auto load_tile = [&](int t) {                           // K and V of key tile t, one copy group (empty past the end)
     if (t * kKeyTile < n) {
       float* st = kv_s + (t & 1) * 2 * S::kKv;
-      load_rows(st, kg, t * kKeyTile, kKeyTile, n);
-      load_rows(st + S::kKv, vg, t * kKeyTile, kKeyTile, n);
+      load_rows(Rows<kKeyTile>{}, st, kg, t * kKeyTile, n);
+      load_rows(Rows<kKeyTile>{}, st + S::kKv, vg, t * kKeyTile, n);
     }
     f32::cp_async_commit();
   };
-  load_rows(q_s, qg, 0, S::kBM, n - q0);
+  load_rows(Rows<S::kBM>{}, q_s, qg, 0, n - q0);
   load_tile(0);
   load_tile(1);
   // which of the rows are deciders?  (strictly ascending list: binary search)
@@ -282,9 +285,9 @@ namespace {
 template <typename T, int DHP, int RW, int NW>
 int launch_simt(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s) {
   using S = SimtSmem<DHP, RW, NW>;
-  // 16-byte copies and stores where the caller's buffers allow them (head_dim is a multiple of 4)
+  // copies and stores of four elements where the caller's buffers allow them (head_dim is a multiple of 4)
   const uintptr_t bits = (uintptr_t)a.q | (uintptr_t)a.k | (uintptr_t)a.v | (uintptr_t)a.out;
-  const bool vec = sizeof(T) == 4 && bits % 16 == 0;
+  const bool vec = bits % (4 * sizeof(T)) == 0;
   dim3 grid(ceil_div(a.max_seqlen, S::kBM), a.H, a.B);
   const int smem = spread_smem(ctx, grid, S::kBytes, 4);
   // (the attribute belongs to the current device: set on every call, a process may drive several GPUs; always to the same

@@ -22,7 +22,7 @@ enum { kSimtProj = 0, kSimtLinear = 1, kSimtGateUp = 2 };
 template <typename T> struct SimtGemm {
   const T* a; const T* b;          // A rows of the products, B rows (for the gate-up pass: gate rows, then the up rows from row n_cols on)
   int rows, n_cols, K;
-  bool vec;                        // 16-byte copies are possible
+  bool vec;                        // vectors of four elements are aligned
   T* out[3];                       // projection: q, k, v; otherwise out[0]
   const T* residual;
   int D;                           // projection: columns of one output
@@ -82,8 +82,7 @@ gemm_simt_kernel(SimtGemm<T> p) {
     if (kb_load < nkb) {
       float* dst = stage + lrow * kLd + lcol;
       const int c = kb_load * S::kBK + lcol;
-#pragma unroll
-      for (int u = 0; u < kLoads; ++u) f32::load4<T>(dst + u * kStep * kLd, src[u], c, p.K, (src_ok >> u) & 1u, p.vec);
+      f32::load_vecs<T, kLoads>(dst, kStep * kLd, [&](int u) { return f32::RowRef<T>{src[u], ((src_ok >> u) & 1u) != 0u}; }, c, p.K, p.vec);
       kb_load += kTurns;
       if (kTurns > 1 && kb_load >= nkb) kb_load = ++turn_load < kTurns ? turn_load : nkb;
     }
@@ -176,25 +175,34 @@ gemm_simt_kernel(SimtGemm<T> p) {
         }
       }
   }
+  const int row0 = m0 + wm * 16 + ty, col0 = n0 + wn * 32 + tx;
+  if (EPI == kSimtLinear && p.residual != nullptr) {
+    // all of the lane's residuals are requested before the first result is stored (out may be the residual buffer, so a
+    // store would hold the next load back)
+    T res[4][4];
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int row = m0 + wm * 16 + ty + 4 * r;
-    if (row < rows) {
+    for (int r = 0; r < 4; ++r)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int col = n0 + wn * 32 + tx + 8 * j;
-        if (col >= cols) continue;
-        if (EPI == kSimtProj) {
-          const int which = col / p.D;
-          p.out[which][(size_t)row * p.D + (col - which * p.D)] = Storage<T>::from_float(c[0][r][j]);
-        } else {
-          const size_t o = (size_t)row * cols + col;
-          float y = c[0][r][j];
-          if (EPI == kSimtGateUp) y = y / (1.f + expf(-y)) * c[kMats - 1][r][j];
-          else if (p.residual != nullptr) y += Storage<T>::to_float(p.residual[o]);
-          p.out[0][o] = Storage<T>::from_float(y);
-        }
-      }
+      for (int j = 0; j < 4; ++j)
+        if (row0 + 4 * r < rows && col0 + 8 * j < cols) res[r][j] = p.residual[(size_t)(row0 + 4 * r) * cols + col0 + 8 * j];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (row0 + 4 * r < rows && col0 + 8 * j < cols) c[0][r][j] += Storage<T>::to_float(res[r][j]);
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int col = col0 + 8 * j;
+    if (col >= cols) continue;
+    const int which = EPI == kSimtProj ? col / p.D : 0, ld = EPI == kSimtProj ? p.D : cols;
+    T* out = (which == 0 ? p.out[0] : which == 1 ? p.out[1] : p.out[2]) + (col - which * ld);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      if (row0 + 4 * r >= rows) continue;
+      float y = c[0][r][j];
+      if (EPI == kSimtGateUp) y = y / (1.f + expf(-y)) * c[kMats - 1][r][j];
+      out[(size_t)(row0 + 4 * r) * ld] = Storage<T>::from_float(y);
     }
   }
 }
@@ -217,7 +225,7 @@ int launch_shape(d3tom_ctx* ctx, const SimtGemm<T>& p, cudaStream_t s) {
 template <typename T, int EPI>
 int launch_simt_gemm(d3tom_ctx* ctx, SimtGemm<T> p, cudaStream_t s) {
   const uintptr_t bits = (uintptr_t)p.a | (uintptr_t)p.b;
-  p.vec = sizeof(T) == 4 && p.K % 4 == 0 && bits % 16 == 0;
+  p.vec = p.K % 4 == 0 && bits % (4 * sizeof(T)) == 0;
   const long long sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
   auto cost = [&](int bm, int bn, double scale) {
     const long long tiles = (long long)ceil_div(p.rows, bm) * ceil_div(p.n_cols, bn);
@@ -268,7 +276,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 sim_simt_kernel(const T* __restrict__ hidden, const T* __restrict__ kept_rows, const int32_t* __restrict__ cu_seqlens,
                 const int32_t* __restrict__ cu_vis, const int32_t* __restrict__ cu_kept, const int32_t* __restrict__ assign,
-                const float* __restrict__ inv_norm, const float* __restrict__ inv_norm_kept, int D, int max_kept, bool vec,
+                const float* __restrict__ inv_norm, const float* __restrict__ inv_norm_kept, int D, int max_kept,
                 unsigned long long* __restrict__ best, float* __restrict__ sim_debug) {
   using S = SimSmem<T>;
   constexpr int kVec = S::kVec, kChunk = S::kChunk, kLd = S::kLd;
@@ -300,9 +308,8 @@ sim_simt_kernel(const T* __restrict__ hidden, const T* __restrict__ kept_rows, c
   auto load_chunk = [&](int t) {
     if (t < n_chunks) {
       float* dst = ring + (t % kStages) * S::kStage + lrow * kLd + lcol;
-#pragma unroll
-      for (int u = 0; u < kLoads; ++u)
-        f32::load4<T>(dst + u * kStep * kLd, src[u], t * kChunk + lcol, D, (src_ok >> u) & 1u, vec);
+      f32::load_vecs<T, kLoads>(dst, kStep * kLd, [&](int u) { return f32::RowRef<T>{src[u], ((src_ok >> u) & 1u) != 0u}; },
+                                t * kChunk + lcol, D, true);         // (rows are 16-byte aligned: the preparation reads them so)
     }
     f32::cp_async_commit();
   };
@@ -385,12 +392,11 @@ template <typename T>
 int sim_t(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
   if (a.max_kept <= 0) return D3TOM_OK;
   const T* hidden = static_cast<const T*>(a.hidden);
-  const bool vec = sizeof(T) == 4 && (uintptr_t)hidden % 16 == 0;      // (D is a multiple of 8)
   dim3 grid(ceil_div(a.max_kept, kSimCols), ceil_div(a.max_visual, kSimRows), a.B);
   D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(sim_simt_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, SimSmem<T>::kBytes));
   D3TOM_CUDA_TRY(ctx, launch_serialized(sim_simt_kernel<T>, grid, 256, SimSmem<T>::kBytes, s, hidden,
                                         static_cast<const T*>(ctx->kept_rows), a.cu_seqlens, a.cu_vis, a.cu_kept, a.assign,
-                                        ctx->inv_norm, ctx->inv_norm_kept, a.D, a.max_kept, vec, ctx->best, a.sim_debug));
+                                        ctx->inv_norm, ctx->inv_norm_kept, a.D, a.max_kept, ctx->best, a.sim_debug));
   return D3TOM_OK;
 }
 

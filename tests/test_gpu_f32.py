@@ -76,6 +76,29 @@ def test_linear_and_gate_up_fp32(rows, K, N, aligned):
     _close(out, act.double() @ wd.double().T)
 
 
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("n,K,N", [(33, 130, 65), (70, 36, 40), (200, 256, 96)])
+def test_unaligned_buffers_give_the_same_bits(dt, n, K, N):
+    # fp32: asynchronous copies or scalar loads; bf16 on the CUDA-core kernels: loads of four elements or scalar ones
+    g = torch.Generator().manual_seed(n)
+    x, w, r = (torch.randn(*s, generator=g).cuda().to(dt) for s in ((n, K), (N, K), (n, N)))
+    qkv = [torch.randn(n, 72, generator=g).cuda().to(dt) for _ in range(3)]
+    cu = torch.tensor([0, n], dtype=torch.int32, device="cuda")
+    ctx = B_.Context(n, 1, 2, 36, 1, n)
+    ctx.set_reference_kernels(True)
+    outs = []
+    for move in (lambda t: t, _unaligned):
+        y, o = move(torch.empty(n, N, dtype=dt, device="cuda")), move(torch.empty(n, 72, dtype=dt, device="cuda"))
+        ctx.d3tom_linear(move(x), move(w), move(r), n, K, N, y)
+        ctx.d3tom_attn_varlen(*(move(t) for t in qkv), cu, 1, n, n, 36 ** -0.5, o)
+        torch.cuda.synchronize()
+        outs.append((y.clone(), o.clone()))
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+    # (fp32 sums of at most 256 terms of unit variance; bf16 rounds the result once more)
+    want = r.double() + x.double() @ w.double().T
+    assert ((outs[0][0].double() - want).abs() <= (1e-4 if dt == torch.float32 else 2.0 ** -8) * (1 + want.abs())).all()
+
+
 def _shared_memory_of_kernels(call):
     """Dynamic shared memory that each kernel of `call` asks for, read from a recorded graph."""
     from cuda.bindings import driver
