@@ -388,15 +388,72 @@ sim_simt_kernel(const T* __restrict__ hidden, const T* __restrict__ kept_rows, c
   }
 }
 
+// The same with one block per visual row: warp w scores slots w, w + 8, ..., lane l running chain l.  Same bits.
+template <typename T>
+__global__ void __launch_bounds__(256)
+sim_rows_kernel(const T* __restrict__ hidden, const T* __restrict__ kept_rows, const int32_t* __restrict__ cu_seqlens,
+                const int32_t* __restrict__ cu_vis, const int32_t* __restrict__ cu_kept, const int32_t* __restrict__ assign,
+                const float* __restrict__ inv_norm, const float* __restrict__ inv_norm_kept, int D, int max_kept,
+                unsigned long long* __restrict__ best, float* __restrict__ sim_debug) {
+  constexpr int kVec = Storage<T>::kVec;
+  grid_dependency_enter();
+  const int rq = blockIdx.y, m = blockIdx.x, v0 = cu_vis[rq];
+  if (m >= cu_vis[rq + 1] - v0) return;
+  const int g = v0 + m;
+  if (assign[g] >= 0) return;                                     // a kept token
+  const int k0 = cu_kept[rq], kb = cu_kept[rq + 1] - k0;
+  const T* hm = hidden + (size_t)(cu_seqlens[rq] + m) * D;
+  const float inm = inv_norm[g];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned long long mine = 0ull;
+  for (int s = warp; s < kb; s += 8) {
+    const T* hk = kept_rows + (size_t)(k0 + s) * D;
+    float dot = 0.f;
+    for (int c = lane * kVec; c < D; c += 32 * kVec) {
+      float x[kVec], y[kVec];
+      Storage<T>::load(hm + c, x);
+      Storage<T>::load(hk + c, y);
+#pragma unroll
+      for (int i = 0; i < kVec; ++i) dot = fmaf(x[i], y[i], dot);
+    }
+    dot = warp_sum(dot);
+    const float sim = (dot * inm) * inv_norm_kept[k0 + s] + 0.0f;
+    const unsigned long long packed = ((unsigned long long)ordered_key(sim) << 32) | (0xffffffffu - (unsigned)s);
+    mine = packed > mine ? packed : mine;
+    if (lane == 0 && sim_debug != nullptr) sim_debug[(size_t)g * max_kept + s] = sim;
+  }
+  __shared__ unsigned long long red[8];
+  if (lane == 0) red[warp] = mine;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long r = red[0];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) r = red[w] > r ? red[w] : r;
+    best[g] = r;
+  }
+}
+
 template <typename T>
 int sim_t(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
   if (a.max_kept <= 0) return D3TOM_OK;
   const T* hidden = static_cast<const T*>(a.hidden);
-  dim3 grid(ceil_div(a.max_kept, kSimCols), ceil_div(a.max_visual, kSimRows), a.B);
+  const T* kept_rows = static_cast<const T*>(ctx->kept_rows);
+  const dim3 grid(ceil_div(a.max_kept, kSimCols), ceil_div(a.max_visual, kSimRows), a.B);
+  // One block per row where there are few dot products: a tile is one serial pass over D on one SM, and with few kept
+  // tokens most of its columns are empty.  Whole merges, rows / tiles (us): 9 visual, 3 kept, D = 4096 20.5 / 34.4;
+  // 512, 24, 512 18.9 / 20.6; 512, 32, 512 equal; 1024, 8, 1024 20 / 23; 1024, 16, 1024 25.9 / 24.9; 4096, 8, 4096 equal;
+  // 20000, 8, 4096 620 / 420.
+  const long long rows = (long long)a.max_visual * a.B;
+  if ((a.max_kept <= 24 && rows <= 512) || (a.max_kept <= 8 && rows <= 4096)) {
+    D3TOM_CUDA_TRY(ctx, launch_serialized(sim_rows_kernel<T>, dim3(a.max_visual, a.B), 256, 0, s, hidden, kept_rows, a.cu_seqlens,
+                                          a.cu_vis, a.cu_kept, a.assign, ctx->inv_norm, ctx->inv_norm_kept, a.D, a.max_kept,
+                                          ctx->best, a.sim_debug));
+    return D3TOM_OK;
+  }
   D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(sim_simt_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, SimSmem<T>::kBytes));
-  D3TOM_CUDA_TRY(ctx, launch_serialized(sim_simt_kernel<T>, grid, 256, SimSmem<T>::kBytes, s, hidden,
-                                        static_cast<const T*>(ctx->kept_rows), a.cu_seqlens, a.cu_vis, a.cu_kept, a.assign,
-                                        ctx->inv_norm, ctx->inv_norm_kept, a.D, a.max_kept, ctx->best, a.sim_debug));
+  D3TOM_CUDA_TRY(ctx, launch_serialized(sim_simt_kernel<T>, grid, 256, SimSmem<T>::kBytes, s, hidden, kept_rows, a.cu_seqlens,
+                                        a.cu_vis, a.cu_kept, a.assign, ctx->inv_norm, ctx->inv_norm_kept, a.D, a.max_kept,
+                                        ctx->best, a.sim_debug));
   return D3TOM_OK;
 }
 

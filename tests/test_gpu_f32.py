@@ -207,3 +207,38 @@ def test_attention_importance_and_merge_give_a_request_the_same_bits_alone_and_i
     alone, together = run([0]), run(list(range(len(lens))))
     for a, b in zip(alone, together):
         assert torch.equal(a, b)
+
+
+# kept counts and lengths on either side of the line between one block per row and tiles of 16 x 32: same bits
+@pytest.mark.parametrize("V,k,D", [(9, 3, 4096), (512, 24, 64), (500, 5, 72), (1024, 8, 1000), (33, 32, 256), (4096, 8, 512)])
+def test_similarity_fp32_gives_the_same_bits_by_rows_and_by_tiles(V, k, D):
+    g = torch.Generator().manual_seed(V)
+    n, P, pad, pad_keep = V + 4, 4, 5000, 40
+    x = torch.randn(n + pad, D, generator=g).cuda()
+    kept = torch.randperm(V, generator=g)[:k].sort().values.to(torch.int32)
+    more = torch.randperm(pad, generator=g)[:pad_keep].sort().values.to(torch.int32)
+    i32 = lambda a: torch.tensor(a, dtype=torch.int32, device="cuda")
+    got = []
+    for B in (1, 2):                      # alone, and with a request beside it that is long enough for the tiles
+        vis, keep, lens = [V, pad][:B], [k, pad_keep][:B], [n, pad][:B]
+        cs = lambda a: i32([0] + list(np.cumsum(a)))
+        out_lens = [k + P, pad_keep][:B]
+        ctx = B_.Context(sum(lens), B, D // 8, 8, 1, max(vis))
+        out = torch.empty(sum(out_lens), D, device="cuda")
+        assign, sim = torch.empty(sum(vis), dtype=torch.int32, device="cuda"), torch.full((sum(vis), max(keep)), 7.0, device="cuda")
+        count, src = (torch.empty(m, dtype=torch.int32, device="cuda") for m in (sum(keep), sum(out_lens)))
+        ctx.d3tom_merge(B_.AGG_SUM, x[:sum(lens)], cs(lens), i32(vis), cs(vis), torch.cat([kept, more][:B]).cuda(), cs(keep), B, D,
+                        sum(lens), sum(out_lens), max(vis), max(keep), out, cs(out_lens), assign, count, src, sim)
+        torch.cuda.synchronize()
+        assert ctx.device_status() == 0
+        got.append((assign[:V], sim[:V, :k], out[:k + P], count[:k]))
+        ctx.close()
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
+    unit = torch.nn.functional.normalize(x[:V].double(), dim=1)
+    cos = unit @ unit[kept.long().cuda()].T
+    pruned = torch.ones(V, dtype=torch.bool, device="cuda")
+    pruned[kept.long().cuda()] = False
+    # (32 chains of at most D / 32 products of unit rows, added pairwise: far inside 1e-5)
+    assert (got[0][1][pruned].double() - cos[pruned]).abs().max() <= 1e-5
+    assert torch.equal(got[0][0][pruned].long(), got[0][1][pruned].argmax(dim=1))
