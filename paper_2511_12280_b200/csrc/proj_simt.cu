@@ -418,9 +418,11 @@ sim_rows_kernel(const T* __restrict__ hidden, const T* __restrict__ kept_rows, c
     }
     dot = warp_sum(dot);
     const float sim = (dot * inm) * inv_norm_kept[k0 + s] + 0.0f;
-    const unsigned long long packed = ((unsigned long long)ordered_key(sim) << 32) | (0xffffffffu - (unsigned)s);
-    mine = packed > mine ? packed : mine;
-    if (lane == 0 && sim_debug != nullptr) sim_debug[(size_t)g * max_kept + s] = sim;
+    if (lane == 0) {
+      const unsigned long long packed = ((unsigned long long)ordered_key(sim) << 32) | (0xffffffffu - (unsigned)s);
+      mine = packed > mine ? packed : mine;
+      if (sim_debug != nullptr) sim_debug[(size_t)g * max_kept + s] = sim;
+    }
   }
   __shared__ unsigned long long red[8];
   if (lane == 0) red[warp] = mine;
@@ -440,11 +442,12 @@ int sim_t(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
   const T* kept_rows = static_cast<const T*>(ctx->kept_rows);
   const dim3 grid(ceil_div(a.max_kept, kSimCols), ceil_div(a.max_visual, kSimRows), a.B);
   // One block per row where there are few dot products: a tile is one serial pass over D on one SM, and with few kept
-  // tokens most of its columns are empty.  Whole merges, rows / tiles (us): 9 visual, 3 kept, D = 4096 20.5 / 34.4;
-  // 512, 24, 512 18.9 / 20.6; 512, 32, 512 equal; 1024, 8, 1024 20 / 23; 1024, 16, 1024 25.9 / 24.9; 4096, 8, 4096 equal;
-  // 20000, 8, 4096 620 / 420.
+  // tokens most of its columns are empty.  Whole merges, rows / tiles (us; visual, kept, D): 9, 3, 4096 20.5 / 34.4;
+  // 512, 24, 512 18.9 / 20.6, with 32 kept equal; 1024, 8, 1024 20 / 23, with 16 kept 25.9 / 24.9.  Eight kept tokens or
+  // fewer until the rows no longer come out of L2: 10000, 4, 1024 90 / 108; 4096, 8, 4096 and 6000, 4, 4096 equal; 8000, 8,
+  // 4096 251 / 191.
   const long long rows = (long long)a.max_visual * a.B;
-  if ((a.max_kept <= 24 && rows <= 512) || (a.max_kept <= 8 && rows <= 4096)) {
+  if ((a.max_kept <= 24 && rows <= 512) || (a.max_kept <= 8 && rows * a.D <= (24ll << 20))) {
     D3TOM_CUDA_TRY(ctx, launch_serialized(sim_rows_kernel<T>, dim3(a.max_visual, a.B), 256, 0, s, hidden, kept_rows, a.cu_seqlens,
                                           a.cu_vis, a.cu_kept, a.assign, ctx->inv_norm, ctx->inv_norm_kept, a.D, a.max_kept,
                                           ctx->best, a.sim_debug));

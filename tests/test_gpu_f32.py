@@ -210,7 +210,7 @@ def test_attention_importance_and_merge_give_a_request_the_same_bits_alone_and_i
 
 
 # kept counts and lengths on either side of the line between one block per row and tiles of 16 x 32: same bits
-@pytest.mark.parametrize("V,k,D", [(9, 3, 4096), (512, 24, 64), (500, 5, 72), (1024, 8, 1000), (33, 32, 256), (4096, 8, 512)])
+@pytest.mark.parametrize("V,k,D", [(9, 3, 4096), (512, 24, 64), (500, 5, 72), (1024, 8, 1000), (33, 32, 256), (4096, 8, 512), (4800, 8, 4096)])
 def test_similarity_fp32_gives_the_same_bits_by_rows_and_by_tiles(V, k, D):
     g = torch.Generator().manual_seed(V)
     n, P, pad, pad_keep = V + 4, 4, 5000, 40
