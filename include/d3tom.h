@@ -120,10 +120,17 @@ int d3tom_set_launch_overlap(int on);
  * FFN_l): -1 (default) lets the library choose shape and width per call (pairs from 2048 rows on, and below where
  * they take less time), 0 keeps single-CTA
  * tiles, 256 forces tiles of 256 x 256 computed by a pair of CTAs (cta_group::2) wherever the number of output columns
- * is a multiple of 256.  Results do not depend on the choice: every output is one fp32 accumulator over K in
- * ascending order, rounded once.  Process-wide; not thread-safe against concurrent launches.
+ * is a multiple of 256.  Results agree to rounding whatever the choice: a pair tile is one fp32 accumulator over K in
+ * ascending order, single-CTA tiles of a launch's last round may sum a long K in up to four slices, added in order.
+ * Process-wide; not thread-safe against concurrent launches.
  * Returns D3TOM_ERR_INVALID_ARG for other values. */
 int d3tom_set_pair_tiles(int width);
+
+/* The width of the pair tiles that a bf16 dense layer of `rows` x `n_cols` outputs over K takes on a device of `sms`
+ * multiprocessors that holds `pairs` CTA pairs at once (sms / 2 when nothing else runs), under the current setting of
+ * d3tom_set_pair_tiles; 0 for single-CTA tiles.  n_cols is 3 D for d3tom_proj_qkv, N for d3tom_linear, and 2 m with
+ * gate_up != 0 for the first pass of d3tom_ffn.  Host arithmetic: the rule the launches use. */
+int d3tom_pair_tile_width(int sms, int pairs, int rows, int n_cols, int K, int gate_up);
 
 /* Which tensor-core attention kernel serves d3tom_attn_varlen / d3tom_attn_importance (Sec. 3.2.1): -1 (default) the
  * library's choice per launch, 0 the kernels with two query tiles per CTA, 1 the kernel with one query tile per CTA and

@@ -49,6 +49,7 @@ _SIGNATURES = {
     "d3tom_set_reference_kernels": (_I, [_P, _I]),
     "d3tom_set_launch_overlap": (_I, [_I]),
     "d3tom_set_pair_tiles": (_I, [_I]),
+    "d3tom_pair_tile_width": (_I, [_I, _I, _I, _I, _I, _I]),
     "d3tom_set_single_tile_attention": (_I, [_I]),
     "d3tom_keep_count": (_I, [_I, C.c_double]),
     "d3tom_schedule_alpha": (_I, [_I, _I, C.c_double, C.c_double, _I, C.POINTER(C.c_double)]),
@@ -128,6 +129,11 @@ def d3tom_set_pair_tiles(width: int):
     """Tile shape of the dense layers: -1 chosen per shape (default), 0 single-CTA tiles only, 256 forces
     256 x 256 tiles computed by CTA pairs wherever the layer's width allows."""
     _check(load().d3tom_set_pair_tiles(int(width)), "d3tom_set_pair_tiles")
+
+
+def d3tom_pair_tile_width(sms: int, pairs: int, rows: int, n_cols: int, K: int, gate_up: bool = False) -> int:
+    """Width of the pair tiles that a bf16 dense layer takes, 0 for single-CTA tiles (host arithmetic)."""
+    return load().d3tom_pair_tile_width(sms, pairs, rows, n_cols, K, int(gate_up))
 
 
 def d3tom_set_single_tile_attention(mode: int):

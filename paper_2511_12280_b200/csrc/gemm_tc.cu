@@ -795,19 +795,37 @@ EncodeTiledFn get_encode_fn() {
 // 15 - 18 us; reading the slices back through bulk copies instead of register loads did not change it, so it is the
 // cold start of the short main loops and the fence / counter round trips rather than the read-back), so cutting
 // pays for long K only: the down projection of the feed-forward network, not the 64-k-block projections.
-void plan_tail_split(const d3tom_ctx* ctx, GemmParams& p) {
-  const int tiles = p.m_tiles * p.n_tiles * p.batch, sms = ctx->sm_count;
-  p.k_splits = 1; p.full_tiles = tiles;
+// Returns the number of slices (1: the tiles stay whole).
+int tail_slices(int sms, int tiles, int num_k_blocks) {
   const int rem = tiles % sms;
-  if (rem == 0 || p.split_ws == nullptr) return;
-  int best = p.num_k_blocks, best_s = 1;
-  for (int sp = 2; sp <= kMaxKSplits; ++sp) {
-    if (p.num_k_blocks / sp < 8 || rem * sp > 2 * sms) break;      // slices too short / more parts than the workspace holds
+  int best = num_k_blocks, best_s = 1;
+  for (int sp = 2; sp <= kMaxKSplits && rem > 0; ++sp) {
+    if (num_k_blocks / sp < 8 || rem * sp > 2 * sms) break;      // slices too short / more parts than the workspace holds
     const int rounds = (rem * sp + sms - 1) / sms;
-    const int cost = rounds * ((p.num_k_blocks + sp - 1) / sp) + 30 + 5 * sp;
+    const int cost = rounds * ((num_k_blocks + sp - 1) / sp) + 30 + 5 * sp;
     if (cost < best) { best = cost; best_s = sp; }
   }
-  if (best_s > 1) { p.k_splits = best_s; p.full_tiles = tiles - rem; }
+  return best_s;
+}
+void plan_tail_split(const d3tom_ctx* ctx, GemmParams& p) {
+  const int tiles = p.m_tiles * p.n_tiles * p.batch;
+  p.k_splits = tail_slices(ctx->sm_count, tiles, p.num_k_blocks);
+  p.full_tiles = p.k_splits > 1 ? tiles - tiles % ctx->sm_count : tiles;
+}
+
+// Width of 128-row tiles: fewest (rounds of tiles over the SMs) x (measured cycles per 64-deep k-block at that width:
+// 667 / 633 / 600 for 256 / 192 / 128 columns; narrow tiles pay the per-k-block barrier traffic of the issuing thread
+// more often per unit of work).
+int one_m_tile_width(int sms, int rows, int ncols) {
+  int bn = 128;
+  double best_cost = 1e30;
+  for (int cand : {256, 192, 128}) {
+    if (ncols % cand != 0) continue;
+    const long long tiles = (long long)ceil_div(rows, kBM) * (ncols / cand);
+    const double cost = (double)((tiles + sms - 1) / sms) * (cand == 256 ? 667.0 : cand == 192 ? 633.0 : 600.0);
+    if (cost < best_cost) { best_cost = cost; bn = cand; }
+  }
+  return bn;
 }
 
 // Which tile shape finishes a dense layer sooner, from measured main-loop cycles per 64 of K (projection timings at
@@ -818,8 +836,7 @@ void plan_tail_split(const d3tom_ctx* ctx, GemmParams& p) {
 // cost 0.89 of that per round and sometimes need a round less, or fill the last one better (1216 rows x 12288
 // columns: 275 tiles in two rounds, 93 us against 99 us for the 240 tiles of 256 x 256).
 // Returns the width of the 256-row tile to use (256 or 224), or 0 for 128-row tiles.
-int two_m_tile_width(const d3tom_ctx* ctx, int rows, int ncols, bool allow_224) {
-  const int sms = ctx->sm_count;
+int two_m_tile_width(int sms, int rows, int ncols, bool allow_224) {
   const long long t1 = (long long)ceil_div(rows, kBM) * ceil_div(ncols, 256);
   const double r1 = (double)(t1 % sms);
   const double cost1 = 850.0 * (double)(t1 / sms) + (r1 > 0 ? 150.0 + 3.9 * r1 : 0.0);
@@ -902,16 +919,19 @@ int launch_gemm_pair(d3tom_ctx* ctx, const CUtensorMap& ta, const CUtensorMap& t
 // Width of the CTA-pair tiles for a dense layer of `rows` x `ncols` outputs (for the gate-up pass the columns of both
 // matrices), or 0 for single-CTA tiles.  A round of pair tiles costs the times below per 64 of K whatever it computes, so
 // the width that fills the rounds best wins; against it stand rounds of single-CTA tiles, whose last, partial round is
-// cheaper, and K slices for a long K (plan_tail_split).  All figures in us per 64 of K, fitted to the four layers of a
+// cheaper, and K slices for a long K (tail_slices).  All figures in us per 64 of K, fitted to the four layers of a
 // block (D = 4096, m = 12288) at 128 .. 4288 rows.  What it changes, old shapes / pairs (us): projection 640 rows
 // 56 / 51; output projection 1216 rows 69 / 55, 1536 rows 57 / 49, 2600 rows 81 / 75 (224 columns; 83 with 256); down
 // projection 640 rows 82 / 62, 1800 rows 171 / 155; feed-forward network 1216 rows 308 / 282.  The factor
 // 1.08 is for power: the pairs move half the operand bytes, and the board's limit sets the clock under these layers.
-// From 2048 rows on the pairs are always taken.
-int pair_tile_width(const d3tom_ctx* ctx, int rows, int ncols, int num_k_blocks, int pairs, bool gate_up) {
+// From 2048 rows on the pairs are taken, with two exceptions, measured single-CTA / pairs (us, rows x K x columns):
+//   - all single-CTA tiles together are one round of K slices, which then walk a half to a quarter of K each where a pair
+//     walks all of it: 2100 x 16384 x 128 35 / 78, 2048 x 12288 x 384 30 / 49, 2048 x 8192 x 512 28 / 35;
+//   - widths that 256 does not divide at a K below 1024, where a pair's longer start and drain show: 2100 x 128 x 640
+//     4.5 / 5.3, 2600 x 512 x 384 6.6 / 7.1; with more rounds the pairs win again, 4288 x 512 x 640 9.1 / 7.6.
+int pair_tile_width(int sms, int rows, int ncols, int num_k_blocks, int pairs, bool gate_up) {
   if (pairs <= 0 || g_d3tom_pair_tiles == 0) return 0;
   if (g_d3tom_pair_tiles == 256) return ncols % 256 == 0 ? 256 : 0;
-  const int sms = ctx->sm_count;
   constexpr int kWidths[] = {256, 224, 192, 160, 128};
   constexpr double kPerBlock[] = {0.36, 0.345, 0.31, 0.30, 0.29};
   double best = 1e30;
@@ -921,23 +941,35 @@ int pair_tile_width(const d3tom_ctx* ctx, int rows, int ncols, int num_k_blocks,
     const double cost = kPerBlock[i] * (double)((tiles + pairs - 1) / pairs);
     if (cost < best) { best = cost; width = kWidths[i]; }
   }
-  if (rows >= 2048) return width;
   auto rounds = [&](int bm, int bn, double full, double last0, double last_r) {
     const long long tiles = (long long)ceil_div(rows, bm) * ceil_div(ncols, bn);
     const long long r = tiles % sms;
     return full * (double)(tiles / sms) + (r > 0 ? last0 + last_r * (double)r : 0.0);
   };
-  double single = rounds(kBM, 256, 0.40, 0.26, 0.0009);
-  if (!gate_up) {      // (the pass of two matrices walks whole tiles)
-    const long long tiles = (long long)ceil_div(rows, kBM) * ceil_div(ncols, 256);
-    const int rem = (int)(tiles % sms);
-    for (int sp = 2; sp <= kMaxKSplits && rem > 0; ++sp) {
-      if (num_k_blocks / sp < 8 || rem * sp > 2 * sms) break;
-      const double cut = (double)(ceil_div(rem * sp, sms) * ceil_div(num_k_blocks, sp) + 30 + 5 * sp) / num_k_blocks;
-      if (cut < 1.0) single = fmin(single, 0.40 * (double)(tiles / sms) + 0.42 * cut);
+  if (rows >= 2048) {
+    const int bn = gate_up ? 256 : one_m_tile_width(sms, rows, ncols);
+    const long long tiles = (long long)ceil_div(rows, kBM) * ceil_div(ncols, bn);
+    if (tiles < sms && two_m_tile_width(sms, rows, ncols, !gate_up) == 0) {
+      const int slices = tail_slices(sms, (int)tiles, num_k_blocks);
+      if (slices > 1 && tiles * slices <= sms) return 0;
     }
-    single = fmin(single, rounds(2 * kBM, 224, 0.65, 0.41, 0.0016));
+    if (ncols % 256 != 0 && num_k_blocks < 16) {
+      const double scale = bn == 256 ? 1.0 : bn == 192 ? 0.95 : 0.9;      // (one_m_tile_width's cycles)
+      return best * num_k_blocks + 1.0 < 1.08 * scale * rounds(kBM, bn, 0.40, 0.26, 0.0009) * num_k_blocks ? width : 0;
+    }
+    return width;
   }
+  // (the gate-up pass at a short K is bound by its epilogue: 1900 rows, D = 512, m = 12288 76.9 / 84.7)
+  if (gate_up && num_k_blocks < 16) return 0;
+  double single = rounds(kBM, 256, 0.40, 0.26, 0.0009);
+  const long long tiles = (long long)ceil_div(rows, kBM) * ceil_div(ncols, 256);
+  const int rem = (int)(tiles % sms);
+  for (int sp = 2; sp <= kMaxKSplits && rem > 0; ++sp) {
+    if (num_k_blocks / sp < 8 || rem * sp > 2 * sms) break;
+    const double cut = (double)(ceil_div(rem * sp, sms) * ceil_div(num_k_blocks, sp) + 30 + 5 * sp) / num_k_blocks;
+    if (cut < 1.0) single = fmin(single, 0.40 * (double)(tiles / sms) + 0.42 * cut);
+  }
+  if (!gate_up) single = fmin(single, rounds(2 * kBM, 224, 0.65, 0.41, 0.0016));
   single = fmin(single, rounds(2 * kBM, 256, 0.73, 0.46, 0.0018));
   // (a pair launch costs about 1.5 us more: with a short K the single-CTA tiles keep small layers, 319 x 3072 x 1024: 9.0 / 9.9)
   return best * num_k_blocks + 1.5 < 1.08 * single * num_k_blocks ? width : 0;
@@ -970,25 +1002,13 @@ int launch_proj_tc(d3tom_ctx* ctx, const void* x, const void* w, int total, int 
   p.out[0] = static_cast<__nv_bfloat16*>(q); p.out[1] = static_cast<__nv_bfloat16*>(k); p.out[2] = static_cast<__nv_bfloat16*>(v);
   p.out_rows = total; p.out_cols = D; p.dev_status = ctx->dev_status;
   p.m_tiles = ceil_div(total, kBM); p.batch = 1; p.k_splits = 1;
-  // Tile width: fewest (rounds of tiles over the SMs) x (measured cycles per 64-deep k-block at that
-  // width: 667 / 633 / 600 for 256 / 192 / 128 columns; narrow tiles pay the per-k-block barrier
-  // traffic of the issuing thread more often per unit of work).  192 divides 3 D whenever 64 divides D.
-  int bn = 128;
-  double best_cost = 1e30;
-  for (int cand : {256, 192, 128}) {
-    if ((3 * D) % cand != 0) continue;
-    const long long tiles = (long long)p.m_tiles * (3 * D / cand);
-    const double rounds = (double)((tiles + ctx->sm_count - 1) / ctx->sm_count);
-    const double cost = rounds * (cand == 256 ? 667.0 : cand == 192 ? 633.0 : 600.0);
-    if (cost < best_cost) { best_cost = cost; bn = cand; }
-  }
-  if (const int bn2 = pair_tile_width(ctx, total, 3 * D, p.num_k_blocks, resident_pairs<kEpiProj>(ctx), false)) {
+  if (const int bn2 = pair_tile_width(ctx->sm_count, total, 3 * D, p.num_k_blocks, resident_pairs<kEpiProj>(ctx), false)) {
     r = make_tmap_bf16_2d(&tb, w, (uint64_t)3 * D, (uint64_t)D, (uint64_t)D, (uint32_t)bn2 / 2);   // a CTA's half of the weight tile
     if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
     p.bn = bn2; p.m_tiles = ceil_div(total, 2 * kBM); p.n_tiles = ceil_div(3 * D, bn2);
     return launch_gemm_pair<kEpiProj>(ctx, ta, tb, p, s);
   }
-  if (const int w2 = two_m_tile_width(ctx, total, 3 * D, D % 32 == 0)) {
+  if (const int w2 = two_m_tile_width(ctx->sm_count, total, 3 * D, D % 32 == 0)) {
     r = make_tmap_bf16_2d(&ta, x, (uint64_t)total, (uint64_t)D, (uint64_t)D, 2 * kBM);
     if (r == 0) r = make_tmap_bf16_2d(&tb, w, (uint64_t)3 * D, (uint64_t)D, (uint64_t)D, (uint32_t)w2);
     if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
@@ -996,6 +1016,7 @@ int launch_proj_tc(d3tom_ctx* ctx, const void* x, const void* w, int total, int 
     if (w2 == 224) return launch_gemm<224, kEpiProj, 2>(ctx, ta, tb, p, s);
     return launch_gemm<256, kEpiProj, 2>(ctx, ta, tb, p, s);
   }
+  const int bn = one_m_tile_width(ctx->sm_count, total, 3 * D);      // (128 always divides 3 D)
   r = make_tmap_bf16_2d(&tb, w, (uint64_t)3 * D, (uint64_t)D, (uint64_t)D, (uint32_t)bn);
   if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
   p.n_tiles = 3 * D / bn;
@@ -1015,23 +1036,13 @@ int launch_linear_tc(d3tom_ctx* ctx, const void* x, const void* w, const void* r
   p.lin_out = static_cast<__nv_bfloat16*>(out); p.residual = static_cast<const __nv_bfloat16*>(residual);
   p.ld_out = N; p.out_rows = rows; p.dev_status = ctx->dev_status;
   p.m_tiles = ceil_div(rows, kBM); p.batch = 1; p.k_splits = 1;
-  // tile width as for the Q,K,V projection: fewest rounds of tiles over the SMs, weighted by the cycles per k-block
-  int bn = 128;
-  double best_cost = 1e30;
-  for (int cand : {256, 192, 128}) {
-    if (N % cand != 0) continue;
-    const long long tiles = (long long)p.m_tiles * (N / cand);
-    const double rounds = (double)((tiles + ctx->sm_count - 1) / ctx->sm_count);
-    const double cost = rounds * (cand == 256 ? 667.0 : cand == 192 ? 633.0 : 600.0);
-    if (cost < best_cost) { best_cost = cost; bn = cand; }
-  }
-  if (const int bn2 = pair_tile_width(ctx, rows, N, p.num_k_blocks, resident_pairs<kEpiLinear>(ctx), false)) {
+  if (const int bn2 = pair_tile_width(ctx->sm_count, rows, N, p.num_k_blocks, resident_pairs<kEpiLinear>(ctx), false)) {
     r = make_tmap_bf16_2d(&tb, w, (uint64_t)N, (uint64_t)K, (uint64_t)K, (uint32_t)bn2 / 2);
     if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
     p.bn = bn2; p.m_tiles = ceil_div(rows, 2 * kBM); p.n_tiles = ceil_div(N, bn2);
     return launch_gemm_pair<kEpiLinear>(ctx, ta, tb, p, s);
   }
-  if (const int w2 = two_m_tile_width(ctx, rows, N, true)) {
+  if (const int w2 = two_m_tile_width(ctx->sm_count, rows, N, true)) {
     r = make_tmap_bf16_2d(&ta, x, (uint64_t)rows, (uint64_t)K, (uint64_t)K, 2 * kBM);
     if (r == 0) r = make_tmap_bf16_2d(&tb, w, (uint64_t)N, (uint64_t)K, (uint64_t)K, (uint32_t)w2);
     if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
@@ -1039,6 +1050,7 @@ int launch_linear_tc(d3tom_ctx* ctx, const void* x, const void* w, const void* r
     if (w2 == 224) return launch_gemm<224, kEpiLinear, 2>(ctx, ta, tb, p, s);
     return launch_gemm<256, kEpiLinear, 2>(ctx, ta, tb, p, s);
   }
+  const int bn = one_m_tile_width(ctx->sm_count, rows, N);
   r = make_tmap_bf16_2d(&tb, w, (uint64_t)N, (uint64_t)K, (uint64_t)K, (uint32_t)bn);
   if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
   p.n_tiles = N / bn;
@@ -1059,14 +1071,14 @@ int launch_gate_up_tc(d3tom_ctx* ctx, const void* x, const void* w_gate_up, int 
   p.lin_out = static_cast<__nv_bfloat16*>(act); p.ld_out = m; p.up_row_offset = m; p.out_rows = rows;
   p.dev_status = ctx->dev_status;
   p.m_tiles = ceil_div(rows, kBM); p.n_tiles = m / 128; p.batch = 1; p.k_splits = 1;
-  if (const int bn2 = pair_tile_width(ctx, rows, 2 * m, p.num_k_blocks, resident_pairs<kEpiGateUp>(ctx), true)) {
+  if (const int bn2 = pair_tile_width(ctx->sm_count, rows, 2 * m, p.num_k_blocks, resident_pairs<kEpiGateUp>(ctx), true)) {
     r = make_tmap_bf16_2d(&tb, w_gate_up, (uint64_t)2 * m, (uint64_t)D, (uint64_t)D, (uint32_t)bn2 / 2);   // gate rows or up rows
     if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
     p.bn = bn2; p.m_tiles = ceil_div(rows, 2 * kBM); p.n_tiles = ceil_div(m, bn2 / 2);
     return launch_gemm_pair<kEpiGateUp>(ctx, ta, tb, p, s);
   }
   {
-    if (two_m_tile_width(ctx, rows, 2 * m, false) == 256) {
+    if (two_m_tile_width(ctx->sm_count, rows, 2 * m, false) == 256) {
       r = make_tmap_bf16_2d(&ta, x, (uint64_t)rows, (uint64_t)D, (uint64_t)D, 2 * kBM);
       if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
       p.m_tiles = ceil_div(rows, 2 * kBM);
@@ -1112,4 +1124,9 @@ int launch_sim_tc(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
   }
   p.n_tiles = ceil_div(a.max_kept, 128);
   return launch_gemm<128, kEpiSim>(ctx, ta, tb, p, s);
+}
+
+extern "C" int d3tom_pair_tile_width(int sms, int pairs, int rows, int n_cols, int K, int gate_up) {
+  if (sms <= 0 || pairs < 0 || rows <= 0 || n_cols <= 0 || K <= 0 || K % kBK != 0 || n_cols % 128 != 0) return 0;
+  return pair_tile_width(sms, rows, n_cols, K / kBK, pairs, gate_up != 0);
 }

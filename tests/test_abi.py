@@ -113,3 +113,28 @@ def test_log_line_per_call_when_the_environment_asks_for_it():
         assert r.returncode == 0, r.stderr
         has = "[d3tom] d3tom_create device 0: tokens 128 batch 1 heads 2 x 64" in r.stderr
         assert has == expect, (val, r.stderr)
+
+
+def test_pair_tile_width_rule(lib):
+    w = lambda rows, n_cols, K, gate_up=False: B_.d3tom_pair_tile_width(148, 74, rows, n_cols, K, gate_up)
+    for rows in (1, 64, 640, 1216, 2048, 4288, 8000):
+        for n_cols in (128, 384, 1024, 4096, 12288):
+            for K in (64, 512, 4096, 16384):
+                for gate_up in (False, True):
+                    assert w(rows, n_cols, K, gate_up) in (0, 128, 160, 192, 224, 256)
+    # the layers of a block (D = 4096, m = 12288) on long sequences
+    assert all(w(4288, n, k, g) == 256 for n, k, g in ((12288, 4096, False), (4096, 4096, False), (24576, 4096, True), (4096, 12288, False)))
+    # one round of K slices on single SMs beats a pair that walks all of K; so do few columns at a short K
+    assert w(2100, 128, 16384) == 0 and w(2048, 384, 12288) == 0 and w(2048, 512, 8192) == 0
+    assert w(2100, 640, 128) == 0 and w(4288, 640, 512) == 160
+    # the gate-up pass is cut along a long K like the other layers
+    assert w(319, 2048, 16384, gate_up=True) == 0
+    # no pairs on the device, switched off, or forced
+    assert B_.d3tom_pair_tile_width(148, 0, 4288, 4096, 4096) == 0 and w(0, 4096, 4096) == 0 and w(4288, 100, 4096) == 0
+    B_.d3tom_set_pair_tiles(0)
+    try:
+        assert w(4288, 4096, 4096) == 0
+        B_.d3tom_set_pair_tiles(256)
+        assert w(100, 256, 64) == 256 and w(100, 384, 64) == 0
+    finally:
+        B_.d3tom_set_pair_tiles(-1)

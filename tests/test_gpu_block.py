@@ -112,21 +112,47 @@ def test_long_dense_layers_take_cta_pairs_by_default():
     run_ffn(2100, 256, 256, "bf16", seed=9)
 
 
+def pair_width(rows, n_cols, K, gate_up=False):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    return B_.d3tom_pair_tile_width(sms, sms // 2, rows, n_cols, K, gate_up)
+
+
 # nine 256-row tiles on 74 pairs: eight column tiles fill one round, so the width follows the number of columns: 128, 160,
-# 160 with an overhang, 192, 192 with an overhang, 224, 224 with an overhang, 256; K of one, three and four 64-deep blocks
-# (the narrower tiles take two blocks per ring stage)
-@pytest.mark.parametrize("N,K", [(1024, 192), (1280, 64), (1152, 192), (1536, 256), (1408, 192), (1792, 192), (1664, 256), (2048, 192)])
-def test_pair_tiles_of_every_width(N, K):
+# 160 with an overhang, 192, 192 with an overhang, 224, 224 with an overhang, 256; K of one, three, four and seventeen
+# 64-deep blocks (the narrower tiles take two blocks per ring stage)
+@pytest.mark.parametrize("N,K,width", [(1024, 192, 128), (1280, 64, 160), (1152, 1088, 160), (1536, 256, 192), (1408, 192, 192),
+                                       (1792, 192, 224), (1664, 256, 224), (2048, 192, 256)])
+def test_pair_tiles_of_every_width(N, K, width):
+    assert pair_width(2100, N, K) == width
     run_linear(2100, K, N, "bf16", residual=True, seed=N)
 
 
-def test_pair_tiles_of_every_width_projection_and_gate_up():
-    run_proj(2100, 4, 128, seed=21)          # 3 D = 1536: width 192 straddles q | k and k | v
-    run_proj(2100, 3, 128, seed=22)          # 3 D = 1152: width 160, overhang
-    run_ffn(2100, 128, 640, "bf16", seed=23)        # 160: halves of 80 gate and 80 up rows
-    run_ffn(2100, 256, 896, "bf16", seed=24)        # 224: halves of 112
-    run_ffn(2100, 128, 1152, "bf16", seed=25)       # 160 in two rounds, the last tile hangs over the edge of both matrices
-    run_linear(600, 320, 5120, "bf16", residual=True, seed=26)      # below 2048 rows: pairs where their rounds are cheaper
+# rows, H (heads of 128), width: 192 straddles q | k and k | v; 256 and 128 columns of 1152, which 256 does not divide; a
+# layer below 2048 rows
+@pytest.mark.parametrize("rows,H,width", [(2100, 4, 192), (3333, 3, 256), (4000, 3, 128), (400, 13, 160)])
+def test_pair_tiles_projection(rows, H, width):
+    assert pair_width(rows, 3 * H * 128, H * 128) == width
+    run_proj(rows, H, 128, seed=20 + H)
+
+
+# halves of 80 gate and 80 up rows; of 112; 160 in two rounds, the last tile hanging over the edge of both matrices; a layer
+# below 2048 rows
+@pytest.mark.parametrize("rows,D,m,width", [(2100, 128, 640, 160), (2100, 256, 896, 224), (2100, 128, 1152, 160), (400, 2048, 1920, 128)])
+def test_pair_tiles_gate_up(rows, D, m, width):
+    assert pair_width(rows, 2 * m, D, gate_up=True) == width
+    run_ffn(rows, D, m, "bf16", seed=23)
+
+
+def test_pair_tiles_below_2048_rows_with_an_overhang():
+    assert pair_width(1930, 4736, 512) == 192          # 4736 = 24 tiles of 192 and one of 128
+    run_linear(1930, 512, 4736, "bf16", residual=True, seed=26)
+
+
+# single-CTA tiles from 2048 rows on: one round of K slices, and a width that 256 does not divide at a short K
+@pytest.mark.parametrize("rows,K,N", [(2100, 16384, 128), (2048, 8192, 384), (2100, 128, 640), (2600, 512, 384)])
+def test_long_layers_that_keep_single_cta_tiles(rows, K, N):
+    assert pair_width(rows, N, K) == 0
+    run_linear(rows, K, N, "bf16", residual=True, seed=K)
 
 
 def test_linear_fp32_odd_sizes():
