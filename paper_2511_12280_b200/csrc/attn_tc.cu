@@ -62,7 +62,8 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
 
 // kImp: the launch also feeds the importance map (decider rows look themselves up and store their scores); the
 // plain instance carries none of that code, which keeps its softmax loop at the registers and schedule it had.
-template <int DH, bool kImp>
+// kShort: requests of at most 48 rows (how the output is stored, see store_rows_64b).
+template <int DH, bool kImp, bool kShort>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                const __grid_constant__ CUtensorMap tmap_v, AttnArgs a) {
@@ -386,7 +387,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
 #pragma unroll
           for (int t = 0; t < 16; ++t)
             w[t] = pack_bf16x2(__uint_as_float(r[2 * t]) * inv_l, __uint_as_float(r[2 * t + 1]) * inv_l);
-          ptx::store_rows_64b(dst + c0, (size_t)a.H * DH * 2, n - warp_row, w);
+          ptx::store_rows_64b<kShort>(dst + c0, (size_t)a.H * DH * 2, n - warp_row, w);
         }
         if (dec_slot >= 0) a.lse_scratch[(size_t)h * a.max_deciders + dec_slot] = make_float2(m_used, l_sum);
       }
@@ -405,7 +406,9 @@ int launch(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s) {
   if (r == 0) r = make_tmap_bf16_2d(&tk, a.k, rows, cols, cols, kTile);
   if (r == 0) r = make_tmap_bf16_2d(&tv, a.v, rows, cols, cols, kTile);
   if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
-  auto kernel = a.decider_pos != nullptr ? attn_tc_kernel<DH, true> : attn_tc_kernel<DH, false>;
+  const bool short_call = a.max_seqlen <= 48;
+  auto kernel = a.decider_pos != nullptr ? (short_call ? attn_tc_kernel<DH, true, true> : attn_tc_kernel<DH, true, false>)
+                                         : (short_call ? attn_tc_kernel<DH, false, true> : attn_tc_kernel<DH, false, false>);
   D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<DH>::kBytes));
   AttnArgs k = a;
   k.nqb = ceil_div(a.max_seqlen, 2 * kTile);

@@ -31,6 +31,7 @@ constexpr int kBM = 128, kBK = 64;
 constexpr int kGemmThreads = 224;      // warps: 0 A loads, 1 MMA, 2..5 epilogue, 6 B loads
 
 enum { kEpiProj = 0, kEpiSim = 1, kEpiLinear = 2, kEpiGateUp = 3 };
+constexpr int kShortRows = 96;        // calls of at most this many rows store row by row
 constexpr int kMaxKSplits = 4;        // K slices per tile at most when the last slice to arrive adds them all
 constexpr int kCoopSlices = 16;       // K slices per similarity tile at most (every slice adds its own share of the columns)
 constexpr uint64_t kSliceWaitNs = 200000ull;   // after this long a slice leaves its share of a tile to the last one
@@ -126,7 +127,8 @@ struct TileCoord {
 
 constexpr int kMaxPrefixBatch = 64;     // ragged batches up to this many requests number only the tiles that exist
 
-template <int BN, int EPI, int MT = 1>
+// kShort: dense layers without a residual of at most kShortRows rows (how the results are stored, see store_rows_64b)
+template <int BN, int EPI, int MT = 1, bool kShort = false>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b, GemmParams p) {
   static_assert(MT == 1 || (BN >= 224 && BN % 32 == 0 && EPI != kEpiSim), "the 256-row tile serves the dense layers at 224 or 256 columns");
@@ -459,7 +461,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
               __nv_bfloat162 h2 = __floats2bfloat162_rn(r[2 * j], r[2 * j + 1]);
               w[j] = *reinterpret_cast<uint32_t*>(&h2);
             }
-            ptx::store_rows_64b(p.out[which] + (size_t)warp_row * p.out_cols + (gcol - which * p.out_cols),
+            ptx::store_rows_64b<kShort>(p.out[which] + (size_t)warp_row * p.out_cols + (gcol - which * p.out_cols),
                                 (size_t)p.out_cols * 2, n_valid, w);
           }
         }
@@ -470,7 +472,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           load32(c, r);
           if (tc.n0 + c < p.ld_out) {
             uint32_t w[16];
-            if (p.residual != nullptr) {
+            if (!kShort && p.residual != nullptr) {
               ptx::load_rows_64b(p.residual + (size_t)warp_row * p.ld_out + tc.n0 + c, (size_t)p.ld_out * 2, n_valid, w);
             } else {
 #pragma unroll
@@ -483,7 +485,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
               w[j] = *reinterpret_cast<uint32_t*>(&h2);
             }
             // (out may be the residual buffer: the piece of a row is read and written by the same lane)
-            ptx::store_rows_64b(p.lin_out + (size_t)warp_row * p.ld_out + tc.n0 + c, (size_t)p.ld_out * 2, n_valid, w);
+            ptx::store_rows_64b<kShort>(p.lin_out + (size_t)warp_row * p.ld_out + tc.n0 + c, (size_t)p.ld_out * 2, n_valid, w);
           }
         }
       } else if (EPI == kEpiGateUp) {
@@ -501,7 +503,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
                                                       __fdividef(g1, 1.f + __expf(-g1)) * up[2 * j + 1]);
             w[j] = *reinterpret_cast<uint32_t*>(&h2);
           }
-          ptx::store_rows_64b(p.lin_out + (size_t)warp_row * p.ld_out + tc.n0 + c, (size_t)p.ld_out * 2, n_valid, w);
+          ptx::store_rows_64b<kShort>(p.lin_out + (size_t)warp_row * p.ld_out + tc.n0 + c, (size_t)p.ld_out * 2, n_valid, w);
         }
       } else {
         const int m = m_base + row;
@@ -861,9 +863,12 @@ int launch_gemm(d3tom_ctx* ctx, const CUtensorMap& ta, const CUtensorMap& tb, Ge
   const long long units = p.full_tiles + (tiles - p.full_tiles) * p.k_splits;
   if (units <= 0) return D3TOM_OK;
   const int grid = (int)(units < ctx->sm_count ? units : ctx->sm_count);          // persistent: one CTA per SM
-  D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           GemmSmem<BN, MT>::kBytes));
-  D3TOM_CUDA_TRY(ctx, launch_serialized(gemm_tc_kernel<BN, EPI, MT>, grid, kGemmThreads, GemmSmem<BN, MT>::kBytes, s, ta, tb, p));
+  auto kernel = gemm_tc_kernel<BN, EPI, MT>;
+  if constexpr (EPI != kEpiSim && MT == 1) {
+    if (p.out_rows <= kShortRows && p.residual == nullptr) kernel = gemm_tc_kernel<BN, EPI, MT, true>;
+  }
+  D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmSmem<BN, MT>::kBytes));
+  D3TOM_CUDA_TRY(ctx, launch_serialized(kernel, grid, kGemmThreads, GemmSmem<BN, MT>::kBytes, s, ta, tb, p));
   return D3TOM_OK;
 }
 

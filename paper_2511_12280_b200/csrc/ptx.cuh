@@ -252,8 +252,21 @@ __device__ __forceinline__ void transpose_pieces(uint32_t (&w)[16]) {
 // on are not touched (loaded as zeros).  An access takes 64 contiguous bytes of eight rows.  In the row-per-lane layout it
 // would touch 32 lines with 16 bytes each: 32 passes and half-used sectors, microseconds at the end of every tile of 128
 // rows (output projection with residual, 640 rows x 4096: 30.6 -> 26.7 us; attention 640 rows x 32 heads x 128: 16.0 -> 14.8).
+// kShort: the row-per-lane layout, for kernels that serve calls of so few rows that the stores of an SM do not queue up.
+// There the exchange between lanes is the longer way, as code to fetch and to run (a choice at run time cost half of
+// it again, also for the longer calls): projection 64 rows x 384 x 128 3.6 us by rows, 4.0 with the exchange, attention of
+// one row x 32 heads 5.9 / 6.3; from 64 (attention) and 128 rows on the exchange is the faster one.
+template <bool kShort = false>
 __device__ __forceinline__ void store_rows_64b(void* base, size_t stride, int n_valid, uint32_t (&w)[16]) {
   const int lane = threadIdx.x & 31;
+  if constexpr (kShort) {
+    uint8_t* row = static_cast<uint8_t*>(base) + (size_t)lane * stride;
+    if (lane < n_valid)
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        *reinterpret_cast<uint4*>(row + t * 16) = make_uint4(w[4 * t], w[4 * t + 1], w[4 * t + 2], w[4 * t + 3]);
+    return;
+  }
   transpose_pieces(w);
   uint8_t* dst = static_cast<uint8_t*>(base) + (size_t)(lane & 28) * stride + (lane & 3) * 16;
 #pragma unroll

@@ -152,6 +152,14 @@ def run_attention_only(lens, H, seed=0):
     ctx.close()
 
 
+def test_attention_of_short_requests():
+    # launches of requests of up to 48 rows store the output row by row, others 64 bytes of eight rows at a time
+    run_attention_only([48], 3, seed=11)
+    run_attention_only([49], 3, seed=12)
+    run_attention_only([40, 48, 1, 33, 7], 2, seed=13)
+    run_attention_only([40, 64, 65, 1, 130], 2, seed=14)
+
+
 def test_attention_with_one_query_tile_per_cta():
     # the kernel with three score buffers: one key block only (the second warpgroup has nothing to do), two, three, four
     # (the buffers come round), ragged last blocks, one-row requests, a batch of unequal lengths (longest first), and a
