@@ -23,10 +23,31 @@ def _close(got, want):
     assert np.isfinite(err).all() and (err <= 1e-5 + 1e-4 * np.abs(want)).all(), err.max()
 
 
-# rows and heads that take 16, 8 and 4 rows per warp; head sizes below, at and above the padded widths 32 / 64 / 128
+def _launches(call):
+    """(grid, dynamic shared memory) of each kernel of `call`, read from a recorded graph."""
+    from cuda.bindings import driver
+    call()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    raw = driver.CUgraph(graph.raw_cuda_graph())
+    _, _, n = driver.cuGraphGetNodes(raw)
+    err, nodes, n = driver.cuGraphGetNodes(raw, n)
+    assert err == driver.CUresult.CUDA_SUCCESS
+    out = []
+    for node in nodes[:n]:
+        if driver.cuGraphNodeGetType(node)[1] == driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            p = driver.cuGraphKernelNodeGetParams(node)[1]
+            out.append(((p.gridDimX, p.gridDimY, p.gridDimZ), p.sharedMemBytes))
+    return out
+
+
+# rows and heads that take 4, 8 and (from ceil(rows / 8) x heads x requests > 16 x SMs on: the 1400-row batch with 64 columns, 620
+# rows with 100 and 128, 700 and 2400 with 32) 16 rows per warp; head sizes below, at and above the padded widths 32 / 64 / 128
 @pytest.mark.parametrize("lens,H,dh", [([1], 2, 64), ([15, 16, 17], 4, 64), ([31, 33], 2, 32), ([255, 257], 1, 36),
                                        ([130], 3, 128), ([65, 1, 200], 2, 100), ([1152], 8, 64), ([700], 32, 4), ([288], 4, 64),
-                                       ([600], 4, 128), ([2400], 8, 32)])
+                                       ([600], 4, 128), ([2400], 8, 32), ([1400, 1400], 8, 64), ([620], 32, 100), ([620], 32, 128)])
 @pytest.mark.parametrize("aligned", [True, False])
 def test_attention_and_importance_fp32(lens, H, dh, aligned):
     g = torch.Generator().manual_seed(sum(lens) + dh)
@@ -55,9 +76,37 @@ def test_attention_and_importance_fp32(lens, H, dh, aligned):
     assert ctx.device_status() == 0
 
 
-# products that take 64 x 64, 32 x 64 and 32 x 32 tiles, K with and without a remainder of the k-blocks and of the vectors
-@pytest.mark.parametrize("rows,K,N", [(1, 4, 4), (33, 130, 65), (70, 31, 40), (200, 256, 512), (640, 512, 1536), (65, 1000, 33),
-                                      (384, 96, 3000)])
+# products in 32 x 32, 64 x 64 and 32 x 64 tiles (linear and gate-up; the down product of a feed-forward network has its own),
+# K with and without a remainder of the k-blocks and of the vectors
+SHAPES = [(1, 4, 4), (33, 130, 65), (70, 31, 40), (200, 256, 512), (640, 512, 1536), (65, 1000, 33), (384, 96, 3000), (384, 100, 768),
+          (384, 768, 768), (512, 130, 1536), (256, 33, 1024)]
+
+
+def tile_that_runs(rows, n_cols, call):
+    """The tile shape of a dense layer's launch, from its grid."""
+    (grid, _), = _launches(call)
+    ran = [(bm, bn) for bm, bn in ((32, 32), (32, 64), (64, 64)) if grid == (-(-n_cols // bn), -(-rows // bm), 1)]
+    assert ran, grid
+    return ran[0]
+
+
+def test_the_dense_shapes_cover_every_tile():
+    def linear(rows, K, N):
+        x, w, y = torch.zeros(rows, K, device="cuda"), torch.zeros(N, K, device="cuda"), torch.empty(rows, N, device="cuda")
+        return tile_that_runs(rows, N, lambda: ctx.d3tom_linear(x, w, None, rows, K, N, y))
+
+    def proj(rows, D):
+        x, w = torch.zeros(rows, D, device="cuda"), torch.zeros(3 * D, D, device="cuda")
+        out = [torch.empty(rows, D, device="cuda") for _ in range(3)]
+        return tile_that_runs(rows, 3 * D, lambda: ctx.d3tom_proj_qkv(x, w, rows, D, *out))
+
+    ctx = B_.Context(2000, 1, 1, 4, 1, 1)
+    assert {linear(*s) for s in SHAPES} == {(32, 32), (32, 64), (64, 64)}
+    assert linear(384, 768, 768) == proj(512, 512) == proj(384, 130) == (32, 64)
+    assert proj(1500, 100) == (64, 64) and proj(33, 100) == (32, 32)
+
+
+@pytest.mark.parametrize("rows,K,N", SHAPES)
 @pytest.mark.parametrize("aligned", [True, False])
 def test_linear_and_gate_up_fp32(rows, K, N, aligned):
     g = torch.Generator().manual_seed(rows + K)
@@ -74,6 +123,22 @@ def test_linear_and_gate_up_fp32(rows, K, N, aligned):
     h = torch.nn.functional.silu(x.double() @ w[:N].double().T) * (x.double() @ w[N:].double().T)
     _close(act, h)
     _close(out, act.double() @ wd.double().T)
+
+
+# 32 x 64 tiles (with and without remainders), 64 x 64 and 32 x 32
+@pytest.mark.parametrize("rows,H,dh", [(512, 8, 64), (384, 13, 10), (1500, 5, 20), (33, 5, 20)])
+@pytest.mark.parametrize("aligned", [True, False])
+def test_projection_fp32(rows, H, dh, aligned):
+    g = torch.Generator().manual_seed(rows)
+    D = H * dh
+    x, w = torch.randn(rows, D, generator=g).cuda(), torch.randn(3 * D, D, generator=g).cuda() * 0.05
+    if not aligned:
+        x, w = _unaligned(x), _unaligned(w)
+    ctx = B_.Context(rows, 1, H, 4, 1, 1)
+    out = [torch.full((rows, D), float("nan"), device="cuda") for _ in range(3)]
+    ctx.d3tom_proj_qkv(x, w, rows, D, *out)
+    for i, t in enumerate(out):
+        _close(t, x.double() @ w[i * D:(i + 1) * D].double().T)
 
 
 @pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
@@ -99,25 +164,6 @@ def test_unaligned_buffers_give_the_same_bits(dt, n, K, N):
     assert ((outs[0][0].double() - want).abs() <= (1e-4 if dt == torch.float32 else 2.0 ** -8) * (1 + want.abs())).all()
 
 
-def _shared_memory_of_kernels(call):
-    """Dynamic shared memory that each kernel of `call` asks for, read from a recorded graph."""
-    from cuda.bindings import driver
-    call()
-    torch.cuda.synchronize()
-    graph = torch.cuda.CUDAGraph(keep_graph=True)
-    with torch.cuda.graph(graph):
-        call()
-    raw = driver.CUgraph(graph.raw_cuda_graph())
-    _, _, n = driver.cuGraphGetNodes(raw)
-    err, nodes, n = driver.cuGraphGetNodes(raw, n)
-    assert err == driver.CUresult.CUDA_SUCCESS
-    out = []
-    for node in nodes[:n]:
-        if driver.cuGraphNodeGetType(node)[1] == driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
-            out.append(driver.cuGraphKernelNodeGetParams(node)[1].sharedMemBytes)
-    return out
-
-
 def test_small_calls_fill_an_sm_with_shared_memory_only_under_launch_overlap():
     n, H, dh = 64, 2, 64
     q, k, v = (torch.randn(n, H * dh, device="cuda") for _ in range(3))
@@ -129,11 +175,11 @@ def test_small_calls_fill_an_sm_with_shared_memory_only_under_launch_overlap():
         ctx.d3tom_attn_varlen(q, k, v, cu, 1, n, n, 0.125, out)
         ctx.d3tom_linear(q, w, None, n, H * dh, H * dh, y)
 
-    with_overlap = _shared_memory_of_kernels(call)
+    with_overlap = [b for _, b in _launches(call)]
     got = out.clone(), y.clone()
     B_.d3tom_set_launch_overlap(False)
     try:
-        without = _shared_memory_of_kernels(call)
+        without = [b for _, b in _launches(call)]
         assert torch.equal(got[0], out) and torch.equal(got[1], y)
     finally:
         B_.d3tom_set_launch_overlap(True)

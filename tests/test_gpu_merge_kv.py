@@ -65,7 +65,7 @@ def run_case(w, mode, keep_ratio=0.25, seed=0):
     ek = pu.assert_close(pu.f64(k_out), res["k_out"], dt, "merged key cache")
     ev = pu.assert_close(pu.f64(v_out), res["v_out"], dt, "merged value cache")
     ctx.close()
-    return ek, ev
+    return dict(err=(ek, ev), total_out=total_out, members=member_count.cpu().numpy(), pruned=total - total_out)
 
 
 @pytest.mark.parametrize("mode", [B_.AGG_SUM, B_.AGG_MEAN])
@@ -84,11 +84,28 @@ def test_merge_kv_llada_shape():
     run_case(wl.config("C1"), B_.AGG_MEAN, keep_ratio=0.10)
 
 
-@pytest.mark.parametrize("V,r", [(4700, 0.92), (9000, 0.2), (17000, 0.02)])
-def test_merge_kv_both_caches_in_one_launch_of_either_aggregation(V, r):
-    # 4.3 K output rows take the streaming pipeline; 9 K and 17 K visual tokens with few kept ones have long member lists
-    # (more heavy kept tokens x chunks than blocks) and lie on either side of what the list kernel keeps in registers
-    run_case(wl.make_workload("kvl", "bf16", 2, 64, 43, 64, [dict(V=V, P=9, O=4, n_dec=1, r=r)]), B_.AGG_MEAN)
+HEAVY = 32            # a kept token with this many members or more is aggregated by whole blocks
+STREAM_ROWS = 4096    # from this many output rows on the streaming pipeline aggregates
+
+
+@pytest.mark.parametrize("mode", [B_.AGG_SUM, B_.AGG_MEAN])
+def test_merge_kv_both_caches_in_one_launch_of_the_streaming_pipeline(mode):
+    res = run_case(wl.make_workload("kvl", "bf16", 2, 64, 43, 64, [dict(V=4700, P=9, O=4, n_dec=1, r=0.92)]), mode, keep_ratio=0.92)
+    assert res["total_out"] >= STREAM_ROWS
+
+
+# long member lists: on either side of what the list kernel keeps in registers (8192 visual tokens), and rows of 16 chunks
+# with more than eight heavy (row, chunk) items per SM possible, so that more blocks than SMs walk over them
+@pytest.mark.parametrize("mode", [B_.AGG_SUM, B_.AGG_MEAN])
+@pytest.mark.parametrize("V,r,H,dh", [(8000, 0.01, 2, 64), (9000, 0.01, 2, 64), (17000, 0.02, 2, 64), (3000, 0.02, 32, 128)])
+def test_merge_kv_both_caches_in_one_launch_with_long_member_lists(V, r, H, dh, mode):
+    res = run_case(wl.make_workload("kvh", "bf16", H, dh, 43, 64, [dict(V=V, P=9, O=4, n_dec=1, r=r)]), mode, keep_ratio=r)
+    heavy, chunks = int((res["members"] >= HEAVY).sum()), max(1, H * dh // 256)
+    assert res["total_out"] < STREAM_ROWS and heavy >= 30
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    if chunks > 1:
+        blocks = res["pruned"] // HEAVY * chunks // 8
+        assert blocks > sms and heavy * chunks > 2 * blocks       # several items per block
 
 
 def test_merge_kv_value_cache_written_over_the_key_cache():
