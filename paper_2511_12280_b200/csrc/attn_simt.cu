@@ -11,9 +11,9 @@
 // the score scratch and their final (M, l) pair to the lse scratch; the
 // finishing kernel turns those into S_j = sum_h sum_{i in D} A_ij.
 //
-// Bound: the fp32 pipe and the latency of one to three warps per scheduler.  One warp per query row, every lane walking a
-// key of its own through global memory, took 1139 us at 1152 rows x 8 heads x 64 where this takes 98, and 111 us at
-// 288 x 4 x 64 where this takes 17.
+// Bound: issue slots and shared memory at one to three warps per scheduler (1152 rows x 8 heads x 64: fp32 pipe 49 % busy,
+// issue 58 %, shared-memory wavefronts 66 %).  One warp per query row, every lane walking a key of its own through global
+// memory, took 1139 us at 1152 rows x 8 heads x 64 where this takes 83, and 111 us at 288 x 4 x 64 where this takes 11.4.
 #include "common.cuh"
 #include "f32_tile.cuh"
 
@@ -297,17 +297,21 @@ int launch_simt(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s) {
   return D3TOM_OK;
 }
 
-// Rows per warp: with 16 a score needs fewer shared-memory reads, with 8 there are twice the warps to hide latency, which
-// wins until the SMs are full of warps anyway (from 16 eight-row warps per SM on).  Measured, 8 / 16 rows (us): 288 rows x
-// 4 heads x 64: 19.4 / 28.0; 600 x 8 x 64: 51.7 / 55.6; 1152 x 8 x 64: 95.8 / 102.0; 700 x 4 x 128: 73.7 / 130.7;
-// 1152 x 32 x 128: 639 / 564.  With 4 rows (so few warps that most schedulers would idle): 288 x 4 x 64 17.1, 300 x 4 x 128
-// 25.9 against 40.2, but 384 x 8 x 64 29.0 against 25.9.
+// Rows per warp: 8, or 4 where there are so few warps that most schedulers would idle (up to two eight-row warps per SM),
+// or 16 for rows of up to 32 channels once the SMs are full of warps (from 16 eight-row warps per SM on): there a score's
+// shared-memory reads weigh most and sixteen rows share them.  Measured, 4 / 8 / 16 rows (us): 288 rows x 4 heads x 64
+// 11.4 / 16.7 / 29.2; 500 x 4 x 64 19.3 / 28.1 / 51.8; 600 x 4 x 64 35.6 / 32.9 / 63.3; 1152 x 8 x 64 111 / 82.6 / 132;
+// with 16 eight-row warps per SM and more, 8 / 16: 2400 x 8 x 64 396 / 438, 1152 x 32 x 128 614 / 665, 2400 x 8 x 128
+// 785 / 929, 2400 x 8 x 32 290 / 252.
 template <typename T, int DHP>
 int launch_simt_dh(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s) {
   const long long sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
   const long long warps8 = (long long)ceil_div(a.max_seqlen, 8) * a.H * a.B;
   if (warps8 <= 2 * sms) return launch_simt<T, DHP, 4, 4>(ctx, a, s);
-  return warps8 > 16 * sms ? launch_simt<T, DHP, 16, 4>(ctx, a, s) : launch_simt<T, DHP, 8, 4>(ctx, a, s);
+  if constexpr (DHP == 32) {
+    if (warps8 > 16 * sms) return launch_simt<T, DHP, 16, 4>(ctx, a, s);
+  }
+  return launch_simt<T, DHP, 8, 4>(ctx, a, s);
 }
 
 template <typename T>

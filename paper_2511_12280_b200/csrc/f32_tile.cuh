@@ -2,12 +2,12 @@
 // operands in shared memory, and 16-byte asynchronous copies into rows padded by 16 bytes.
 //
 // Lane layout of a warp tile: ty (0..3) owns rows ty + 4 r, tx (0..7) owns columns tx + 8 j (r, j = 0..3), the bits of ty
-// and tx interleaved over the lane number.  A vector read then finds equal addresses in lanes that differ in bit 0 (first
-// operand) or bit 1 (second operand), and takes 2 passes over the banks instead of 4: with ty = lane / 8 the second
-// operand took 4, and a 1152 x 6144 x 2048 product ran at 32 TFLOP/s instead of 35.
-// Both operands are read as 16-byte vectors along K from rows whose length is a multiple of 4 floats plus 4: the eight
-// rows (or four rows, for the first operand) that a warp touches then start in different bank groups, so a vector read
-// costs one pass over the banks.  Per 4 of K a lane reads 8 vectors for 32 packed multiply-adds (fma.f32x2 along K).
+// and tx interleaved over the lane number, so that equal addresses lie in lanes that differ in bit 0 (first operand) or
+// bit 1 (second operand).  Both operands are read as 16-byte vectors along K from rows whose length is a multiple of 4
+// floats plus 4: the eight rows (or four rows, for the first operand) that a warp touches start in different bank groups.
+// A vector read then takes 2 passes over the banks without conflicts (counted: 1.93 wavefronts per read); with
+// ty = lane / 8 the second operand took 4, and a 1152 x 6144 x 2048 product ran at 32 TFLOP/s instead of 35.
+// Per 4 of K a lane reads 8 vectors for 32 packed multiply-adds (fma.f32x2 along K).
 #pragma once
 
 #include "common.cuh"

@@ -9,8 +9,9 @@
 // the 32-deep pieces c, c + 4, c + 8, ... of K, and the four are added in this order.  A warp that owns more than one
 // chain walks its k-blocks chain by chain (the sums so far wait in shared memory: in registers they would cost the second
 // CTA per SM).  So a row has the same bits alone and in any batch, whichever tile serves it.
-// Bound: the fp32 pipe and shared memory (a lane reads 8 vectors per 64 multiply-adds): 42 TFLOP/s at 1152 x 12288 x 4096,
-// 30 at 384 x 1536 x 512 (20 us; one output per thread and two shared-memory reads per multiply-add took 83).
+// Bound: the fp32 pipe and shared memory (a lane reads 8 vectors per 64 multiply-adds): 42 TFLOP/s at 1152 x 12288 x 4096
+// (pipe 60 % busy, shared-memory wavefronts 59 %), 31 at 384 x 1536 x 512 (19 us; one output per thread and two
+// shared-memory reads per multiply-add took 83).
 #include "common.cuh"
 #include "f32_tile.cuh"
 

@@ -43,8 +43,8 @@ def _launches(call):
     return out
 
 
-# rows and heads that take 4, 8 and (from ceil(rows / 8) x heads x requests > 16 x SMs on: the 1400-row batch with 64 columns, 620
-# rows with 100 and 128, 700 and 2400 with 32) 16 rows per warp; head sizes below, at and above the padded widths 32 / 64 / 128
+# rows and heads that take 4, 8 and (up to 32 channels, from ceil(rows / 8) x heads x requests > 16 x SMs on: 700 x 32 x 4 and
+# 2400 x 8 x 32) 16 rows per warp; head sizes below, at and above the padded widths 32 / 64 / 128
 @pytest.mark.parametrize("lens,H,dh", [([1], 2, 64), ([15, 16, 17], 4, 64), ([31, 33], 2, 32), ([255, 257], 1, 36),
                                        ([130], 3, 128), ([65, 1, 200], 2, 100), ([1152], 8, 64), ([700], 32, 4), ([288], 4, 64),
                                        ([600], 4, 128), ([2400], 8, 32), ([1400, 1400], 8, 64), ([620], 32, 100), ([620], 32, 128)])
@@ -216,8 +216,8 @@ def test_dense_layers_give_a_row_the_same_bits_alone_and_in_a_batch(n, K, N):
             assert torch.equal(got, want[a:b]), (a, b)
 
 
-# one request among others, with lengths at which 4, 8 and 16 rows per warp serve the launch
-@pytest.mark.parametrize("lens,H,dh", [([288, 40], 4, 64), ([288, 900, 100], 4, 64), ([288, 1400, 1400], 8, 64), ([150, 700], 32, 128),
+# one request among others, with lengths at which 4, 8 and (32 channels) 16 rows per warp serve the launch
+@pytest.mark.parametrize("lens,H,dh", [([288, 40], 4, 64), ([290, 1200, 1300], 8, 32), ([288, 900, 100], 4, 64), ([288, 1400, 1400], 8, 64), ([150, 700], 32, 128),
                                        ([75, 31], 2, 36)])
 def test_attention_importance_and_merge_give_a_request_the_same_bits_alone_and_in_a_batch(lens, H, dh):
     g = torch.Generator().manual_seed(sum(lens))
