@@ -31,7 +31,7 @@ constexpr int kBM = 128, kBK = 64;
 constexpr int kGemmThreads = 224;      // warps: 0 A loads, 1 MMA, 2..5 epilogue, 6 B loads
 
 enum { kEpiProj = 0, kEpiSim = 1, kEpiLinear = 2, kEpiGateUp = 3 };
-constexpr int kShortRows = 96;        // calls of at most this many rows store row by row
+constexpr int kShortRows = 127;       // calls of at most this many rows (less than a row tile) store row by row
 constexpr int kMaxKSplits = 4;        // K slices per tile at most when the last slice to arrive adds them all
 constexpr int kCoopSlices = 16;       // K slices per similarity tile at most (every slice adds its own share of the columns)
 constexpr uint64_t kSliceWaitNs = 200000ull;   // after this long a slice leaves its share of a tile to the last one

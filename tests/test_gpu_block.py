@@ -155,8 +155,8 @@ def test_long_layers_that_keep_single_cta_tiles(rows, K, N):
     run_linear(rows, K, N, "bf16", residual=True, seed=K)
 
 
-# calls of up to 96 rows store row by row, longer ones 64 bytes of eight rows at a time
-@pytest.mark.parametrize("rows", [1, 31, 96, 97, 129])
+# calls of up to 127 rows store row by row, longer ones 64 bytes of eight rows at a time
+@pytest.mark.parametrize("rows", [1, 31, 127, 128, 129])
 def test_dense_layers_at_the_ends_of_the_short_calls(rows):
     run_proj(rows, 2, 128, seed=rows)
     run_linear(rows, 128, 256, "bf16", residual=False, seed=rows)
