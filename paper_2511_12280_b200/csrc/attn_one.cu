@@ -72,7 +72,7 @@ attn_one_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
   const int per_req = a.H * a.nqb;
   int b = (int)blockIdx.x / per_req;
   const int lin = (int)blockIdx.x - b * per_req;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = ptx::uniform_warp();
   if (a.B > 1 && a.B <= 32) {
     const int nl = lane < a.B ? a.cu_seqlens[lane + 1] - a.cu_seqlens[lane] : -1;
     int rank = 0;
@@ -128,7 +128,7 @@ attn_one_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));
     if (warp == 8) {
       // ------------------------------------------------------------ TMA producer
-      if (lane == 0) {
+      if (ptx::elect_one()) {
         ptx::prefetch_tensormap(&tmap_q); ptx::prefetch_tensormap(&tmap_k); ptx::prefetch_tensormap(&tmap_v);
         auto load_tile = [&](uint8_t* dst, const CUtensorMap* tm, uint64_t* bar, int row) {
           ptx::mbar_arrive_expect_tx(bar, kTileBytes);
@@ -151,7 +151,7 @@ attn_one_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
       }
     } else if (warp == 9) {
       // ------------------------------------------------------------ MMA issuer
-      if (lane == 0) {
+      if (ptx::elect_one()) {
         constexpr uint32_t idesc_qk = ptx::idesc_bf16_f32(kTile, kTile, 0, 0);   // S = Q K^T, both K-major
         constexpr uint32_t idesc_pv = ptx::idesc_bf16_f32(kTile, kDH, 0, 1);     // O += P V, V is MN-major
         const ptx::SmemDesc q_desc = ptx::smem_desc_kmajor_sw128(ptx::smem_u32(q_s));

@@ -146,7 +146,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   float* ink_s = reinterpret_cast<float*>(smem + kStages * (S::kABytes + S::kBBytes) + 256);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = ptx::uniform_warp(), lane = threadIdx.x & 31;
   // barriers and tensor memory first (on-chip only), then wait for the kernels before this one
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) { ptx::mbar_init(&full[s], 2); ptx::mbar_init(&empty[s], 1); }   // A and B loaders
@@ -186,7 +186,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     // ------------------------------------------------------------ TMA producers: warp 0 streams A, warp 6 streams B
     // (issuing a load and its barrier traffic costs the issuing thread a few hundred cycles per
     // k-block; two threads keep ahead of 128 x 192 tiles, one does not)
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       const bool is_a = warp == 0;
       const CUtensorMap* tm = is_a ? &tmap_a : &tmap_b;
       uint8_t* ring = is_a ? a_s : b_s;
@@ -215,7 +215,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       constexpr uint32_t idesc = ptx::idesc_bf16_f32(kBM, BN, 0, 0);
       const ptx::SmemDesc a_desc0 = ptx::smem_desc_kmajor_sw128(ptx::smem_u32(a_s));
       const ptx::SmemDesc b_desc0 = ptx::smem_desc_kmajor_sw128(ptx::smem_u32(b_s));
@@ -602,7 +602,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = ptx::uniform_warp(), lane = threadIdx.x & 31;
   const uint32_t rank = ptx::cluster_ctarank();
   const bool leader = rank == 0;
   if (threadIdx.x == 0) {
@@ -626,7 +626,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
 
   if (warp == 0 || warp == 6) {
     // ------------------------------------------------------------ TMA producers: warp 0 streams A, warp 6 streams B
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       const bool is_a = warp == 0;
       const CUtensorMap* tm = is_a ? &tmap_a : &tmap_b;
       uint8_t* ring = is_a ? a_s : b_s;
@@ -656,7 +656,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (rank 0 only)
-    if (lane == 0 && leader) {
+    if (leader && ptx::elect_one()) {
       const uint32_t idesc = ptx::idesc_bf16_f32(2 * kBM, bn, 0, 0);
       const ptx::SmemDesc a_desc0 = ptx::smem_desc_kmajor_sw128(ptx::smem_u32(a_s));
       const ptx::SmemDesc b_desc0 = ptx::smem_desc_kmajor_sw128(ptx::smem_u32(b_s));

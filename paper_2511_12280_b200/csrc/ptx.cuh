@@ -19,6 +19,18 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
   return t;
 }
 
+// One lane of a converged warp, the same one at every call.  A region under this predicate has one active thread as far as the
+// compiler is concerned, where `lane == 0` leaves it to provide for several with different operands of tcgen05.mma, TMA
+// copies and commits; the issuing and loading loops paid for that per instruction.  `lane == 0` / elected (us): projection
+// 319 rows x 3072 x 1024 8.2 / 6.0, attention of 4096 rows x 37 heads 256 / 245, linear 1216 x 4096 x 4096 56.7 / 53.5.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+  return e != 0;
+}
+// the warp's number, known to be the same in all its lanes
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
 // ------------------------------------------------------------------ mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
