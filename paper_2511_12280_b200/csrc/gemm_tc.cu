@@ -71,14 +71,10 @@ struct Unit {
   }
 };
 
-// MT = 1: a CTA tile is 128 x BN with two accumulators (the epilogue of a tile overlaps the main loop of the next).
-// MT = 2: a CTA tile is 256 x BN: two 128-row A tiles share every B tile in shared memory, so a k-block moves
-//         32 + 32 KB for 1024 tensor cycles (62 B/clk) where the 128 x 256 tile moves 16 + 32 KB for 512 (96 B/clk);
-//         the dense layers are bound by what the SMs can pull out of L2, so this is the faster shape whenever there
-//         are enough rows.  Both accumulators belong to the one tile (no overlap of epilogue and main loop).
-template <int BN, int MT = 1> struct GemmSmem {
-  static constexpr int kABytes = MT * kBM * kBK * 2, kBBytes = BN * kBK * 2;
-  static constexpr int kStages = (MT == 2) ? 3 : (BN == 256 ? 4 : (BN == 192 ? 5 : 6));   // as many as fit in 227 KB
+// A CTA tile is 128 x BN with two accumulators (the epilogue of a tile overlaps the main loop of the next).
+template <int BN> struct GemmSmem {
+  static constexpr int kABytes = kBM * kBK * 2, kBBytes = BN * kBK * 2;
+  static constexpr int kStages = BN == 256 ? 4 : (BN == 192 ? 5 : 6);   // as many as fit in 227 KB
   static constexpr int kAccStride = BN <= 128 ? 128 : 256;              // TMEM columns between the two accumulators
   static constexpr int kBytes = kStages * (kABytes + kBBytes) + 1024 /*alignment slack*/ + 256 /*barriers*/ + BN * 4;
 };
@@ -87,7 +83,7 @@ template <int N> struct Const { static constexpr int value = N; };
 
 // Where tile `t` of the walk lies: rows of A, rows of B, and for the similarity the request
 // it belongs to.  Returns false for a tile of the bounding grid that a request does not reach.
-template <int BN, int EPI, int MT = 1>
+template <int BN, int EPI>
 struct TileCoord {
   int m0, n0, a_row, b_row, b, Vb, kb, v0, k0;
   const int* prefix;      // similarity with a ragged batch: tiles before request b (shared memory), or null
@@ -112,7 +108,7 @@ struct TileCoord {
     ni = rest % p.n_tiles;
     b = rest / p.n_tiles;
     // (a gate-up tile covers BN / 2 output features: its B rows are 128 gate rows and 128 up rows)
-    m0 = mi * (MT * kBM); n0 = ni * (EPI == kEpiGateUp ? BN / 2 : BN); a_row = m0; b_row = n0;
+    m0 = mi * kBM; n0 = ni * (EPI == kEpiGateUp ? BN / 2 : BN); a_row = m0; b_row = n0;
     Vb = kb = v0 = k0 = 0;
     if (EPI == kEpiSim) {
       v0 = p.cu_vis[b]; Vb = p.cu_vis[b + 1] - v0;
@@ -128,11 +124,10 @@ struct TileCoord {
 constexpr int kMaxPrefixBatch = 64;     // ragged batches up to this many requests number only the tiles that exist
 
 // kShort: dense layers without a residual of at most kShortRows rows (how the results are stored, see store_rows_64b)
-template <int BN, int EPI, int MT = 1, bool kShort = false>
+template <int BN, int EPI, bool kShort = false>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b, GemmParams p) {
-  static_assert(MT == 1 || (BN >= 224 && BN % 32 == 0 && EPI != kEpiSim), "the 256-row tile serves the dense layers at 224 or 256 columns");
-  using S = GemmSmem<BN, MT>;
+  using S = GemmSmem<BN>;
   constexpr int kStages = S::kStages;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -179,7 +174,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   ptx::tc_fence_after_sync();
   if (use_prefix) total_units = tile_prefix[p.batch] * p.k_splits;      // (the similarity cuts every tile or none)
   const uint32_t tmem_base = *tmem_slot;
-  TileCoord<BN, EPI, MT> tc;
+  TileCoord<BN, EPI> tc;
   tc.prefix = use_prefix ? tile_prefix : nullptr;
 
   if (warp == 0 || warp == 6) {
@@ -226,8 +221,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         un.set(p, u);
         if (!tc.set(p, un.t)) continue;
         const int kb0 = un.kb0, kb1 = un.kb1;
-        const int buf = MT == 2 ? 0 : (lt & 1);               // (a 256-row tile owns both accumulators)
-        const uint32_t acc_use = MT == 2 ? (uint32_t)lt : (uint32_t)(lt >> 1);   // how often this buffer has been used
+        const int buf = lt & 1;
+        const uint32_t acc_use = (uint32_t)(lt >> 1);               // how often this buffer has been used
         ok = ptx::mbar_wait(&acc_empty[buf], (acc_use & 1) ^ 1, abort_flag, p.dev_status);   // epilogue done with it
         if (!ok) break;
         ptx::tc_fence_after_sync();
@@ -239,13 +234,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           ptx::tc_fence_after_sync();
           const ptx::SmemDesc ad = ptx::smem_desc_advance(a_desc0, s * S::kABytes), bd = ptx::smem_desc_advance(b_desc0, s * S::kBBytes);
 #pragma unroll
-          for (int kk = 0; kk < kBK / 16; ++kk) {
+          for (int kk = 0; kk < kBK / 16; ++kk)
             ptx::mma_ss(tmem_acc, ptx::smem_desc_advance(ad, kk * 32), ptx::smem_desc_advance(bd, kk * 32), idesc,
                         (kbk > kb0 || kk > 0) ? 1u : 0u);
-            if (MT == 2)   // rows 128..255 of the A stage against the same B tile, into the second accumulator
-              ptx::mma_ss(tmem_acc + S::kAccStride, ptx::smem_desc_advance(ad, kBM * kBK * 2 + kk * 32),
-                          ptx::smem_desc_advance(bd, kk * 32), idesc, (kbk > kb0 || kk > 0) ? 1u : 0u);
-          }
           ptx::mma_commit(&empty[s]);     // frees the stage once these MMAs have read it
         }
         if (ok) ptx::mma_commit(&acc_full[buf]);
@@ -264,8 +255,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       un.set(p, u);
       const int t = un.t, sp = un.sp;
       if (!tc.set(p, t)) continue;
-      const int buf = MT == 2 ? 0 : (lt & 1);
-      const uint32_t acc_use = MT == 2 ? (uint32_t)lt : (uint32_t)(lt >> 1);
+      const int buf = lt & 1;
+      const uint32_t acc_use = (uint32_t)(lt >> 1);
       if (EPI == kEpiSim) {
         // inverse norms of this tile's kept rows; the four epilogue warps share them (named barrier 1)
         asm volatile("bar.sync 1, 128;" ::: "memory");          // everyone is done with the previous tile's values
@@ -275,8 +266,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       const bool ok = __all_sync(0xffffffffu, ptx::mbar_wait(&acc_full[buf], acc_use & 1, abort_flag, p.dev_status));
       if (!ok) break;
       ptx::tc_fence_after_sync();
-      uint32_t t_row = tmem_base + (uint32_t)buf * S::kAccStride + ((uint32_t)(quarter * 32) << 16);
-      int m_base = tc.m0;                                       // first row of the 128-row half in hand
+      const uint32_t t_row = tmem_base + (uint32_t)buf * S::kAccStride + ((uint32_t)(quarter * 32) << 16);
       // A tile whose K range is cut into slices on different SMs: every unit writes its partial sums out (column-major, so
       // a warp's 32 rows are one 128-byte line) and counts itself in.  Dense layers: the unit that completes the tile
       // adds the parts in the order of the K slices and runs the epilogue on the sums (the counter is left at zero
@@ -373,7 +363,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         const int nsp = un.nsp;                                  // 2 .. 16
         const int groups = (min(BN, tc.kb - tc.n0) + 7) >> 3;
         const int shares = s_prev;
-        const int m = m_base + row;
+        const int m = tc.m0 + row;
         const int g = tc.v0 + m;
         const bool active = m < tc.Vb && p.assign[g] < 0;
         const float inm = active ? p.inv_norm[g] : 0.f;
@@ -443,10 +433,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         ++lt;
         continue;
       }
-      // (a 256-row tile: the same epilogue once per 128-row half, each half in its own accumulator)
-#pragma unroll 1
-      for (int mh = 0; mh < MT; ++mh, t_row += S::kAccStride, m_base += kBM) {
-      const int warp_row = m_base + quarter * 32, n_valid = p.out_rows - warp_row;      // dense layers: this warp's 32 rows
+      const int warp_row = tc.m0 + quarter * 32, n_valid = p.out_rows - warp_row;      // dense layers: this warp's 32 rows
       if (EPI == kEpiProj) {
 #pragma unroll 1
         for (int c = 0; c < BN; c += 32) {
@@ -506,7 +493,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           ptx::store_rows_64b<kShort>(p.lin_out + (size_t)warp_row * p.ld_out + tc.n0 + c, (size_t)p.ld_out * 2, n_valid, w);
         }
       } else {
-        const int m = m_base + row;
+        const int m = tc.m0 + row;
         const int g = tc.v0 + m;
         const bool active = m < tc.Vb && p.assign[g] < 0;     // a pruned token of this request
         const float inm = active ? p.inv_norm[g] : 0.f;
@@ -535,7 +522,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
               ((unsigned long long)ordered_key(best_sim) << 32) | (0xffffffffu - (unsigned)best_slot);
           atomicMax(p.best + g, mine);
         }
-      }
       }
       if (split) { ++lt; continue; }                      // (its accumulator was released when the partial went out)
       // the accumulator may be overwritten once all four warps have read it
@@ -815,60 +801,55 @@ void plan_tail_split(const d3tom_ctx* ctx, GemmParams& p) {
   p.full_tiles = p.k_splits > 1 ? tiles - tiles % ctx->sm_count : tiles;
 }
 
-// Width of 128-row tiles: fewest (rounds of tiles over the SMs) x (measured cycles per 64-deep k-block at that width:
-// 667 / 633 / 600 for 256 / 192 / 128 columns; narrow tiles pay the per-k-block barrier traffic of the issuing thread
-// more often per unit of work).
-int one_m_tile_width(int sms, int rows, int ncols) {
+// What a dense layer costs in tiles of one shape (us): `start` once, per 64 of K `round` for each full round of tiles over the
+// SMs (or the pairs) and `part` + `part_r` x (its share of the SMs) for an incomplete last one, which leaves more of L2 to
+// each, and `more` for every round after the first (an epilogue that nothing hides).  Fitted to 250 layers (64 .. 8000 rows,
+// K 512 .. 12288, 1024 .. 12288 columns) timed in every shape; over them the cheapest shape by these figures is 0.4 % slower
+// than the fastest one.
+struct TileCost { int width; double start, round, part, part_r, more; };
+constexpr TileCost kOneCost[] = {{256, 7.13, 0.401, 0.283, 0.093, 1.80}, {192, 6.13, 0.284, 0.214, 0.084, 1.78},
+                                 {128, 4.96, 0.222, 0.144, 0.067, 0.72}};
+constexpr TileCost kPairCost[] = {{256, 7.89, 0.345, 0.267, 0.088, 2.12}, {224, 7.42, 0.299, 0.225, 0.089, 1.41},
+                                  {192, 7.09, 0.255, 0.191, 0.087, 1.55}, {160, 6.55, 0.221, 0.162, 0.068, 1.15},
+                                  {128, 6.04, 0.192, 0.122, 0.078, 1.18}};
+double tile_time(const TileCost& c, long long tiles, int units, int num_k_blocks) {
+  const double full = (double)(tiles / units), rest = (double)(tiles % units) / units;
+  const double rounds = full + (rest > 0 ? 1.0 : 0.0);
+  return c.start + num_k_blocks * (c.round * full + (rest > 0 ? c.part + c.part_r * rest : 0.0)) + c.more * (rounds - 1.0);
+}
+
+// Width of single-CTA tiles (one that divides the columns; 128 always does).  By rounds alone, weighed 667 / 633 / 600 for 256 /
+// 192 / 128 columns, it took 256 too often at a long K (2600 rows x 6144 x 2048: 1.20 x the time of 128); a K below 1024 is
+// start and epilogue, where fewer rounds are right (130 x 256 x 12288: 192 columns 8.2 us, 128 9.3).
+int one_m_tile_width(int sms, int rows, int ncols, int num_k_blocks) {
   int bn = 128;
-  double best_cost = 1e30;
-  for (int cand : {256, 192, 128}) {
-    if (ncols % cand != 0) continue;
-    const long long tiles = (long long)ceil_div(rows, kBM) * (ncols / cand);
-    const double cost = (double)((tiles + sms - 1) / sms) * (cand == 256 ? 667.0 : cand == 192 ? 633.0 : 600.0);
-    if (cost < best_cost) { best_cost = cost; bn = cand; }
+  double best = 1e30;
+  for (const TileCost& c : kOneCost) {
+    if (ncols % c.width != 0) continue;
+    const long long tiles = (long long)ceil_div(rows, kBM) * (ncols / c.width);
+    const double t = num_k_blocks >= 16 ? tile_time(c, tiles, sms, num_k_blocks)
+                                        : (double)((tiles + sms - 1) / sms) * (c.width == 256 ? 667.0 : c.width == 192 ? 633.0 : 600.0);
+    if (t < best) { best = t; bn = c.width; }
   }
   return bn;
 }
 
-// Which tile shape finishes a dense layer sooner, from measured main-loop cycles per 64 of K (projection timings at
-// 128 .. 7600 rows).  128 x 256 tiles: 850 per full round over the SMs (48 KB of operands per k-block: what the SMs
-// together can pull out of L2), and 150 + 3.9 r for a last round of r tiles, which runs faster per tile because
-// fewer SMs share L2.  256 x 256 tiles: 1450 per full round (64 KB per k-block in three 64 KB stages: bound by the
-// load latency of one SM, so a round of few tiles is no cheaper), 900 + 3.5 r for the last round; 256 x 224 tiles
-// cost 0.89 of that per round and sometimes need a round less, or fill the last one better (1216 rows x 12288
-// columns: 275 tiles in two rounds, 93 us against 99 us for the 240 tiles of 256 x 256).
-// Returns the width of the 256-row tile to use (256 or 224), or 0 for 128-row tiles.
-int two_m_tile_width(int sms, int rows, int ncols, bool allow_224) {
-  const long long t1 = (long long)ceil_div(rows, kBM) * ceil_div(ncols, 256);
-  const double r1 = (double)(t1 % sms);
-  const double cost1 = 850.0 * (double)(t1 / sms) + (r1 > 0 ? 150.0 + 3.9 * r1 : 0.0);
-  auto cost2 = [&](int width, double scale) {
-    const long long t2 = (long long)ceil_div(rows, 2 * kBM) * ceil_div(ncols, width);
-    const double r2 = (double)(t2 % sms);
-    return scale * (1450.0 * (double)(t2 / sms) + (r2 > 0 ? 900.0 + 3.5 * r2 : 0.0));
-  };
-  const double c256 = ncols % 256 == 0 ? cost2(256, 1.0) : 1e30, c224 = allow_224 ? cost2(224, 0.89) : 1e30;
-  if (c224 < 0.97 * c256 && c224 < 0.97 * cost1) return 224;
-  return c256 < 0.97 * cost1 ? 256 : 0;
-}
-
-template <int BN, int EPI, int MT = 1>
+template <int BN, int EPI>
 int launch_gemm(d3tom_ctx* ctx, const CUtensorMap& ta, const CUtensorMap& tb, GemmParams p, cudaStream_t s) {
-  if (EPI != kEpiSim && MT == 1) {
+  if (EPI != kEpiSim) {
     p.split_ws = ctx->gemm_split_ws; p.split_counters = ctx->gemm_split_counters;
     plan_tail_split(ctx, p);
   }
-  if (MT == 2) { p.k_splits = 1; p.full_tiles = p.m_tiles * p.n_tiles * p.batch; }   // whole tiles only
   const long long tiles = (long long)p.m_tiles * p.n_tiles * p.batch;
   const long long units = p.full_tiles + (tiles - p.full_tiles) * p.k_splits;
   if (units <= 0) return D3TOM_OK;
   const int grid = (int)(units < ctx->sm_count ? units : ctx->sm_count);          // persistent: one CTA per SM
-  auto kernel = gemm_tc_kernel<BN, EPI, MT>;
-  if constexpr (EPI != kEpiSim && MT == 1) {
-    if (p.out_rows <= kShortRows && p.residual == nullptr) kernel = gemm_tc_kernel<BN, EPI, MT, true>;
+  auto kernel = gemm_tc_kernel<BN, EPI>;
+  if constexpr (EPI != kEpiSim) {
+    if (p.out_rows <= kShortRows && p.residual == nullptr) kernel = gemm_tc_kernel<BN, EPI, true>;
   }
-  D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmSmem<BN, MT>::kBytes));
-  D3TOM_CUDA_TRY(ctx, launch_serialized(kernel, grid, kGemmThreads, GemmSmem<BN, MT>::kBytes, s, ta, tb, p));
+  D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmSmem<BN>::kBytes));
+  D3TOM_CUDA_TRY(ctx, launch_serialized(kernel, grid, kGemmThreads, GemmSmem<BN>::kBytes, s, ta, tb, p));
   return D3TOM_OK;
 }
 
@@ -922,18 +903,20 @@ int launch_gemm_pair(d3tom_ctx* ctx, const CUtensorMap& ta, const CUtensorMap& t
 }
 
 // Width of the CTA-pair tiles for a dense layer of `rows` x `ncols` outputs (for the gate-up pass the columns of both
-// matrices), or 0 for single-CTA tiles.  A round of pair tiles costs the times below per 64 of K whatever it computes, so
-// the width that fills the rounds best wins; against it stand rounds of single-CTA tiles, whose last, partial round is
-// cheaper, and K slices for a long K (tail_slices).  All figures in us per 64 of K, fitted to the four layers of a
-// block (D = 4096, m = 12288) at 128 .. 4288 rows.  What it changes, old shapes / pairs (us): projection 640 rows
-// 56 / 51; output projection 1216 rows 69 / 55, 1536 rows 57 / 49, 2600 rows 81 / 75 (224 columns; 83 with 256); down
-// projection 640 rows 82 / 62, 1800 rows 171 / 155; feed-forward network 1216 rows 308 / 282.  The factor
-// 1.08 is for power: the pairs move half the operand bytes, and the board's limit sets the clock under these layers.
-// From 2048 rows on the pairs are taken, with two exceptions, measured single-CTA / pairs (us, rows x K x columns):
-//   - all single-CTA tiles together are one round of K slices, which then walk a half to a quarter of K each where a pair
-//     walks all of it: 2100 x 16384 x 128 35 / 78, 2048 x 12288 x 384 30 / 49, 2048 x 8192 x 512 28 / 35;
-//   - widths that 256 does not divide at a K below 1024, where a pair's longer start and drain show: 2100 x 128 x 640
-//     4.5 / 5.3, 2600 x 512 x 384 6.6 / 7.1; with more rounds the pairs win again, 4288 x 512 x 640 9.1 / 7.6.
+// matrices), or 0 for single-CTA tiles.
+//   - 513 .. 2047 rows, K of 1024 and more: the shape that is cheapest by the costs above.  A rule by rounds that weighed 256-row
+//     single-CTA tiles against pairs took neither the best width nor the better kind (us, rule / now): linear 1216 x 4096 x 4096
+//     48.4 / 33.4, 1408 x 4096 x 4096 52.7 / 39.9, 1216 x 12288 x 4096 109 / 90, 1216 x 4096 x 12288 110 / 90,
+//     1408 x 1024 x 6144 22.6 / 19.3; the 256-row tiles, never the fastest of the 250 layers, are gone.
+//   - other layers below 2048 rows: rounds, in us per 64 of K, against rounds of single-CTA tiles and K slices (tail_slices);
+//     1.08 is for power (the pairs move half the operand bytes).
+//   - from 2048 rows on pairs, in the width that fills the rounds best, except where (single-CTA / pairs, us, rows x K x columns)
+//     all single-CTA tiles together are one round of K slices, which then walk a half to a quarter of K each where a pair walks
+//     all of it: 2100 x 16384 x 128 35 / 78, 2048 x 12288 x 384 30 / 49, 2048 x 8192 x 512 28 / 35; or the costs above are
+//     3 % in favour of single-CTA tiles at a K of 1024 or more: 2176 x 1024 x 1024 8.0 / 9.5, 2600 x 1024 x 6144 35.2 / 38.8,
+//     8000 x 1024 x 3072 53.3 / 58.9; or 256 does not divide the width and K is below 1024, where a pair's longer start and
+//     drain show: 2100 x 128 x 640 4.5 / 5.3, 2600 x 512 x 384 6.6 / 7.1; with more rounds the pairs win again,
+//     4288 x 512 x 640 9.1 / 7.6.
 int pair_tile_width(int sms, int rows, int ncols, int num_k_blocks, int pairs, bool gate_up) {
   if (pairs <= 0 || g_d3tom_pair_tiles == 0) return 0;
   if (g_d3tom_pair_tiles == 256) return ncols % 256 == 0 ? 256 : 0;
@@ -951,10 +934,27 @@ int pair_tile_width(int sms, int rows, int ncols, int num_k_blocks, int pairs, b
     const long long r = tiles % sms;
     return full * (double)(tiles / sms) + (r > 0 ? last0 + last_r * (double)r : 0.0);
   };
-  if (rows >= 2048) {
-    const int bn = gate_up ? 256 : one_m_tile_width(sms, rows, ncols);
+  auto pair_time = [&](int w) {
+    const TileCost& c = kPairCost[(256 - w) / 32];
+    return tile_time(c, (long long)ceil_div(rows, 2 * kBM) * ceil_div(ncols, w), pairs, num_k_blocks);
+  };
+  auto one_time = [&] {
+    const int bn = gate_up ? 256 : one_m_tile_width(sms, rows, ncols, num_k_blocks);
+    const TileCost& c = kOneCost[(256 - bn) / 64];
     const long long tiles = (long long)ceil_div(rows, kBM) * ceil_div(ncols, bn);
-    if (tiles < sms && two_m_tile_width(sms, rows, ncols, !gate_up) == 0) {
+    const int slices = tail_slices(sms, (int)tiles, num_k_blocks);
+    if (slices == 1) return tile_time(c, tiles, sms, num_k_blocks);
+    // whole rounds, the rounds of slices, and the exchange of their sums
+    const double full = (double)(tiles / sms);
+    const int units = (int)(tiles % sms) * slices;
+    return c.start + full * (num_k_blocks * c.round + c.more) +
+           ceil_div(num_k_blocks, slices) * (c.round * (ceil_div(units, sms) - 1) + c.part + c.part_r * fmin(1.0, (double)units / sms)) +
+           4.6 + (2.6 * slices - 3.0) * bn / 128;
+  };
+  if (rows >= 2048) {
+    const int bn = gate_up ? 256 : one_m_tile_width(sms, rows, ncols, num_k_blocks);
+    const long long tiles = (long long)ceil_div(rows, kBM) * ceil_div(ncols, bn);
+    if (tiles < sms) {
       const int slices = tail_slices(sms, (int)tiles, num_k_blocks);
       if (slices > 1 && tiles * slices <= sms) return 0;
     }
@@ -962,10 +962,15 @@ int pair_tile_width(int sms, int rows, int ncols, int num_k_blocks, int pairs, b
       const double scale = bn == 256 ? 1.0 : bn == 192 ? 0.95 : 0.9;      // (one_m_tile_width's cycles)
       return best * num_k_blocks + 1.0 < 1.08 * scale * rounds(kBM, bn, 0.40, 0.26, 0.0009) * num_k_blocks ? width : 0;
     }
+    if (num_k_blocks >= 16) return 1.03 * one_time() < pair_time(width) ? 0 : width;
     return width;
   }
   // (the gate-up pass at a short K is bound by its epilogue: 1900 rows, D = 512, m = 12288 76.9 / 84.7)
   if (gate_up && num_k_blocks < 16) return 0;
+  if (rows > 512 && num_k_blocks >= 16) {
+    for (int w : kWidths) if (pair_time(w) < pair_time(width)) width = w;
+    return one_time() < 1.02 * pair_time(width) ? 0 : width;     // (ties to the single-CTA tiles)
+  }
   double single = rounds(kBM, 256, 0.40, 0.26, 0.0009);
   const long long tiles = (long long)ceil_div(rows, kBM) * ceil_div(ncols, 256);
   const int rem = (int)(tiles % sms);
@@ -974,8 +979,6 @@ int pair_tile_width(int sms, int rows, int ncols, int num_k_blocks, int pairs, b
     const double cut = (double)(ceil_div(rem * sp, sms) * ceil_div(num_k_blocks, sp) + 30 + 5 * sp) / num_k_blocks;
     if (cut < 1.0) single = fmin(single, 0.40 * (double)(tiles / sms) + 0.42 * cut);
   }
-  if (!gate_up) single = fmin(single, rounds(2 * kBM, 224, 0.65, 0.41, 0.0016));
-  single = fmin(single, rounds(2 * kBM, 256, 0.73, 0.46, 0.0018));
   // (a pair launch costs about 1.5 us more: with a short K the single-CTA tiles keep small layers, 319 x 3072 x 1024: 9.0 / 9.9)
   return best * num_k_blocks + 1.5 < 1.08 * single * num_k_blocks ? width : 0;
 }
@@ -1013,15 +1016,7 @@ int launch_proj_tc(d3tom_ctx* ctx, const void* x, const void* w, int total, int 
     p.bn = bn2; p.m_tiles = ceil_div(total, 2 * kBM); p.n_tiles = ceil_div(3 * D, bn2);
     return launch_gemm_pair<kEpiProj>(ctx, ta, tb, p, s);
   }
-  if (const int w2 = two_m_tile_width(ctx->sm_count, total, 3 * D, D % 32 == 0)) {
-    r = make_tmap_bf16_2d(&ta, x, (uint64_t)total, (uint64_t)D, (uint64_t)D, 2 * kBM);
-    if (r == 0) r = make_tmap_bf16_2d(&tb, w, (uint64_t)3 * D, (uint64_t)D, (uint64_t)D, (uint32_t)w2);
-    if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
-    p.m_tiles = ceil_div(total, 2 * kBM); p.n_tiles = ceil_div(3 * D, w2);
-    if (w2 == 224) return launch_gemm<224, kEpiProj, 2>(ctx, ta, tb, p, s);
-    return launch_gemm<256, kEpiProj, 2>(ctx, ta, tb, p, s);
-  }
-  const int bn = one_m_tile_width(ctx->sm_count, total, 3 * D);      // (128 always divides 3 D)
+  const int bn = one_m_tile_width(ctx->sm_count, total, 3 * D, p.num_k_blocks);      // (128 always divides 3 D)
   r = make_tmap_bf16_2d(&tb, w, (uint64_t)3 * D, (uint64_t)D, (uint64_t)D, (uint32_t)bn);
   if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
   p.n_tiles = 3 * D / bn;
@@ -1047,15 +1042,7 @@ int launch_linear_tc(d3tom_ctx* ctx, const void* x, const void* w, const void* r
     p.bn = bn2; p.m_tiles = ceil_div(rows, 2 * kBM); p.n_tiles = ceil_div(N, bn2);
     return launch_gemm_pair<kEpiLinear>(ctx, ta, tb, p, s);
   }
-  if (const int w2 = two_m_tile_width(ctx->sm_count, rows, N, true)) {
-    r = make_tmap_bf16_2d(&ta, x, (uint64_t)rows, (uint64_t)K, (uint64_t)K, 2 * kBM);
-    if (r == 0) r = make_tmap_bf16_2d(&tb, w, (uint64_t)N, (uint64_t)K, (uint64_t)K, (uint32_t)w2);
-    if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
-    p.m_tiles = ceil_div(rows, 2 * kBM); p.n_tiles = ceil_div(N, w2);
-    if (w2 == 224) return launch_gemm<224, kEpiLinear, 2>(ctx, ta, tb, p, s);
-    return launch_gemm<256, kEpiLinear, 2>(ctx, ta, tb, p, s);
-  }
-  const int bn = one_m_tile_width(ctx->sm_count, rows, N);
+  const int bn = one_m_tile_width(ctx->sm_count, rows, N, p.num_k_blocks);
   r = make_tmap_bf16_2d(&tb, w, (uint64_t)N, (uint64_t)K, (uint64_t)K, (uint32_t)bn);
   if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
   p.n_tiles = N / bn;
@@ -1081,14 +1068,6 @@ int launch_gate_up_tc(d3tom_ctx* ctx, const void* x, const void* w_gate_up, int 
     if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
     p.bn = bn2; p.m_tiles = ceil_div(rows, 2 * kBM); p.n_tiles = ceil_div(m, bn2 / 2);
     return launch_gemm_pair<kEpiGateUp>(ctx, ta, tb, p, s);
-  }
-  {
-    if (two_m_tile_width(ctx->sm_count, rows, 2 * m, false) == 256) {
-      r = make_tmap_bf16_2d(&ta, x, (uint64_t)rows, (uint64_t)D, (uint64_t)D, 2 * kBM);
-      if (r != 0) { ctx->last_cuda_error = r; return D3TOM_ERR_CUDA; }
-      p.m_tiles = ceil_div(rows, 2 * kBM);
-      return launch_gemm<256, kEpiGateUp, 2>(ctx, ta, tb, p, s);
-    }
   }
   return launch_gemm<256, kEpiGateUp>(ctx, ta, tb, p, s);
 }

@@ -155,6 +155,14 @@ def test_long_layers_that_keep_single_cta_tiles(rows, K, N):
     run_linear(rows, K, N, "bf16", residual=True, seed=K)
 
 
+# between 513 and 2047 rows, and single-CTA tiles from 2048 rows on, by the fitted costs: each width of either kind, ragged rows
+@pytest.mark.parametrize("rows,K,N,width", [(513, 1024, 384, 0), (769, 1024, 2816, 160), (700, 1024, 3968, 192), (513, 2048, 4736, 224),
+                                            (2047, 1024, 768, 0), (2049, 1024, 384, 0), (2600, 1024, 1024, 192)])
+def test_tile_shapes_by_cost(rows, K, N, width):
+    assert pair_width(rows, N, K) == width
+    run_linear(rows, K, N, "bf16", residual=True, seed=rows)
+
+
 # calls of up to 127 rows store row by row, longer ones 64 bytes of eight rows at a time
 @pytest.mark.parametrize("rows", [1, 31, 127, 128, 129])
 def test_dense_layers_at_the_ends_of_the_short_calls(rows):
