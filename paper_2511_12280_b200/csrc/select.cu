@@ -147,10 +147,11 @@ select_kernel(const float* __restrict__ importance, const int32_t* __restrict__ 
 
 // Requests of up to 1024 x IPT visual tokens (IPT 1 .. 16; 12287 tokens: 14.4 us, 20.5 with
 // the staged kernel above): every thread keeps IPT CONSECUTIVE keys in registers, so the ordered
-// output needs a single block-wide prefix sum and the keys are read once.  The radix select takes three passes of
-// 12, 10 and 10 bits; the wide first digit (sign, exponent, three mantissa bits) spreads scores that share their
-// leading bits over many bins, after which few keys remain candidates.  A thread owns the same bins in every pass
-// and clears them as it reads them, which saves the barrier of a separate clearing phase.
+// output needs a single block-wide prefix sum and the keys are read once.  The radix select takes digits of 12 bits
+// from the highest bit of (key - smallest key) on (the first digit then spreads them over many bins, where the sign and
+// the exponent they share would crowd a few) and stops as soon as every key that shares the digits so far is kept: mostly after
+// the second digit.  A thread owns the same four bins in every pass and clears them as it reads them, which saves the barrier
+// of a separate clearing phase.  Bound: latency of one block, three barriers a pass.
 constexpr int kRegBinsMax = 4096;
 
 template <int IPT>
@@ -158,9 +159,10 @@ __global__ void __launch_bounds__(kThreads)
 select_reg_kernel(const float* __restrict__ importance, const int32_t* __restrict__ cu_vis,
                   const int32_t* __restrict__ keep_count, const int32_t* __restrict__ cu_kept,
                   int32_t* __restrict__ kept_idx, uint8_t* __restrict__ keep_mask) {
-  __shared__ unsigned hist[kRegBinsMax];
-  __shared__ unsigned warp_tot[kWarps];
-  __shared__ unsigned sh_prefix, sh_remaining;
+  __shared__ uint4 hist4[kRegBinsMax / 4];
+  __shared__ unsigned warp_tot[kWarps], warp_lo[kWarps], warp_hi[kWarps];
+  __shared__ unsigned sh_prefix, sh_remaining, sh_whole;
+  unsigned* hist = reinterpret_cast<unsigned*>(hist4);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int d = tid; d < kRegBinsMax; d += kThreads) hist[d] = 0u;      // on-chip only: before the dependency wait
   grid_dependency_enter();
@@ -174,8 +176,6 @@ select_reg_kernel(const float* __restrict__ importance, const int32_t* __restric
   uint32_t key[IPT];
 #pragma unroll
   for (int i = 0; i < IPT; ++i) key[i] = (j0 + i < V) ? ordered_key(sc[j0 + i]) : 0u;
-  if (tid == 0) { sh_prefix = 0u; sh_remaining = (unsigned)k; }
-  __syncthreads();
 
   // inclusive prefix sum of `val` over the block in thread order; every warp scans the 32 warp totals itself
   auto block_scan = [&](unsigned val, unsigned& total) -> unsigned {
@@ -198,61 +198,69 @@ select_reg_kernel(const float* __restrict__ importance, const int32_t* __restric
     return incl + before;
   };
 
-  uint32_t mask = 0u;
-  if (k > 0) {
+  // The keys are taken relative to the smallest one, so that the radix select starts at the highest bit of their range; it
+  // stops as soon as all keys that share the digits so far are kept.
+  uint32_t lo_key = 0xffffffffu, hi_key = 0u;
 #pragma unroll
-    for (int pass = 0; pass < 3; ++pass) {
-      const int bits = pass == 0 ? 12 : 10;
-      const int shift = pass == 0 ? 20 : (pass == 1 ? 10 : 0);
-      const int bpt = (1 << bits) / kThreads;              // bins per thread: 4, 1, 1
-      const uint32_t prefix = sh_prefix;
-      const unsigned rem = sh_remaining;
+  for (int i = 0; i < IPT; ++i)
+    if (j0 + i < V) { lo_key = min(lo_key, key[i]); hi_key = max(hi_key, key[i]); }
+  lo_key = __reduce_min_sync(0xffffffffu, lo_key);
+  hi_key = __reduce_max_sync(0xffffffffu, hi_key);
+  if (lane == 0) { warp_lo[warp] = lo_key; warp_hi[warp] = hi_key; }
+  __syncthreads();                          // (the cleared histogram as well)
+  lo_key = __reduce_min_sync(0xffffffffu, warp_lo[lane]);
+  hi_key = __reduce_max_sync(0xffffffffu, warp_hi[lane]);
 #pragma unroll
-      for (int i = 0; i < IPT; ++i)
-        if (j0 + i < V && (key[i] & mask) == prefix) atomicAdd(&hist[(key[i] >> shift) & ((1u << bits) - 1u)], 1u);
-      __syncthreads();
-      // thread t owns the bins (bins - 1 - bpt * t) downwards: the running count from the top digit
-      const int top = (1 << bits) - 1 - bpt * tid;
-      unsigned cnt[4], mine = 0u;
+  for (int i = 0; i < IPT; ++i) key[i] -= lo_key;                // (those past the end are never looked at)
+  int top = 32 - __clz((int)(hi_key - lo_key));                  // no key has a bit from `top` on
+  uint32_t prefix = 0u;
+  unsigned rem = (unsigned)k;
+  bool whole = k == V;                      // every key with this prefix is kept
+  if (k <= 0) { top = 0; prefix = 0xffffffffu; }                 // (nothing is kept: no key above, none of the equal ones)
+  while (top > 0 && !whole) {
+    const int shift = top > 12 ? top - 12 : 0;
+    const uint32_t mask = top < 32 ? 0xffffffffu << top : 0u, digits = (1u << (top - shift)) - 1u;
+#pragma unroll
+    for (int i = 0; i < IPT; ++i)
+      if (j0 + i < V && (key[i] & mask) == prefix) atomicAdd(&hist[(key[i] >> shift) & digits], 1u);
+    __syncthreads();
+    // thread t owns four bins, 4095 - 4 t downwards (the running count goes from the top digit), and leaves them clear
+    uint4* mine4 = hist4 + (kThreads - 1 - tid);
+    const uint4 c4 = *mine4;
+    *mine4 = make_uint4(0u, 0u, 0u, 0u);
+    const unsigned cnt[4] = {c4.w, c4.z, c4.y, c4.x};
+    const unsigned mine = (c4.x + c4.y) + (c4.z + c4.w);
+    unsigned total;
+    const unsigned incl = block_scan(mine, total);
+    const unsigned excl = incl - mine;
+    if (excl < rem && rem <= incl) {                      // exactly one thread: the digit of the key of rank k
+      unsigned run = excl;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        cnt[i] = 0u;
-        if (i < bpt) { cnt[i] = hist[top - i]; mine += cnt[i]; }
-      }
-      if (pass == 0) {                                      // the 4096 bins are clear again for the next passes
-#pragma unroll
-        for (int i = 0; i < 4; ++i) hist[top - i] = 0u;
-      } else {
-        hist[top] = 0u;
-      }
-      unsigned total;
-      const unsigned incl = block_scan(mine, total);
-      const unsigned excl = incl - mine;
-      if (excl < rem && rem <= incl) {                      // exactly one thread: the digit of the key of rank k
-        unsigned run = excl;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          if (i < bpt && run < rem && rem <= run + cnt[i]) {
-            sh_prefix = prefix | ((uint32_t)(top - i) << shift);
-            sh_remaining = rem - run;
-          }
-          run += cnt[i];
+        if (run < rem && rem <= run + cnt[i]) {
+          sh_prefix = prefix | ((uint32_t)(4 * (kThreads - 1 - tid) + 3 - i) << shift);
+          sh_remaining = rem - run;
+          sh_whole = rem - run == cnt[i] ? 1u : 0u;
         }
+        run += cnt[i];
       }
-      mask |= ((1u << bits) - 1u) << shift;
-      __syncthreads();
     }
+    __syncthreads();
+    prefix = sh_prefix;
+    rem = sh_remaining;
+    whole = sh_whole != 0u;
+    top = shift;
   }
-  const uint32_t T = sh_prefix;            // key of rank k
-  const unsigned need_eq = k > 0 ? sh_remaining : 0u;    // keys equal to T that are kept: the lowest positions
+  // kept: the keys above T, and of the keys equal to T the `need_eq` at the lowest positions
+  uint32_t T = prefix;                      // the key of rank k; or, if its lower digits were not looked at, ...
+  unsigned need_eq = rem;
+  if (whole && T > 0u) { T -= 1u; need_eq = 0u; }       // ... the largest value below every key with its upper digits
 
   // ---- ordered output: one prefix sum over the per-thread counts (greater << 16 | equal)
   unsigned val = 0u;
-  if (k > 0) {
 #pragma unroll
-    for (int i = 0; i < IPT; ++i)
-      if (j0 + i < V) val += (key[i] > T ? 0x10000u : 0u) + (key[i] == T ? 1u : 0u);
-  }
+  for (int i = 0; i < IPT; ++i)
+    if (j0 + i < V) val += (key[i] > T ? 0x10000u : 0u) + (key[i] == T ? 1u : 0u);
   __syncthreads();                          // warp_tot is reused
   unsigned total;
   const unsigned incl = block_scan(val, total);
@@ -263,7 +271,7 @@ select_reg_kernel(const float* __restrict__ importance, const int32_t* __restric
   for (int i = 0; i < IPT; ++i) {
     const int j = j0 + i;
     if (j < V) {
-      const bool gt = k > 0 && key[i] > T, eq = k > 0 && key[i] == T;
+      const bool gt = key[i] > T, eq = key[i] == T;
       const bool keep = gt || (eq && eq_before < need_eq);
       mk[j] = keep ? 1 : 0;
       if (keep) out[gt_before + min(eq_before, need_eq)] = j;

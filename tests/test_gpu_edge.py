@@ -280,6 +280,21 @@ def test_select_at_the_ends_of_the_key_in_registers_range(V):
     run_select([rng.integers(0, 5, V) / 8.0, rng.random(9)], [V - 3, 2])        # long runs of ties
 
 
+# The first digit starts at the top of the keys' range, and the passes end as soon as a digit's keys are all kept: ranges that
+# cross the sign and powers of two, the smallest key kept, everything kept, one token, infinities and zeros of both signs
+@pytest.mark.parametrize("V", [1, 2, 1024, 1025, 5000])
+def test_select_digits_from_the_range_of_the_keys(V):
+    rng = np.random.default_rng(100 + V)
+    wide = rng.random(V) * 6.0 - 3.0
+    wide[rng.integers(0, V)] = np.inf
+    wide[rng.integers(0, V)] = -0.0
+    spread = np.exp(rng.uniform(-80, 80, V)) * rng.choice([-1.0, 1.0], V)
+    two = np.where(np.arange(V) % 5 == 0, 1.0, -1.0)
+    for x in (wide, spread, two, 1.75 + np.arange(V) * 2.0 ** -12):
+        for k in {0, 1, V // 3, max(V - 1, 0), V}:
+            run_select([x, x[::-1].copy()], [k, V - k])
+
+
 def test_host_made_failures_return_status_codes():
     w = small(post=0)
     step = pu.make_step(w, sim_debug=False)
