@@ -288,3 +288,33 @@ def test_similarity_fp32_gives_the_same_bits_by_rows_and_by_tiles(V, k, D):
     # (32 chains of at most D / 32 products of unit rows, added pairwise: far inside 1e-5)
     assert (got[0][1][pruned].double() - cos[pruned]).abs().max() <= 1e-5
     assert torch.equal(got[0][0][pruned].long(), got[0][1][pruned].argmax(dim=1))
+
+
+# one block per 32 keys with a warp per head (up to four heads), and the kernel with partial sums beyond: deciders below, at and
+# above a warp's width, ragged numbers of keys
+@pytest.mark.parametrize("H", [1, 4, 5])
+@pytest.mark.parametrize("V,n_dec", [(1, 1), (31, 16), (32, 17), (33, 32), (300, 33), (95, 70)])
+def test_importance_of_few_heads(H, V, n_dec):
+    dev, dh = torch.device("cuda", 0), 32
+    g = torch.Generator().manual_seed(V + H)
+    n_vis, n_resp = [V, 2 * V + 3], [n_dec + 2, n_dec]
+    lens = [a + b for a, b in zip(n_vis, n_resp)]
+    N, cu = sum(lens), np.concatenate([[0], np.cumsum(lens)])
+    q, k, v = (torch.randn(N, H * dh, generator=g).to(dev) for _ in range(3))
+    dec = [np.arange(a, a + n_dec, dtype=np.int32) for a in n_vis]
+    i32 = lambda a: torch.as_tensor(np.asarray(a, np.int32), device=dev)
+    ctx = B_.Context(N, 2, H, dh, 2 * n_dec, max(n_vis))
+    out, imp = torch.empty_like(q), torch.full((sum(n_vis) + 1,), -7.0, device=dev)
+    ctx.d3tom_attn_importance(q, k, v, i32(cu), i32(n_vis), i32(np.concatenate(dec)), i32([0, n_dec, 2 * n_dec]), 2, N, max(lens),
+                              max(n_vis), 2 * n_dec, dh ** -0.5, out, imp, i32([0, n_vis[0], sum(n_vis)]))
+    torch.cuda.synchronize()
+    want = []
+    for b in range(2):
+        rows = slice(int(cu[b]), int(cu[b + 1]))
+        qh, kh = (t[rows].double().reshape(lens[b], H, dh).transpose(0, 1) for t in (q, k))
+        a = torch.softmax(qh[:, torch.as_tensor(dec[b], dtype=torch.int64, device=dev)] @ kh.transpose(1, 2) * dh ** -0.5, dim=2)
+        want.append(a[:, :, : n_vis[b]].sum((0, 1)))
+    want = torch.cat(want)
+    # every term is a probability with an fp32 relative error of about 1e-5 (scores of magnitude 10 in the exponent)
+    assert imp[-1].item() == -7.0 and ((imp[:-1].double() - want).abs() <= 1e-4 * want + 1e-7 * n_dec * H).all()
+    ctx.close()
