@@ -198,6 +198,7 @@ int launch_sim_simt(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s);        
 int launch_sim_tc(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s);            // similarity + argmax, tcgen05
 int launch_merge_finish(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s);      // members, aggregate, compact
 int launch_merge_aggregate(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s);   // aggregate, compact (lists already built), both payloads
+constexpr int kStreamMinRows = 4096;       // fewer output rows than this do not go to the bulk-copy pipeline
 int launch_merge_aggregate_stream(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s);   // the same as a bulk-copy pipeline
 
 int launch_wait_timeout_selftest(d3tom_ctx* ctx, long long limit_ns, cudaStream_t s);   // a wait that cannot end

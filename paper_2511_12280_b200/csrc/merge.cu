@@ -11,6 +11,8 @@
 // The arg-max is a 64-bit maximum over (order-preserving similarity bits << 32
 // | ~slot): the largest similarity wins and, among equals, the lowest slot, no
 // matter in which order candidates arrive.
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace {
@@ -452,6 +454,230 @@ aggregate_compact_kernel(const T* __restrict__ hidden_1, const T* __restrict__ h
     }
 }
 
+// Aggregation and compaction without member lists, for calls whose requests have up to kScanVisual visual tokens.  A block
+// takes eight consecutive output rows, one per warp, and one of `col_blocks` parts of their columns (blockIdx.y: payload).  It
+// finds their members itself: it reads the request's packed arg-max words once and marks every token whose slot is one of its
+// rows in a bitmap per row, out of which the positions come in ascending order.  That takes the place of a launch of one block
+// per request that counted, listed and sorted (4 - 9 us in which the other SMs waited) and of the lists' round trip; it costs
+// V x 8 bytes out of L2 per block.  Bound: three dependent rounds of loads, then HBM / L2.
+// The sums run in the order of aggregate_compact_kernel: the kept row, then its members by position, fp32, one rounding; rows
+// with kHeavy members or more (few): eight partial sums, 32-member segment s in sum s % 8, added in order.
+constexpr int kScanRows = kAggWarps;
+constexpr int kScanVisual = 12 * 1024;   // 8 bitmaps and a list of 16-bit positions: 36 KB
+constexpr int kHeavyUnroll = 8;          // rows of a heavy list in flight per lane
+constexpr long long kScanTokens = 256 * 1024;
+constexpr int kScanBlocksPerSm = 2;      // what fits at 128 registers; more parts of the columns scan more than they gain
+
+template <typename T>
+__global__ void __launch_bounds__(kAggWarps * 32, kScanBlocksPerSm)
+aggregate_scan_kernel(const T* __restrict__ hidden_1, const T* __restrict__ hidden_2, const int32_t* __restrict__ cu_seqlens,
+                      const int32_t* __restrict__ cu_vis, const int32_t* __restrict__ kept_idx,
+                      const int32_t* __restrict__ cu_kept, const int32_t* __restrict__ cu_seqlens_out,
+                      const unsigned long long* __restrict__ best, int B, int D, int chunks, int total_out, int col_blocks,
+                      int words, int mean, int32_t* __restrict__ assign, int32_t* __restrict__ member_count,
+                      T* __restrict__ out_1, T* __restrict__ out_2, int32_t* __restrict__ src_of_dst) {
+  constexpr int kVec = Storage<T>::kVec;
+  extern __shared__ unsigned scan_s[];                           // [kScanRows][words] bitmaps, then the lists of heavy rows
+  __shared__ int light_s[kScanRows][32];
+  __shared__ int heavy_s[kScanRows];                             // members of a heavy row, 0: not heavy
+  __shared__ int4 heavy_at[kScanRows];                           // heavy rows in hand: {row, start in the list, position, request}
+  unsigned short* list_s = reinterpret_cast<unsigned short*>(scan_s + kScanRows * words);
+  grid_dependency_enter();
+  const T* __restrict__ hidden = blockIdx.y == 0 ? hidden_1 : hidden_2;
+  T* __restrict__ hidden_out = blockIdx.y == 0 ? out_1 : out_2;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rg = (int)blockIdx.x / col_blocks, cb = (int)blockIdx.x - rg * col_blocks;
+  const int r0 = rg * kScanRows, r1 = min(r0 + kScanRows, total_out);
+  const bool reports = cb == 0 && blockIdx.y == 0;               // one block per row group writes what it found
+  const int groups = (chunks + kAggCpw - 1) / kAggCpw;
+  const int cg0 = cb * groups / col_blocks, cg1 = (cb + 1) * groups / col_blocks;
+
+  // ---- the members of this block's rows
+  for (int i = tid; i < kScanRows * words; i += kAggWarps * 32) scan_s[i] = 0u;
+  const int b_first = find_segment(cu_seqlens_out, B, r0);
+  __syncthreads();
+  for (int b = b_first; b < B; ++b) {
+    const int out0 = cu_seqlens_out[b];
+    if (out0 >= r1) break;
+    const int v0 = cu_vis[b], V = cu_vis[b + 1] - v0, kb = cu_kept[b + 1] - cu_kept[b];
+    const int s0 = max(r0 - out0, 0), s1 = min(r1 - out0, kb);   // the request's slots among the rows
+    if (s0 >= s1 || kb >= V) continue;                           // (or nothing pruned in this request)
+    constexpr int kInFlight = 8;
+    for (int base = 0; base < V; base += kInFlight * kAggWarps * 32) {
+      unsigned low[kInFlight];                                   // ~slot of a pruned token, 0 of a kept one
+#pragma unroll
+      for (int u = 0; u < kInFlight; ++u) {
+        const int m = base + u * kAggWarps * 32 + tid;
+        low[u] = m < V ? (unsigned)(best[v0 + m] & 0xffffffffull) : 0u;
+      }
+#pragma unroll
+      for (int u = 0; u < kInFlight; ++u) {
+        const unsigned slot = 0xffffffffu - low[u];
+        if (slot - (unsigned)s0 < (unsigned)(s1 - s0)) {
+          const int m = base + u * kAggWarps * 32 + tid;
+          atomicOr(&scan_s[(out0 + (int)slot - r0) * words + (m >> 5)], 1u << (m & 31));
+          if (reports) assign[v0 + m] = (int)slot;
+        }
+      }
+    }
+  }
+  __syncthreads();
+
+  // ---- one warp per row
+  const int row = r0 + warp;
+  int cnt = -1, pos = 0, lo = 0;                                 // members (-1: a copied row), position and first row of the request
+  const unsigned* bm = scan_s + warp * words;
+  int row_words = 0;
+  if (row < r1) {
+    const int b = find_segment(cu_seqlens_out, B, row);
+    const int r = row - cu_seqlens_out[b], k0 = cu_kept[b], kb = cu_kept[b + 1] - k0, V = cu_vis[b + 1] - cu_vis[b];
+    lo = cu_seqlens[b];
+    pos = V + (r - kb);
+    if (r < kb) {
+      pos = kept_idx[k0 + r];
+      row_words = (V + 31) >> 5;
+      cnt = 0;
+      for (int w = lane; w < row_words; w += 32) cnt += __popc(bm[w]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+      if (reports && lane == 0) member_count[k0 + r] = cnt;
+    }
+    if (reports && lane == 0) src_of_dst[row] = lo + pos;
+  }
+  // the positions marked in the warp's bitmap, in order, to dst
+  auto list_positions = [&](auto* dst) {
+    int written = 0;
+    for (int w0 = 0; w0 < row_words; w0 += 32) {
+      unsigned v = w0 + lane < row_words ? bm[w0 + lane] : 0u;
+      const int n = __popc(v);
+      int incl = n;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+      }
+      int at = written + incl - n;
+      while (v) {
+        dst[at++] = ((w0 + lane) << 5) + __ffs(v) - 1;
+        v &= v - 1;
+      }
+      written += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    __syncwarp();
+  };
+  const bool heavy = cnt >= kHeavy;
+  if (lane == 0) heavy_s[warp] = heavy ? cnt : 0;
+  if (row < r1 && !heavy) {
+    const T* req = hidden + (size_t)lo * D;
+    T* dst = hidden_out + (size_t)row * D;
+    int ordered = pos;                                           // lane t: the t-th row to add
+    if (cnt > 0) {
+      list_positions(light_s[warp]);
+      if (lane > 0 && lane <= cnt) ordered = light_s[warp][lane - 1];
+    }
+    const int n = cnt + 1;
+    const float inv_denom = mean ? 1.0f / (float)(1 + cnt) : 1.f;
+    for (int cg = cg0; cg < cg1; ++cg) {
+      int col[kAggCpw];
+      bool live[kAggCpw];
+#pragma unroll
+      for (int j = 0; j < kAggCpw; ++j) {
+        col[j] = ((cg * kAggCpw + j) * 32 + lane) * kVec;
+        live[j] = col[j] < D;
+        if (!live[j]) col[j] = 0;                                // lanes past the row end read column 0, write nothing
+      }
+      if (cnt < 0) {                                             // prompt / response row: copy
+        uint4 raw[kAggCpw];
+#pragma unroll
+        for (int j = 0; j < kAggCpw; ++j) raw[j] = *reinterpret_cast<const uint4*>(req + (size_t)pos * D + col[j]);
+#pragma unroll
+        for (int j = 0; j < kAggCpw; ++j) if (live[j]) *reinterpret_cast<uint4*>(dst + col[j]) = raw[j];
+        continue;
+      }
+      float accs[kAggCpw][kVec];
+#pragma unroll
+      for (int j = 0; j < kAggCpw; ++j)
+#pragma unroll
+        for (int e = 0; e < kVec; ++e) accs[j][e] = 0.f;
+      for (int i = 0; i < n; i += kAggUnroll) {                  // kAggUnroll rows x kAggCpw chunks in flight
+        uint4 raw[kAggUnroll][kAggCpw];
+#pragma unroll
+        for (int u = 0; u < kAggUnroll; ++u) {
+          const int rr = __shfl_sync(0xffffffffu, ordered, (i + u) & 31);
+          if (i + u < n) {
+#pragma unroll
+            for (int j = 0; j < kAggCpw; ++j) raw[u][j] = *reinterpret_cast<const uint4*>(req + (size_t)rr * D + col[j]);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < kAggUnroll; ++u)
+          if (i + u < n) {
+#pragma unroll
+            for (int j = 0; j < kAggCpw; ++j) add_raw<T>(accs[j], raw[u][j]);
+          }
+      }
+#pragma unroll
+      for (int j = 0; j < kAggCpw; ++j)
+        if (live[j]) {
+#pragma unroll
+          for (int e = 0; e < kVec; ++e) accs[j][e] *= inv_denom;
+          Storage<T>::store(dst + col[j], accs[j]);
+        }
+    }
+  }
+  __syncthreads();
+
+  // ---- the heavy rows among the eight: one warp per (row, chunk).  The lists of as many rows as fit are written first (those
+  // of one request always do: no token is in two)
+  const int capacity = words * 32, n_chunks = min(cg1 * kAggCpw, chunks) - cg0 * kAggCpw;
+  for (int h0 = 0; h0 < kScanRows;) {
+    int h1 = h0, n_list = 0, n_rows = 0;
+    for (; h1 < kScanRows && n_list + heavy_s[h1] <= capacity; ++h1) {
+      if (heavy_s[h1] == 0) continue;
+      if (warp == h1) {
+        list_positions(list_s + n_list);
+        if (lane == 0) { heavy_at[n_rows] = make_int4(h1, n_list, pos, lo); }
+      }
+      n_list += heavy_s[h1];
+      ++n_rows;
+    }
+    if (n_rows == 0) break;                                      // uniform: none left
+    __syncthreads();
+    for (int t = warp; t < n_rows * n_chunks; t += kAggWarps) {
+      const int4 at = heavy_at[t / n_chunks];
+      const int hc = heavy_s[at.x], c = ((cg0 * kAggCpw + t % n_chunks) * 32 + lane) * kVec;
+      const bool live = c < D;
+      const T* src = hidden + (size_t)at.w * D + (live ? c : 0);
+      const unsigned short* list = list_s + at.y;
+      float total[kVec];
+      for (int w = 0; w < min(kAggWarps, (hc + 31) >> 5); ++w) {        // partial sum w: the segments w, w + 8, ...
+        float acc[kVec];
+#pragma unroll
+        for (int e = 0; e < kVec; ++e) acc[e] = 0.f;
+        if (w == 0) add_raw<T>(acc, *reinterpret_cast<const uint4*>(src + (size_t)at.z * D));
+        for (int seg = w; seg * 32 < hc; seg += kAggWarps)
+          for (int i = seg * 32; i < min(hc, seg * 32 + 32); i += kHeavyUnroll) {
+            uint4 raw[kHeavyUnroll];
+#pragma unroll
+            for (int u = 0; u < kHeavyUnroll; ++u)
+              if (i + u < hc) raw[u] = *reinterpret_cast<const uint4*>(src + (size_t)list[i + u] * D);
+#pragma unroll
+            for (int u = 0; u < kHeavyUnroll; ++u)
+              if (i + u < hc) add_raw<T>(acc, raw[u]);
+          }
+#pragma unroll
+        for (int e = 0; e < kVec; ++e) total[e] = w == 0 ? acc[e] : total[e] + acc[e];
+      }
+      const float inv_denom = mean ? 1.0f / (float)(1 + hc) : 1.f;
+#pragma unroll
+      for (int e = 0; e < kVec; ++e) total[e] *= inv_denom;
+      if (live) Storage<T>::store(hidden_out + (size_t)(r0 + at.x) * D + c, total);
+    }
+    __syncthreads();                                             // the lists are reused
+    h0 = h1;
+  }
+}
+
 }  // namespace
 
 int launch_merge_prepare(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
@@ -469,7 +695,18 @@ int launch_merge_prepare(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
   return D3TOM_OK;
 }
 
+// Calls that aggregate without lists (aggregate_scan_kernel): while the blocks together scan few tokens (every eight rows one
+// request's), or where nothing was pruned.  With lists / without, per merge (us, tokens -> kept x D): 256 -> 64 x 256 fp32
+// 13.1 / 11.7, 577 -> 173 x 1024 19.1 / 17.7, 1024 -> 102 x 4096 28.0 / 26.8, 2048 -> 512 x 4096 37.6 / 36.3, K and V of
+// 1500 -> 300 x 2048 33.4 / 31.8, 2048 -> 2048 x 4096 21.3 / 17.2; but 4096 -> 1024 x 4096 56.3 / 58.1, its K and V 68 / 76,
+// 8000 -> 2000 x 4096 148 / 161.
+static bool scans(const MergeArgs& a) {
+  if (a.max_visual > kScanVisual || a.total_out >= kStreamMinRows) return false;
+  return a.total_out == a.total_tokens || (long long)a.max_visual * ceil_div(a.total_out, kScanRows) <= kScanTokens;
+}
+
 int launch_merge_finish(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
+  if (scans(a)) return launch_merge_aggregate(ctx, a, s);
   // (the attribute belongs to the current device: set on every call, a process may drive several GPUs)
   D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(members_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            kMemberSmemSlots * (int)sizeof(int) + kBitmapBytes));
@@ -522,6 +759,24 @@ int launch_merge_aggregate(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
   }
   const int vec = a.dt == D3TOM_FP32 ? 4 : 8;
   const int chunks = ceil_div(a.D, 32 * vec);                       // 512-byte chunks per row
+  if (scans(a)) {
+    const int row_groups = ceil_div(a.total_out, kScanRows), payloads = a.second != nullptr ? 2 : 1, groups = ceil_div(chunks, kAggCpw);
+    const int want = ceil_div(kScanBlocksPerSm * ctx->sm_count, row_groups * payloads);
+    int col_blocks = 1;                                              // (a power of two: uneven parts wait for the largest)
+    while (col_blocks < want && col_blocks * 2 <= groups) col_blocks *= 2;
+    const int words = ceil_div(a.max_visual, 32);
+    const size_t smem = (size_t)words * (kScanRows * 4 + 64);
+    const dim3 grid(row_groups * col_blocks, payloads);
+    auto launch = [&](auto* tag) -> cudaError_t {
+      using T = typename std::remove_pointer<decltype(tag)>::type;
+      return launch_serialized(aggregate_scan_kernel<T>, grid, kAggWarps * 32, smem, s, static_cast<const T*>(a.hidden),
+                               static_cast<const T*>(a.second), a.cu_seqlens, a.cu_vis, a.kept_idx, a.cu_kept, a.cu_seqlens_out,
+                               ctx->best, a.B, a.D, chunks, a.total_out, col_blocks, words, mean, a.assign, a.member_count,
+                               static_cast<T*>(a.hidden_out), static_cast<T*>(a.second_out), a.src_of_dst);
+    };
+    D3TOM_CUDA_TRY(ctx, a.dt == D3TOM_FP32 ? launch(static_cast<float*>(nullptr)) : launch(static_cast<__nv_bfloat16*>(nullptr)));
+    return D3TOM_OK;
+  }
   const long long warps = (long long)a.total_out * ceil_div(chunks, kAggCpw);
   const int light_blocks = (int)((warps + kAggWarps - 1) / kAggWarps);
   // at most (pruned tokens) / kHeavy kept tokens can be heavy; the blocks beyond the actual number leave at once

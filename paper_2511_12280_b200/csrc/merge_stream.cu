@@ -21,7 +21,6 @@ constexpr int kStreamThreads = 32 * (1 + kConsumerWarps);
 constexpr int kMaxSlots = 32;
 constexpr int kRingBytes = 32 * 1024;
 constexpr int kMaxVecPerThread = 4;        // 16-byte vectors of a segment per consumer thread
-constexpr int kStreamMinRows = 4096;       // fewer output rows than this go to the plain kernel
 constexpr int kHeavyList = 32;             // lists of this many members or more are already sorted in memory
 
 __device__ __forceinline__ void bulk_load(void* smem_dst, const void* gsrc, uint32_t bytes, uint64_t* bar) {

@@ -152,3 +152,68 @@ def test_merge_kv_key_cache_written_over_the_value_cache(V, k, v_over_k):
         outs.append((k_out.clone(), v_out.clone()))
     assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
     ctx.close()
+
+
+# Aggregation that finds a row's members itself: lists at both sides of what one warp adds (31, 32, 33 members, several parts of
+# eight and of thirty-two), kept tokens without members, eight rows that span requests, rows of odd numbers of 16-byte vectors, one
+# and two payloads, nothing pruned.  Every visual token is a multiple of its kept token's unit vector, so the assignment and the
+# sums over K are exact in either type; the sums over V are compared with float64.
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("H,counts", [(4, [[0, 1, 31, 32, 33, 0, 2], [64, 65], [255, 0, 0, 257, 3]]), (9, [[7] * 60, [0] * 9]),
+                                      (4, [[1500, 2, 0, 40, 41, 33, 32, 31, 100]]), (5, [[0], [1], [0, 0, 0], [5, 0, 90]])])
+def test_members_found_by_scanning(H, counts, dtype):
+    dev, dh = torch.device("cuda", 0), 64
+    D, dt = H * dh, torch.float32 if dtype == "fp32" else torch.bfloat16
+    rng = np.random.default_rng(len(counts) + H)
+    K, owner, kept, n_vis, n_prompt = [], [], [], [], [3, 0, 9, 1][: len(counts)]
+    for c in counts:
+        ids = rng.permutation(np.repeat(np.arange(len(c)), np.asarray(c) + 1))
+        first = np.array([np.flatnonzero(ids == i)[0] for i in range(len(c))])          # a kept token: its group's first
+        order = np.argsort(first)                                                      # slots follow positions
+        slot_of = np.empty(len(c), np.int64)
+        slot_of[order] = np.arange(len(c))
+        x = np.zeros((len(ids), D))
+        x[np.arange(len(ids)), ids] = rng.integers(1, 3, len(ids))
+        K.append(x)
+        owner.append(slot_of[ids])
+        kept.append(np.sort(first))
+        n_vis.append(len(ids))
+    B = len(counts)
+    lens, keep = [v + p for v, p in zip(n_vis, n_prompt)], [len(k) for k in kept]
+    cs = lambda a: np.concatenate([[0], np.cumsum(a)]).astype(np.int32)
+    cu, cu_vis, cu_kept, cu_out = cs(lens), cs(n_vis), cs(keep), cs([n - v + k for n, v, k in zip(lens, n_vis, keep)])
+    k_h = np.concatenate([np.concatenate([x, rng.integers(-3, 4, (p, D))]) for x, p in zip(K, n_prompt)])
+    k_d = torch.as_tensor(k_h, device=dev).to(dt)
+    v_d = torch.as_tensor(rng.standard_normal(k_h.shape), device=dev).to(dt)
+    t = lambda a: torch.as_tensor(np.asarray(a, np.int32), device=dev)
+    total, total_out = int(cu[-1]), int(cu_out[-1])
+    ctx = B_.Context(total, B, H, dh, 1, max(n_vis))
+    for second in (True, False):
+        outs = [torch.full((total_out + 1, D), float("nan"), dtype=dt, device=dev) for _ in range(2)]
+        ints = [torch.full((n + 1,), -9, dtype=torch.int32, device=dev) for n in (cu_vis[-1], cu_kept[-1], total_out)]
+        tail = (t(cu), t(n_vis), t(cu_vis), t(np.concatenate(kept)), t(cu_kept), B, D, total, total_out, max(n_vis), max(keep))
+        if second:
+            ctx.d3tom_merge_kv(B_.AGG_SUM, k_d, v_d, *tail, outs[0], outs[1], t(cu_out), *ints)
+        else:
+            ctx.d3tom_merge(B_.AGG_SUM, k_d, *tail, outs[0], t(cu_out), *ints)
+        torch.cuda.synchronize()
+        assign, count, src = (x.cpu().numpy() for x in ints)
+        assert assign[-1] == count[-1] == src[-1] == -9
+        for b in range(B):
+            s, o, lo = slice(cu_vis[b], cu_vis[b + 1]), cu_out[b], cu[b]
+            assert np.array_equal(assign[s], owner[b])
+            assert np.array_equal(count[cu_kept[b]:cu_kept[b + 1]], np.bincount(owner[b], minlength=keep[b]) - 1)
+            assert np.array_equal(src[o:cu_out[b + 1]] - lo, np.concatenate([kept[b], np.arange(n_vis[b], lens[b])]))
+            for got, x in zip(outs[: 2 if second else 1], (k_d, v_d)):
+                rows = x[lo:cu[b + 1]].double().cpu().numpy()
+                want = np.zeros((keep[b], D))
+                np.add.at(want, owner[b], rows[: n_vis[b]])
+                scale = np.zeros((keep[b], D))
+                np.add.at(scale, owner[b], np.abs(rows[: n_vis[b]]))
+                want, scale = np.concatenate([want, rows[n_vis[b]:]]), np.concatenate([scale, np.abs(rows[n_vis[b]:])])
+                err = np.abs(got[o:cu_out[b + 1]].double().cpu().numpy() - want)
+                # fp32 sums of up to 1500 terms (each rounding 2^-24 of the running sum), one rounding to the storage type
+                eps = 2.0 ** -24 * 64 * scale + (2.0 ** -8 * np.abs(want) if dtype == "bf16" else 0)
+                assert (err <= eps + 1e-30).all()
+        assert torch.isnan(outs[0][-1]).all()
+    ctx.close()
