@@ -176,6 +176,7 @@ struct AttnArgs {
 
 int launch_attn_simt(d3tom_ctx* ctx, d3tom_dtype dt, const AttnArgs& a, cudaStream_t s);
 int launch_attn_tc(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s);
+int launch_attn_short(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s);   // short calls: a query tile per SM, QK^T ahead
 int launch_attn_sk(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s);      // one request, work balanced over the SMs
 int launch_attn_one(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s);     // one query tile per CTA, three score buffers
 int launch_importance_finish(d3tom_ctx* ctx, const AttnArgs& a, int max_visual, float* importance,

@@ -422,3 +422,42 @@ def test_similarity_slices_beside_another_stream_that_holds_the_sms():
             assert c.device_status() == 0
             c.close()
     att.close()
+
+
+# Calls whose query tiles all have an SM of their own run a kernel of their own (QK^T two key tiles ahead of PV); the entry point
+# with static scratch always takes whole items of two query tiles: the same arithmetic, hence the same bits.  One to nine key tiles
+# (rings of three tiles, four barriers), ragged last tiles, a request without rows, the last call that still fits and the first
+# that does not; sharp rows, so that the running maximum is raised in later key tiles as well.
+@pytest.mark.parametrize("dh,H,lens,n_dec", [(128, 2, [1], 0), (64, 3, [48, 49], 4), (128, 4, [127, 128, 129], 5), (64, 8, [300, 0, 641], 17),
+                                             (128, 4, [513], 33), (64, 16, [1150], 20), (128, 4, [900, 385, 260], 0), (64, 148, [128], 1),
+                                             (64, 149, [100], 1), (64, 4, [1024, 700, 90], 40)])
+def test_short_calls_equal_whole_items_bit_for_bit(dh, H, lens, n_dec):
+    dev = torch.device("cuda", 0)
+    g = torch.Generator().manual_seed(sum(lens) + dh)
+    cs = lambda a: np.concatenate([[0], np.cumsum(a)]).astype(np.int32)
+    t = lambda a: torch.as_tensor(np.asarray(a, np.int32), device=dev)
+    n, B = sum(lens), len(lens)
+    q, k, v = (torch.randn(n, H * dh, generator=g).to(torch.bfloat16).to(dev) for _ in range(3))
+    q *= 6
+    n_vis = [max(0, x - n_dec - 2) for x in lens]
+    dec = [np.arange(x - n_dec, x, dtype=np.int32) if x > n_dec + 2 else np.zeros(0, np.int32) for x in lens]
+    cu, cu_vis, cu_dec = cs(lens), cs(n_vis), cs([len(d) for d in dec])
+    n_d = int(cu_dec[-1])
+    pos = t(np.concatenate(dec + [np.zeros(1, np.int32)]))
+    ctx = B_.Context(n, B, H, dh, max(n_d, 1), max(max(n_vis), 1))
+    outs = []
+    for call in (ctx.d3tom_attn_importance, lambda *a: B_.d3tom_attn_importance_static(H, dh, *a)):
+        out = torch.full((n + 1, H * dh), float("nan"), dtype=torch.bfloat16, device=dev)
+        imp = torch.full((int(cu_vis[-1]) + 1,), -3.0, device=dev)
+        call(q, k, v, t(cu), t(n_vis), pos, t(cu_dec), B, n, max(lens), max(n_vis), n_d, dh ** -0.5, out, imp, t(cu_vis))
+        torch.cuda.synchronize()
+        outs.append((out, imp))
+    assert ctx.device_status() == 0
+    assert torch.isfinite(outs[0][0][:n].float()).all() and torch.isnan(outs[0][0][n]).all()
+    assert torch.equal(outs[0][0][:n], outs[1][0][:n])
+    for b in range(B):
+        if len(dec[b]):
+            rows = slice(int(cu_vis[b]), int(cu_vis[b + 1]))
+            assert torch.equal(outs[0][1][rows], outs[1][1][rows])
+    assert outs[0][1][-1].item() == -3.0
+    ctx.close()
