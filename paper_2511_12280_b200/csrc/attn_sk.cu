@@ -23,7 +23,6 @@ namespace {
 
 constexpr int kTile = 128;
 constexpr int kAttnThreads = 384;
-constexpr int kSoftmaxRegs = 208, kOtherRegs = 88;   // 256 * 208 + 128 * 88 = 384 * 168; with 64 the issuing and loading warps spill: 1216 rows 35.9 -> 35.0 us
 constexpr int kKvSlots = 4;
 constexpr float kRescaleThreshold = 8.0f;
 
@@ -107,6 +106,11 @@ attn_sk_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
   constexpr int kHalfBytes = kTile * 128;
   constexpr int kHalves = DH / 64;
   constexpr int kSlotFloats = 2 * (128 + 2) * kTile;     // per CTA: two tiles of [128 columns][128 rows] + (m, l) per row
+  // Who issues, and the split of the registers, as measured (us; lane 0 with 216 / 64 registers against elected threads with 208 /
+  // 88, where the issuing and loading warps spill less): plain at head_dim 128 the latter, 1216 rows x 32 heads 35.5 / 35.0,
+  // 4288 281 / 275; with the importance map 4288 rows 282 / 292, 10770 1806 / 1941; at head_dim 64 6602 rows x 16 heads 247 / 258.
+  constexpr bool kElected = DH == 128 && !kImp;
+  constexpr int kSoftmaxRegs = kElected ? 208 : 216, kOtherRegs = kElected ? 88 : 64;   // 256 x + 128 y <= 384 * 168
   grid_dependency_enter();
   const int lo = a.cu_seqlens[0], n = a.cu_seqlens[1] - lo;
   // deciders are response rows: rows below the visual count cannot be any, and their segments skip the look-up
@@ -140,7 +144,7 @@ attn_sk_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 18);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int warp = ptx::uniform_warp(), lane = threadIdx.x & 31;
+  const int warp = kElected ? ptx::uniform_warp() : (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) {
       ptx::mbar_init(&q_full[i], 1); ptx::mbar_init(&q_empty[i], 4);
@@ -164,7 +168,7 @@ attn_sk_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));
     if (warp == 8) {
       // ------------------------------------------------------------ TMA producer
-      if (ptx::elect_one()) {
+      if (kElected ? ptx::elect_one() : lane == 0) {
         ptx::prefetch_tensormap(&tmap_q); ptx::prefetch_tensormap(&tmap_k); ptx::prefetch_tensormap(&tmap_v);
         Walk w = walk0;
         int g = 0, segs[2] = {0, 0};
@@ -199,7 +203,7 @@ attn_sk_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant
       }
     } else if (warp == 9) {
       // ------------------------------------------------------------ MMA issuer
-      if (ptx::elect_one()) {
+      if (kElected ? ptx::elect_one() : lane == 0) {
         constexpr uint32_t idesc_qk = ptx::idesc_bf16_f32(kTile, kTile, 0, 0);
         constexpr uint32_t idesc_pv = ptx::idesc_bf16_f32(kTile, DH, 0, 1);
         const ptx::SmemDesc q_desc[2] = {ptx::smem_desc_kmajor_sw128(ptx::smem_u32(q_s)),

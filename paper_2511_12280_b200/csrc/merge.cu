@@ -454,96 +454,86 @@ aggregate_compact_kernel(const T* __restrict__ hidden_1, const T* __restrict__ h
     }
 }
 
-// Aggregation and compaction without member lists, for calls whose requests have up to kScanVisual visual tokens.  A block
-// takes eight consecutive output rows, one per warp, and one of `col_blocks` parts of their columns (blockIdx.y: payload).  It
-// finds their members itself: it reads the request's packed arg-max words once and marks every token whose slot is one of its
-// rows in a bitmap per row, out of which the positions come in ascending order.  That takes the place of a launch of one block
-// per request that counted, listed and sorted (4 - 9 us in which the other SMs waited) and of the lists' round trip; it costs
-// V x 8 bytes out of L2 per block.  Bound: three dependent rounds of loads, then HBM / L2.
+// Aggregation and compaction of ONE request of up to kScanVisual visual tokens without member lists.  A block takes eight
+// consecutive output rows, one per warp, and one of `col_blocks` parts of their columns (blockIdx.y: payload).  It finds their
+// members itself: it reads the request's packed arg-max words once and marks every token whose slot is one of its rows in a
+// bitmap per row, out of which the positions come in ascending order.  That takes the place of a launch of one block that
+// counted, listed and sorted (4 - 9 us in which the other SMs waited) and of the lists' round trip; it costs V x 8 bytes out of
+// L2 per block.  Bound: three dependent rounds of loads, then HBM / L2.
 // The sums run in the order of aggregate_compact_kernel: the kept row, then its members by position, fp32, one rounding; rows
 // with kHeavy members or more (few): eight partial sums, 32-member segment s in sum s % 8, added in order.
 constexpr int kScanRows = kAggWarps;
 constexpr int kScanVisual = 12 * 1024;   // 8 bitmaps and a list of 16-bit positions: 36 KB
-constexpr int kHeavyUnroll = 8;          // rows of a heavy list in flight per lane
 constexpr long long kScanTokens = 256 * 1024;
-constexpr int kScanBlocksPerSm = 2;      // what fits at 128 registers; more parts of the columns scan more than they gain
 
-template <typename T>
-__global__ void __launch_bounds__(kAggWarps * 32, kScanBlocksPerSm)
+// kHeavyUnroll: rows of a heavy list in flight per lane; kBlocks: blocks per SM it leaves registers for
+template <typename T, int kHeavyUnroll, int kBlocks>
+__global__ void __launch_bounds__(kAggWarps * 32, kBlocks)
 aggregate_scan_kernel(const T* __restrict__ hidden_1, const T* __restrict__ hidden_2, const int32_t* __restrict__ cu_seqlens,
                       const int32_t* __restrict__ cu_vis, const int32_t* __restrict__ kept_idx,
-                      const int32_t* __restrict__ cu_kept, const int32_t* __restrict__ cu_seqlens_out,
-                      const unsigned long long* __restrict__ best, int B, int D, int chunks, int total_out, int col_blocks,
-                      int words, int mean, int32_t* __restrict__ assign, int32_t* __restrict__ member_count,
-                      T* __restrict__ out_1, T* __restrict__ out_2, int32_t* __restrict__ src_of_dst) {
+                      const int32_t* __restrict__ cu_kept, const unsigned long long* __restrict__ best, int D, int chunks,
+                      int total_out, int col_blocks, int words, int mean, int32_t* __restrict__ assign,
+                      int32_t* __restrict__ member_count, T* __restrict__ out_1, T* __restrict__ out_2,
+                      int32_t* __restrict__ src_of_dst) {
   constexpr int kVec = Storage<T>::kVec;
-  extern __shared__ unsigned scan_s[];                           // [kScanRows][words] bitmaps, then the lists of heavy rows
+  extern __shared__ unsigned scan_s[];                           // [kScanRows][words] bitmaps, then the lists of the heavy rows
   __shared__ int light_s[kScanRows][32];
   __shared__ int heavy_s[kScanRows];                             // members of a heavy row, 0: not heavy
-  __shared__ int4 heavy_at[kScanRows];                           // heavy rows in hand: {row, start in the list, position, request}
+  __shared__ int4 heavy_at[kScanRows];                           // the heavy rows: {row, start of the list, position, members}
+  __shared__ int next_task;
   unsigned short* list_s = reinterpret_cast<unsigned short*>(scan_s + kScanRows * words);
   grid_dependency_enter();
-  const T* __restrict__ hidden = blockIdx.y == 0 ? hidden_1 : hidden_2;
+  const T* __restrict__ hidden = (blockIdx.y == 0 ? hidden_1 : hidden_2) + (size_t)cu_seqlens[0] * D;
   T* __restrict__ hidden_out = blockIdx.y == 0 ? out_1 : out_2;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rg = (int)blockIdx.x / col_blocks, cb = (int)blockIdx.x - rg * col_blocks;
-  const int r0 = rg * kScanRows, r1 = min(r0 + kScanRows, total_out);
+  const int r0 = rg * kScanRows, r1 = min(r0 + kScanRows, total_out), row = r0 + warp;
   const bool reports = cb == 0 && blockIdx.y == 0;               // one block per row group writes what it found
   const int groups = (chunks + kAggCpw - 1) / kAggCpw;
   const int cg0 = cb * groups / col_blocks, cg1 = (cb + 1) * groups / col_blocks;
+  const int V = cu_vis[1] - cu_vis[0], kb = cu_kept[1] - cu_kept[0];
+  const int pos = row < kb ? kept_idx[cu_kept[0] + row] : V + (row - kb);      // source row in the request (rows past the end: unused)
 
   // ---- the members of this block's rows
   for (int i = tid; i < kScanRows * words; i += kAggWarps * 32) scan_s[i] = 0u;
-  const int b_first = find_segment(cu_seqlens_out, B, r0);
+  if (tid == 0) next_task = 0;
   __syncthreads();
-  for (int b = b_first; b < B; ++b) {
-    const int out0 = cu_seqlens_out[b];
-    if (out0 >= r1) break;
-    const int v0 = cu_vis[b], V = cu_vis[b + 1] - v0, kb = cu_kept[b + 1] - cu_kept[b];
-    const int s0 = max(r0 - out0, 0), s1 = min(r1 - out0, kb);   // the request's slots among the rows
-    if (s0 >= s1 || kb >= V) continue;                           // (or nothing pruned in this request)
+  const int s1 = min(r1, kb);                                    // [r0, s1): the kept slots among the rows
+  if (r0 < s1 && kb < V) {                                       // (else nothing was pruned)
     constexpr int kInFlight = 8;
+    const unsigned long long* words_in = best + cu_vis[0];
     for (int base = 0; base < V; base += kInFlight * kAggWarps * 32) {
       unsigned low[kInFlight];                                   // ~slot of a pruned token, 0 of a kept one
 #pragma unroll
       for (int u = 0; u < kInFlight; ++u) {
         const int m = base + u * kAggWarps * 32 + tid;
-        low[u] = m < V ? (unsigned)(best[v0 + m] & 0xffffffffull) : 0u;
+        low[u] = m < V ? (unsigned)(words_in[m] & 0xffffffffull) : 0u;
       }
 #pragma unroll
       for (int u = 0; u < kInFlight; ++u) {
         const unsigned slot = 0xffffffffu - low[u];
-        if (slot - (unsigned)s0 < (unsigned)(s1 - s0)) {
+        if (slot - (unsigned)r0 < (unsigned)(s1 - r0)) {
           const int m = base + u * kAggWarps * 32 + tid;
-          atomicOr(&scan_s[(out0 + (int)slot - r0) * words + (m >> 5)], 1u << (m & 31));
-          if (reports) assign[v0 + m] = (int)slot;
+          atomicOr(&scan_s[((int)slot - r0) * words + (m >> 5)], 1u << (m & 31));
+          if (reports) assign[cu_vis[0] + m] = (int)slot;
         }
       }
     }
   }
   __syncthreads();
 
-  // ---- one warp per row
-  const int row = r0 + warp;
-  int cnt = -1, pos = 0, lo = 0;                                 // members (-1: a copied row), position and first row of the request
+  // ---- one warp per row: its members are counted and, where they are many, listed for all warps
+  const int row_words = row < s1 ? (V + 31) >> 5 : 0;
   const unsigned* bm = scan_s + warp * words;
-  int row_words = 0;
-  if (row < r1) {
-    const int b = find_segment(cu_seqlens_out, B, row);
-    const int r = row - cu_seqlens_out[b], k0 = cu_kept[b], kb = cu_kept[b + 1] - k0, V = cu_vis[b + 1] - cu_vis[b];
-    lo = cu_seqlens[b];
-    pos = V + (r - kb);
-    if (r < kb) {
-      pos = kept_idx[k0 + r];
-      row_words = (V + 31) >> 5;
-      cnt = 0;
-      for (int w = lane; w < row_words; w += 32) cnt += __popc(bm[w]);
+  int cnt = -1;                                                  // (a copied row)
+  if (row < s1) {
+    cnt = 0;
+    for (int w = lane; w < row_words; w += 32) cnt += __popc(bm[w]);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-      if (reports && lane == 0) member_count[k0 + r] = cnt;
-    }
-    if (reports && lane == 0) src_of_dst[row] = lo + pos;
+    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+    if (reports && lane == 0) member_count[cu_kept[0] + row] = cnt;
   }
+  if (row < r1 && reports && lane == 0) src_of_dst[row] = cu_seqlens[0] + pos;
   // the positions marked in the warp's bitmap, in order, to dst
   auto list_positions = [&](auto* dst) {
     int written = 0;
@@ -567,8 +557,22 @@ aggregate_scan_kernel(const T* __restrict__ hidden_1, const T* __restrict__ hidd
   };
   const bool heavy = cnt >= kHeavy;
   if (lane == 0) heavy_s[warp] = heavy ? cnt : 0;
+  __syncthreads();
+  int n_heavy = 0, n_list = 0;                                   // (no token is in two lists: together at most V positions)
+#pragma unroll
+  for (int r = 0; r < kScanRows; ++r) {
+    const int hc = heavy_s[r];
+    if (hc == 0) continue;
+    if (warp == r) {
+      list_positions(list_s + n_list);
+      if (lane == 0) heavy_at[n_heavy] = make_int4(r0 + r, n_list, pos, hc);
+    }
+    n_list += hc;
+    ++n_heavy;
+  }
+  if (n_heavy > 0) __syncthreads();                              // uniform
+
   if (row < r1 && !heavy) {
-    const T* req = hidden + (size_t)lo * D;
     T* dst = hidden_out + (size_t)row * D;
     int ordered = pos;                                           // lane t: the t-th row to add
     if (cnt > 0) {
@@ -589,7 +593,7 @@ aggregate_scan_kernel(const T* __restrict__ hidden_1, const T* __restrict__ hidd
       if (cnt < 0) {                                             // prompt / response row: copy
         uint4 raw[kAggCpw];
 #pragma unroll
-        for (int j = 0; j < kAggCpw; ++j) raw[j] = *reinterpret_cast<const uint4*>(req + (size_t)pos * D + col[j]);
+        for (int j = 0; j < kAggCpw; ++j) raw[j] = *reinterpret_cast<const uint4*>(hidden + (size_t)pos * D + col[j]);
 #pragma unroll
         for (int j = 0; j < kAggCpw; ++j) if (live[j]) *reinterpret_cast<uint4*>(dst + col[j]) = raw[j];
         continue;
@@ -606,7 +610,7 @@ aggregate_scan_kernel(const T* __restrict__ hidden_1, const T* __restrict__ hidd
           const int rr = __shfl_sync(0xffffffffu, ordered, (i + u) & 31);
           if (i + u < n) {
 #pragma unroll
-            for (int j = 0; j < kAggCpw; ++j) raw[u][j] = *reinterpret_cast<const uint4*>(req + (size_t)rr * D + col[j]);
+            for (int j = 0; j < kAggCpw; ++j) raw[u][j] = *reinterpret_cast<const uint4*>(hidden + (size_t)rr * D + col[j]);
           }
         }
 #pragma unroll
@@ -625,56 +629,42 @@ aggregate_scan_kernel(const T* __restrict__ hidden_1, const T* __restrict__ hidd
         }
     }
   }
-  __syncthreads();
 
-  // ---- the heavy rows among the eight: one warp per (row, chunk).  The lists of as many rows as fit are written first (those
-  // of one request always do: no token is in two)
-  const int capacity = words * 32, n_chunks = min(cg1 * kAggCpw, chunks) - cg0 * kAggCpw;
-  for (int h0 = 0; h0 < kScanRows;) {
-    int h1 = h0, n_list = 0, n_rows = 0;
-    for (; h1 < kScanRows && n_list + heavy_s[h1] <= capacity; ++h1) {
-      if (heavy_s[h1] == 0) continue;
-      if (warp == h1) {
-        list_positions(list_s + n_list);
-        if (lane == 0) { heavy_at[n_rows] = make_int4(h1, n_list, pos, lo); }
-      }
-      n_list += heavy_s[h1];
-      ++n_rows;
+  // ---- the heavy rows: (row, chunk) by whichever warp is free
+  const int n_chunks = min(cg1 * kAggCpw, chunks) - cg0 * kAggCpw, n_tasks = n_heavy * n_chunks;
+  while (n_tasks > 0) {
+    int t = 0;
+    if (lane == 0) t = atomicAdd(&next_task, 1);
+    t = __shfl_sync(0xffffffffu, t, 0);
+    if (t >= n_tasks) break;
+    const int4 at = heavy_at[t / n_chunks];
+    const int hc = at.w, c = ((cg0 * kAggCpw + t % n_chunks) * 32 + lane) * kVec;
+    const bool live = c < D;
+    const T* src = hidden + (live ? c : 0);
+    const unsigned short* list = list_s + at.y;
+    float total[kVec];
+    for (int w = 0; w < min(kAggWarps, (hc + 31) >> 5); ++w) {   // partial sum w: the segments w, w + 8, ...
+      float acc[kVec];
+#pragma unroll
+      for (int e = 0; e < kVec; ++e) acc[e] = 0.f;
+      if (w == 0) add_raw<T>(acc, *reinterpret_cast<const uint4*>(src + (size_t)at.z * D));
+      for (int seg = w; seg * 32 < hc; seg += kAggWarps)
+        for (int i = seg * 32; i < min(hc, seg * 32 + 32); i += kHeavyUnroll) {
+          uint4 raw[kHeavyUnroll];
+#pragma unroll
+          for (int u = 0; u < kHeavyUnroll; ++u)
+            if (i + u < hc) raw[u] = *reinterpret_cast<const uint4*>(src + (size_t)list[i + u] * D);
+#pragma unroll
+          for (int u = 0; u < kHeavyUnroll; ++u)
+            if (i + u < hc) add_raw<T>(acc, raw[u]);
+        }
+#pragma unroll
+      for (int e = 0; e < kVec; ++e) total[e] = w == 0 ? acc[e] : total[e] + acc[e];
     }
-    if (n_rows == 0) break;                                      // uniform: none left
-    __syncthreads();
-    for (int t = warp; t < n_rows * n_chunks; t += kAggWarps) {
-      const int4 at = heavy_at[t / n_chunks];
-      const int hc = heavy_s[at.x], c = ((cg0 * kAggCpw + t % n_chunks) * 32 + lane) * kVec;
-      const bool live = c < D;
-      const T* src = hidden + (size_t)at.w * D + (live ? c : 0);
-      const unsigned short* list = list_s + at.y;
-      float total[kVec];
-      for (int w = 0; w < min(kAggWarps, (hc + 31) >> 5); ++w) {        // partial sum w: the segments w, w + 8, ...
-        float acc[kVec];
+    const float inv_denom = mean ? 1.0f / (float)(1 + hc) : 1.f;
 #pragma unroll
-        for (int e = 0; e < kVec; ++e) acc[e] = 0.f;
-        if (w == 0) add_raw<T>(acc, *reinterpret_cast<const uint4*>(src + (size_t)at.z * D));
-        for (int seg = w; seg * 32 < hc; seg += kAggWarps)
-          for (int i = seg * 32; i < min(hc, seg * 32 + 32); i += kHeavyUnroll) {
-            uint4 raw[kHeavyUnroll];
-#pragma unroll
-            for (int u = 0; u < kHeavyUnroll; ++u)
-              if (i + u < hc) raw[u] = *reinterpret_cast<const uint4*>(src + (size_t)list[i + u] * D);
-#pragma unroll
-            for (int u = 0; u < kHeavyUnroll; ++u)
-              if (i + u < hc) add_raw<T>(acc, raw[u]);
-          }
-#pragma unroll
-        for (int e = 0; e < kVec; ++e) total[e] = w == 0 ? acc[e] : total[e] + acc[e];
-      }
-      const float inv_denom = mean ? 1.0f / (float)(1 + hc) : 1.f;
-#pragma unroll
-      for (int e = 0; e < kVec; ++e) total[e] *= inv_denom;
-      if (live) Storage<T>::store(hidden_out + (size_t)(r0 + at.x) * D + c, total);
-    }
-    __syncthreads();                                             // the lists are reused
-    h0 = h1;
+    for (int e = 0; e < kVec; ++e) total[e] *= inv_denom;
+    if (live) Storage<T>::store(hidden_out + (size_t)at.x * D + c, total);
   }
 }
 
@@ -695,18 +685,33 @@ int launch_merge_prepare(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
   return D3TOM_OK;
 }
 
-// Calls that aggregate without lists (aggregate_scan_kernel): while the blocks together scan few tokens (every eight rows one
-// request's), or where nothing was pruned.  With lists / without, per merge (us, tokens -> kept x D): 256 -> 64 x 256 fp32
-// 13.1 / 11.7, 577 -> 173 x 1024 19.1 / 17.7, 1024 -> 102 x 4096 28.0 / 26.8, 2048 -> 512 x 4096 37.6 / 36.3, K and V of
-// 1500 -> 300 x 2048 33.4 / 31.8, 2048 -> 2048 x 4096 21.3 / 17.2; but 4096 -> 1024 x 4096 56.3 / 58.1, its K and V 68 / 76,
-// 8000 -> 2000 x 4096 148 / 161.
-static bool scans(const MergeArgs& a) {
-  if (a.max_visual > kScanVisual || a.total_out >= kStreamMinRows) return false;
-  return a.total_out == a.total_tokens || (long long)a.max_visual * ceil_div(a.total_out, kScanRows) <= kScanTokens;
+// How a call aggregates without lists (aggregate_scan_kernel): parts of the columns per row group, and whether sixteen rows of a
+// heavy list are in flight (one block per SM then); col_blocks 0: with lists.  One request, where the blocks together scan few
+// tokens or nothing was pruned, and heavy rows are either few (up to four members per kept token on average) or added sixteen at
+// a time.  With lists / without, per merge (us, tokens -> kept x D): 256 -> 64 x 256 fp32 13.1 / 11.4, 485 -> 48 x 512 fp32
+// 17.8 / 15.5, 577 -> 173 x 1024 19.2 / 17.3, 1024 -> 102 x 4096 27.4 / 23.7, 2048 -> 512 x 4096 38.0 / 35.9, K and V of
+// 1500 -> 300 x 2048 32.7 / 30.2, 2048 -> 2048 x 4096 21.3 / 17.6; but 4096 -> 1024 x 4096 56 / 58, its K and V 68 / 76,
+// 8000 -> 2000 x 4096 148 / 161, K and V of five requests of up to 653 tokens x 2048, a tenth kept, 37 / 38.5.
+struct ScanPlan { int col_blocks; bool wide; };
+static ScanPlan scan_plan(const d3tom_ctx* ctx, const MergeArgs& a) {
+  ScanPlan p = {0, false};
+  if (a.B != 1 || a.max_visual > kScanVisual || a.total_out >= kStreamMinRows || a.total_out <= 0) return p;
+  const int row_groups = ceil_div(a.total_out, kScanRows), payloads = a.second != nullptr ? 2 : 1, pruned = a.total_tokens - a.total_out;
+  if (pruned > 0 && (long long)a.max_visual * row_groups > kScanTokens) return p;
+  const int groups = ceil_div(ceil_div(a.D, 32 * (a.dt == D3TOM_FP32 ? 4 : 8)), kAggCpw);
+  const int want = ceil_div(2 * ctx->sm_count, row_groups * payloads);     // (two blocks per SM fit at 128 registers)
+  int col_blocks = 1;                                                      // (a power of two: uneven parts wait for the largest)
+  while (col_blocks < want && col_blocks * 2 <= groups) col_blocks *= 2;
+  p.wide = row_groups * payloads * col_blocks <= ctx->sm_count;
+  if (p.wide || pruned <= 4 * a.max_kept) p.col_blocks = col_blocks;
+  return p;
 }
 
-int launch_merge_finish(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
-  if (scans(a)) return launch_merge_aggregate(ctx, a, s);
+int launch_merge_finish(d3tom_ctx* ctx, const MergeArgs& args, cudaStream_t s) {
+  MergeArgs a = args;
+  const ScanPlan plan = scan_plan(ctx, a);               // (decided once: payloads launched one by one follow it too)
+  a.scan_col_blocks = plan.col_blocks; a.scan_wide = plan.wide;
+  if (a.scan_col_blocks > 0) return launch_merge_aggregate(ctx, a, s);
   // (the attribute belongs to the current device: set on every call, a process may drive several GPUs)
   D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(members_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            kMemberSmemSlots * (int)sizeof(int) + kBitmapBytes));
@@ -759,19 +764,15 @@ int launch_merge_aggregate(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
   }
   const int vec = a.dt == D3TOM_FP32 ? 4 : 8;
   const int chunks = ceil_div(a.D, 32 * vec);                       // 512-byte chunks per row
-  if (scans(a)) {
-    const int row_groups = ceil_div(a.total_out, kScanRows), payloads = a.second != nullptr ? 2 : 1, groups = ceil_div(chunks, kAggCpw);
-    const int want = ceil_div(kScanBlocksPerSm * ctx->sm_count, row_groups * payloads);
-    int col_blocks = 1;                                              // (a power of two: uneven parts wait for the largest)
-    while (col_blocks < want && col_blocks * 2 <= groups) col_blocks *= 2;
+  if (a.scan_col_blocks > 0) {
     const int words = ceil_div(a.max_visual, 32);
     const size_t smem = (size_t)words * (kScanRows * 4 + 64);
-    const dim3 grid(row_groups * col_blocks, payloads);
+    const dim3 grid(ceil_div(a.total_out, kScanRows) * a.scan_col_blocks, a.second != nullptr ? 2 : 1);
     auto launch = [&](auto* tag) -> cudaError_t {
       using T = typename std::remove_pointer<decltype(tag)>::type;
-      return launch_serialized(aggregate_scan_kernel<T>, grid, kAggWarps * 32, smem, s, static_cast<const T*>(a.hidden),
-                               static_cast<const T*>(a.second), a.cu_seqlens, a.cu_vis, a.kept_idx, a.cu_kept, a.cu_seqlens_out,
-                               ctx->best, a.B, a.D, chunks, a.total_out, col_blocks, words, mean, a.assign, a.member_count,
+      return launch_serialized(a.scan_wide ? aggregate_scan_kernel<T, 16, 1> : aggregate_scan_kernel<T, 8, 2>, grid, kAggWarps * 32, smem, s, static_cast<const T*>(a.hidden),
+                               static_cast<const T*>(a.second), a.cu_seqlens, a.cu_vis, a.kept_idx, a.cu_kept, ctx->best, a.D, chunks,
+                               a.total_out, a.scan_col_blocks, words, mean, a.assign, a.member_count,
                                static_cast<T*>(a.hidden_out), static_cast<T*>(a.second_out), a.src_of_dst);
     };
     D3TOM_CUDA_TRY(ctx, a.dt == D3TOM_FP32 ? launch(static_cast<float*>(nullptr)) : launch(static_cast<__nv_bfloat16*>(nullptr)));
