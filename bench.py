@@ -268,7 +268,9 @@ def step_kernel_labels(step):
            ("prepare_rows", "prepare_rows")]
     if step.total_out < step.total:
         seq.append(("similarity_gemm", "gemm_"))
-    seq += [("members", "members"), ("aggregate_compact", "aggregate")]
+    if step.uses_member_lists():
+        seq.append(("members", "members"))
+    seq.append(("aggregate_compact", "aggregate"))
     for _ in range(step.n_post):
         seq += [("proj_qkv", "gemm_"), ("attn_post", "attn_")]       # gemm_tc_kernel, or gemm_pair_kernel for long layers
     return seq

@@ -286,7 +286,7 @@ importance_finish_kernel(const float* __restrict__ score, const float2* __restri
 // dependent rounds of loads instead of five (no partials through global memory, no counter): what a small call costs is that
 // chain.
 __global__ void __launch_bounds__(1024)
-importance_block_kernel(const float* __restrict__ score, const float2* __restrict__ lse,
+importance_finish_block_kernel(const float* __restrict__ score, const float2* __restrict__ lse,
                         const int32_t* __restrict__ n_visual, const int32_t* __restrict__ cu_deciders,
                         const int32_t* __restrict__ cu_vis, int max_deciders, int vis_stride, float scale_log2, int H,
                         float* __restrict__ importance) {
@@ -375,7 +375,7 @@ int launch_importance_finish(d3tom_ctx* ctx, const AttnArgs& a, int max_visual, 
                              const int32_t* cu_vis, cudaStream_t s) {
   if (max_visual <= 0) return D3TOM_OK;
   if (a.H <= kImpBlockHeads) {
-    D3TOM_CUDA_TRY(ctx, launch_serialized(importance_block_kernel, dim3(ceil_div(max_visual, 32), a.B), a.H * 32, 0, s,
+    D3TOM_CUDA_TRY(ctx, launch_serialized(importance_finish_block_kernel, dim3(ceil_div(max_visual, 32), a.B), a.H * 32, 0, s,
                                           a.score_scratch, a.lse_scratch, a.n_visual, a.cu_deciders, cu_vis, a.max_deciders,
                                           a.vis_stride, a.scale_log2, a.H, importance));
     return D3TOM_OK;

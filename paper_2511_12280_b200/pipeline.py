@@ -156,12 +156,22 @@ class MergeLayerStep:
             self.run(q, k, v, w_post)
         return graph
 
+    def uses_member_lists(self) -> bool:
+        """Whether the merge of the current problem launches the kernel that lists members (the rule of scan_plan in merge.cu)."""
+        rows, pruned, chunks = -(-self.total_out // 8), self.total - self.total_out, -(-self.D * self.attn_out.element_size() // 512)
+        if self.nB != 1 or self.max_visual > 12288 or self.total_out >= 4096 or (pruned and self.max_visual * rows > 256 * 1024):
+            return True
+        groups, parts, sms = -(-chunks // 4), 1, torch.cuda.get_device_properties(self.dev).multi_processor_count
+        while parts * rows < 2 * sms and parts * 2 <= groups:
+            parts *= 2
+        return rows * parts > sms and pruned > 4 * self.max_kept
+
     def launches_per_step(self) -> int:
         """Kernels of this library launched by one run(): attention 1 + importance finish 1,
-        select 1, merge 1 (prepare) + 1 (similarity, when something is pruned) + 2 (members,
-        aggregate/compact), and 2 per post-merge layer."""
+        select 1, merge 1 (prepare) + 1 (similarity, when something is pruned) + 1 (members, where lists are used)
+        + 1 (aggregate/compact), and 2 per post-merge layer."""
         sim = 1 if self.total_out < self.total else 0
-        return 2 + 1 + 1 + sim + 2 + 2 * self.n_post
+        return 2 + 1 + 1 + sim + int(self.uses_member_lists()) + 1 + 2 * self.n_post
 
 
 class HostFedStep:
