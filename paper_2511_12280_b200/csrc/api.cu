@@ -267,7 +267,7 @@ static int attn_common(d3tom_ctx* ctx, d3tom_dtype dt, const void* q, const void
   if (dt == D3TOM_BF16 && !ctx->reference_kernels) {
     st = D3TOM_ERR_UNSUPPORTED;
     if (g_d3tom_single_tile_attention == 1) st = launch_attn_one(ctx, a, stream);   // one query tile per CTA
-    if (st == D3TOM_ERR_UNSUPPORTED) st = launch_attn_short(ctx, a, stream);   // every query tile has an SM of its own
+    if (st == D3TOM_ERR_UNSUPPORTED && g_d3tom_single_tile_attention != 0) st = launch_attn_short(ctx, a, stream);   // every query tile has an SM of its own
     if (st == D3TOM_ERR_UNSUPPORTED) st = launch_attn_sk(ctx, a, stream);   // one request whose items do not fill whole rounds of SMs
     if (st == D3TOM_ERR_UNSUPPORTED) st = launch_attn_tc(ctx, a, stream);
   } else {
