@@ -276,7 +276,7 @@ static int attn_common(d3tom_ctx* ctx, d3tom_dtype dt, const void* q, const void
   if (st != D3TOM_OK) return st;
   if (with_importance) {
     a.cu_deciders = cu_deciders;
-    st = launch_importance_finish(ctx, a, max_visual, importance, cu_vis, stream);
+    st = launch_importance_finish(ctx, a, n_deciders_total, max_visual, importance, cu_vis, stream);
   }
   return st;
 }

@@ -226,9 +226,10 @@ attn_simt_kernel(AttnArgs a, bool vec) {
 // so the result does not depend on which block that is: no float atomics, reproducible.
 constexpr int kImpThreads = 256;
 constexpr int kImpDecChunk = 128;
-// Up to this many heads one block per 32 keys (below): attention + importance, partial sums / one pass (us): 256 keys x 4 heads
-// 17.8 / 14.8; but 1024 keys x 8 heads 90.3 / 93.3, 1024 x 32 47.2 / 53.1, where a block's 128-byte pieces of many rows are the
-// longer way to the same bytes.
+// Up to this many heads and deciders one block per 32 keys (below): attention + importance, partial sums / one pass (us): 256
+// keys x 4 heads, 8 deciders 17.5 / 14.4; but 800 x 4, 16 deciders 54.7 / 55.2, 364 x 4, 32 deciders 31.0 / 35.2, and 1024 keys
+// x 8 heads 90.3 / 93.3, 1024 x 32 47.2 / 53.1, where a block's 128-byte pieces of many rows are the longer way to the same bytes.
+constexpr int kImpBlockDeciders = 8;
 constexpr int kImpBlockHeads = 4;
 
 __global__ void __launch_bounds__(kImpThreads)
@@ -285,34 +286,29 @@ importance_finish_kernel(const float* __restrict__ score, const float2* __restri
 // The same sums in one pass: one block = 32 visual keys of a request, one warp per head; the heads meet in shared memory.  Two
 // dependent rounds of loads instead of five (no partials through global memory, no counter): what a small call costs is that
 // chain.
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(32 * kImpBlockHeads)
 importance_finish_block_kernel(const float* __restrict__ score, const float2* __restrict__ lse,
                         const int32_t* __restrict__ n_visual, const int32_t* __restrict__ cu_deciders,
                         const int32_t* __restrict__ cu_vis, int max_deciders, int vis_stride, float scale_log2, int H,
                         float* __restrict__ importance) {
-  __shared__ float part[32][32];
+  __shared__ float part[kImpBlockHeads][32];
   grid_dependency_enter();
   const int b = blockIdx.y, h = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int Vb = n_visual[b], j = blockIdx.x * 32 + lane;
   const int d0 = cu_deciders[b], d1 = cu_deciders[b + 1], g0 = cu_vis[b];
   if ((int)blockIdx.x * 32 >= Vb) return;                       // uniform: no key of this request in the range
   const int jj = j < Vb ? j : Vb - 1;                           // lanes past the end read a valid column, write nothing
-  float acc = 0.f;
-  for (int dc = d0; dc < d1; dc += 32) {
-    const int nd = min(32, d1 - dc);
-    const float2 ml = lane < nd ? lse[(size_t)h * max_deciders + dc + lane] : make_float2(0.f, 1.f);
-    const float neg_m = -ml.x, inv_l = 1.0f / ml.y;
-    const float* col = score + ((size_t)h * max_deciders + dc) * vis_stride + jj;
-    for (int u0 = 0; u0 < nd; u0 += 16) {                       // 16 deciders in flight; the sum runs in ascending order
-      float x[16];
+  const int nd = d1 - d0;                                       // at most kImpBlockDeciders
+  const float2 ml = lane < nd ? lse[(size_t)h * max_deciders + d0 + lane] : make_float2(0.f, 1.f);
+  const float neg_m = -ml.x, inv_l = 1.0f / ml.y;
+  const float* col = score + ((size_t)h * max_deciders + d0) * vis_stride + jj;
+  float x[kImpBlockDeciders], acc = 0.f;                        // (all loads in flight; the sum runs in ascending order)
 #pragma unroll
-      for (int u = 0; u < 16; ++u) if (u0 + u < nd) x[u] = col[(size_t)(u0 + u) * vis_stride];
+  for (int u = 0; u < kImpBlockDeciders; ++u) if (u < nd) x[u] = col[(size_t)u * vis_stride];
 #pragma unroll
-      for (int u = 0; u < 16; ++u)
-        if (u0 + u < nd)
-          acc = fmaf(exp2f(fmaf(x[u], scale_log2, __shfl_sync(0xffffffffu, neg_m, u0 + u))), __shfl_sync(0xffffffffu, inv_l, u0 + u), acc);
-    }
-  }
+  for (int u = 0; u < kImpBlockDeciders; ++u)
+    if (u < nd)
+      acc = fmaf(exp2f(fmaf(x[u], scale_log2, __shfl_sync(0xffffffffu, neg_m, u))), __shfl_sync(0xffffffffu, inv_l, u), acc);
   part[h][lane] = acc;
   __syncthreads();
   if (h == 0 && j < Vb) {
@@ -371,10 +367,10 @@ int launch_attn_simt(d3tom_ctx* ctx, d3tom_dtype dt, const AttnArgs& a, cudaStre
   return launch_simt_t<__nv_bfloat16>(ctx, a, s);
 }
 
-int launch_importance_finish(d3tom_ctx* ctx, const AttnArgs& a, int max_visual, float* importance,
+int launch_importance_finish(d3tom_ctx* ctx, const AttnArgs& a, int n_deciders, int max_visual, float* importance,
                              const int32_t* cu_vis, cudaStream_t s) {
   if (max_visual <= 0) return D3TOM_OK;
-  if (a.H <= kImpBlockHeads) {
+  if (a.H <= kImpBlockHeads && n_deciders <= kImpBlockDeciders) {
     D3TOM_CUDA_TRY(ctx, launch_serialized(importance_finish_block_kernel, dim3(ceil_div(max_visual, 32), a.B), a.H * 32, 0, s,
                                           a.score_scratch, a.lse_scratch, a.n_visual, a.cu_deciders, cu_vis, a.max_deciders,
                                           a.vis_stride, a.scale_log2, a.H, importance));

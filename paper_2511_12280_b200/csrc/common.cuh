@@ -179,7 +179,7 @@ int launch_attn_tc(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s);
 int launch_attn_short(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s);   // short calls: a query tile per SM, QK^T ahead
 int launch_attn_sk(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s);      // one request, work balanced over the SMs
 int launch_attn_one(d3tom_ctx* ctx, const AttnArgs& a, cudaStream_t s);     // one query tile per CTA, three score buffers
-int launch_importance_finish(d3tom_ctx* ctx, const AttnArgs& a, int max_visual, float* importance,
+int launch_importance_finish(d3tom_ctx* ctx, const AttnArgs& a, int n_deciders, int max_visual, float* importance,
                              const int32_t* cu_vis, cudaStream_t s);
 int launch_select(d3tom_ctx* ctx, const float* importance, const int32_t* cu_vis, const int32_t* keep_count,
                   const int32_t* cu_kept, int B, int max_visual, int32_t* kept_idx, uint8_t* keep_mask,

@@ -127,7 +127,7 @@ extern "C" int d3tom_attn_importance_static(d3tom_dtype dt, int heads, int head_
   a.dev_status = c.dev_status;
   st = dt == D3TOM_BF16 ? launch_attn_tc(&c, a, s) : launch_attn_simt(&c, dt, a, s);
   if (st != D3TOM_OK) return st;
-  st = launch_importance_finish(&c, a, max_visual, importance, cu_vis, s);
+  st = launch_importance_finish(&c, a, n_deciders_total, max_visual, importance, cu_vis, s);
   if (st != D3TOM_OK) return st;
   if (device_status_out != nullptr &&
       cudaMemcpyAsync(device_status_out, c.dev_status, sizeof(int), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
