@@ -290,7 +290,10 @@ def test_select_digits_from_the_range_of_the_keys(V):
     wide[rng.integers(0, V)] = -0.0
     spread = np.exp(rng.uniform(-80, 80, V)) * rng.choice([-1.0, 1.0], V)
     two = np.where(np.arange(V) % 5 == 0, 1.0, -1.0)
-    for x in (wide, spread, two, 1.75 + np.arange(V) * 2.0 ** -12):
+    # a range of 31 bits that only the last digit (9 bits, under a prefix) resolves, and the same with many equal scores
+    last = np.where(np.arange(V) % 3 == 0, 0.0, 3.0 + rng.integers(0, 4096, V) * 2.0 ** -22)
+    few = np.where(np.arange(V) % 3 == 0, 0.0, 3.0 + rng.integers(0, 4, V) * 2.0 ** -22)
+    for x in (wide, spread, two, 1.75 + np.arange(V) * 2.0 ** -12, last, few):
         for k in {0, 1, V // 3, max(V - 1, 0), V}:
             run_select([x, x[::-1].copy()], [k, V - k])
 
