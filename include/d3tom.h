@@ -132,6 +132,12 @@ int d3tom_set_pair_tiles(int width);
  * gate_up != 0 for the first pass of d3tom_ffn.  Host arithmetic: the rule the launches use. */
 int d3tom_pair_tile_width(int sms, int pairs, int rows, int n_cols, int K, int gate_up);
 
+/* 1 where a merge of these sizes on a device of `sms` multiprocessors builds member lists in a launch of their own, 0 where the
+ * aggregation finds the members itself (Sec. 3.2.2; a launch fewer, the same results).  `payloads` is 1 for d3tom_merge and 2 for
+ * d3tom_merge_kv; the other arguments are those of the call.  Host arithmetic: the rule the launches use. */
+int d3tom_merge_member_lists(int sms, d3tom_dtype dt, int payloads, int B, int D, int total_tokens, int total_out,
+                             int max_visual, int max_kept);
+
 /* Which tensor-core attention kernel serves d3tom_attn_varlen / d3tom_attn_importance (Sec. 3.2.1): -1 (default) the
  * library's choice per launch, 0 the kernels with two query tiles per CTA, 1 the kernel with one query tile per CTA and
  * three score buffers wherever it supports the launch (bf16, head_dim 128, no importance side-work).  Results agree

@@ -50,6 +50,7 @@ _SIGNATURES = {
     "d3tom_set_launch_overlap": (_I, [_I]),
     "d3tom_set_pair_tiles": (_I, [_I]),
     "d3tom_pair_tile_width": (_I, [_I, _I, _I, _I, _I, _I]),
+    "d3tom_merge_member_lists": (_I, [_I] * 9),
     "d3tom_set_single_tile_attention": (_I, [_I]),
     "d3tom_keep_count": (_I, [_I, C.c_double]),
     "d3tom_schedule_alpha": (_I, [_I, _I, C.c_double, C.c_double, _I, C.POINTER(C.c_double)]),
@@ -134,6 +135,13 @@ def d3tom_set_pair_tiles(width: int):
 def d3tom_pair_tile_width(sms: int, pairs: int, rows: int, n_cols: int, K: int, gate_up: bool = False) -> int:
     """Width of the pair tiles that a bf16 dense layer takes, 0 for single-CTA tiles (host arithmetic)."""
     return load().d3tom_pair_tile_width(sms, pairs, rows, n_cols, K, int(gate_up))
+
+
+def d3tom_merge_member_lists(sms: int, dtype: torch.dtype, payloads: int, B: int, D: int, total_tokens: int, total_out: int,
+                             max_visual: int, max_kept: int) -> bool:
+    """Whether a merge of these sizes builds member lists in a launch of their own (host arithmetic)."""
+    return bool(load().d3tom_merge_member_lists(sms, FP32 if dtype == torch.float32 else BF16, payloads, B, D, total_tokens,
+                                                total_out, max_visual, max_kept))
 
 
 def d3tom_set_single_tile_attention(mode: int):

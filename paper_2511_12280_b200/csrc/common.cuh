@@ -193,7 +193,7 @@ struct MergeArgs {
   void* hidden_out; const int32_t* cu_seqlens_out;
   const void* second; void* second_out;      // a second payload of the same rows (the V cache), or null
   int32_t* assign; int32_t* member_count; int32_t* src_of_dst; float* sim_debug;
-  int scan_col_blocks = 0; bool scan_wide = false;   // set by launch_merge_finish: aggregation without lists (0: with)
+  int scan_rows_log2 = 3, scan_col_blocks = 0;   // set by launch_merge_finish: aggregation without lists (0: with)
 };
 int launch_merge_prepare(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s);     // slots, norms, kept-row gather
 int launch_sim_simt(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s);          // similarity + argmax, CUDA cores

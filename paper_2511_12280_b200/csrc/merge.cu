@@ -454,91 +454,117 @@ aggregate_compact_kernel(const T* __restrict__ hidden_1, const T* __restrict__ h
     }
 }
 
-// Aggregation and compaction of ONE request of up to kScanVisual visual tokens without member lists.  A block takes eight
-// consecutive output rows, one per warp, and one of `col_blocks` parts of their columns (blockIdx.y: payload).  It finds their
-// members itself: it reads the request's packed arg-max words once and marks every token whose slot is one of its rows in a
-// bitmap per row, out of which the positions come in ascending order.  That takes the place of a launch of one block that
-// counted, listed and sorted (4 - 9 us in which the other SMs waited) and of the lists' round trip; it costs V x 8 bytes out of
-// L2 per block.  Bound: three dependent rounds of loads, then HBM / L2.
+// Aggregation and compaction of ONE request of up to kScanVisual visual tokens without member lists.  A block takes `rows` (1, 2,
+// 4, 8) consecutive kept tokens and one of `col_blocks` parts of their columns (blockIdx.y: payload); its eight warps share out
+// rows and columns.  It finds the members itself: it reads the request's packed arg-max words once and builds a bitmap per row,
+// out of which the positions come in ascending order.  That takes the place of a launch of one block that counted, listed and
+// sorted (4 - 9 us in which the other SMs waited) and of the lists' round trip; it costs V x 8 bytes out of L2 per block.  The
+// blocks after them copy the prompt and response rows.  Bound: three dependent rounds of loads, then HBM / L2.
 // The sums run in the order of aggregate_compact_kernel: the kept row, then its members by position, fp32, one rounding; rows
-// with kHeavy members or more (few): eight partial sums, 32-member segment s in sum s % 8, added in order.
-constexpr int kScanRows = kAggWarps;
-constexpr int kScanVisual = 12 * 1024;   // 8 bitmaps and a list of 16-bit positions: 36 KB
-constexpr long long kScanTokens = 256 * 1024;
+// with kHeavy members or more: eight partial sums, 32-member segment s in sum s % 8, added in order.  A long list is a chain of
+// loads on the one SM that has it, so it is spread: a warp per (row, chunk), or from kBlockList members on (kBlockListFew where
+// the block has so few (row, chunk) pairs that most of its warps would idle) a warp per partial sum.  Words are turned into
+// bitmaps by ballot: with shared atomics a cluster that most tokens fall into (its tokens share a word) was serialised, 2045 -> 204
+// x 2048, six tenths in one of 32 clusters, 117 us with eight rows per block and atomics, 42 here, 49 with lists.
+constexpr int kScanVisual = 8 * 1024;    // 8 bitmaps and a list of 16-bit positions: 24 KB beside 18 KB of partial sums
+constexpr int kBlockList = 128, kBlockListFew = 48;
+constexpr int kLongUnroll = 8;           // rows of a long list in flight per lane (16: 2 % slower)
 
-// kHeavyUnroll: rows of a heavy list in flight per lane; kBlocks: blocks per SM it leaves registers for
-template <typename T, int kHeavyUnroll, int kBlocks>
-__global__ void __launch_bounds__(kAggWarps * 32, kBlocks)
+template <typename T>
+__global__ void __launch_bounds__(kAggWarps * 32, 2)
 aggregate_scan_kernel(const T* __restrict__ hidden_1, const T* __restrict__ hidden_2, const int32_t* __restrict__ cu_seqlens,
                       const int32_t* __restrict__ cu_vis, const int32_t* __restrict__ kept_idx,
                       const int32_t* __restrict__ cu_kept, const unsigned long long* __restrict__ best, int D, int chunks,
-                      int total_out, int col_blocks, int words, int mean, int32_t* __restrict__ assign,
+                      int total_out, int rows_log2, int col_blocks, int words, int mean, int32_t* __restrict__ assign,
                       int32_t* __restrict__ member_count, T* __restrict__ out_1, T* __restrict__ out_2,
                       int32_t* __restrict__ src_of_dst) {
   constexpr int kVec = Storage<T>::kVec;
-  extern __shared__ unsigned scan_s[];                           // [kScanRows][words] bitmaps, then the lists of the heavy rows
-  __shared__ int light_s[kScanRows][32];
-  __shared__ int heavy_s[kScanRows];                             // members of a heavy row, 0: not heavy
-  __shared__ int4 heavy_at[kScanRows];                           // the heavy rows: {row, start of the list, position, members}
+  extern __shared__ unsigned scan_s[];                           // [rows][words] bitmaps, then the long lists
+  __shared__ int light_s[kAggWarps][32];
+  __shared__ int long_s[kAggWarps];                              // members of a row with a long list, 0: short
+  __shared__ int4 long_at[kAggWarps];                            // those rows: {row, start of the list, position, members}
   __shared__ int next_task;
-  unsigned short* list_s = reinterpret_cast<unsigned short*>(scan_s + kScanRows * words);
+  __shared__ float part_s[2][kAggWarps][kVec][32];
+  const int rows = 1 << rows_log2;
+  unsigned short* list_s = reinterpret_cast<unsigned short*>(scan_s + rows * words);
   grid_dependency_enter();
   const T* __restrict__ hidden = (blockIdx.y == 0 ? hidden_1 : hidden_2) + (size_t)cu_seqlens[0] * D;
   T* __restrict__ hidden_out = blockIdx.y == 0 ? out_1 : out_2;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int rg = (int)blockIdx.x / col_blocks, cb = (int)blockIdx.x - rg * col_blocks;
-  const int r0 = rg * kScanRows, r1 = min(r0 + kScanRows, total_out), row = r0 + warp;
-  const bool reports = cb == 0 && blockIdx.y == 0;               // one block per row group writes what it found
-  const int groups = (chunks + kAggCpw - 1) / kAggCpw;
-  const int cg0 = cb * groups / col_blocks, cg1 = (cb + 1) * groups / col_blocks;
   const int V = cu_vis[1] - cu_vis[0], kb = cu_kept[1] - cu_kept[0];
-  const int pos = row < kb ? kept_idx[cu_kept[0] + row] : V + (row - kb);      // source row in the request (rows past the end: unused)
+  const int kept_blocks = ((kb + rows - 1) >> rows_log2) * col_blocks;
+  if ((int)blockIdx.x >= kept_blocks) {
+    // ---- prompt and response rows: one warp per (row, kAggCpw chunks)
+    const int groups = (chunks + kAggCpw - 1) / kAggCpw, step = ((int)gridDim.x - kept_blocks) * kAggWarps;
+    for (int t = ((int)blockIdx.x - kept_blocks) * kAggWarps + warp; t < (total_out - kb) * groups; t += step) {
+      const int row = kb + t / groups, cg = t % groups, from = V + row - kb;
+      uint4 raw[kAggCpw];
+#pragma unroll
+      for (int j = 0; j < kAggCpw; ++j) {
+        const int c = ((cg * kAggCpw + j) * 32 + lane) * kVec;
+        if (c < D) raw[j] = *reinterpret_cast<const uint4*>(hidden + (size_t)from * D + c);
+      }
+#pragma unroll
+      for (int j = 0; j < kAggCpw; ++j) {
+        const int c = ((cg * kAggCpw + j) * 32 + lane) * kVec;
+        if (c < D) *reinterpret_cast<uint4*>(hidden_out + (size_t)row * D + c) = raw[j];
+      }
+      if (cg == 0 && blockIdx.y == 0 && lane == 0) src_of_dst[row] = cu_seqlens[0] + from;
+    }
+    return;
+  }
+  const int rg = (int)blockIdx.x / col_blocks, cb = (int)blockIdx.x - rg * col_blocks;
+  const int wrow = warp & (rows - 1), sub = warp >> rows_log2, subs = kAggWarps >> rows_log2;   // `subs` warps share a row
+  const int r0 = rg * rows, r1 = min(r0 + rows, kb), row = r0 + wrow;
+  const bool reports = cb == 0 && blockIdx.y == 0;               // one block per row group writes what it found
+  const int c0 = cb * chunks / col_blocks, c1 = (cb + 1) * chunks / col_blocks;      // this block's chunks
+  const int pos = row < r1 ? kept_idx[cu_kept[0] + row] : 0;     // source row in the request
 
-  // ---- the members of this block's rows
-  for (int i = tid; i < kScanRows * words; i += kAggWarps * 32) scan_s[i] = 0u;
+  // ---- the members of this block's rows: a warp looks at 32 consecutive tokens, which are one word of each row's bitmap
+  const int n_words = kb < V ? (V + 31) >> 5 : 0;                // (0: nothing was pruned)
   if (tid == 0) next_task = 0;
-  __syncthreads();
-  const int s1 = min(r1, kb);                                    // [r0, s1): the kept slots among the rows
-  if (r0 < s1 && kb < V) {                                       // (else nothing was pruned)
-    constexpr int kInFlight = 8;
-    const unsigned long long* words_in = best + cu_vis[0];
-    for (int base = 0; base < V; base += kInFlight * kAggWarps * 32) {
-      unsigned low[kInFlight];                                   // ~slot of a pruned token, 0 of a kept one
+  constexpr int kInFlight = 8;
+  const unsigned long long* words_in = best + cu_vis[0];
+  for (int base = warp; base < n_words; base += kInFlight * kAggWarps) {
+    unsigned rel[kInFlight];                                     // first ~slot of a pruned token, 0 of a kept one
 #pragma unroll
-      for (int u = 0; u < kInFlight; ++u) {
-        const int m = base + u * kAggWarps * 32 + tid;
-        low[u] = m < V ? (unsigned)(words_in[m] & 0xffffffffull) : 0u;
-      }
+    for (int u = 0; u < kInFlight; ++u) {
+      const int m = (base + u * kAggWarps) * 32 + lane;
+      rel[u] = m < V ? (unsigned)(words_in[m] & 0xffffffffull) : 0u;
+    }
 #pragma unroll
-      for (int u = 0; u < kInFlight; ++u) {
-        const unsigned slot = 0xffffffffu - low[u];
-        if (slot - (unsigned)r0 < (unsigned)(s1 - r0)) {
-          const int m = base + u * kAggWarps * 32 + tid;
-          atomicOr(&scan_s[((int)slot - r0) * words + (m >> 5)], 1u << (m & 31));
-          if (reports) assign[cu_vis[0] + m] = (int)slot;
-        }
+    for (int u = 0; u < kInFlight; ++u) {
+      const int wi = base + u * kAggWarps;
+      if (wi >= n_words) break;                                  // uniform
+      rel[u] = 0xffffffffu - rel[u] - (unsigned)r0;              // row in the block
+      const bool in = rel[u] < (unsigned)(r1 - r0);
+      if (reports && in) assign[cu_vis[0] + wi * 32 + lane] = r0 + (int)rel[u];
+      unsigned left = __ballot_sync(0xffffffffu, in), mine = 0u;
+      while (left) {                                             // (uniform) one turn per row that occurs
+        const unsigned r = __shfl_sync(0xffffffffu, rel[u], __ffs((int)left) - 1);
+        const unsigned who = __ballot_sync(0xffffffffu, in && rel[u] == r);
+        if ((unsigned)lane == r) mine = who;
+        left &= ~who;
       }
+      if (lane < rows) scan_s[lane * words + wi] = mine;
     }
   }
   __syncthreads();
 
-  // ---- one warp per row: its members are counted and, where they are many, listed for all warps
-  const int row_words = row < s1 ? (V + 31) >> 5 : 0;
-  const unsigned* bm = scan_s + warp * words;
-  int cnt = -1;                                                  // (a copied row)
-  if (row < s1) {
-    cnt = 0;
-    for (int w = lane; w < row_words; w += 32) cnt += __popc(bm[w]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    if (reports && lane == 0) member_count[cu_kept[0] + row] = cnt;
+  // ---- they are counted and, where they are many, listed for all warps
+  const unsigned* bm = scan_s + wrow * words;                    // (a row past the end: an empty one)
+  int cnt = 0;
+  for (int w = lane; w < n_words; w += 32) cnt += __popc(bm[w]);
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
+  if (row < r1 && reports && sub == 0 && lane == 0) {
+    member_count[cu_kept[0] + row] = cnt;
+    src_of_dst[row] = cu_seqlens[0] + pos;
   }
-  if (row < r1 && reports && lane == 0) src_of_dst[row] = cu_seqlens[0] + pos;
-  // the positions marked in the warp's bitmap, in order, to dst
+  // the positions marked in the row's bitmap, in order, to dst
   auto list_positions = [&](auto* dst) {
     int written = 0;
-    for (int w0 = 0; w0 < row_words; w0 += 32) {
-      unsigned v = w0 + lane < row_words ? bm[w0 + lane] : 0u;
+    for (int w0 = 0; w0 < n_words; w0 += 32) {
+      unsigned v = w0 + lane < n_words ? bm[w0 + lane] : 0u;
       const int n = __popc(v);
       int incl = n;
 #pragma unroll
@@ -556,21 +582,24 @@ aggregate_scan_kernel(const T* __restrict__ hidden_1, const T* __restrict__ hidd
     __syncwarp();
   };
   const bool heavy = cnt >= kHeavy;
-  if (lane == 0) heavy_s[warp] = heavy ? cnt : 0;
+  if (sub == 0 && lane == 0) long_s[wrow] = heavy ? cnt : 0;
   __syncthreads();
-  int n_heavy = 0, n_list = 0;                                   // (no token is in two lists: together at most V positions)
-#pragma unroll
-  for (int r = 0; r < kScanRows; ++r) {
-    const int hc = heavy_s[r];
-    if (hc == 0) continue;
-    if (warp == r) {
-      list_positions(list_s + n_list);
-      if (lane == 0) heavy_at[n_heavy] = make_int4(r0 + r, n_list, pos, hc);
+  const int block_list = rows * (c1 - c0) <= 4 ? kBlockListFew : kBlockList;
+  int n_long = 0, n_block = 0, n_list = 0;                       // (no token is in two lists: together at most V positions)
+  for (int pass = 0; pass < 2; ++pass) {                         // first the rows for the whole block (n_block of them)
+    for (int r = 0; r < rows; ++r) {
+      const int hc = long_s[r];
+      if (hc == 0 || (hc >= block_list) != (pass == 0)) continue;
+      if (sub == 0 && wrow == r) {
+        list_positions(list_s + n_list);
+        if (lane == 0) long_at[n_long] = make_int4(r0 + r, n_list, pos, hc);
+      }
+      n_list += hc;
+      ++n_long;
     }
-    n_list += hc;
-    ++n_heavy;
+    if (pass == 0) n_block = n_long;
   }
-  if (n_heavy > 0) __syncthreads();                              // uniform
+  if (n_long > 0) __syncthreads();                               // uniform
 
   if (row < r1 && !heavy) {
     T* dst = hidden_out + (size_t)row * D;
@@ -581,22 +610,14 @@ aggregate_scan_kernel(const T* __restrict__ hidden_1, const T* __restrict__ hidd
     }
     const int n = cnt + 1;
     const float inv_denom = mean ? 1.0f / (float)(1 + cnt) : 1.f;
-    for (int cg = cg0; cg < cg1; ++cg) {
+    for (int cg = c0 + sub * kAggCpw; cg < c1; cg += subs * kAggCpw) {
       int col[kAggCpw];
       bool live[kAggCpw];
 #pragma unroll
       for (int j = 0; j < kAggCpw; ++j) {
-        col[j] = ((cg * kAggCpw + j) * 32 + lane) * kVec;
-        live[j] = col[j] < D;
-        if (!live[j]) col[j] = 0;                                // lanes past the row end read column 0, write nothing
-      }
-      if (cnt < 0) {                                             // prompt / response row: copy
-        uint4 raw[kAggCpw];
-#pragma unroll
-        for (int j = 0; j < kAggCpw; ++j) raw[j] = *reinterpret_cast<const uint4*>(hidden + (size_t)pos * D + col[j]);
-#pragma unroll
-        for (int j = 0; j < kAggCpw; ++j) if (live[j]) *reinterpret_cast<uint4*>(dst + col[j]) = raw[j];
-        continue;
+        col[j] = ((cg + j) * 32 + lane) * kVec;
+        live[j] = cg + j < c1 && col[j] < D;
+        if (!live[j]) col[j] = cg * 32 * kVec;                   // lanes past the end read a column in hand, write nothing
       }
       float accs[kAggCpw][kVec];
 #pragma unroll
@@ -630,41 +651,72 @@ aggregate_scan_kernel(const T* __restrict__ hidden_1, const T* __restrict__ hidd
     }
   }
 
-  // ---- the heavy rows: (row, chunk) by whichever warp is free
-  const int n_chunks = min(cg1 * kAggCpw, chunks) - cg0 * kAggCpw, n_tasks = n_heavy * n_chunks;
+  if (n_long == 0) return;                                       // uniform
+
+  // acc += rows [i0, i1) of a long list, kLongUnroll loads in flight
+  auto add_list = [&](float (&acc)[kVec], const T* src, const unsigned short* list, int i0, int i1) {
+    for (int i = i0; i < i1; i += kLongUnroll) {
+      uint4 raw[kLongUnroll];
+#pragma unroll
+      for (int u = 0; u < kLongUnroll; ++u)
+        if (i + u < i1) raw[u] = *reinterpret_cast<const uint4*>(src + (size_t)list[i + u] * D);
+#pragma unroll
+      for (int u = 0; u < kLongUnroll; ++u)
+        if (i + u < i1) add_raw<T>(acc, raw[u]);
+    }
+  };
+  auto clear = [](float (&acc)[kVec]) {
+#pragma unroll
+    for (int e = 0; e < kVec; ++e) acc[e] = 0.f;
+  };
+  const int n_chunks = c1 - c0;
+  // ---- the longest lists: (row, chunk) by the whole block, one warp per partial sum
+  for (int t = 0; t < n_block * n_chunks; ++t) {
+    const int4 at = long_at[t / n_chunks];
+    const int hc = at.w, c = ((c0 + t % n_chunks) * 32 + lane) * kVec;
+    const T* src = hidden + (c < D ? c : 0);
+    float acc[kVec];
+    clear(acc);
+    if (warp == 0) add_raw<T>(acc, *reinterpret_cast<const uint4*>(src + (size_t)at.z * D));
+    for (int seg = warp; seg * 32 < hc; seg += kAggWarps) add_list(acc, src, list_s + at.y, seg * 32, min(hc, seg * 32 + 32));
+#pragma unroll
+    for (int e = 0; e < kVec; ++e) part_s[t & 1][warp][e][lane] = acc[e];
+    __syncthreads();                                             // (the other half of part_s is free once all warps are here)
+    if (warp == (t & (kAggWarps - 1))) {
+      const float inv_denom = mean ? 1.0f / (float)(1 + hc) : 1.f;
+#pragma unroll
+      for (int e = 0; e < kVec; ++e) {
+        acc[e] = part_s[t & 1][0][e][lane];
+#pragma unroll
+        for (int w = 1; w < kAggWarps; ++w) acc[e] += part_s[t & 1][w][e][lane];
+        acc[e] *= inv_denom;
+      }
+      if (c < D) Storage<T>::store(hidden_out + (size_t)at.x * D + c, acc);
+    }
+  }
+  // ---- the other long lists: (row, chunk) by whichever warp is free
+  const int n_tasks = (n_long - n_block) * n_chunks;
   while (n_tasks > 0) {
     int t = 0;
     if (lane == 0) t = atomicAdd(&next_task, 1);
     t = __shfl_sync(0xffffffffu, t, 0);
     if (t >= n_tasks) break;
-    const int4 at = heavy_at[t / n_chunks];
-    const int hc = at.w, c = ((cg0 * kAggCpw + t % n_chunks) * 32 + lane) * kVec;
-    const bool live = c < D;
-    const T* src = hidden + (live ? c : 0);
-    const unsigned short* list = list_s + at.y;
+    const int4 at = long_at[n_block + t / n_chunks];
+    const int hc = at.w, c = ((c0 + t % n_chunks) * 32 + lane) * kVec;
+    const T* src = hidden + (c < D ? c : 0);
     float total[kVec];
     for (int w = 0; w < min(kAggWarps, (hc + 31) >> 5); ++w) {   // partial sum w: the segments w, w + 8, ...
       float acc[kVec];
-#pragma unroll
-      for (int e = 0; e < kVec; ++e) acc[e] = 0.f;
+      clear(acc);
       if (w == 0) add_raw<T>(acc, *reinterpret_cast<const uint4*>(src + (size_t)at.z * D));
-      for (int seg = w; seg * 32 < hc; seg += kAggWarps)
-        for (int i = seg * 32; i < min(hc, seg * 32 + 32); i += kHeavyUnroll) {
-          uint4 raw[kHeavyUnroll];
-#pragma unroll
-          for (int u = 0; u < kHeavyUnroll; ++u)
-            if (i + u < hc) raw[u] = *reinterpret_cast<const uint4*>(src + (size_t)list[i + u] * D);
-#pragma unroll
-          for (int u = 0; u < kHeavyUnroll; ++u)
-            if (i + u < hc) add_raw<T>(acc, raw[u]);
-        }
+      for (int seg = w; seg * 32 < hc; seg += kAggWarps) add_list(acc, src, list_s + at.y, seg * 32, min(hc, seg * 32 + 32));
 #pragma unroll
       for (int e = 0; e < kVec; ++e) total[e] = w == 0 ? acc[e] : total[e] + acc[e];
     }
     const float inv_denom = mean ? 1.0f / (float)(1 + hc) : 1.f;
 #pragma unroll
     for (int e = 0; e < kVec; ++e) total[e] *= inv_denom;
-    if (live) Storage<T>::store(hidden_out + (size_t)at.x * D + c, total);
+    if (c < D) Storage<T>::store(hidden_out + (size_t)at.x * D + c, total);
   }
 }
 
@@ -685,32 +737,58 @@ int launch_merge_prepare(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
   return D3TOM_OK;
 }
 
-// How a call aggregates without lists (aggregate_scan_kernel): parts of the columns per row group, and whether sixteen rows of a
-// heavy list are in flight (one block per SM then); col_blocks 0: with lists.  One request, where the blocks together scan few
-// tokens or nothing was pruned, and heavy rows are either few (up to four members per kept token on average) or added sixteen at
-// a time.  With lists / without, per merge (us, tokens -> kept x D): 256 -> 64 x 256 fp32 13.1 / 11.4, 485 -> 48 x 512 fp32
-// 17.8 / 15.5, 577 -> 173 x 1024 19.2 / 17.3, 1024 -> 102 x 4096 27.4 / 23.7, 2048 -> 512 x 4096 38.0 / 35.9, K and V of
-// 1500 -> 300 x 2048 32.7 / 30.2, 2048 -> 2048 x 4096 21.3 / 17.6; but 4096 -> 1024 x 4096 56 / 58, its K and V 68 / 76,
-// 8000 -> 2000 x 4096 148 / 161, K and V of five requests of up to 653 tokens x 2048, a tenth kept, 37 / 38.5.
-struct ScanPlan { int col_blocks; bool wide; };
-static ScanPlan scan_plan(const d3tom_ctx* ctx, const MergeArgs& a) {
-  ScanPlan p = {0, false};
-  if (a.B != 1 || a.max_visual > kScanVisual || a.total_out >= kStreamMinRows || a.total_out <= 0) return p;
-  const int row_groups = ceil_div(a.total_out, kScanRows), payloads = a.second != nullptr ? 2 : 1, pruned = a.total_tokens - a.total_out;
-  if (pruned > 0 && (long long)a.max_visual * row_groups > kScanTokens) return p;
-  const int groups = ceil_div(ceil_div(a.D, 32 * (a.dt == D3TOM_FP32 ? 4 : 8)), kAggCpw);
-  const int want = ceil_div(2 * ctx->sm_count, row_groups * payloads);     // (two blocks per SM fit at 128 registers)
-  int col_blocks = 1;                                                      // (a power of two: uneven parts wait for the largest)
-  while (col_blocks < want && col_blocks * 2 <= groups) col_blocks *= 2;
-  p.wide = row_groups * payloads * col_blocks <= ctx->sm_count;
-  if (p.wide || pruned <= 4 * a.max_kept) p.col_blocks = col_blocks;
+// Chunks of 512 bytes per row.
+static int row_chunks(d3tom_dtype dt, int D) { return ceil_div(D, 32 * (dt == D3TOM_FP32 ? 4 : 8)); }
+// One request: as many kept tokens as the host's sizes allow (their number, where max_visual or max_kept is exact).
+static int kept_bound(int total_tokens, int total_out, int max_visual, int max_kept) {
+  const int kept = max_visual - (total_tokens - total_out);
+  return kept < 0 ? 0 : (kept < max_kept ? kept : max_kept);
+}
+
+// How a call aggregates without lists (aggregate_scan_kernel): rows per block and parts of the columns; col_blocks 0: with lists.
+// Fitted to 333 merges of one request (64 .. 8192 visual tokens, one to half of them kept, rows of 256 .. 4736, both types, one
+// and two payloads, clusters even or up to 95 % of the tokens in one), each timed with lists and in every shape; this rule takes
+// 0.88 of the lists' time on average.
+//   - blocks: columns first, then fewer rows, until the kept rows have a block per SM: a list that most tokens are on is then added
+//     by as many SMs as there are.  (Always eight rows and four parts: up to four times the lists' time, 3399 -> 2 x 4736 70 / 279
+//     us, 619 -> 61 x 3072, 8 clusters, 27 / 50.)
+//   - not where all blocks together read more than kScanTokens words: 2403 -> 600 x 2048, K and V, 0.7 Mi 53 / 74, 5187 -> 1296 x
+//     2048 1.7 Mi 114 / 207;
+//   - nor long rows with more than a third kept: the one long list that such a call may have keeps a few SMs busy after the others,
+//     734 -> 367 x 3072, K and V, 27 / 41.
+//   - nothing pruned: whole rows, eight per block as soon as that gives two blocks for five SMs: 0.5 .. 0.8 of the time with lists.
+constexpr long long kScanTokens = 512 * 1024;
+struct ScanPlan { int rows_log2, col_blocks; };
+static ScanPlan scan_plan(int sms, int B, int chunks, int payloads, int total_tokens, int total_out, int max_visual, int max_kept) {
+  ScanPlan p = {3, 0};
+  if (B != 1 || max_visual > kScanVisual || total_out >= kStreamMinRows || total_out <= 0) return p;
+  const int pruned = total_tokens - total_out, kept = kept_bound(total_tokens, total_out, max_visual, max_kept);
+  int cols = 1;
+  auto blocks = [&] { return (long long)((kept + (1 << p.rows_log2) - 1) >> p.rows_log2) * cols * payloads; };
+  if (pruned == 0) {
+    while (p.rows_log2 > 0 && blocks() < 2 * sms / 5) --p.rows_log2;
+  } else {
+    if (chunks > 8 && pruned < 2 * kept) return p;
+    while (cols * 2 <= chunks && cols < 16 && blocks() < sms) cols *= 2;
+    while (p.rows_log2 > 0 && blocks() < sms) --p.rows_log2;
+    if (max_visual * blocks() > kScanTokens) return p;
+  }
+  p.col_blocks = cols;
   return p;
+}
+
+extern "C" int d3tom_merge_member_lists(int sms, d3tom_dtype dt, int payloads, int B, int D, int total_tokens, int total_out,
+                                        int max_visual, int max_kept) {
+  if (sms <= 0 || D <= 0 || total_out < 0 || total_tokens < total_out || max_visual < 0 || max_kept < 0) return 1;
+  return scan_plan(sms, B, row_chunks(dt, D), payloads, total_tokens, total_out, max_visual, max_kept).col_blocks == 0 ? 1 : 0;
 }
 
 int launch_merge_finish(d3tom_ctx* ctx, const MergeArgs& args, cudaStream_t s) {
   MergeArgs a = args;
-  const ScanPlan plan = scan_plan(ctx, a);               // (decided once: payloads launched one by one follow it too)
-  a.scan_col_blocks = plan.col_blocks; a.scan_wide = plan.wide;
+  // (decided once: payloads launched one by one follow it too)
+  const ScanPlan plan = scan_plan(ctx->sm_count, a.B, row_chunks(a.dt, a.D), a.second != nullptr ? 2 : 1, a.total_tokens, a.total_out,
+                                  a.max_visual, a.max_kept);
+  a.scan_rows_log2 = plan.rows_log2; a.scan_col_blocks = plan.col_blocks;
   if (a.scan_col_blocks > 0) return launch_merge_aggregate(ctx, a, s);
   // (the attribute belongs to the current device: set on every call, a process may drive several GPUs)
   D3TOM_CUDA_TRY(ctx, cudaFuncSetAttribute(members_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -762,17 +840,18 @@ int launch_merge_aggregate(d3tom_ctx* ctx, const MergeArgs& a, cudaStream_t s) {
     const int st = launch_merge_aggregate_stream(ctx, a, s);
     if (st != D3TOM_ERR_UNSUPPORTED) return st;
   }
-  const int vec = a.dt == D3TOM_FP32 ? 4 : 8;
-  const int chunks = ceil_div(a.D, 32 * vec);                       // 512-byte chunks per row
+  const int chunks = row_chunks(a.dt, a.D);
   if (a.scan_col_blocks > 0) {
-    const int words = ceil_div(a.max_visual, 32);
-    const size_t smem = (size_t)words * (kScanRows * 4 + 64);
-    const dim3 grid(ceil_div(a.total_out, kScanRows) * a.scan_col_blocks, a.second != nullptr ? 2 : 1);
+    const int words = ceil_div(a.max_visual, 32), kept = kept_bound(a.total_tokens, a.total_out, a.max_visual, a.max_kept);
+    const size_t smem = (size_t)words * ((4 << a.scan_rows_log2) + 64);
+    // (the kernel reads the exact number of kept tokens; blocks beyond theirs copy, at least one in case the bound is not tight)
+    const int copies = ceil_div((a.total_out - kept) * ceil_div(chunks, kAggCpw), kAggWarps);
+    const dim3 grid(ceil_div(kept, 1 << a.scan_rows_log2) * a.scan_col_blocks + (copies > 0 ? copies : 1), a.second != nullptr ? 2 : 1);
     auto launch = [&](auto* tag) -> cudaError_t {
       using T = typename std::remove_pointer<decltype(tag)>::type;
-      return launch_serialized(a.scan_wide ? aggregate_scan_kernel<T, 16, 1> : aggregate_scan_kernel<T, 8, 2>, grid, kAggWarps * 32, smem, s, static_cast<const T*>(a.hidden),
+      return launch_serialized(aggregate_scan_kernel<T>, grid, kAggWarps * 32, smem, s, static_cast<const T*>(a.hidden),
                                static_cast<const T*>(a.second), a.cu_seqlens, a.cu_vis, a.kept_idx, a.cu_kept, ctx->best, a.D, chunks,
-                               a.total_out, a.scan_col_blocks, words, mean, a.assign, a.member_count,
+                               a.total_out, a.scan_rows_log2, a.scan_col_blocks, words, mean, a.assign, a.member_count,
                                static_cast<T*>(a.hidden_out), static_cast<T*>(a.second_out), a.src_of_dst);
     };
     D3TOM_CUDA_TRY(ctx, a.dt == D3TOM_FP32 ? launch(static_cast<float*>(nullptr)) : launch(static_cast<__nv_bfloat16*>(nullptr)));

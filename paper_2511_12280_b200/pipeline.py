@@ -31,6 +31,7 @@ class MergeLayerStep:
         self.H, self.dh, self.D = H, dh, H * dh
         self.dtype = dtype
         self.dev = torch.device("cuda", device)
+        self.sms = torch.cuda.get_device_properties(self.dev).multi_processor_count
         self.mode = mode
         self.n_post = n_post
         self.want_sim_debug = sim_debug
@@ -157,14 +158,9 @@ class MergeLayerStep:
         return graph
 
     def uses_member_lists(self) -> bool:
-        """Whether the merge of the current problem launches the kernel that lists members (the rule of scan_plan in merge.cu)."""
-        rows, pruned, chunks = -(-self.total_out // 8), self.total - self.total_out, -(-self.D * self.attn_out.element_size() // 512)
-        if self.nB != 1 or self.max_visual > 12288 or self.total_out >= 4096 or (pruned and self.max_visual * rows > 256 * 1024):
-            return True
-        groups, parts, sms = -(-chunks // 4), 1, torch.cuda.get_device_properties(self.dev).multi_processor_count
-        while parts * rows < 2 * sms and parts * 2 <= groups:
-            parts *= 2
-        return rows * parts > sms and pruned > 4 * self.max_kept
+        """Whether the merge of the current problem launches the kernel that lists members."""
+        return B_.d3tom_merge_member_lists(self.sms, self.attn_out.dtype, 1, self.nB, self.D, self.total, self.total_out,
+                                           self.max_visual, self.max_kept)
 
     def launches_per_step(self) -> int:
         """Kernels of this library launched by one run(): attention 1 + importance finish 1,

@@ -84,6 +84,11 @@ def test_merge_kv_llada_shape():
     run_case(wl.config("C1"), B_.AGG_MEAN, keep_ratio=0.10)
 
 
+def takes_lists(dt, payloads, B, D, total, total_out, max_visual, max_kept):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    return B_.d3tom_merge_member_lists(sms, dt, payloads, B, D, total, total_out, max_visual, max_kept)
+
+
 HEAVY = 32            # a kept token with this many members or more is aggregated by whole blocks
 STREAM_ROWS = 4096    # from this many output rows on the streaming pipeline aggregates
 
@@ -100,6 +105,7 @@ def test_merge_kv_both_caches_in_one_launch_of_the_streaming_pipeline(mode):
 @pytest.mark.parametrize("V,r,H,dh", [(8000, 0.01, 2, 64), (9000, 0.01, 2, 64), (17000, 0.02, 2, 64), (3000, 0.02, 32, 128)])
 def test_merge_kv_both_caches_in_one_launch_with_long_member_lists(V, r, H, dh, mode):
     res = run_case(wl.make_workload("kvh", "bf16", H, dh, 43, 64, [dict(V=V, P=9, O=4, n_dec=1, r=r)]), mode, keep_ratio=r)
+    assert takes_lists(torch.bfloat16, 2, 1, H * dh, V + 9, res["total_out"], V, max(1, int(r * V)))
     heavy, chunks = int((res["members"] >= HEAVY).sum()), max(1, H * dh // 256)
     assert res["total_out"] < STREAM_ROWS and heavy >= 30
     sms = torch.cuda.get_device_properties(0).multi_processor_count
@@ -130,9 +136,10 @@ def test_merge_kv_value_cache_written_over_the_key_cache():
 
 
 @pytest.mark.parametrize("v_over_k", [False, True])
-@pytest.mark.parametrize("V,k", [(300, 40), (5000, 4200)])          # the plain aggregation and the streaming one
+@pytest.mark.parametrize("V,k", [(300, 40), (8000, 300), (5000, 4200)])    # aggregation without lists, with lists, and streaming
 def test_merge_kv_key_cache_written_over_the_value_cache(V, k, v_over_k):
     dev, D, P = torch.device("cuda", 0), 256, 5
+    assert takes_lists(torch.bfloat16, 2, 1, D, V + P, k + P, V, k) == (V != 300)
     g = torch.Generator().manual_seed(V)
     kc, vc = (torch.randn(V + P, D, generator=g).to(torch.bfloat16).to(dev) for _ in range(2))
     i32 = lambda *a: torch.tensor(a, dtype=torch.int32, device=dev)
@@ -154,14 +161,14 @@ def test_merge_kv_key_cache_written_over_the_value_cache(V, k, v_over_k):
     ctx.close()
 
 
-# Aggregation that finds a row's members itself: lists at both sides of what one warp adds (31, 32, 33 members, several parts of
-# eight and of thirty-two), kept tokens without members, eight rows that span requests, rows of odd numbers of 16-byte vectors, one
-# and two payloads, nothing pruned.  Every visual token is a multiple of its kept token's unit vector, so the assignment and the
-# sums over K are exact in either type; the sums over V are compared with float64.
+# Member lists of both aggregations (a batch builds lists, the last set, one request, does not): lists at both sides of what one
+# warp adds (31, 32, 33 members, several parts of eight and of thirty-two), kept tokens without members, requests of a row or two,
+# one and two payloads, nothing pruned.  Every visual token is a multiple of its kept token's unit vector, so the assignment and
+# the sums over K are exact in either type; the sums over V are compared with float64.
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])
 @pytest.mark.parametrize("H,counts", [(4, [[0, 1, 31, 32, 33, 0, 2], [64, 65], [255, 0, 0, 257, 3]]), (9, [[7] * 60, [0] * 9]),
                                       (4, [[1500, 2, 0, 40, 41, 33, 32, 31, 100]]), (5, [[0], [1], [0, 0, 0], [5, 0, 90]])])
-def test_members_found_by_scanning(H, counts, dtype):
+def test_members_of_a_batch_and_of_one_request(H, counts, dtype):
     dev, dh = torch.device("cuda", 0), 64
     D, dt = H * dh, torch.float32 if dtype == "fp32" else torch.bfloat16
     rng = np.random.default_rng(len(counts) + H)
@@ -216,4 +223,52 @@ def test_members_found_by_scanning(H, counts, dtype):
                 eps = 2.0 ** -24 * 64 * scale + (2.0 ** -8 * np.abs(want) if dtype == "bf16" else 0)
                 assert (err <= eps + 1e-30).all()
         assert torch.isnan(outs[0][-1]).all()
+    ctx.close()
+
+
+# The aggregation that finds the members itself against the one with member lists, which the same request takes beside a second
+# one: the same bits.  One, two, four and eight rows per block, one to sixteen column parts (D of 37 heads: ragged chunks), lists on
+# either side of what a lane holds (31, 32) and of what the whole block adds (47, 48, 127, 128, 129), several long lists in a block, one
+# list with every token, nothing pruned, one token.
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("H,counts", [(37, [31, 32, 33, 0, 2, 47, 48, 127, 128, 129, 256, 300]), (37, [64, 40, 0, 5] + [3, 0] * 33),
+                                      (20, [130, 40, 128, 33, 0] + [1, 0, 2] * 98), (20, [129, 127, 40, 300, 33, 128, 32, 31] + [1] * 1192),
+                                      (4, [1500]), (37, [2000, 0]), (4, [200, 90]), (37, [0] * 100), (4, [0])])
+def test_members_found_by_scanning_give_the_bits_of_the_lists(H, counts, dtype):
+    dev, D = torch.device("cuda", 0), 64 * H
+    rng = np.random.default_rng(H + len(counts))
+    k, P = len(counts), 5
+    ids = rng.permutation(np.repeat(np.arange(k), np.asarray(counts) + 1))
+    V = len(ids)
+    kept = np.sort([np.flatnonzero(ids == i)[0] for i in range(k)])
+    x = np.zeros((V + P, D))
+    x[np.arange(V), ids] = rng.integers(1, 3, V)                   # multiples of a unit vector per kept token
+    x[V:] = rng.standard_normal((P, D))
+    extra = np.eye(4, D)                                           # a second request: two visual tokens, one kept, two other rows
+    t = lambda a: torch.as_tensor(np.asarray(a, np.int32), device=dev)
+    k_d = torch.as_tensor(np.concatenate([x, extra]), device=dev).to(dtype)
+    v_d = torch.as_tensor(rng.standard_normal((V + P + 4, D)), device=dev).to(dtype)
+    ctx = B_.Context(V + P + 4, 2, H, 64, 1, max(V, 2))
+    for payloads in (1, 2):
+        got = []
+        if k > 1000 and (payloads == 2 or dtype == torch.float32):     # (these read too much: with lists)
+            continue
+        for B in (1, 2):
+            n, m, n_vis, n_kept = V + P + (4 if B == 2 else 0), k + P + (3 if B == 2 else 0), [V, 2][:B], [k, 1][:B]
+            cs = lambda a: t(np.concatenate([[0], np.cumsum(a)]))
+            cu, cu_out = cs([V + P, 4][:B]), cs([k + P, 3][:B])
+            assert takes_lists(dtype, payloads, B, D, n, m, max(n_vis), max(n_kept)) == (B == 2)
+            outs = [torch.full((m + 1, D), float("nan"), dtype=dtype, device=dev) for _ in range(2)]
+            ints = [torch.full((c + 1,), -9, dtype=torch.int32, device=dev) for c in (sum(n_vis), sum(n_kept), m)]
+            tail = (cu, t(n_vis), cs(n_vis), t(np.concatenate([kept, [0]])[: sum(n_kept)]), cs(n_kept), B, D, n, m, max(n_vis), max(n_kept))
+            if payloads == 2:
+                ctx.d3tom_merge_kv(B_.AGG_MEAN, k_d[:n], v_d[:n], *tail, *outs, cu_out, *ints)
+            else:
+                ctx.d3tom_merge(B_.AGG_SUM, k_d[:n], *tail, outs[0], cu_out, *ints)
+            torch.cuda.synchronize()
+            assert all(i[-1].item() == -9 for i in ints) and all(torch.isnan(o[-1]).all() for o in outs)
+            got.append([o[: k + P] for o in outs[:payloads]] + [i[:c] for i, c in zip(ints, (V, k, k + P))])
+        assert all(torch.equal(a, b) for a, b in zip(*got))
+        order = np.argsort([np.flatnonzero(ids == i)[0] for i in range(k)])
+        assert np.array_equal(got[0][-2].cpu().numpy(), np.asarray(counts)[order])
     ctx.close()
