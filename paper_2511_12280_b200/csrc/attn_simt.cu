@@ -292,7 +292,10 @@ importance_finish_block_kernel(const float* __restrict__ score, const float2* __
                         const int32_t* __restrict__ cu_vis, int max_deciders, int vis_stride, float scale_log2, int H,
                         float* __restrict__ importance) {
   __shared__ float part[kImpBlockHeads][32];
-  grid_dependency_enter();
+  grid_dependency_wait();
+  // (a batch keeps the next kernel back until it ends: blocks of an fp32 attention launch that came in beside this kernel's many
+  // small ones piled up on some SMs, eight requests x 1 head x 64 called back to back 150 -> 257 us, 160 so)
+  if (gridDim.y == 1) grid_dependency_release();
   const int b = blockIdx.y, h = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int Vb = n_visual[b], j = blockIdx.x * 32 + lane;
   const int d0 = cu_deciders[b], d1 = cu_deciders[b + 1], g0 = cu_vis[b];
