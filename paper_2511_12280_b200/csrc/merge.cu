@@ -463,12 +463,13 @@ aggregate_compact_kernel(const T* __restrict__ hidden_1, const T* __restrict__ h
 // The sums run in the order of aggregate_compact_kernel: the kept row, then its members by position, fp32, one rounding; rows
 // with kHeavy members or more: eight partial sums, 32-member segment s in sum s % 8, added in order.  A long list is a chain of
 // loads on the one SM that has it, so it is spread: a warp per (row, chunk), or from kBlockList members on (kBlockListFew where
-// the block has so few (row, chunk) pairs that most of its warps would idle) a warp per partial sum.  Words are turned into
+// the block has so few (row, chunk) pairs that most of its warps would idle) a warp per partial sum, two chunks at a time (one at a
+// time: 2048 -> 205 x 4096 with six tenths in one cluster 60 us, 53 so).  Words are turned into
 // bitmaps by ballot: with shared atomics a cluster that most tokens fall into (its tokens share a word) was serialised, 2045 -> 204
-// x 2048, six tenths in one of 32 clusters, 117 us with eight rows per block and atomics, 42 here, 49 with lists.
+// x 2048, six tenths in one of 32 clusters, 117 us with eight rows per block and atomics, 42 by ballot, 49 with lists.
 constexpr int kScanVisual = 8 * 1024;    // 8 bitmaps and a list of 16-bit positions: 24 KB beside 18 KB of partial sums
 constexpr int kBlockList = 128, kBlockListFew = 48;
-constexpr int kLongUnroll = 8;           // rows of a long list in flight per lane (16: 2 % slower)
+constexpr int kLongUnroll = 8;           // rows of a long list in flight per lane
 
 template <typename T>
 __global__ void __launch_bounds__(kAggWarps * 32, 2)
@@ -539,13 +540,10 @@ aggregate_scan_kernel(const T* __restrict__ hidden_1, const T* __restrict__ hidd
       rel[u] = 0xffffffffu - rel[u] - (unsigned)r0;              // row in the block
       const bool in = rel[u] < (unsigned)(r1 - r0);
       if (reports && in) assign[cu_vis[0] + wi * 32 + lane] = r0 + (int)rel[u];
-      unsigned left = __ballot_sync(0xffffffffu, in), mine = 0u;
-      while (left) {                                             // (uniform) one turn per row that occurs
-        const unsigned r = __shfl_sync(0xffffffffu, rel[u], __ffs((int)left) - 1);
-        const unsigned who = __ballot_sync(0xffffffffu, in && rel[u] == r);
-        if ((unsigned)lane == r) mine = who;
-        left &= ~who;
-      }
+      // lane r: the tokens whose row has the three bits of r
+      const unsigned b_in = __ballot_sync(0xffffffffu, in), b0 = __ballot_sync(0xffffffffu, rel[u] & 1u),
+                     b1 = __ballot_sync(0xffffffffu, rel[u] & 2u), b2 = __ballot_sync(0xffffffffu, rel[u] & 4u);
+      const unsigned mine = b_in & (lane & 1 ? b0 : ~b0) & (lane & 2 ? b1 : ~b1) & (lane & 4 ? b2 : ~b2);
       if (lane < rows) scan_s[lane * words + wi] = mine;
     }
   }
@@ -670,29 +668,65 @@ aggregate_scan_kernel(const T* __restrict__ hidden_1, const T* __restrict__ hidd
     for (int e = 0; e < kVec; ++e) acc[e] = 0.f;
   };
   const int n_chunks = c1 - c0;
-  // ---- the longest lists: (row, chunk) by the whole block, one warp per partial sum
-  for (int t = 0; t < n_block * n_chunks; ++t) {
-    const int4 at = long_at[t / n_chunks];
-    const int hc = at.w, c = ((c0 + t % n_chunks) * 32 + lane) * kVec;
-    const T* src = hidden + (c < D ? c : 0);
-    float acc[kVec];
-    clear(acc);
-    if (warp == 0) add_raw<T>(acc, *reinterpret_cast<const uint4*>(src + (size_t)at.z * D));
-    for (int seg = warp; seg * 32 < hc; seg += kAggWarps) add_list(acc, src, list_s + at.y, seg * 32, min(hc, seg * 32 + 32));
+  // ---- the longest lists: (row, two chunks) by the whole block, one warp per partial sum
+  const int n_pairs = (n_chunks + 1) >> 1;
+  for (int t = 0; t < n_block * n_pairs; ++t) {
+    const int4 at = long_at[t / n_pairs];
+    const int hc = at.w, cc = c0 + 2 * (t % n_pairs);
+    const bool two = cc + 1 < c1;                                // uniform
+    int c[2];
+    bool live[2];
 #pragma unroll
-    for (int e = 0; e < kVec; ++e) part_s[t & 1][warp][e][lane] = acc[e];
-    __syncthreads();                                             // (the other half of part_s is free once all warps are here)
-    if (warp == (t & (kAggWarps - 1))) {
+    for (int j = 0; j < 2; ++j) {
+      c[j] = ((cc + j) * 32 + lane) * kVec;
+      live[j] = (j == 0 || two) && c[j] < D;
+      if (!live[j]) c[j] = cc * 32 * kVec;
+    }
+    float acc[2][kVec];
+    clear(acc[0]);
+    clear(acc[1]);
+    if (warp == 0) {
+#pragma unroll
+      for (int j = 0; j < 2; ++j) add_raw<T>(acc[j], *reinterpret_cast<const uint4*>(hidden + (size_t)at.z * D + c[j]));
+    }
+    const unsigned short* list = list_s + at.y;
+    for (int seg = warp; seg * 32 < hc; seg += kAggWarps) {
+      const int i1 = min(hc, seg * 32 + 32);
+      for (int i = seg * 32; i < i1; i += kLongUnroll) {
+        uint4 raw[kLongUnroll][2];
+#pragma unroll
+        for (int u = 0; u < kLongUnroll; ++u)
+          if (i + u < i1) {
+            const T* src = hidden + (size_t)list[i + u] * D;
+            raw[u][0] = *reinterpret_cast<const uint4*>(src + c[0]);
+            if (two) raw[u][1] = *reinterpret_cast<const uint4*>(src + c[1]);
+          }
+#pragma unroll
+        for (int u = 0; u < kLongUnroll; ++u)
+          if (i + u < i1) {
+            add_raw<T>(acc[0], raw[u][0]);
+            if (two) add_raw<T>(acc[1], raw[u][1]);
+          }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int e = 0; e < kVec; ++e) part_s[j][warp][e][lane] = acc[j][e];
+    __syncthreads();
+    if (warp < 2 && (warp == 0 ? live[0] : live[1])) {
       const float inv_denom = mean ? 1.0f / (float)(1 + hc) : 1.f;
+      float sum[kVec];
 #pragma unroll
       for (int e = 0; e < kVec; ++e) {
-        acc[e] = part_s[t & 1][0][e][lane];
+        sum[e] = part_s[warp][0][e][lane];
 #pragma unroll
-        for (int w = 1; w < kAggWarps; ++w) acc[e] += part_s[t & 1][w][e][lane];
-        acc[e] *= inv_denom;
+        for (int w = 1; w < kAggWarps; ++w) sum[e] += part_s[warp][w][e][lane];
+        sum[e] *= inv_denom;
       }
-      if (c < D) Storage<T>::store(hidden_out + (size_t)at.x * D + c, acc);
+      Storage<T>::store(hidden_out + (size_t)at.x * D + (warp == 0 ? c[0] : c[1]), sum);
     }
+    __syncthreads();
   }
   // ---- the other long lists: (row, chunk) by whichever warp is free
   const int n_tasks = (n_long - n_block) * n_chunks;
@@ -746,32 +780,35 @@ static int kept_bound(int total_tokens, int total_out, int max_visual, int max_k
 }
 
 // How a call aggregates without lists (aggregate_scan_kernel): rows per block and parts of the columns; col_blocks 0: with lists.
-// Fitted to 333 merges of one request (64 .. 8192 visual tokens, one to half of them kept, rows of 256 .. 4736, both types, one
-// and two payloads, clusters even or up to 95 % of the tokens in one), each timed with lists and in every shape; this rule takes
-// 0.88 of the lists' time on average.
-//   - blocks: columns first, then fewer rows, until the kept rows have a block per SM: a list that most tokens are on is then added
-//     by as many SMs as there are.  (Always eight rows and four parts: up to four times the lists' time, 3399 -> 2 x 4736 70 / 279
-//     us, 619 -> 61 x 3072, 8 clusters, 27 / 50.)
-//   - not where all blocks together read more than kScanTokens words: 2403 -> 600 x 2048, K and V, 0.7 Mi 53 / 74, 5187 -> 1296 x
-//     2048 1.7 Mi 114 / 207;
-//   - nor long rows with more than a third kept: the one long list that such a call may have keeps a few SMs busy after the others,
-//     734 -> 367 x 3072, K and V, 27 / 41.
+// Fitted to merges of one request (64 .. 8192 visual tokens, one to half of them kept, rows of 256 .. 4736, both types, one and
+// two payloads, clusters even or up to 95 % of the tokens in one), each timed with lists and in every shape; over 260 of them this
+// rule takes 0.93 of the lists' time, and more than 1.03 of it four times, 1.12 at worst.
+//   - blocks: columns down to two chunks, then fewer rows, then single chunks, until the kept rows have seven blocks for five SMs: a
+//     list that most tokens are on is then added by as many SMs as there are.  (Always eight rows and four parts: up to four times
+//     the lists' time, 3399 -> 2 x 4736 70 / 279 us, 619 -> 61 x 3072, 8 clusters, 27 / 50.)  1024 -> 102 x 4096 25.1 / 23.6, with half
+//     of the tokens in one cluster 30.6 / 32.3; fewer and larger blocks are up to 1.5 us faster with even clusters and up to 70 slower.
+//   - not where all blocks together read more than kScanTokens words: 2048 -> 512 x 4096 36.8 / 35.7, with 60 % in one cluster 56 /
+//     81; 5187 -> 1296 x 2048 114 / 207;
+//   - nor long rows with a quarter kept and more: the one long list that such a call may have keeps a few SMs busy after the others,
+//     1367 -> 341 x 4096 51 / 72, 734 -> 367 x 3072, K and V, 27 / 41.
 //   - nothing pruned: whole rows, eight per block as soon as that gives two blocks for five SMs: 0.5 .. 0.8 of the time with lists.
-constexpr long long kScanTokens = 512 * 1024;
+constexpr long long kScanTokens = 300 * 1000;
 struct ScanPlan { int rows_log2, col_blocks; };
 static ScanPlan scan_plan(int sms, int B, int chunks, int payloads, int total_tokens, int total_out, int max_visual, int max_kept) {
   ScanPlan p = {3, 0};
   if (B != 1 || max_visual > kScanVisual || total_out >= kStreamMinRows || total_out <= 0) return p;
   const int pruned = total_tokens - total_out, kept = kept_bound(total_tokens, total_out, max_visual, max_kept);
   int cols = 1;
-  auto blocks = [&] { return (long long)((kept + (1 << p.rows_log2) - 1) >> p.rows_log2) * cols * payloads; };
+  auto blocks = [&] { return (long long)((kept + (1 << p.rows_log2) - 1) >> p.rows_log2) * cols; };      // per payload
   if (pruned == 0) {
-    while (p.rows_log2 > 0 && blocks() < 2 * sms / 5) --p.rows_log2;
+    while (p.rows_log2 > 0 && blocks() * payloads < 2 * sms / 5) --p.rows_log2;
   } else {
-    if (chunks > 8 && pruned < 2 * kept) return p;
-    while (cols * 2 <= chunks && cols < 16 && blocks() < sms) cols *= 2;
-    while (p.rows_log2 > 0 && blocks() < sms) --p.rows_log2;
-    if (max_visual * blocks() > kScanTokens) return p;
+    if (chunks > 8 && pruned <= 3 * kept) return p;
+    const int target = 7 * sms / 5, most = chunks < 16 ? chunks : 16;
+    while (cols * 4 <= chunks && cols * 2 <= most && blocks() < target) cols *= 2;
+    while (p.rows_log2 > 0 && blocks() < target) --p.rows_log2;
+    while (cols * 2 <= most && blocks() < target) cols *= 2;
+    if (max_visual * blocks() * payloads > kScanTokens) return p;
   }
   p.col_blocks = cols;
   return p;

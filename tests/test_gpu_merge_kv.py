@@ -231,8 +231,9 @@ def test_members_of_a_batch_and_of_one_request(H, counts, dtype):
 # either side of what a lane holds (31, 32) and of what the whole block adds (47, 48, 127, 128, 129), several long lists in a block, one
 # list with every token, nothing pruned, one token.
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
-@pytest.mark.parametrize("H,counts", [(37, [31, 32, 33, 0, 2, 47, 48, 127, 128, 129, 256, 300]), (37, [64, 40, 0, 5] + [3, 0] * 33),
-                                      (20, [130, 40, 128, 33, 0] + [1, 0, 2] * 98), (20, [129, 127, 40, 300, 33, 128, 32, 31] + [1] * 1192),
+@pytest.mark.parametrize("H,counts", [(37, [31, 32, 33, 0, 2, 47, 48, 127, 128, 129, 256, 300]), (37, [64, 40, 0, 5] + [4, 0] * 33),
+                                      (64, [300, 60, 130] + [5] * 99), (20, [130, 40, 128, 33, 0] + [1] * 294),
+                                      (16, [129, 127, 40, 33] + [0] * 828), (4, [129, 127, 40, 30, 33, 128, 32, 31] + [0, 1] * 100),
                                       (4, [1500]), (37, [2000, 0]), (4, [200, 90]), (37, [0] * 100), (4, [0])])
 def test_members_found_by_scanning_give_the_bits_of_the_lists(H, counts, dtype):
     dev, D = torch.device("cuda", 0), 64 * H
@@ -251,13 +252,13 @@ def test_members_found_by_scanning_give_the_bits_of_the_lists(H, counts, dtype):
     ctx = B_.Context(V + P + 4, 2, H, 64, 1, max(V, 2))
     for payloads in (1, 2):
         got = []
-        if k > 1000 and (payloads == 2 or dtype == torch.float32):     # (these read too much: with lists)
-            continue
+        single_lists = takes_lists(dtype, payloads, 1, D, V + P, k + P, V, k)
+        assert not single_lists or payloads == 2 or dtype == torch.float32
         for B in (1, 2):
             n, m, n_vis, n_kept = V + P + (4 if B == 2 else 0), k + P + (3 if B == 2 else 0), [V, 2][:B], [k, 1][:B]
             cs = lambda a: t(np.concatenate([[0], np.cumsum(a)]))
             cu, cu_out = cs([V + P, 4][:B]), cs([k + P, 3][:B])
-            assert takes_lists(dtype, payloads, B, D, n, m, max(n_vis), max(n_kept)) == (B == 2)
+            assert takes_lists(dtype, payloads, B, D, n, m, max(n_vis), max(n_kept)) == (B == 2 or single_lists)
             outs = [torch.full((m + 1, D), float("nan"), dtype=dtype, device=dev) for _ in range(2)]
             ints = [torch.full((c + 1,), -9, dtype=torch.int32, device=dev) for c in (sum(n_vis), sum(n_kept), m)]
             tail = (cu, t(n_vis), cs(n_vis), t(np.concatenate([kept, [0]])[: sum(n_kept)]), cs(n_kept), B, D, n, m, max(n_vis), max(n_kept))
