@@ -301,17 +301,21 @@ importance_finish_block_kernel(const float* __restrict__ score, const float2* __
   const int d0 = cu_deciders[b], d1 = cu_deciders[b + 1], g0 = cu_vis[b];
   if ((int)blockIdx.x * 32 >= Vb) return;                       // uniform: no key of this request in the range
   const int jj = j < Vb ? j : Vb - 1;                           // lanes past the end read a valid column, write nothing
-  const int nd = d1 - d0;                                       // at most kImpBlockDeciders
-  const float2 ml = lane < nd ? lse[(size_t)h * max_deciders + d0 + lane] : make_float2(0.f, 1.f);
-  const float neg_m = -ml.x, inv_l = 1.0f / ml.y;
-  const float* col = score + ((size_t)h * max_deciders + d0) * vis_stride + jj;
-  float x[kImpBlockDeciders], acc = 0.f;                        // (all loads in flight; the sum runs in ascending order)
+  float acc = 0.f;
+  // (the host's count chose this kernel, the device's list is what is summed: a captured call may be replayed with a longer one)
+  for (int d = d0; d < d1; d += kImpBlockDeciders) {
+    const int nd = min(kImpBlockDeciders, d1 - d);
+    const float2 ml = lane < nd ? lse[(size_t)h * max_deciders + d + lane] : make_float2(0.f, 1.f);
+    const float neg_m = -ml.x, inv_l = 1.0f / ml.y;
+    const float* col = score + ((size_t)h * max_deciders + d) * vis_stride + jj;
+    float x[kImpBlockDeciders];                                 // (all loads in flight; the sum runs in ascending order)
 #pragma unroll
-  for (int u = 0; u < kImpBlockDeciders; ++u) if (u < nd) x[u] = col[(size_t)u * vis_stride];
+    for (int u = 0; u < kImpBlockDeciders; ++u) if (u < nd) x[u] = col[(size_t)u * vis_stride];
 #pragma unroll
-  for (int u = 0; u < kImpBlockDeciders; ++u)
-    if (u < nd)
-      acc = fmaf(exp2f(fmaf(x[u], scale_log2, __shfl_sync(0xffffffffu, neg_m, u))), __shfl_sync(0xffffffffu, inv_l, u), acc);
+    for (int u = 0; u < kImpBlockDeciders; ++u)
+      if (u < nd)
+        acc = fmaf(exp2f(fmaf(x[u], scale_log2, __shfl_sync(0xffffffffu, neg_m, u))), __shfl_sync(0xffffffffu, inv_l, u), acc);
+  }
   part[h][lane] = acc;
   __syncthreads();
   if (h == 0 && j < Vb) {

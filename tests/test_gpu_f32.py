@@ -318,3 +318,29 @@ def test_importance_of_few_heads(H, V, n_dec):
     # every term is a probability with an fp32 relative error of about 1e-5 (scores of magnitude 10 in the exponent)
     assert imp[-1].item() == -7.0 and ((imp[:-1].double() - want).abs() <= 1e-4 * want + 1e-7 * n_dec * H).all()
     ctx.close()
+
+
+def test_importance_of_a_replay_with_more_deciders_than_were_captured():
+    # the host's count is that of the capture; what is summed is the device's list, whichever kernel sums it
+    dev, H, dh, V, n = torch.device("cuda", 0), 2, 32, 70, 90
+    g = torch.Generator().manual_seed(5)
+    q, k, v = (torch.randn(n, H * dh, generator=g).to(dev) for _ in range(3))
+    i32 = lambda *a: torch.tensor(a, dtype=torch.int32, device=dev)
+    pos, cu_dec, imp, out = torch.arange(V, V + 17, dtype=torch.int32, device=dev), i32(0, 8), torch.zeros(V, device=dev), torch.empty_like(q)
+    ctx = B_.Context(n, 1, H, dh, 17, V)
+    cu, nv, cu_vis = i32(0, n), i32(V), i32(0, V)
+    call = lambda n_dec: ctx.d3tom_attn_importance(q, k, v, cu, nv, pos, cu_dec, 1, n, n, V, n_dec, dh ** -0.5, out, imp, cu_vis)
+    call(8)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call(8)
+    for n_dec in (8, 9, 17):
+        cu_dec.copy_(i32(0, n_dec))
+        graph.replay()
+        torch.cuda.synchronize()
+        got = imp.clone()
+        call(17)                                   # the kernel for longer lists
+        torch.cuda.synchronize()
+        assert (got - imp).abs().max() <= 1e-6 * n_dec * H     # probabilities, summed in another order
+    ctx.close()
