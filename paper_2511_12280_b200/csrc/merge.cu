@@ -608,47 +608,55 @@ aggregate_scan_kernel(const T* __restrict__ hidden_1, const T* __restrict__ hidd
     }
     const int n = cnt + 1;
     const float inv_denom = mean ? 1.0f / (float)(1 + cnt) : 1.f;
-    for (int cg = c0 + sub * kAggCpw; cg < c1; cg += subs * kAggCpw) {
-      int col[kAggCpw];
-      bool live[kAggCpw];
+    // kCpw chunks of the row from chunk cg on, kUnroll rows in flight
+    auto add_light = [&](int cg, auto chunks_at_once, auto rows_at_once) {
+      constexpr int kCpw = decltype(chunks_at_once)::value, kUnroll = decltype(rows_at_once)::value;
+      int col[kCpw];
+      bool live[kCpw];
 #pragma unroll
-      for (int j = 0; j < kAggCpw; ++j) {
+      for (int j = 0; j < kCpw; ++j) {
         col[j] = ((cg + j) * 32 + lane) * kVec;
         live[j] = cg + j < c1 && col[j] < D;
         if (!live[j]) col[j] = cg * 32 * kVec;                   // lanes past the end read a column in hand, write nothing
       }
-      float accs[kAggCpw][kVec];
+      float accs[kCpw][kVec];
 #pragma unroll
-      for (int j = 0; j < kAggCpw; ++j)
+      for (int j = 0; j < kCpw; ++j)
 #pragma unroll
         for (int e = 0; e < kVec; ++e) accs[j][e] = 0.f;
-      for (int i = 0; i < n; i += kAggUnroll) {                  // kAggUnroll rows x kAggCpw chunks in flight
-        uint4 raw[kAggUnroll][kAggCpw];
+      for (int i = 0; i < n; i += kUnroll) {
+        uint4 raw[kUnroll][kCpw];
 #pragma unroll
-        for (int u = 0; u < kAggUnroll; ++u) {
+        for (int u = 0; u < kUnroll; ++u) {
           const int rr = __shfl_sync(0xffffffffu, ordered, (i + u) & 31);
           if (i + u < n) {
 #pragma unroll
-            for (int j = 0; j < kAggCpw; ++j) raw[u][j] = *reinterpret_cast<const uint4*>(hidden + (size_t)rr * D + col[j]);
+            for (int j = 0; j < kCpw; ++j) raw[u][j] = *reinterpret_cast<const uint4*>(hidden + (size_t)rr * D + col[j]);
           }
         }
 #pragma unroll
-        for (int u = 0; u < kAggUnroll; ++u)
+        for (int u = 0; u < kUnroll; ++u)
           if (i + u < n) {
 #pragma unroll
-            for (int j = 0; j < kAggCpw; ++j) add_raw<T>(accs[j], raw[u][j]);
+            for (int j = 0; j < kCpw; ++j) add_raw<T>(accs[j], raw[u][j]);
           }
       }
 #pragma unroll
-      for (int j = 0; j < kAggCpw; ++j)
+      for (int j = 0; j < kCpw; ++j)
         if (live[j]) {
 #pragma unroll
           for (int e = 0; e < kVec; ++e) accs[j][e] *= inv_denom;
           Storage<T>::store(dst + col[j], accs[j]);
         }
+    };
+    // (a chunk for every warp of the row: more rows at a time instead; 1024 -> 102 x 4096 24.6 / 23.0, 256 -> 64 x 256 fp32 10.8 / 9.8)
+    if (c1 - c0 <= subs) {
+      if (sub < c1 - c0) add_light(c0 + sub, std::integral_constant<int, 1>(), std::integral_constant<int, 12>());
+    } else {
+      for (int cg = c0 + sub * kAggCpw; cg < c1; cg += subs * kAggCpw)
+        add_light(cg, std::integral_constant<int, kAggCpw>(), std::integral_constant<int, kAggUnroll>());
     }
   }
-
   if (n_long == 0) return;                                       // uniform
 
   // acc += rows [i0, i1) of a long list, kLongUnroll loads in flight
@@ -785,8 +793,8 @@ static int kept_bound(int total_tokens, int total_out, int max_visual, int max_k
 // rule takes 0.93 of the lists' time, and more than 1.03 of it four times, 1.12 at worst.
 //   - blocks: columns down to two chunks, then fewer rows, then single chunks, until the kept rows have seven blocks for five SMs: a
 //     list that most tokens are on is then added by as many SMs as there are.  (Always eight rows and four parts: up to four times
-//     the lists' time, 3399 -> 2 x 4736 70 / 279 us, 619 -> 61 x 3072, 8 clusters, 27 / 50.)  1024 -> 102 x 4096 25.1 / 23.6, with half
-//     of the tokens in one cluster 30.6 / 32.3; fewer and larger blocks are up to 1.5 us faster with even clusters and up to 70 slower.
+//     the lists' time, 3399 -> 2 x 4736 70 / 279 us, 619 -> 61 x 3072, 8 clusters, 27 / 50.)  1024 -> 102 x 4096 26.0 / 23.0, with half
+//     of the tokens in one cluster 34.8 / 35.6; fewer and larger blocks were up to 1.5 us faster with even clusters and up to 70 slower.
 //   - not where all blocks together read more than kScanTokens words: 2048 -> 512 x 4096 36.8 / 35.7, with 60 % in one cluster 56 /
 //     81; 5187 -> 1296 x 2048 114 / 207;
 //   - nor long rows with a quarter kept and more: the one long list that such a call may have keeps a few SMs busy after the others,
