@@ -56,16 +56,14 @@ def test_linear_and_ffn_bf16_long_k_few_tiles_cut_into_k_slices():
     run_ffn(300, 4096, 256, "bf16", seed=4)
 
 
-def test_linear_and_ffn_bf16_shapes_that_take_256_row_tiles():
-    # 1500 rows x 48 column tiles: 256-row CTA tiles finish sooner than 128-row ones here (two rounds over the SMs
-    # instead of four), for the linear layer and for the gate/up pass; the last tile has 220 of 256 rows
-    run_linear(1500, 64, 12288, "bf16", residual=True, seed=5)
-    run_linear(1500, 128, 12288, "bf16", residual=False, seed=6)
+def test_linear_and_ffn_bf16_many_single_cta_tiles_at_a_short_k():
+    # 1500 rows x 12288 columns: four rounds of 128-row tiles over the SMs, for the linear layer and for the gate/up pass; the
+    # last row tile has 92 of 128 rows.  1216 rows: 9.5 row tiles
+    for rows, K in ((1500, 64), (1500, 128), (1216, 64), (1216, 128)):
+        assert pair_width(rows, 12288, K) == 0
+        run_linear(rows, K, 12288, "bf16", residual=K == 64, seed=rows + K)
+    assert pair_width(1500, 12288, 128, gate_up=True) == 0
     run_ffn(1500, 128, 6144, "bf16", seed=7)
-    # 1216 rows x 12288 columns: 256 x 224 tiles (275 of them fill two rounds over 148 SMs better than 240 tiles of
-    # 256 x 256); 224 does not divide 12288, so the last column tile hangs over the edge of the matrix
-    run_linear(1216, 64, 12288, "bf16", residual=True, seed=8)
-    run_linear(1216, 128, 12288, "bf16", residual=False, seed=9)
 
 
 def run_proj(rows, H, dh, seed=0):

@@ -131,10 +131,10 @@ def test_similarity_tiles_cut_into_two_to_four_slices(H, reqs):
     pu.check_step(w, full_attention=False, n_sample_rows=8)
 
 
-def run_attention_only(lens, H, seed=0):
+def run_attention_only(lens, H, seed=0, dh=128):
     """d3tom_attn_varlen on random Q, K, V of a ragged batch against the oracle, every row."""
     dev = torch.device("cuda", 0)
-    dh, total = 128, int(sum(lens))
+    total = int(sum(lens))
     g = torch.Generator().manual_seed(seed)
     q, k, v = (torch.randn(total, H * dh, generator=g).to(torch.bfloat16) for _ in range(3))
     cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
@@ -158,6 +158,11 @@ def test_attention_of_short_requests():
     run_attention_only([49], 3, seed=12)
     run_attention_only([40, 48, 1, 33, 7], 2, seed=13)
     run_attention_only([40, 64, 65, 1, 130], 2, seed=14)
+    # the same where the (head, request) pairs are more than the SMs: whole items instead of the kernel for short calls
+    for dh in (64, 128):
+        run_attention_only([40, 48, 1, 33, 7, 20], 32, seed=15, dh=dh)
+        run_attention_only([40, 49, 1, 33, 7, 20], 32, seed=16, dh=dh)
+        run_attention_only([48, 5], 3, seed=17, dh=dh)
 
 
 def test_attention_with_one_query_tile_per_cta():
@@ -222,7 +227,7 @@ def test_mixed_decider_counts_and_single_decider():
 
 def test_duplicate_rows_and_heavy_slots():
     # many identical visual rows: cosine ties resolve to the lowest kept position and
-    # some kept tokens collect far more than 32 members (the long-list aggregation path)
+    # some kept tokens collect far more than 32 members (a list for whole blocks; one request: found without member lists)
     w = small(post=0, reqs=[dict(V=400, P=8, O=8, n_dec=4, r=0.02)])
     w.k[:400] = w.k[:1]
     w.v[5:400] = w.v[5:6]
@@ -433,7 +438,8 @@ def test_similarity_slices_beside_another_stream_that_holds_the_sms():
 # that does not; sharp rows, so that the running maximum is raised in later key tiles as well.
 @pytest.mark.parametrize("dh,H,lens,n_dec", [(128, 2, [1], 0), (64, 3, [48, 49], 4), (128, 4, [127, 128, 129], 5), (64, 8, [300, 0, 641], 17),
                                              (128, 4, [513], 33), (64, 16, [1150], 20), (128, 4, [900, 385, 260], 0), (64, 148, [128], 1),
-                                             (64, 149, [100], 1), (64, 4, [1024, 700, 90], 40)])
+                                             (64, 149, [100], 1), (64, 4, [1024, 700, 90], 40), (64, 4, [48, 33, 1, 7], 4),
+                                             (128, 2, [48, 33, 1, 7], 4)])
 def test_short_calls_equal_whole_items_bit_for_bit(dh, H, lens, n_dec):
     dev = torch.device("cuda", 0)
     g = torch.Generator().manual_seed(sum(lens) + dh)
@@ -462,5 +468,11 @@ def test_short_calls_equal_whole_items_bit_for_bit(dh, H, lens, n_dec):
         if len(dec[b]):
             rows = slice(int(cu_vis[b]), int(cu_vis[b + 1]))
             assert torch.equal(outs[0][1][rows], outs[1][1][rows])
+            if lens[b] <= 48:                  # both kernels store these row by row: the map against float64 as well
+                req = slice(int(cu[b]), int(cu[b + 1]))
+                qh, kh = (t[req].double().reshape(lens[b], H, dh).transpose(0, 1) for t in (q, k))
+                a = torch.softmax(qh[:, -n_dec:] @ kh.transpose(1, 2) * dh ** -0.5, dim=2)[:, :, : n_vis[b]].sum((0, 1))
+                # terms in (0, 1) with a relative error of about 2^-24 x |score| x a few
+                assert ((outs[0][1][rows].double() - a).abs() <= 1e-4 * a + 1e-6).all()
     assert outs[0][1][-1].item() == -3.0
     ctx.close()
