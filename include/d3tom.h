@@ -118,8 +118,9 @@ int d3tom_set_launch_overlap(int on);
 
 /* Tile shape of the dense layers (d3tom_proj_qkv, d3tom_linear, d3tom_ffn; Sec. 3.2.1 "Q = H W_Q", Algorithm 1
  * FFN_l): -1 (default) lets the library choose shape and width per call (pairs from 2048 rows on, and below where
- * they take less time), 0 keeps single-CTA
- * tiles, 256 forces tiles of 256 x 256 computed by a pair of CTAs (cta_group::2) wherever the number of output columns
+ * they take less time), 0 keeps single-CTA tiles of 128 rows (a switch for comparison: most layers of more than about
+ * five hundred rows are slower so), 256 forces tiles of 256 x 256 computed by a pair of CTAs (cta_group::2) wherever the number of
+ * output columns
  * is a multiple of 256.  Results agree to rounding whatever the choice: a pair tile is one fp32 accumulator over K in
  * ascending order, single-CTA tiles of a launch's last round may sum a long K in up to four slices, added in order.
  * Process-wide; not thread-safe against concurrent launches.

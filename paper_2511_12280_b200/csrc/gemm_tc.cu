@@ -804,8 +804,9 @@ void plan_tail_split(const d3tom_ctx* ctx, GemmParams& p) {
 // What a dense layer costs in tiles of one shape (us): `start` once, per 64 of K `round` for each full round of tiles over the
 // SMs (or the pairs) and `part` + `part_r` x (its share of the SMs) for an incomplete last one, which leaves more of L2 to
 // each, and `more` for every round after the first (an epilogue that nothing hides).  Fitted to 250 layers (64 .. 8000 rows,
-// K 512 .. 12288, 1024 .. 12288 columns) timed in every shape; over them the cheapest shape by these figures is 0.4 % slower
-// than the fastest one.
+// K 512 .. 12288, 1024 .. 12288 columns) timed in every shape, each after a pause, with the operands in L2; over them the cheapest
+// shape by these figures is 0.4 % slower than the fastest one.  pair_tile_width asks them for the shape between 513 and 2047 rows
+// only; below and above its older rules stand, which were fitted back to back under the board's power limit.
 struct TileCost { int width; double start, round, part, part_r, more; };
 constexpr TileCost kOneCost[] = {{256, 7.13, 0.401, 0.283, 0.093, 1.80}, {192, 6.13, 0.284, 0.214, 0.084, 1.78},
                                  {128, 4.96, 0.222, 0.144, 0.067, 0.72}};
@@ -907,9 +908,12 @@ int launch_gemm_pair(d3tom_ctx* ctx, const CUtensorMap& ta, const CUtensorMap& t
 //   - 513 .. 2047 rows, K of 1024 and more: the shape that is cheapest by the costs above.  A rule by rounds that weighed 256-row
 //     single-CTA tiles against pairs took neither the best width nor the better kind (us, rule / now): linear 1216 x 4096 x 4096
 //     48.4 / 33.4, 1408 x 4096 x 4096 52.7 / 39.9, 1216 x 12288 x 4096 109 / 90, 1216 x 4096 x 12288 110 / 90,
-//     1408 x 1024 x 6144 22.6 / 19.3; the 256-row tiles, never the fastest of the 250 layers, are gone.
+//     1408 x 1024 x 6144 22.6 / 19.3; the 256-row tiles, never the fastest of the 250 layers, are gone.  (With pairs switched off, or
+//     where none fits, 128-row tiles serve these layers too: of 200 random ones of 300 .. 3000 rows 185 are as fast as with 256-row
+//     tiles or faster, the others up to 15 % slower, 1133 x 12288 x 6400 141 / 163 us.)
 //   - other layers below 2048 rows: rounds, in us per 64 of K, against rounds of single-CTA tiles and K slices (tail_slices);
-//     1.08 is for power (the pairs move half the operand bytes).
+//     1.08 is for power (the pairs move half the operand bytes).  By the costs above up to 512 rows this choice is 1 % off the
+//     cheapest on average and 32 % at worst (263 x 4096 x 6144), and the next one 2.5 % and 12 %: not timed in alternation.
 //   - from 2048 rows on pairs, in the width that fills the rounds best, except where (single-CTA / pairs, us, rows x K x columns)
 //     all single-CTA tiles together are one round of K slices, which then walk a half to a quarter of K each where a pair walks
 //     all of it: 2100 x 16384 x 128 35 / 78, 2048 x 12288 x 384 30 / 49, 2048 x 8192 x 512 28 / 35; or the costs above are
