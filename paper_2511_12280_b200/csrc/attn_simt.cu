@@ -226,11 +226,14 @@ attn_simt_kernel(AttnArgs a, bool vec) {
 // so the result does not depend on which block that is: no float atomics, reproducible.
 constexpr int kImpThreads = 256;
 constexpr int kImpDecChunk = 128;
-// Up to this many heads and deciders one block per 32 keys (below): attention + importance, partial sums / one pass (us): 256
-// keys x 4 heads, 8 deciders 17.5 / 14.4; but 800 x 4, 16 deciders 54.7 / 55.2, 364 x 4, 32 deciders 31.0 / 35.2, and 1024 keys
-// x 8 heads 90.3 / 93.3, 1024 x 32 47.2 / 53.1, where a block's 128-byte pieces of many rows are the longer way to the same bytes.
-constexpr int kImpBlockDeciders = 8;
-constexpr int kImpBlockHeads = 4;
+// Up to this many heads and deciders one block per 32 keys (below).  One request, attention + importance, partial sums / one pass
+// (us), by deciders at 1024 keys x 4 heads x 64 fp32: 4 64.3 / 61.0, 8 65.0 / 61.4, 16 64.4 / 62.5, 32 64.9 / 64.4, 64 67.6 / 68.9;
+// 256 keys x 4: 8 19.5 / 15.8, 16 18.7 / 16.9, 64 19.7 / 22.0; 12000 keys x 4 bf16: 8 232 / 227, 16 232 / 229, 64 284 / 285;
+// 256 keys x 8: 8 26.8 / 22.5, 16 25.0 / 23.7, 64 27.2 / 29.0.  With many heads (1024 keys x 32, 32 deciders 47.2 / 53.1) a block's
+// 128-byte pieces of many rows are the longer way to the same bytes.
+constexpr int kImpBlockDeciders = 16;
+constexpr int kImpBlockHeads = 8;
+constexpr int kImpBlockLoads = 8;      // scores in flight per lane
 
 __global__ void __launch_bounds__(kImpThreads)
 importance_finish_kernel(const float* __restrict__ score, const float2* __restrict__ lse,
@@ -303,16 +306,16 @@ importance_finish_block_kernel(const float* __restrict__ score, const float2* __
   const int jj = j < Vb ? j : Vb - 1;                           // lanes past the end read a valid column, write nothing
   float acc = 0.f;
   // (the host's count chose this kernel, the device's list is what is summed: a captured call may be replayed with a longer one)
-  for (int d = d0; d < d1; d += kImpBlockDeciders) {
-    const int nd = min(kImpBlockDeciders, d1 - d);
+  for (int d = d0; d < d1; d += kImpBlockLoads) {
+    const int nd = min(kImpBlockLoads, d1 - d);
     const float2 ml = lane < nd ? lse[(size_t)h * max_deciders + d + lane] : make_float2(0.f, 1.f);
     const float neg_m = -ml.x, inv_l = 1.0f / ml.y;
     const float* col = score + ((size_t)h * max_deciders + d) * vis_stride + jj;
-    float x[kImpBlockDeciders];                                 // (all loads in flight; the sum runs in ascending order)
+    float x[kImpBlockLoads];                                    // (all loads in flight; the sum runs in ascending order)
 #pragma unroll
-    for (int u = 0; u < kImpBlockDeciders; ++u) if (u < nd) x[u] = col[(size_t)u * vis_stride];
+    for (int u = 0; u < kImpBlockLoads; ++u) if (u < nd) x[u] = col[(size_t)u * vis_stride];
 #pragma unroll
-    for (int u = 0; u < kImpBlockDeciders; ++u)
+    for (int u = 0; u < kImpBlockLoads; ++u)
       if (u < nd)
         acc = fmaf(exp2f(fmaf(x[u], scale_log2, __shfl_sync(0xffffffffu, neg_m, u))), __shfl_sync(0xffffffffu, inv_l, u), acc);
   }

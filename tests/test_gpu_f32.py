@@ -290,10 +290,10 @@ def test_similarity_fp32_gives_the_same_bits_by_rows_and_by_tiles(V, k, D):
     assert torch.equal(got[0][0][pruned].long(), got[0][1][pruned].argmax(dim=1))
 
 
-# one block per 32 keys with a warp per head (up to four heads and eight deciders), and the kernel with partial sums beyond:
+# one block per 32 keys with a warp per head (up to eight heads and sixteen deciders), and the kernel with partial sums beyond:
 # deciders below, at and above either limit, ragged numbers of keys
-@pytest.mark.parametrize("H", [1, 4, 5])
-@pytest.mark.parametrize("V,n_dec", [(1, 1), (31, 4), (33, 4), (300, 3), (95, 5), (31, 16), (32, 17), (33, 32), (300, 33), (95, 70)])
+@pytest.mark.parametrize("H", [1, 4, 5, 8, 9])
+@pytest.mark.parametrize("V,n_dec", [(1, 1), (31, 4), (33, 4), (300, 3), (95, 5), (64, 8), (33, 9), (31, 16), (32, 17), (33, 32), (300, 33), (95, 70)])
 def test_importance_of_few_heads(H, V, n_dec):
     dev, dh = torch.device("cuda", 0), 32
     g = torch.Generator().manual_seed(V + H)
