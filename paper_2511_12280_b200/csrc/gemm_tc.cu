@@ -907,8 +907,8 @@ int launch_gemm_pair(d3tom_ctx* ctx, const CUtensorMap& ta, const CUtensorMap& t
 // matrices), or 0 for single-CTA tiles.
 //   - 513 .. 2047 rows, K of 1024 and more: the shape that is cheapest by the costs above.  A rule by rounds that weighed 256-row
 //     single-CTA tiles against pairs took neither the best width nor the better kind (us, rule / now): linear 1216 x 4096 x 4096
-//     48.4 / 33.4, 1408 x 4096 x 4096 52.7 / 39.9, 1216 x 12288 x 4096 109 / 90, 1216 x 4096 x 12288 110 / 90,
-//     1408 x 1024 x 6144 22.6 / 19.3; the 256-row tiles, never the fastest of the 250 layers, are gone.  (With pairs switched off, or
+//     48.9 / 33.1, 1408 x 4096 x 4096 53.4 / 40.1, 1216 x 12288 x 4096 119 / 97, 1216 x 4096 x 12288 107 / 92,
+//     1408 x 1024 x 6144 23.2 / 19.2; the 256-row tiles, never the fastest of the 250 layers, are gone.  (With pairs switched off, or
 //     where none fits, 128-row tiles serve these layers too: of 200 random ones of 300 .. 3000 rows 185 are as fast as with 256-row
 //     tiles or faster, the others up to 15 % slower, 1133 x 12288 x 6400 141 / 163 us.)
 //   - other layers below 2048 rows: rounds, in us per 64 of K, against rounds of single-CTA tiles and K slices (tail_slices);
